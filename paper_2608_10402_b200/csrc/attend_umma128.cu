@@ -1,22 +1,32 @@
-// Append-prefill attention for resume rows on the 5th-generation tensor cores, 128-key tiles.
+// Append-prefill attention for resume rows on the 5th-generation tensor cores, 128-key tiles, head sizes 64 and 128.
 //
-// Same work item and results as attend_umma.cu (256 packed rows r = q_index * G + g as two 128-row tiles A and B
-// against keys [kv_begin, kv_end) of one KV head; paper Section 4: the appended observation tokens attend to the
-// whole preserved KV state).  What differs is the arrangement around the tensor pipe:
-//   * key tiles of 128: S_t = Q_t . K_j^T is 8 MMAs of 128x128x16 and O_t += P_t . V_j another 8, so there are a
-//     third fewer MMA instructions per key than with 64-key tiles (QK at N = 64 only half fills an instruction)
-//     and half as many hand-offs between the softmax warps and the MMA warp;
-//   * Q sits in shared memory (both operands of QK from shared memory run at the rate of the TMEM-A form once
-//     N = 128), which frees TMEM for S tiles of 128 columns: S_A S_B 2 x 128 (P_t, packed bf16, overwrites the
-//     first 64 columns of S_t), O_A O_B 2 x 128;
-//   * K tiles and V tiles are separate 32-KB units of one ring (K0 V0 K1 V1 ...), 5 units beside the 64 KB of Q,
-//     each unit filled by one bulk copy per page (the K block or the V block of a (page, head) is contiguous in the
-//     pool and already in operand layout), K by warp 8 and V by warp 10;
-//   * a share of the exponentials is computed on the FMA pipe (range reduction and a cubic), because the unit that
-//     serves ex2 needs as long for a tile as the tensor pipe does and the two softmax warpgroups would otherwise
-//     queue for it.
-// The two row tiles ping-pong: while warpgroup A works on S_A(j) the tensor pipe runs PV_B(j-1) and QK_B(j).
-// Every wait is bounded; a wait that runs out sets TIDE_ERR_DEVICE_TIMEOUT and the CTA drains and exits.
+// Work item: 256 packed rows r = q_index * G + g (two 128-row tiles A and B) against keys [kv_begin, kv_end) of one KV
+// head (paper Section 4: the appended observation tokens attend to the whole preserved KV state).
+//
+// A thread block is PERSISTENT: one per SM, twelve warps, every role walking the same sequence of items.  The grid has
+// one block per item; a running block takes over the index of a block that has not started yet
+// (clusterlaunchcontrol.try_cancel), so items are handed out one at a time, in order, to whichever SM is free, with no
+// counter in memory.  Warp 11 asks for the next item while the current one runs, works out its geometry once and
+// publishes it; the K and V producers then run ahead into it, its queries are copied as soon as the last QK of the
+// current item has retired, and its first QK is issued behind the current item's last PV.  Of an item's fixed cost only
+// the epilogue and the fill of the softmax pipeline remain (one block per item spent 14 us outside the key loop - 2.3
+// launch and TMEM set-up, 4.6 staging Q, 0.8 first QK, 0.8 last PV, 4.3 epilogue, 1.1 between blocks - against 1.6 us per
+// 128-key tile, i.e. 44 % of a batch of prompts of 200 to 4000 tokens and 21 % of the long-horizon batch).
+//   * S_t = Q_t . K_j^T is D/16 MMAs of 128x128x16, O_t += P_t . V_j eight of 128xDx16;
+//   * Q sits in shared memory (both operands of QK from shared memory run at the rate of the TMEM-A form once N = 128);
+//     K tiles and V tiles are separate units of one ring (K0 V0 K1 V1 ...), each filled by one bulk copy per page (the K
+//     block or the V block of a (page, head) is contiguous in the pool and already in operand layout), K by warp 8 and V
+//     by warp 10; warp 9 issues the MMAs;
+//   * D = 128: TMEM holds S_A S_B 2 x 128 columns (P_t, packed bf16, overwrites the first 64 of S_t) and O_A O_B 2 x 128.
+//     The two row tiles ping-pong: while warpgroup A works on S_A(j) the tensor pipe runs PV_B(j-1) and QK_B(j);
+//   * D = 64: O needs half the columns, so P_t gets columns of its own and QK_t(j+1) is issued as soon as the softmax
+//     warps have S_t(j) in registers: they always find their next S tile waiting, and the kernel is bound by the
+//     exponentials (a 64-wide head has half the MMA work per exponential);
+//   * every exponential is an ex2.  A quarter of them as a cubic on the FMA pipe shortens an isolated tile (the ex2 unit
+//     needs as long for a D = 128 tile as the tensor pipe does) but costs six times the instructions, and what bounds a
+//     long batch is the board's 1 kW: mixed text batch 7.06 ms with the share, 7.00 without, multimodal batch 18.2 and
+//     18.0, prompts 0.722 and 0.702 (0.3 s and more into a run, SM clock 1.5 to 1.7 GHz).
+// Every wait is bounded; a wait that runs out sets TIDE_ERR_DEVICE_TIMEOUT and the block drains and exits.
 #include <climits>
 #include <type_traits>
 
@@ -26,31 +36,30 @@ namespace tide {
 
 namespace umma128 {
 
-constexpr int D = 128;
 constexpr int kTileKeys = 128;
-constexpr int kThreads = 384;   // 3 warpgroups: softmax A, softmax B, {K producer 8, MMA issuer 9, V producer 10, idle 11}
-constexpr int kNumUnits = 5;                        // ring of operand tiles in the order K0 V0 K1 V1 ...
-constexpr int kGroupBytes = (D / 64) * 1024;        // one 8-key group of a K (or V) tile: two 1-KB atoms
-constexpr int kUnitBytes = (kTileKeys / 8) * kGroupBytes;   // one K or V tile: 32 KB
-constexpr int kQSlabBytes = 128 * 128;              // 128 rows x 128 bytes
-constexpr int kQTileBytes = 2 * kQSlabBytes;        // the queries of one 128-row tile
-constexpr int kQBytes = 2 * kQTileBytes;
-constexpr int kSmemBytes = kQBytes + kNumUnits * kUnitBytes;   // 224 KB; with the static part (below 3 KB) the whole 227 KB of an SM
+constexpr int kThreads = 384;   // 3 warpgroups: softmax A, softmax B, {K producer 8, MMA issuer 9, V producer 10, scheduler and Q loader 11}
+constexpr int kItemSlots = 4;   // published items
 constexpr float kRescaleThreshold = 8.0f;           // log2 units
-constexpr uint32_t kColS = 0, kColO = 256;          // S_t at kColS + t*128 (P_t over its first 64 columns), O_t at kColO + t*128
-#ifndef TIDE_UMMA128_EMU_PAIRS
-#define TIDE_UMMA128_EMU_PAIRS 1                    // of every 4 pairs of exponentials, how many take the polynomial
-#endif
-constexpr int kEmuPairs = TIDE_UMMA128_EMU_PAIRS;
-#ifndef TIDE_UMMA128_P_PARTS
-#define TIDE_UMMA128_P_PARTS 2                      // P_t is handed to the MMA warp in this many parts (2 or 4)
-#endif
-constexpr int kPParts = TIDE_UMMA128_P_PARTS;
+constexpr int kPParts = 2;      // P_t is handed to the MMA warp in two halves
 
-// instruction descriptor: fp32 accumulate, bf16 A and B, M = 128, N = 128; bit 16 = B is MN-major
-constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24) | ((128u >> 3) << 17);
-constexpr uint32_t kIdescQK = kIdescBase;
-constexpr uint32_t kIdescPV = kIdescBase | (1u << 16);
+template <int D>
+struct Cfg {
+  static constexpr bool kSepP = D == 64;                       // P_t has TMEM columns of its own
+  static constexpr int kNumUnits = D == 128 ? 5 : 10;          // ring of operand tiles in the order K0 V0 K1 V1 ...
+  static constexpr int kGroupBytes = (D / 64) * 1024;          // one 8-key group of a K (or V) tile: D/64 1-KB atoms
+  static constexpr int kUnitBytes = (kTileKeys / 8) * kGroupBytes;   // one K or V tile
+  static constexpr int kQSlabBytes = 128 * 128;                // 128 rows x 128 bytes
+  static constexpr int kQTileBytes = (D / 64) * kQSlabBytes;   // the queries of one 128-row tile
+  static constexpr int kQBytes = 2 * kQTileBytes;
+  static constexpr int kSmemBytes = kQBytes + kNumUnits * kUnitBytes;   // D = 128: 224 KB; with the static part the whole 227 KB of an SM
+  static constexpr uint32_t kColS = 0;                                  // S_t at kColS + t*128
+  static constexpr uint32_t kColP = kSepP ? 256 : 0, kColPStep = kSepP ? 64 : 128;
+  static constexpr uint32_t kColO = kSepP ? 384 : 256;                  // O_t at kColO + t*D
+  // instruction descriptors: fp32 accumulate, bf16 A and B, M = 128; N = 128 keys (QK) or D columns (PV); bit 16 = B is MN-major
+  static constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
+  static constexpr uint32_t kIdescQK = kIdescBase | ((128u >> 3) << 17);
+  static constexpr uint32_t kIdescPV = kIdescBase | (((uint32_t)D >> 3) << 17) | (1u << 16);
+};
 
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
   uint64_t d = 0;
@@ -163,86 +172,97 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// Two base-2 exponentials on the FMA and integer pipes: n = round(x) by the magic-number addition (n lands in the
-// low mantissa bits), a cubic for 2^r on r = x - n in [-0.5, 0.5] (relative error 7.5e-5, far below the bf16
-// rounding of P), and n added to the exponent field.  Arguments below -126 are clamped (result 2^-126, not 0).
-__device__ __forceinline__ void poly_exp2_pair(float x0, float x1, float& e0, float& e1) {
-  const uint64_t xc = pack2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
-  const uint64_t t = add2(xc, pack2(12582912.f, 12582912.f));
-  const uint64_t n = add2(t, pack2(-12582912.f, -12582912.f));
-  const uint64_t r = fma2(n, pack2(-1.f, -1.f), xc);
-  uint64_t p = fma2(pack2(0.05517132f, 0.05517132f), r, pack2(0.24261054f, 0.24261054f));
-  p = fma2(p, r, pack2(0.69326097f, 0.69326097f));
-  p = fma2(p, r, pack2(0.99992812f, 0.99992812f));
-  float p0, p1, t0, t1;
-  unpack2(p, p0, p1);
-  unpack2(t, t0, t1);
-  e0 = __int_as_float((__float_as_int(t0) << 23) + __float_as_int(p0));
-  e1 = __int_as_float((__float_as_int(t1) << 23) + __float_as_int(p1));
+// Ask the hardware for the index of a block of this launch that has not started: the 16-byte answer lands at `resp`
+// and is counted on `bar`.  After an answer "none left" nothing more may be asked.
+__device__ __forceinline__ void next_block_ask(uint32_t resp, uint32_t bar) {
+  mbar_expect_tx(bar, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(resp), "r"(bar) : "memory");
+}
+__device__ __forceinline__ int next_block_answer(uint32_t resp) {        // -1: none left
+  int x;
+  asm volatile(
+      "{\n\t.reg .b128 r;\n\t.reg .pred p;\n\t"
+      "ld.shared.b128 r, [%1];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "mov.b32 %0, -1;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}"
+      : "=r"(x) : "r"(resp) : "memory");
+  return x;
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {     // zero-fills when not valid
+  const int n = valid ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+// 32 bytes per lane, in one instruction where the address allows it: a lane writes whole sectors of its own row (the
+// rows of a warp are apart)
+__device__ __forceinline__ void st_32bytes(void* p, const uint32_t (&v)[8], bool wide) {
+  if (wide)
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]),
+                 "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+  else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+  }
 }
 
-struct Bars {
-  uint64_t kv_full[kNumUnits];
-  uint64_t kv_empty[kNumUnits];
-  uint64_t q_full;
-  uint64_t s_full[2];   // S_t(j) is in TMEM (and every earlier MMA, PV_t(j-1) included, has retired)
-  uint64_t p_part[2][kPParts];   // part q of P_t(j) (keys [q, q+1) * 128 / kPParts) is in TMEM
-  uint64_t o_full[2];   // the last PV_t has retired
-  uint64_t mma_done;    // every MMA of the item has retired
+// One work item as every role sees it.
+struct __align__(16) Item {
+  int run;             // 0: there is no further item
+  int table_off, kvh, kv_begin, kv_end, n_tiles;
+  int tiles[2];        // per 128-row tile: number of 128-key tiles to process (0: the tile has no rows or sees no key),
+  int end[2];          // one past the last key any of its rows sees,
+  int min_limit[2];    // and the first key that its first row does not see
+  int row0, R;         // first packed row; packed rows of the (row, kv head)
+  int p, causal;
+  int q_row0;          // (token, head) row of the segment's first token in q (and out): q_off * Hq
+  int dst_row0;        // (token, head) row of its first token in out, or in the partials of this split
+  int direct;          // 1: results go to out / lse; 0: to the partials
+  int drop;            // test hook: K tile 0 never arrives
 };
 
+template <int NU>
+struct Bars {
+  uint64_t kv_full[NU];
+  uint64_t kv_empty[NU];
+  uint64_t q_full[2];   // Q_t of the item is in shared memory
+  uint64_t q_empty[2];  // the item's last QK_t has retired
+  uint64_t s_full[2];   // S_t(j) is in TMEM (D = 128: and every earlier MMA of the row tile, PV_t(j-1) included, has retired)
+  uint64_t s_free[2];   // D = 64: S_t(j) is in registers
+  uint64_t p_part[2][kPParts];   // part q of P_t(j) (keys [q, q+1) * 128 / kPParts) is in TMEM
+  uint64_t o_full[2];   // D = 128: the item's last PV_t has retired; D = 64: PV_t(j) has
+  uint64_t item_full[kItemSlots];
+  uint64_t item_empty[kItemSlots];
+  uint64_t k_issued;    // the copies of the item's last K tile are on their way
+  uint64_t next;        // the answer of next_block_ask has landed
+  uint64_t mma_done;    // every MMA of the block has retired
+};
+constexpr int kItemReaders = 3 + 8;   // K producer, V producer, MMA warp, eight softmax warps: one arrival each
+
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const AttendParams P) {
+  using C = Cfg<D>;
   // The swizzled operand layouts need their tiles on 1-KB boundaries; there is no room for alignment slack, so the
   // dynamic part is declared with that alignment (and checked below).
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) Bars bars;
+  __shared__ __align__(8) Bars<C::kNumUnits> bars;
+  __shared__ Item items[kItemSlots];
+  __shared__ __align__(16) uint4 s_next;
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
 
   const uint32_t smem_q = smem_u32(smem_raw);                      // Q tiles A and B, then the operand ring
-  const uint32_t smem_ring = smem_q + kQBytes;
-  uint8_t* q_gen = smem_raw;
-  uint8_t* ring_gen = q_gen + kQBytes;
+  const uint32_t smem_ring = smem_q + C::kQBytes;
+  uint8_t* ring_gen = smem_raw + C::kQBytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Geom& g = P.g;
-
-  // ---- which item ----
-  const int item = blockIdx.x;
-  int n_segs = P.n_segs;
-  if (P.dyn != nullptr) {                      // fixed grid: the batch's counts live in device memory
-    if (item >= P.dyn[0]) return;
-    n_segs = P.dyn[1];
-  }
-  const int si = find_segment(n_segs, item, [&](int i) { return P.segs[i].item_base; });
-  const Segment seg = P.segs[si];
-  int local = item - seg.item_base;
-  const int m_tile = local % seg.n_mtiles;
-  local /= seg.n_mtiles;
-  const int split = local % seg.n_splits;
-  const int kvh = local / seg.n_splits;
-  const int R = seg.n * g.G;
-  const int item_row0 = m_tile * kUmmaTileRows * 2;
-  const int kv_begin = seg.origin + split * seg.chunk;
-  const bool direct = seg.n_splits == 1 && seg.partial == 0;
-  // per 128-row tile: rows present, last key any of its rows sees, number of 128-key tiles to process
-  int t_rows[2], t_end[2], t_tiles[2], t_min_limit[2];
-#pragma unroll
-  for (int t = 0; t < 2; ++t) {
-    const int r0 = item_row0 + t * 128;
-    t_rows[t] = max(0, min(128, R - r0));
-    if (t_rows[t] > 0) {
-      t_end[t] = min(kv_begin + seg.chunk, seg.p + ((r0 + t_rows[t] - 1) / g.G) * seg.causal + 1);
-      t_min_limit[t] = min(t_end[t], seg.p + (r0 / g.G) * seg.causal + 1);
-      t_tiles[t] = t_end[t] > kv_begin ? (t_end[t] - kv_begin + kTileKeys - 1) / kTileKeys : 0;
-    } else {
-      t_end[t] = kv_begin; t_min_limit[t] = kv_begin; t_tiles[t] = 0;
-    }
-  }
-  const int n_tiles = max(t_tiles[0], t_tiles[1]);
-  const int kv_end = max(t_end[0], t_end[1]);
+  const int n_items = P.dyn ? P.dyn[0] : P.n_items;                // fixed grid: the batch's counts live in device memory
+  if ((int)blockIdx.x >= n_items) return;
 
   // The status word is set when a bounded wait runs out and stays set until tide_status clears it; while it is set
-  // no CTA starts work, so outputs are undefined from the time-out until the caller has read the status.
+  // no block starts work, so outputs are undefined from the time-out until the caller has read the status.
   __shared__ int s_skip;
   if (threadIdx.x == 0) {
     s_skip = *reinterpret_cast<volatile int*>(P.status);
@@ -250,22 +270,24 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
       atomicExch(P.status, (int)TIDE_ERR_CUDA);
       s_skip = 1;
     }
-  }
-  __syncthreads();
-  if (s_skip != 0) return;
-
-  if (threadIdx.x == 0) {
     s_abort = 0;
-    for (int i = 0; i < kNumUnits; ++i) { mbar_init(smem_u32(&bars.kv_full[i]), 1); mbar_init(smem_u32(&bars.kv_empty[i]), 1); }
-    mbar_init(smem_u32(&bars.q_full), 256);
+    for (int i = 0; i < C::kNumUnits; ++i) { mbar_init(smem_u32(&bars.kv_full[i]), 1); mbar_init(smem_u32(&bars.kv_empty[i]), 1); }
     for (int t = 0; t < 2; ++t) {
+      mbar_init(smem_u32(&bars.q_full[t]), 32);
+      mbar_init(smem_u32(&bars.q_empty[t]), 1);
       mbar_init(smem_u32(&bars.s_full[t]), 1);
+      mbar_init(smem_u32(&bars.s_free[t]), 128);
       for (int q = 0; q < kPParts; ++q) mbar_init(smem_u32(&bars.p_part[t][q]), 128);
       mbar_init(smem_u32(&bars.o_full[t]), 1);
     }
+    for (int i = 0; i < kItemSlots; ++i) { mbar_init(smem_u32(&bars.item_full[i]), 1); mbar_init(smem_u32(&bars.item_empty[i]), kItemReaders); }
+    mbar_init(smem_u32(&bars.k_issued), 1);
+    mbar_init(smem_u32(&bars.next), 1);
     mbar_init(smem_u32(&bars.mma_done), 1);
     mbar_fence_init();
   }
+  __syncthreads();
+  if (s_skip != 0) return;
   if (warp == 9) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -275,6 +297,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
   tc_fence_after();
   const uint32_t tmem = s_tmem_base;
   volatile int* abort_flag = &s_abort;
+  auto wait = [&](uint64_t& bar, int parity) -> bool {
+    return mbar_wait(smem_u32(&bar), (uint32_t)parity, abort_flag, P.status, P.wait_limit_ns);
+  };
+  // the same where a warp branches on the outcome: its lanes stay together
+  auto wait_all = [&](uint64_t& bar, int parity) -> bool { return __all_sync(0xffffffffu, wait(bar, parity)) != 0; };
 
   // register budget: the data-movement warpgroup gives registers to the two softmax warpgroups.  setmaxnreg
   // moves registers inside the CTA's own launch allocation (384 x 168), so the new counts must not add up to
@@ -283,135 +310,286 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     if (warp == 8 || warp == 10) {
       // ================= producers: warp 8 the K tiles (units 0, 2, 4, ...), warp 10 the V tiles (1, 3, 5, ...) =================
-      if (n_tiles > 0) {
-        const int is_v = warp == 10 ? 1 : 0;
-        const int pages_per_tile = kTileKeys / g.S;            // 8 or 4: one copy each
+      const int is_v = warp == 10 ? 1 : 0;
+      const int pages_per_tile = kTileKeys / g.S;              // 8 or 4: one copy each
+      const int tiles_per_group = 32 / pages_per_tile;
+      int slot = is_v, use = 0;                                // this warp's next unit of the ring
+      int issued = 0;                                          // tiles this warp has issued its copies of
+      bool ok = true;
+      for (int it = 0; ok; ++it) {
+        if (!wait_all(bars.item_full[it % kItemSlots], (it / kItemSlots) & 1)) break;
+        const Item& w = items[it % kItemSlots];
+        if (!w.run) break;
+        const int n_tiles = w.n_tiles, kv_begin = w.kv_begin, kv_end = w.kv_end, drop = w.drop;
+        const int32_t* trow = P.table + w.table_off;
+        const uint8_t* head_base = P.pool + (long long)w.kvh * g.head_bytes + is_v * g.kblock_bytes;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.item_empty[it % kItemSlots]));
         // page ids are fetched 32 logical pages at a time, one per lane, a whole group ahead of their use,
         // so that no bulk copy waits for a dependent page-table load
-        const int tiles_per_group = 32 / pages_per_tile;
         const int lp0 = kv_begin / g.S;
-        const int32_t* trow = P.table + seg.table_off;
         auto load_ids = [&](int grp) -> int {
           const int lp = lp0 + grp * 32 + lane;
           return lp < g.max_pages_per_task ? trow[lp] : 0;
         };
         int ids_cur = load_ids(0), ids_nxt = load_ids(1), cur_grp = 0;
-        int issued = 0;                                        // tiles this warp has issued its copies of
         for (int j = 0; j < n_tiles; ++j) {
-          const int u = 2 * j + is_v, slot = u % kNumUnits, use = u / kNumUnits;
           const int grp = j / tiles_per_group;
           if (grp != cur_grp) { ids_cur = ids_nxt; ids_nxt = load_ids(grp + 1); cur_grp = grp; }
           // a wait that gave up means the ring can no longer be trusted: issue nothing more
-          if (use > 0 && !mbar_wait(smem_u32(&bars.kv_empty[slot]), (use - 1) & 1, abort_flag, P.status, P.wait_limit_ns)) break;
-          issued = j + 1;
-          if (P.debug_drop_first_stage != 0 && item == 0 && j == 0 && is_v == 0) continue;   // test hook: K tile 0 never arrives
+          if (use > 0 && !wait_all(bars.kv_empty[slot], (use - 1) & 1)) { ok = false; break; }
+          ++issued;
           const int key0 = kv_begin + j * kTileKeys;
           const int npages = min(pages_per_tile, (kv_end - key0 + g.S - 1) / g.S);
           const uint32_t bar = smem_u32(&bars.kv_full[slot]);
           const long long page = __shfl_sync(0xffffffffu, ids_cur, ((j % tiles_per_group) * pages_per_tile + lane) & 31);
-          if (lane == 0) mbar_expect_tx(bar, (uint32_t)(npages * g.kblock_bytes));
-          __syncwarp();
-          if (lane < npages)
-            bulk_g2s(smem_ring + slot * kUnitBytes + lane * g.kblock_bytes,
-                     P.pool + page * g.page_bytes + (long long)kvh * g.head_bytes + is_v * g.kblock_bytes, (uint32_t)g.kblock_bytes, bar);
-        }
-        if (*abort_flag && lane == 0) {
-          // a wait gave up somewhere: this warp does not leave while copies it issued into the CTA's shared memory
-          // can still be landing.  Those are among its last kNumUnits tiles; each wait is bounded like every other.
-          for (int j = max(0, issued - kNumUnits); j < issued; ++j) {
-            const int u = 2 * j + is_v;
-            const uint32_t bar = smem_u32(&bars.kv_full[u % kNumUnits]);
-            const long long t0 = global_ns();
-            while (!mbar_try(bar, (u / kNumUnits) & 1) && global_ns() - t0 < P.wait_limit_ns) {}
+          if (!(drop != 0 && j == 0 && is_v == 0)) {                           // test hook: K tile 0 never arrives
+            if (lane == 0) mbar_expect_tx(bar, (uint32_t)(npages * g.kblock_bytes));
+            __syncwarp();
+            if (lane < npages)
+              bulk_g2s(smem_ring + slot * C::kUnitBytes + lane * g.kblock_bytes, head_base + page * g.page_bytes, (uint32_t)g.kblock_bytes, bar);
           }
+          slot += 2;
+          if (slot >= C::kNumUnits) { slot -= C::kNumUnits; ++use; }
+        }
+        if (is_v == 0 && lane == 0) mbar_arrive(smem_u32(&bars.k_issued));
+      }
+      if (*abort_flag && lane == 0) {
+        // a wait gave up somewhere: this warp does not leave while copies it issued into the CTA's shared memory
+        // can still be landing.  Those are among its last kNumUnits tiles; each wait is bounded like every other.
+        for (int j = max(0, issued - C::kNumUnits); j < issued; ++j) {
+          const int u = 2 * j + is_v;
+          const uint32_t bar = smem_u32(&bars.kv_full[u % C::kNumUnits]);
+          const long long t0 = global_ns();
+          while (!mbar_try(bar, (u / C::kNumUnits) & 1) && global_ns() - t0 < P.wait_limit_ns) {}
         }
       }
     } else if (warp == 9) {
       // ================= MMA issuer (whole warp converged, one elected lane issues) =================
-      if (n_tiles > 0) {
-        mbar_wait(smem_u32(&bars.q_full), 0, abort_flag, P.status, P.wait_limit_ns);
-        tc_fence_after();
-        // Descriptors are built once; moving an operand's start address is one 32-bit add on the low word (the
-        // address field counts 16-byte units and cannot overflow its 14 bits inside this CTA's shared memory).
-        const uint64_t kd0 = make_desc(smem_ring, 16, kGroupBytes);        // a K tile in unit 0 (K-major, 8-key groups 2 KB apart)
-        const uint64_t vd0 = make_desc(smem_ring, 1024, kGroupBytes);      // a V tile in unit 0 (MN-major: slabs 1 KB, groups 2 KB apart)
-        const uint64_t qd0 = make_desc(smem_q, 16, 1024);                  // a Q tile (K-major, 8-row groups 1 KB apart)
-        const uint32_t kd_lo = (uint32_t)kd0, kd_hi = (uint32_t)(kd0 >> 32), vd_lo = (uint32_t)vd0, vd_hi = (uint32_t)(vd0 >> 32);
-        const uint32_t qd_lo = (uint32_t)qd0, qd_hi = (uint32_t)(qd0 >> 32);
-        constexpr uint32_t kUnitStep = kUnitBytes >> 4;
-        auto issue_qk = [&](int t, int slot) {
-          const uint32_t k_lo = kd_lo + slot * kUnitStep;
-          const uint32_t q_lo = qd_lo + t * (kQTileBytes >> 4);
+      // Descriptors are built once; moving an operand's start address is one 32-bit add on the low word (the
+      // address field counts 16-byte units and cannot overflow its 14 bits inside this CTA's shared memory).
+      const uint64_t kd0 = make_desc(smem_ring, 16, C::kGroupBytes);        // a K tile in unit 0 (K-major, 8-key groups apart)
+      const uint64_t vd0 = make_desc(smem_ring, 1024, C::kGroupBytes);      // a V tile in unit 0 (MN-major: slabs 1 KB apart)
+      const uint64_t qd0 = make_desc(smem_q, 16, 1024);                     // a Q tile (K-major, 8-row groups 1 KB apart)
+      const uint32_t kd_lo = (uint32_t)kd0, kd_hi = (uint32_t)(kd0 >> 32), vd_lo = (uint32_t)vd0, vd_hi = (uint32_t)(vd0 >> 32);
+      const uint32_t qd_lo = (uint32_t)qd0, qd_hi = (uint32_t)(qd0 >> 32);
+      constexpr uint32_t kUnitStep = C::kUnitBytes >> 4;
+      int n_qk[2] = {0, 0}, n_pv[2] = {0, 0}, n_q[2] = {0, 0};    // QKs, PVs and queries of each row tile so far (their barriers' phases)
+      auto issue_qk = [&](int t, int slot, bool last) {
+        if (C::kSepP && n_qk[t] > 0) { wait(bars.s_free[t], (n_qk[t] - 1) & 1); tc_fence_after(); }
+        const uint32_t k_lo = kd_lo + slot * kUnitStep;
+        const uint32_t q_lo = qd_lo + t * (C::kQTileBytes >> 4);
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks)
-            mma_ss(tmem + kColS + t * 128, desc64(q_lo + (((ks >> 2) * kQSlabBytes + (ks & 3) * 32) >> 4), qd_hi),
-                   desc64(k_lo + (((ks >> 2) * 1024 + (ks & 3) * 32) >> 4), kd_hi), kIdescQK, ks > 0);
-          mma_commit(smem_u32(&bars.s_full[t]));
-        };
-        auto issue_pv = [&](int t, int j, int slot, int part) {      // the PV MMAs of part `part` of the keys
-          const uint32_t v_lo = vd_lo + slot * kUnitStep;
+        for (int ks = 0; ks < D / 16; ++ks)
+          mma_ss(tmem + C::kColS + t * 128, desc64(q_lo + (((ks >> 2) * C::kQSlabBytes + (ks & 3) * 32) >> 4), qd_hi),
+                 desc64(k_lo + (((ks >> 2) * 1024 + (ks & 3) * 32) >> 4), kd_hi), C::kIdescQK, ks > 0);
+        mma_commit(smem_u32(&bars.s_full[t]));
+        if (last) mma_commit(smem_u32(&bars.q_empty[t]));
+        ++n_qk[t];
+      };
+      auto issue_pv = [&](int t, int j, int slot) {
+        const uint32_t v_lo = vd_lo + slot * kUnitStep;
+#pragma unroll
+        for (int q = 0; q < kPParts; ++q) {
+          wait(bars.p_part[t][q], n_pv[t] & 1);
+          tc_fence_after();
 #pragma unroll
           for (int k4 = 0; k4 < kTileKeys / 16 / kPParts; ++k4) {
-            const int ks = part * (kTileKeys / 16 / kPParts) + k4;
-            mma_ts(tmem + kColO + t * 128, tmem + kColS + t * 128 + ks * 8, desc64(v_lo + ((ks * 2 * kGroupBytes) >> 4), vd_hi), kIdescPV,
-                   (j > 0 || ks > 0) ? 1u : 0u);
+            const int ks = q * (kTileKeys / 16 / kPParts) + k4;
+            mma_ts(tmem + C::kColO + t * D, tmem + C::kColP + t * C::kColPStep + ks * 8, desc64(v_lo + ((ks * 2 * C::kGroupBytes) >> 4), vd_hi),
+                   C::kIdescPV, (j > 0 || ks > 0) ? 1u : 0u);
           }
-        };
-        // operand u of the sequence K0 V0 K1 V1 ... sits in unit u % kNumUnits on its (u / kNumUnits)-th use
-        auto wait_full = [&](int slot, int use) {
-          mbar_wait(smem_u32(&bars.kv_full[slot]), use & 1, abort_flag, P.status, P.wait_limit_ns);
-        };
-        wait_full(0, 0);
+        }
+        ++n_pv[t];
+      };
+      int kslot = 0, kuse = 0, vslot = 1, vuse = 0;             // operand u of the sequence sits in unit u % kNumUnits
+      auto advance = [&](int& slot, int& use) { slot += 2; if (slot >= C::kNumUnits) { slot -= C::kNumUnits; ++use; } };
+      for (int it = 0; ; ++it) {
+        if (!wait_all(bars.item_full[it % kItemSlots], (it / kItemSlots) & 1)) break;
+        const Item& w = items[it % kItemSlots];
+        if (!w.run) break;
+        const int n_tiles = w.n_tiles, kv_begin = w.kv_begin, kv_end = w.kv_end;
+        const int t_tiles[2] = {w.tiles[0], w.tiles[1]};
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.item_empty[it % kItemSlots]));
+        if (n_tiles == 0) continue;
+        wait(bars.kv_full[kslot], kuse & 1);
         tc_fence_after();
-        for (int t = 0; t < 2; ++t) if (t_tiles[t] > 0) issue_qk(t, 0);
-        mma_commit(smem_u32(&bars.kv_empty[0]));          // K(0) is consumed once these retire
-        int vslot = 1, vuse = 0;                          // V(j): operand 2j + 1
-        int kslot = 2, kuse = 0;                          // K(j+1): operand 2j + 2
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+          if (t_tiles[t] > 0) {
+            wait(bars.q_full[t], n_q[t] & 1);
+            ++n_q[t];
+            tc_fence_after();
+            issue_qk(t, kslot, t_tiles[t] == 1);
+          }
+        mma_commit(smem_u32(&bars.kv_empty[kslot]));          // K(0) is consumed once these retire
+        advance(kslot, kuse);
         for (int j = 0; j < n_tiles; ++j) {
-          wait_full(vslot, vuse);
+          wait(bars.kv_full[vslot], vuse & 1);
           if (kv_end < kv_begin + (j + 1) * kTileKeys) {
             // rows of the V tile past the end of the item were not loaded (or hold stale page slots): clear
             // them so that weight 0 times leftover bits cannot produce NaN
             const int first = kv_end - (kv_begin + j * kTileKeys);
-            uint8_t* vgen = ring_gen + vslot * kUnitBytes;
-            for (int i = lane; i < (kTileKeys - first) * 16; i += 32) {
-              const int rr = first + (i >> 4), c = i & 15;     // whole rows are cleared, so the swizzle does not matter
-              *reinterpret_cast<uint4*>(vgen + (rr >> 3) * kGroupBytes + (c >> 3) * 1024 + (rr & 7) * 128 + (c & 7) * 16) = make_uint4(0, 0, 0, 0);
+            uint8_t* vgen = ring_gen + vslot * C::kUnitBytes;
+            for (int i = lane; i < (kTileKeys - first) * (D / 8); i += 32) {
+              const int rr = first + i / (D / 8), c = i % (D / 8);     // whole rows are cleared, so the swizzle does not matter
+              *reinterpret_cast<uint4*>(vgen + (rr >> 3) * C::kGroupBytes + (c >> 3) * 1024 + (rr & 7) * 128 + (c & 7) * 16) = make_uint4(0, 0, 0, 0);
             }
             fence_async_smem();
             __syncwarp();
           }
           bool k_ready = false;
-          for (int t = 0; t < 2; ++t) {
-            if (j < t_tiles[t]) {
+          auto next_qk = [&](int t) {                          // QK_t(j+1)
+            if (!k_ready) { wait(bars.kv_full[kslot], kuse & 1); tc_fence_after(); k_ready = true; }
+            issue_qk(t, kslot, j + 2 == t_tiles[t]);
+          };
 #pragma unroll
-              for (int q = 0; q < kPParts; ++q) {
-                mbar_wait(smem_u32(&bars.p_part[t][q]), j & 1, abort_flag, P.status, P.wait_limit_ns);
-                tc_fence_after();
-                issue_pv(t, j, vslot, q);
-              }
-              if (j + 1 < t_tiles[t]) {
-                if (!k_ready) { wait_full(kslot, kuse); tc_fence_after(); k_ready = true; }
-                issue_qk(t, kslot);                          // overwrites S_t / P_t after PV_t(j), in order
-              } else {
-                mma_commit(smem_u32(&bars.o_full[t]));
-              }
+          for (int t = 0; t < 2; ++t) {
+            if (C::kSepP && j + 1 < t_tiles[t]) next_qk(t);
+            if (C::kSepP && t == 1 && j + 1 < n_tiles) mma_commit(smem_u32(&bars.kv_empty[kslot]));
+            if (j < t_tiles[t]) {
+              issue_pv(t, j, vslot);
+              if (!C::kSepP && j + 1 < t_tiles[t]) next_qk(t); // overwrites S_t / P_t after PV_t(j), in order
+              if (C::kSepP || j + 1 == t_tiles[t]) mma_commit(smem_u32(&bars.o_full[t]));
             }
           }
           // V(j) and K(j+1) are consumed once these MMAs retire
           mma_commit(smem_u32(&bars.kv_empty[vslot]));
-          if (j + 1 < n_tiles) mma_commit(smem_u32(&bars.kv_empty[kslot]));
-          vslot += 2; if (vslot >= kNumUnits) { vslot -= kNumUnits; ++vuse; }
-          kslot += 2; if (kslot >= kNumUnits) { kslot -= kNumUnits; ++kuse; }
+          advance(vslot, vuse);
+          if (j + 1 < n_tiles) {
+            if (!C::kSepP) mma_commit(smem_u32(&bars.kv_empty[kslot]));
+            advance(kslot, kuse);
+          }
         }
-        // Every MMA has retired before this warp leaves (TMEM is freed after the CTA's last barrier): one more commit
-        // covers all of them.  This wait does not look at the abort flag - MMAs retire whatever else went wrong.
-        mma_commit(smem_u32(&bars.mma_done));
-        {
-          const uint32_t bar = smem_u32(&bars.mma_done);
-          const long long t0 = global_ns();
-          while (!mbar_try(bar, 0) && global_ns() - t0 < P.wait_limit_ns) {}
+      }
+      // Every MMA has retired before this warp leaves (TMEM is freed after the CTA's last barrier): one more commit
+      // covers all of them.  This wait does not look at the abort flag - MMAs retire whatever else went wrong.
+      mma_commit(smem_u32(&bars.mma_done));
+      {
+        const uint32_t bar = smem_u32(&bars.mma_done);
+        const long long t0 = global_ns();
+        while (!mbar_try(bar, 0) && global_ns() - t0 < P.wait_limit_ns) {}
+      }
+    } else {
+      // ================= warp 11: hands out the items and copies their queries =================
+      const int n_segs = P.dyn ? P.dyn[1] : P.n_segs;
+      // copies of Q: lane -> row (mod 8) and 16-byte chunk (mod 4); eight rows on is dq tokens and dg heads on
+      const int my_row = lane >> 2, my_chunk = lane & 3;
+      const uint32_t my_swz0 = (uint32_t)((my_chunk ^ my_row) << 4), my_swz1 = (uint32_t)(((my_chunk + 4) ^ my_row) << 4);
+      const int dq = 8 / g.G, dg = 8 - dq * g.G;
+      const int src_step = (dq * g.Hq + dg) * D * 2, src_wrap = (g.Hq - g.G) * D * 2;
+      int n_q[2] = {0, 0};
+      int item = (int)blockIdx.x, asks = 0;
+      bool open = false;                                           // a question without an answer yet
+      for (int it = 0; ; ++it) {
+        const int slot = it % kItemSlots;
+        if (it >= kItemSlots && !wait_all(bars.item_empty[slot], (it / kItemSlots - 1) & 1)) break;
+        Item& w = items[slot];
+        if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(P.status), 0) != 0) item = -1;
+        if (item < 0) {
+          if (lane == 0) { w.run = 0; mbar_arrive(smem_u32(&bars.item_full[slot])); }
+          break;
         }
+        const int si = find_segment(n_segs, item, [&](int i) { return P.segs[i].item_base; });
+        const Segment seg = P.segs[si];
+        int local = item - seg.item_base;
+        const int m_tile = local % seg.n_mtiles;
+        local /= seg.n_mtiles;
+        const int split = local % seg.n_splits;
+        const int kvh = local / seg.n_splits;
+        const int R = seg.n * g.G, row0 = m_tile * kUmmaTileRows * 2;
+        const int kv_begin = seg.origin + split * seg.chunk;
+        int t_rows[2], t_end[2], t_tiles[2], t_min_limit[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const int r0 = row0 + t * 128;
+          t_rows[t] = max(0, min(128, R - r0));
+          t_end[t] = kv_begin; t_min_limit[t] = kv_begin; t_tiles[t] = 0;
+          if (t_rows[t] > 0) {
+            t_end[t] = min(kv_begin + seg.chunk, seg.p + ((r0 + t_rows[t] - 1) / g.G) * seg.causal + 1);
+            t_min_limit[t] = min(t_end[t], seg.p + (r0 / g.G) * seg.causal + 1);
+            t_tiles[t] = t_end[t] > kv_begin ? (t_end[t] - kv_begin + kTileKeys - 1) / kTileKeys : 0;
+          }
+        }
+        if (lane == 0) {
+          w.run = 1;
+          w.table_off = seg.table_off; w.kvh = kvh; w.kv_begin = kv_begin; w.kv_end = max(t_end[0], t_end[1]);
+          w.n_tiles = max(t_tiles[0], t_tiles[1]);
+          for (int t = 0; t < 2; ++t) { w.tiles[t] = t_tiles[t]; w.end[t] = t_end[t]; w.min_limit[t] = t_min_limit[t]; }
+          w.row0 = row0; w.R = R; w.p = seg.p; w.causal = seg.causal;
+          w.direct = seg.n_splits == 1 && seg.partial == 0;
+          w.q_row0 = seg.q_off * g.Hq;
+          w.dst_row0 = w.direct ? seg.q_off * g.Hq : seg.part_base + split * seg.n * g.Hq;
+          w.drop = P.debug_drop_first_stage != 0 && item == 0;
+          mbar_arrive(smem_u32(&bars.item_full[slot]));
+        }
+        // The rows of Q (zeros past the last one) as the A operand of S = Q.K^T: K-major, 128-byte swizzle.  One
+        // instruction copies 64 bytes of eight rows; a lane's rows are eight apart, so their place in the swizzle is
+        // fixed and a row costs it one pointer step for its D / 32 copies.  (One softmax thread per row, 16 bytes at a
+        // time, needed 4.6 us per item; whole rows per instruction with an address per copy 2.4 us per tile.)
+        auto copy_q = [&](int t) {
+          int row = row0 + t * 128 + my_row;
+          const int qi = row / g.G;
+          int gi = row - qi * g.G;
+          const uint8_t* src = reinterpret_cast<const uint8_t*>(P.q) +
+                               (((long long)(seg.q_off + qi) * g.Hq + kvh * g.G + gi) * D + my_chunk * 8) * 2;
+          uint32_t dst = smem_q + t * C::kQTileBytes + my_row * 128;
+#pragma unroll 2
+          for (int i = 0; i < 16; ++i) {
+            const bool valid = row < R;
+            const uint8_t* from = valid ? src : reinterpret_cast<const uint8_t*>(P.q);
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c)
+              cp_async16(dst + (c >> 1) * C::kQSlabBytes + ((c & 1) ? my_swz1 : my_swz0), from + (valid ? c * 64 : 0), valid);
+            row += 8;
+            gi += dg;
+            src += src_step;
+            if (gi >= g.G) { gi -= g.G; src += src_wrap; }
+            dst += 1024;
+          }
+          cp_async_commit();
+        };
+        auto q_done = [&](int t) { fence_async_smem(); mbar_arrive(smem_u32(&bars.q_full[t])); };
+        bool fine = true, a_open = false;                          // a_open: A's copy is under way and not yet reported
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          if (t_tiles[t] == 0 || !fine) continue;
+          if (n_q[t] > 0) {
+            // B's buffer is free half a tile after A's: A's copy is not held back by that
+            if (a_open && __any_sync(0xffffffffu, !mbar_try(smem_u32(&bars.q_empty[t]), (n_q[t] - 1) & 1))) {
+              cp_async_wait<0>();
+              q_done(0);
+              a_open = false;
+            }
+            fine = wait_all(bars.q_empty[t], (n_q[t] - 1) & 1);
+          }
+          if (!fine) continue;
+          copy_q(t);
+          ++n_q[t];
+          if (t == 0) a_open = true;
+        }
+        if (a_open && t_tiles[1] > 0 && fine) { cp_async_wait<1>(); q_done(0); a_open = false; }
+        cp_async_wait<0>();
+        if (!fine) break;
+        if (a_open) q_done(0);
+        if (t_tiles[1] > 0) q_done(1);
+        // The next item is claimed when the K producer has nothing left to do for this one, some two tiles before its
+        // end: claimed at its start, it would bind long items to this SM while others run out of work.
+        if (!wait_all(bars.k_issued, it & 1)) break;
+        if (lane == 0) next_block_ask(smem_u32(&s_next), smem_u32(&bars.next));
+        ++asks;
+        open = true;
+        if (!wait_all(bars.next, (asks - 1) & 1)) break;
+        open = false;
+        item = next_block_answer(smem_u32(&s_next));
+        fence_async_smem();                                        // the answer has been read before the next one may land
+        __syncwarp();
+        if (item >= n_items) item = -1;                            // fixed grid: indices beyond the batch
+      }
+      if (open) {                                                  // only after a wait gave up: the answer lands before the block leaves
+        const long long t0 = global_ns();
+        while (!mbar_try(smem_u32(&bars.next), (asks - 1) & 1) && global_ns() - t0 < P.wait_limit_ns) {}
       }
     }
   } else {
@@ -420,183 +598,188 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
     const int t = warp >> 2;                                   // 0 = A, 1 = B
     const int row = ((warp & 3) << 5) | lane;                  // row of the 128-row tile = TMEM lane
     const uint32_t lane_addr = (uint32_t)((warp & 3) << 5) << 16;
-    const int r = item_row0 + t * 128 + row;
-    const bool valid = r < R;
-    const int qi = r / g.G, hd = kvh * g.G + (r - qi * g.G);
-    const int my_tiles = t_tiles[t];
-    const int limit = valid ? min(t_end[t], seg.p + qi * seg.causal + 1) : t_end[t];   // keys j < limit are visible
-
-    // ---- this row of Q (or zeros) into shared memory as the A operand of S = Q.K^T: K-major, 128-byte swizzle ----
-    {
-      const uint4* src = reinterpret_cast<const uint4*>(P.q + ((long long)(seg.q_off + qi) * g.Hq + hd) * D);
-      uint8_t* qrow = q_gen + t * kQTileBytes + row * 128;
-#pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const uint4 v = valid ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<uint4*>(qrow + (c >> 3) * kQSlabBytes + (((c & 7) ^ (row & 7)) << 4)) = v;
-      }
-      fence_async_smem();
-      mbar_arrive(smem_u32(&bars.q_full));
-    }
-
-    float m = -INFINITY, l = 0.f;       // running max (base-2, scaled) and sum
+    const uint32_t s_addr = tmem + lane_addr + C::kColS + t * 128;
+    const uint32_t p_addr = tmem + lane_addr + C::kColP + t * C::kColPStep;
+    const uint32_t o_addr = tmem + lane_addr + C::kColO + t * D;
     const float sl2 = P.scale_log2e;
-    const uint32_t s_addr = tmem + lane_addr + kColS + t * 128;
-    const uint32_t o_addr = tmem + lane_addr + kColO + t * 128;
+    int n_s = 0, n_o = 0;               // S tiles and finished items of this row tile so far (their barriers' phases)
 
-    // One key tile of this row tile.  The tiles that need the causal (or end-of-range) mask are the last ones of the
-    // item; they get a copy of the body of their own (with every exponential on the ex2 unit, which gives an exact 0
-    // for a masked key), so the compare-and-select instructions of the mask are not part of the code the other tiles run.
-    auto tile = [&](const int j, auto masked_tag) {
-      constexpr bool kMasked = decltype(masked_tag)::value;
-      constexpr int kEmu = kMasked ? 0 : kEmuPairs;
-      mbar_wait(smem_u32(&bars.s_full[t]), j & 1, abort_flag, P.status, P.wait_limit_ns);
-      tc_fence_after();
-      float s[128];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + c * 32, &s[c * 32]);
-      tmem_wait_ld();
-      if constexpr (kMasked) {
-        const int vis = limit - (kv_begin + j * kTileKeys);
-#pragma unroll
-        for (int c = 0; c < 128; ++c) if (c >= vis) s[c] = -INFINITY;
-      }
-      // independent partial reductions (one long dependent chain would expose its latency), three inputs per
-      // instruction: 8 chains over 128 values, then a tree
-      float mxp[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) mxp[i] = max3(s[i], s[i + 8], s[i + 16]);
-#pragma unroll
-      for (int c = 24; c < 120; c += 16) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) mxp[i] = max3(mxp[i], s[c + i], s[c + i + 8]);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) mxp[i] = fmaxf(mxp[i], s[i + 120]);
-      float mx = max3(max3(mxp[0], mxp[1], mxp[2]), max3(mxp[3], mxp[4], mxp[5]), fmaxf(mxp[6], mxp[7]));
-      mx *= sl2;                                               // scale > 0 on this path
-      float m_new = m;
-      if (mx > m + kRescaleThreshold) m_new = mx;             // also the first visible key: -inf + 8 = -inf < any finite mx
-      float alpha = 1.f;
-      if (__any_sync(0xffffffffu, m_new != m)) {               // rare: one vote per tile decides both steps
-        alpha = fast_exp2(m - m_new);                          // m = -inf -> 0, equal -> 1
-        if (j > 0) {
-          // O_t holds tiles < j: S_t(j) was committed after PV_t(j-1)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            float o[32];
-            tmem_ld32(o_addr + c * 32, o);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] *= alpha;
-            tmem_st32(o_addr + c * 32, o);
-          }
-        }
-      }
-      m = m_new;
-      const float mu = (m == -INFINITY) ? 0.f : m;
-      const uint64_t sl2_2 = pack2(sl2, sl2), nmu_2 = pack2(-mu, -mu);
-      uint64_t sp2[4] = {pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f)};
-      // The exponentials run on the ex2 unit (and, for a share of them, on the FMA and integer pipes), the sums and the
-      // bf16 packing on the FMA and ALU pipes.  A warp issues in order, so the three only overlap if independent work
-      // is next to each other in the instruction stream: the stream is written as a software pipeline over groups of
-      // 8 keys - scaled logits for all groups first, then the exponentials of group g+1 ahead of the sum and the
-      // packing of group g, whose exponentials have had a whole group's time to come back.
-      uint64_t x2[64];
-#pragma unroll
-      for (int i = 0; i < 64; ++i) x2[i] = fma2(pack2(s[2 * i], s[2 * i + 1]), sl2_2, nmu_2);
-      float e[2][8];
-      auto exp_group = [&](int gidx, float (&eg)[8]) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float x0, x1;
-          unpack2(x2[gidx * 4 + i], x0, x1);
-          if (i < kEmu) poly_exp2_pair(x0, x1, eg[2 * i], eg[2 * i + 1]);
-          else { eg[2 * i] = fast_exp2(x0); eg[2 * i + 1] = fast_exp2(x1); }
-        }
-      };
-      uint32_t pk[32];
-      exp_group(0, e[0]);
-#pragma unroll
-      for (int gidx = 0; gidx < 16; ++gidx) {
-        if (gidx + 1 < 16) exp_group(gidx + 1, e[(gidx + 1) & 1]);
-        const float (&eg)[8] = e[gidx & 1];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          sp2[i] = add2(sp2[i], pack2(eg[2 * i], eg[2 * i + 1]));
-          pk[(gidx & 7) * 4 + i] = pack_bf16(eg[2 * i], eg[2 * i + 1]);
-        }
-        // P_t over the first 64 columns of S_t; a part is handed over as soon as it is stored, so that its PV runs
-        // while the exponentials of the later parts are computed (the last part is handed over after the row sum)
-        constexpr int kGroupsPerPart = 16 / kPParts;
-        if ((gidx + 1) % kGroupsPerPart == 0) {
-          const int q = gidx / kGroupsPerPart;
-          if constexpr (kPParts == 2) tmem_st32u(s_addr + q * 32, pk);
-          else tmem_st16u(s_addr + q * 16, *reinterpret_cast<const uint32_t(*)[16]>(&pk[(q & 1) * 16]));
-          if (q + 1 < kPParts) {
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(smem_u32(&bars.p_part[t][q]));
-          }
-        }
-      }
-      float sp[8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) unpack2(sp2[i], sp[2 * i], sp[2 * i + 1]);
-      l = l * alpha + (((sp[0] + sp[1]) + (sp[2] + sp[3])) + ((sp[4] + sp[5]) + (sp[6] + sp[7])));
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(smem_u32(&bars.p_part[t][kPParts - 1]));
-    };
-    // tiles j < n_plain end at or before the first row's limit: every key of theirs is visible to every row
-    const int n_plain = min(my_tiles, max(0, (t_min_limit[t] - kv_begin) / kTileKeys));
-    for (int j = 0; j < n_plain; ++j) tile(j, std::false_type{});
-    for (int j = n_plain; j < my_tiles; ++j) tile(j, std::true_type{});
+    for (int it = 0; ; ++it) {
+      if (!wait_all(bars.item_full[it % kItemSlots], (it / kItemSlots) & 1)) break;
+      const Item& w = items[it % kItemSlots];
+      if (!w.run) break;
+      const int my_tiles = w.tiles[t], kv_begin = w.kv_begin;
+      int limit = w.end[t];                                      // keys j < limit are visible
+      if (w.row0 + t * 128 + row < w.R) limit = min(limit, w.p + ((w.row0 + t * 128 + row) / g.G) * w.causal + 1);
+      float m = -INFINITY, l = 0.f;       // running max (base-2, scaled) and sum
 
-    // ---- epilogue: O / l and LSE ----
-    const float kLn2 = 0.6931471805599453f;
-    if (my_tiles > 0) {
-      mbar_wait(smem_u32(&bars.o_full[t]), 0, abort_flag, P.status, P.wait_limit_ns);
-      tc_fence_after();
-    }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
-    const float e2 = l > 0.f ? m + log2f(l) : -INFINITY;
-    const long long orow = (long long)(seg.q_off + qi) * g.Hq + hd;
-    const long long prow_idx = seg.part_base + (long long)(split * seg.n + qi) * g.Hq + hd;
+      // One key tile of this row tile.  The tiles that need the causal (or end-of-range) mask are the last ones of the
+      // item; they get a copy of the body of their own, so the compare-and-select instructions of the mask are not part of the
+      // code the other tiles run.
+      auto tile = [&](const int j, auto masked_tag) {
+        constexpr bool kMasked = decltype(masked_tag)::value;
+        wait(bars.s_full[t], n_s & 1);
+        tc_fence_after();
+        float s[128];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float o[32];
-      if (my_tiles > 0) {                 // uniform over the warpgroup
-        tmem_ld32(o_addr + c * 32, o);
+        for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + c * 32, &s[c * 32]);
         tmem_wait_ld();
-      } else {
+        if constexpr (C::kSepP) {                                // QK_t(j+1) may overwrite S_t
+          tc_fence_before();
+          mbar_arrive(smem_u32(&bars.s_free[t]));
+        }
+        if constexpr (kMasked) {
+          const int vis = limit - (kv_begin + j * kTileKeys);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = 0.f;
-      }
-      if (valid) {
-        if (direct) {
-          uint4* dst = reinterpret_cast<uint4*>(P.out + orow * D + c * 32);
+          for (int c = 0; c < 128; ++c) if (c >= vis) s[c] = -INFINITY;
+        }
+        // independent partial reductions (one long dependent chain would expose its latency), three inputs per
+        // instruction: 8 chains over 128 values, then a tree
+        float mxp[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) mxp[i] = max3(s[i], s[i + 8], s[i + 16]);
+#pragma unroll
+        for (int c = 24; c < 120; c += 16) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mxp[i] = max3(mxp[i], s[c + i], s[c + i + 8]);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) mxp[i] = fmaxf(mxp[i], s[i + 120]);
+        float mx = max3(max3(mxp[0], mxp[1], mxp[2]), max3(mxp[3], mxp[4], mxp[5]), fmaxf(mxp[6], mxp[7]));
+        mx *= sl2;                                               // scale > 0 on this path
+        float m_new = m;
+        if (C::kSepP && n_s > 0) {                               // PV_t(j-1) has read P_t and written O_t (D = 128: implied by s_full)
+          wait(bars.o_full[t], (n_s - 1) & 1);
+          tc_fence_after();
+        }
+        ++n_s;
+        if (mx > m + kRescaleThreshold) m_new = mx;             // also the first visible key: -inf + 8 = -inf < any finite mx
+        float alpha = 1.f;
+        if (__any_sync(0xffffffffu, m_new != m)) {               // rare: one vote per tile decides both steps
+          alpha = fast_exp2(m - m_new);                          // m = -inf -> 0, equal -> 1
+          if (j > 0) {
+            // O_t holds tiles < j: S_t(j) was committed after PV_t(j-1)
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+              float o[32];
+              tmem_ld32(o_addr + c * 32, o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 32; ++i) o[i] *= alpha;
+              tmem_st32(o_addr + c * 32, o);
+            }
+          }
+        }
+        m = m_new;
+        const float mu = (m == -INFINITY) ? 0.f : m;
+        const uint64_t sl2_2 = pack2(sl2, sl2), nmu_2 = pack2(-mu, -mu);
+        uint64_t sp2[4] = {pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f), pack2(0.f, 0.f)};
+        // The exponentials run on the ex2 unit, the sums and the bf16 packing on the FMA and ALU pipes.  A warp issues in
+        // order, so the three only overlap if independent work is next to each other in the instruction stream: the stream
+        // is written as a software pipeline over groups of 8 keys - scaled logits for all groups first, then the exponentials of group g+1 ahead of the sum and the
+        // packing of group g, whose exponentials have had a whole group's time to come back.
+        uint64_t x2[64];
+#pragma unroll
+        for (int i = 0; i < 64; ++i) x2[i] = fma2(pack2(s[2 * i], s[2 * i + 1]), sl2_2, nmu_2);
+        float e[2][8];
+        auto exp_group = [&](int gidx, float (&eg)[8]) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            uint4 v;
-            v.x = pack_bf16(o[i * 8 + 0] * inv, o[i * 8 + 1] * inv);
-            v.y = pack_bf16(o[i * 8 + 2] * inv, o[i * 8 + 3] * inv);
-            v.z = pack_bf16(o[i * 8 + 4] * inv, o[i * 8 + 5] * inv);
-            v.w = pack_bf16(o[i * 8 + 6] * inv, o[i * 8 + 7] * inv);
-            dst[i] = v;
+            float x0, x1;
+            unpack2(x2[gidx * 4 + i], x0, x1);
+            eg[2 * i] = fast_exp2(x0);
+            eg[2 * i + 1] = fast_exp2(x1);
           }
-        } else {
-          float4* dst = reinterpret_cast<float4*>(P.part_o + prow_idx * D + c * 32);
+        };
+        uint32_t pk[32];
+        exp_group(0, e[0]);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) dst[i] = make_float4(o[i * 4] * inv, o[i * 4 + 1] * inv, o[i * 4 + 2] * inv, o[i * 4 + 3] * inv);
+        for (int gidx = 0; gidx < 16; ++gidx) {
+          if (gidx + 1 < 16) exp_group(gidx + 1, e[(gidx + 1) & 1]);
+          const float (&eg)[8] = e[gidx & 1];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            sp2[i] = add2(sp2[i], pack2(eg[2 * i], eg[2 * i + 1]));
+            pk[(gidx & 7) * 4 + i] = pack_bf16(eg[2 * i], eg[2 * i + 1]);
+          }
+          // P_t over the first 64 columns of S_t; a part is handed over as soon as it is stored, so that its PV runs
+          // while the exponentials of the later parts are computed (the last part is handed over after the row sum)
+          constexpr int kGroupsPerPart = 16 / kPParts;
+          if ((gidx + 1) % kGroupsPerPart == 0) {
+            const int q = gidx / kGroupsPerPart;
+            tmem_st32u(p_addr + q * 32, pk);
+            if (q + 1 < kPParts) {
+              tmem_wait_st();
+              tc_fence_before();
+              mbar_arrive(smem_u32(&bars.p_part[t][q]));
+            }
+          }
+        }
+        float sp[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) unpack2(sp2[i], sp[2 * i], sp[2 * i + 1]);
+        l = l * alpha + (((sp[0] + sp[1]) + (sp[2] + sp[3])) + ((sp[4] + sp[5]) + (sp[6] + sp[7])));
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(smem_u32(&bars.p_part[t][kPParts - 1]));
+      };
+      // tiles j < n_plain end at or before the first row's limit: every key of theirs is visible to every row
+      const int n_plain = min(my_tiles, max(0, (w.min_limit[t] - kv_begin) / kTileKeys));
+      for (int j = 0; j < n_plain; ++j) tile(j, std::false_type{});
+      for (int j = n_plain; j < my_tiles; ++j) tile(j, std::true_type{});
+
+      // ---- epilogue: O / l and LSE ----
+      const float kLn2 = 0.6931471805599453f;
+      if (my_tiles > 0) {
+        wait(bars.o_full[t], (C::kSepP ? n_s - 1 : n_o) & 1);
+        ++n_o;
+        tc_fence_after();
+      }
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      const int r = w.row0 + t * 128 + row;
+      const bool valid = r < w.R, direct = w.direct != 0;
+      const bool wide = ((uintptr_t)P.out & 31) == 0;            // callers need only align to 16
+      const int qi = r / g.G;
+      const long long drow = w.dst_row0 + (long long)qi * g.Hq + w.kvh * g.G + (r - qi * g.G);
+#pragma unroll
+      for (int c = 0; c < D / 32; ++c) {
+        float o[32];
+        if (my_tiles > 0) {                 // uniform over the warpgroup
+          tmem_ld32(o_addr + c * 32, o);
+          tmem_wait_ld();
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) o[i] = 0.f;
+        }
+        if (valid) {
+          if (direct) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              uint32_t v[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] = pack_bf16(o[i * 16 + 2 * e] * inv, o[i * 16 + 2 * e + 1] * inv);
+              st_32bytes(P.out + drow * D + c * 32 + i * 16, v, wide);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              uint32_t v[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(o[i * 8 + e] * inv);
+              st_32bytes(P.part_o + drow * D + c * 32 + i * 8, v, true);
+            }
+          }
         }
       }
+      if (valid) {
+        const float e2 = l > 0.f ? m + log2f(l) : -INFINITY;
+        if (direct) { if (P.lse != nullptr) P.lse[drow] = e2 * kLn2; }
+        else P.part_lse[drow] = e2;
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars.item_empty[it % kItemSlots]));
     }
-    if (valid) {
-      if (direct) { if (P.lse != nullptr) P.lse[orow] = e2 * kLn2; }
-      else P.part_lse[prow_idx] = e2;
-    }
-    tc_fence_before();
   }
 
   __syncthreads();
@@ -608,14 +791,20 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
 
 }  // namespace umma128
 
+template <int D>
+static cudaError_t init_one() {
+  return cudaFuncSetAttribute(umma128::attend_umma128_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, umma128::Cfg<D>::kSmemBytes);
+}
 cudaError_t attend_umma128_init() {
-  return cudaFuncSetAttribute(umma128::attend_umma128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, umma128::kSmemBytes);
+  const cudaError_t e = init_one<128>();
+  return e != cudaSuccess ? e : init_one<64>();
 }
 
 cudaError_t launch_attend_umma128(const AttendParams& p, cudaStream_t s) {
   const int grid = p.dyn ? p.grid_cap : p.n_items;
   if (grid <= 0) return cudaSuccess;
-  umma128::attend_umma128_kernel<<<grid, umma128::kThreads, umma128::kSmemBytes, s>>>(p);
+  if (p.g.D == 128) umma128::attend_umma128_kernel<128><<<grid, umma128::kThreads, umma128::Cfg<128>::kSmemBytes, s>>>(p);
+  else umma128::attend_umma128_kernel<64><<<grid, umma128::kThreads, umma128::Cfg<64>::kSmemBytes, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -1007,6 +1007,9 @@ static void find_share_groups(const tide_kv* kv, int32_t n_rows, const tide_row_
   }
 }
 
+// Head sizes the selected tcgen05 kernel is built for: 64-key tiles only 128, 128-key tiles both.
+static bool umma_takes(const tide_kv* kv) { return kv->g.D == 128 || kv->umma_tile_keys == 128; }
+
 // The work plan of one batch: one segment per row, decode-style (<= 16 packed rows), warp-MMA tile-style or
 // tcgen05-style; long contexts are split along the keys so that the grid has about items_per_sm items per SM.
 // A group of rows that share their first pages gets one more segment for the shared range (its tokens are the
@@ -1250,7 +1253,7 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
   int rc = check_rows(kv, n_rows, rows);
   if (rc != TIDE_OK) return rc;
   PlanHost P;
-  if ((rc = build_plan(kv, n_rows, rows, kv->g.D == 128 && scale > 0.f, page_table == nullptr, P)) != TIDE_OK) return rc;
+  if ((rc = build_plan(kv, n_rows, rows, umma_takes(kv) && scale > 0.f, page_table == nullptr, P)) != TIDE_OK) return rc;
   if (P.n_all() * sizeof(Segment) + 256 > kv->lay.slot_bytes) return TIDE_ERR_WORKSPACE;
 
   cudaStream_t st = (cudaStream_t)stream;
@@ -1341,7 +1344,11 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   // The plan needs the lengths after the step only through ctx_len, which the rows already carry, so it is built
   // (and can still be refused) before anything changes.
   PlanHost P;
-  if ((rc = build_plan(kv, n_rows, rows, g.D == 128, true, P)) != TIDE_OK) return rc;
+  // Launch shapes fixed without tcgen05 items (or with too few): head size 64 has the warp-MMA tile kernel as well.
+  bool umma = umma_takes(kv) && !(kv->fixed_grids && g.D == 64 && kv->cap_umma == 0);
+  if ((rc = build_plan(kv, n_rows, rows, umma, true, P)) != TIDE_OK) return rc;
+  if (umma && kv->fixed_grids && g.D == 64 && P.items_umma > kv->cap_umma &&
+      (rc = build_plan(kv, n_rows, rows, false, true, P)) != TIDE_OK) return rc;
   if (kv->fixed_grids && (P.items_dec > kv->cap_dec || P.items_tile > kv->cap_tile || P.items_umma > kv->cap_umma ||
                           P.merge_rows > kv->cap_merge_rows || indptr[(size_t)n_rows] > kv->cap_tokens))
     return TIDE_ERR_WORKSPACE;   // the step does not fit the launch shapes that were fixed

@@ -1,0 +1,67 @@
+"""The tcgen05 kernel runs one persistent thread block per SM that takes over item after item: batches of several
+hundred short items (every block walks many, of one tile and of several, with one row tile and with two), items cut
+along the keys, both head sizes, and launch shapes fixed larger than the batch.  Every output element and every LSE is
+compared with the float64 oracle."""
+import math
+
+import numpy as np
+import pytest
+
+from oracle import cbuild
+from oracle.paged_kv import PagedKVOracle
+from paper_2608_10402_b200 import inputs
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("geom,n_rows,fixed", [((28, 4, 128, 16), 90, False), ((28, 4, 128, 32), 40, True), ((8, 2, 64, 16), 200, False),
+                                               ((16, 1, 64, 32), 230, True), ((12, 4, 64, 16), 6, False)])
+def test_many_short_items_per_thread_block(geom, n_rows, fixed):
+    import torch
+    from paper_2608_10402_b200 import tide
+    HQ, HKV, D, S = geom
+    G = HQ // HKV
+    rng = np.random.default_rng(HQ + D + S + n_rows)
+    scale = 1.0 / math.sqrt(D)
+    edges = [16 // G + 1, 128 // G, 128 // G + 1, 256 // G, 256 // G + 1]        # around one and two row tiles
+    new = [max(1, edges[b % 5]) if b % 2 else int(rng.integers(16 // G + 1, 600 // G + 2)) for b in range(n_rows)]
+    prefix = [int(rng.choice([0, 1, 127, 128, 129])) if b % 3 == 0 else int(rng.integers(0, 700)) for b in range(n_rows)]
+    if n_rows < 16:
+        prefix[0], prefix[1] = 6000, 9001                                       # few items: cut along the keys and merged
+    pages = sum((p + n + S - 1) // S for p, n in zip(prefix, new)) + 4
+    max_pages = max((p + n + S - 1) // S for p, n in zip(prefix, new)) + 1
+    T = sum(new)
+    order = rng.permutation(pages).astype(np.int32)
+    kv = tide.TideKV(HQ, HKV, D, S, pages, n_rows, max_pages, n_rows, T, free_order=order)
+    orc = PagedKVOracle(pages, S, HKV, D, n_rows, max_pages, free_order=order)
+    ids = list(range(n_rows))
+    for o in (kv, orc):
+        for t in ids:
+            o.alloc(t)
+    ip = np.concatenate([[0], np.cumsum(prefix)]).astype(np.int32)
+    pk, pv = inputs.normal_bf16(rng, (int(ip[-1]), HKV, D)), inputs.normal_bf16(rng, (int(ip[-1]), HKV, D))
+    kv.append(ids, ip, H.to_dev(pk, torch), H.to_dev(pv, torch))
+    orc.append(ids, ip, pk, pv)
+    ip = np.concatenate([[0], np.cumsum(new)]).astype(np.int32)
+    nk, nv = inputs.normal_bf16(rng, (T, HKV, D)), inputs.normal_bf16(rng, (T, HKV, D))
+    q = inputs.normal_bf16(rng, (T, HQ, D))
+    rows = [(t, n, p + n) for t, (p, n) in enumerate(zip(prefix, new))]
+    # results start 16 bytes behind a 32-byte boundary: the smallest alignment the call takes
+    out = torch.zeros(T * HQ * D + 8, dtype=torch.int16, device="cuda")[8:].view(T, HQ, D)
+    lse = torch.zeros((T, HQ), dtype=torch.float32, device="cuda")
+    if fixed:
+        kv.step_fix_grids(max_umma_items=4000, max_tokens=T)
+        kv.step_begin(rows)
+        kv.step_layer(0, H.to_dev(nk, torch), H.to_dev(nv, torch), H.to_dev(q, torch), scale, out, lse)
+    else:
+        kv.append(ids, ip, H.to_dev(nk, torch), H.to_dev(nv, torch))
+        kv.attend(rows, H.to_dev(q, torch), scale, out, lse)
+    assert kv.status() == tide.OK
+    plan = kv.last_plan()
+    assert plan["prefill_items"] > (0 if n_rows < 16 else 200) and plan["decode_items"] == 0
+    assert (plan["merge_rows"] > 0) == (n_rows < 16)
+    orc.append(ids, ip, nk, nv)
+    ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
+    H.check_outputs(H.from_dev(out), lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
+    kv.close()
