@@ -88,10 +88,19 @@ def _ptr(x):
     return ctypes.c_void_p(x.data_ptr())
 
 
+def _raw_stream():
+    """The current stream's handle.  torch.cuda.current_stream() builds a Stream object on every call (3.2 us, twice in a
+    decode step whose kernels take 17 us); the raw handle costs 0.2 us."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch._C._cuda_getDevice())
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return ctypes.c_void_p(_raw_stream())
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
     return ctypes.c_void_p(stream.cuda_stream)
