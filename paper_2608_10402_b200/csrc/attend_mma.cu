@@ -1,5 +1,6 @@
-// Split-KV attention over the paged cache with warp-level tensor-core tiles (mma.sync) — the decode path,
-// and the general path for resume rows that the tcgen05 kernel does not take.
+// Attention of resume rows over the paged cache with warp-level tensor-core tiles (mma.sync): the rows that the tcgen05
+// kernel does not take (a softmax scale that is not positive, launch shapes fixed without tcgen05 items, 64-key tiles
+// selected with head size 64), and the merge of split rows.
 //
 // What it computes (paper Section 4: a resumed task continues from its preserved KV state; the maths is
 // ordinary scaled-dot-product softmax attention with grouped KV heads): for a work item
@@ -9,9 +10,7 @@
 //
 // Structure: one producer warp streams whole (page, head) blocks (K and V, contiguous in the pool) into a
 // ring of shared-memory stages with 1-D bulk copies that complete on mbarriers; four consumer warps run
-// m16n8k16 bf16 MMAs straight from the pre-swizzled blocks with ldmatrix.  Decode items: the four warps
-// split the keys of a stage and merge their (m, l, O) at the end.  Tile items: each warp owns 16 of the
-// 64 packed rows.  Bound by HBM bandwidth for decode: Hkv*D*4 bytes per context token, 4*D*Hq flops.
+// m16n8k16 bf16 MMAs straight from the pre-swizzled blocks with ldmatrix, each on 16 of the 64 packed rows.
 #include <cfloat>
 #include <climits>
 
@@ -29,12 +28,12 @@ struct MmaCfg {
   static constexpr int kSmemBytes = kStages * kStageBytes + 1024;
 };
 
-template <int D, bool DECODE>
-__device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Segment* __restrict__ segs) {
+template <int D>
+__global__ void __launch_bounds__(kAttendThreads, 2) attend_mma_kernel(const AttendParams P) {
   constexpr int KS = D / 16;                 // k-steps of Q.K^T
   constexpr int NT = D / 8;                  // n-tiles of O
-  constexpr int STEP_KB = DECODE ? 1 : 4;    // 16-key blocks per softmax step of one warp
-  constexpr int TILE_M = DECODE ? kDecodeTileRows : kMmaTileRows;
+  constexpr int STEP_KB = 4;                 // 16-key blocks per softmax step of one warp
+  constexpr int TILE_M = kMmaTileRows;
   constexpr int STAGE_BYTES = MmaCfg<D>::kStageBytes;
 
   extern __shared__ uint8_t smem_raw[];
@@ -46,6 +45,7 @@ __device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Seg
   uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Geom& g = P.g;
+  const Segment* __restrict__ segs = P.segs;
 
   // ---- which item ----
   const int item = blockIdx.x;
@@ -70,16 +70,15 @@ __device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Seg
   const float kLn2 = 0.6931471805599453f;
 
   // rows this thread owns inside its warp's 16-row MMA tile
-  const int row_base = tile_row0 + (DECODE ? 0 : warp * 16);
+  const int row_base = tile_row0 + warp * 16;
   const int r_lo = row_base + (lane >> 2), r_hi = r_lo + 8;
   const bool v_lo = r_lo < R, v_hi = r_hi < R;
   const int qi_lo = r_lo / g.G, qi_hi = r_hi / g.G;
   const int hd_lo = kvh * g.G + (r_lo - qi_lo * g.G), hd_hi = kvh * g.G + (r_hi - qi_hi * g.G);
 
-  if (kv_end <= kv_begin && seg.partial != 2) {
-    // nothing visible in this split (only possible when n_splits > 1): neutral partials.  (A segment whose last split
-    // merges walks the normal path with zero stages instead, so that it is counted.)
-    if (warp < kConsumerWarps && (lane & 3) == 0 && (!DECODE || warp == 0)) {
+  if (kv_end <= kv_begin) {
+    // nothing visible in this split (only possible when n_splits > 1): neutral partials
+    if (warp < kConsumerWarps && (lane & 3) == 0) {
       if (v_lo) P.part_lse[seg.part_base + (split * seg.n + qi_lo) * g.Hq + hd_lo] = -INFINITY;
       if (v_hi) P.part_lse[seg.part_base + (split * seg.n + qi_hi) * g.Hq + hd_hi] = -INFINITY;
     }
@@ -174,36 +173,19 @@ __device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Seg
   float m_lo = -INFINITY, m_hi = -INFINITY, l_lo = 0.f, l_hi = 0.f;
   const float sl2 = P.scale_log2e;
 
-  // Decode items: a warp reads the same 16 slots of every stage, so the offsets of its ldmatrix rows inside a stage
-  // are fixed for the whole item (two per K n-tile, four for V; the others are 1 KB further on).
-  uint32_t dk_off[2][2] = {{0u, 0u}, {0u, 0u}}, dv_off[4] = {0u, 0u, 0u, 0u};
-  if (DECODE) {
-    const int koff = warp * 16;
-    const uint32_t page_off = (uint32_t)((koff / g.S) * g.head_bytes);
-    const int row0 = koff % g.S;
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int x = 0; x < 2; ++x) dk_off[nt][x] = page_off + (uint32_t)blk_offset(g, row0 + nt * 8 + (lane & 7), 0, x * 4 + (lane >> 3));
-    const int vrow = row0 + ((lane >> 3) & 1) * 8 + (lane & 7);
-#pragma unroll
-    for (int y = 0; y < 4; ++y) dv_off[y] = page_off + (uint32_t)blk_offset(g, vrow, 1, y * 2 + (lane >> 4));
-  }
-
   for (int st = 0; st < n_st; ++st) {
     const int slot = st % kStages;
     mbar_wait(smem_u32(&s_full[slot]), (st / kStages) & 1, abort_flag, P.status, P.wait_limit_ns);
     const int key0 = kv_begin + st * kStageKeys;
     const uint32_t stage = smem_base + slot * STAGE_BYTES;
-    const int kb_first = DECODE ? warp : 0;
-    const int step_key0 = key0 + kb_first * 16;
+    const int step_key0 = key0;
     if (step_key0 < w_end) {
       const int nkb = min(STEP_KB, (w_end - step_key0 + 15) >> 4);
       float s[STEP_KB * 2][4];
 #pragma unroll
       for (int b = 0; b < STEP_KB; ++b) {
         if (b < nkb) {
-          const int koff = (kb_first + b) * 16;            // key offset inside the stage
+          const int koff = b * 16;            // key offset inside the stage
           const uint32_t pbase = stage + (koff / g.S) * g.head_bytes;
           const int row0 = koff % g.S;
 #pragma unroll
@@ -214,8 +196,7 @@ __device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Seg
 #pragma unroll
             for (int k2 = 0; k2 < KS / 2; ++k2) {
               uint32_t b0, b1, b2, b3;
-              if (DECODE) ldsm_x4(stage + dk_off[nt][k2 & 1] + (k2 >> 1) * 1024, b0, b1, b2, b3);
-              else ldsm_x4(pbase + blk_offset(g, slot_row, 0, k2 * 4 + (lane >> 3)), b0, b1, b2, b3);
+              ldsm_x4(pbase + blk_offset(g, slot_row, 0, k2 * 4 + (lane >> 3)), b0, b1, b2, b3);
               mma_bf16(acc, qa[2 * k2], b0, b1);
               mma_bf16(acc, qa[2 * k2 + 1], b2, b3);
             }
@@ -270,7 +251,7 @@ __device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Seg
 #pragma unroll
       for (int b = 0; b < STEP_KB; ++b) {
         if (b < nkb) {
-          const int koff = (kb_first + b) * 16;
+          const int koff = b * 16;
           const uint32_t vbase = stage + (koff / g.S) * g.head_bytes;   // the page block; V parts through blk_offset(.., 1, ..)
           const int row0 = koff % g.S;
           const int blk_key0 = key0 + koff;
@@ -294,8 +275,7 @@ __device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Seg
 #pragma unroll
           for (int n2 = 0; n2 < NT / 2; ++n2) {
             uint32_t b0, b1, b2, b3;
-            if (DECODE) ldsm_x4_t(stage + dv_off[n2 & 3] + (n2 >> 2) * 1024, b0, b1, b2, b3);
-            else ldsm_x4_t(vbase + blk_offset(g, vrow, 1, n2 * 2 + (lane >> 4)), b0, b1, b2, b3);
+            ldsm_x4_t(vbase + blk_offset(g, vrow, 1, n2 * 2 + (lane >> 4)), b0, b1, b2, b3);
             mma_bf16(o[2 * n2], pa, b0, b1);
             mma_bf16(o[2 * n2 + 1], pa, b2, b3);
           }
@@ -312,194 +292,47 @@ __device__ __forceinline__ void attend_mma_body(const AttendParams& P, const Seg
   l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1);
   l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
 
-  if (!DECODE) {
-    const float inv_lo = l_lo > 0.f ? 1.f / l_lo : 0.f, inv_hi = l_hi > 0.f ? 1.f / l_hi : 0.f;
-    const float e_lo = l_lo > 0.f ? m_lo + log2f(l_lo) : -INFINITY;
-    const float e_hi = l_hi > 0.f ? m_hi + log2f(l_hi) : -INFINITY;
-    const int dcol = 2 * (lane & 3);
-    if (direct) {
-      const long long o_lo = ((long long)(seg.q_off + qi_lo) * g.Hq + hd_lo), o_hi = ((long long)(seg.q_off + qi_hi) * g.Hq + hd_hi);
-#pragma unroll
-      for (int i = 0; i < NT; ++i) {
-        if (v_lo) *reinterpret_cast<uint32_t*>(P.out + o_lo * D + i * 8 + dcol) = pack_bf16(o[i][0] * inv_lo, o[i][1] * inv_lo);
-        if (v_hi) *reinterpret_cast<uint32_t*>(P.out + o_hi * D + i * 8 + dcol) = pack_bf16(o[i][2] * inv_hi, o[i][3] * inv_hi);
-      }
-      if (P.lse != nullptr && (lane & 3) == 0) {
-        if (v_lo) P.lse[o_lo] = e_lo * kLn2;
-        if (v_hi) P.lse[o_hi] = e_hi * kLn2;
-      }
-    } else {
-      const long long p_lo = seg.part_base + (long long)(split * seg.n + qi_lo) * g.Hq + hd_lo;
-      const long long p_hi = seg.part_base + (long long)(split * seg.n + qi_hi) * g.Hq + hd_hi;
-#pragma unroll
-      for (int i = 0; i < NT; ++i) {
-        if (v_lo) *reinterpret_cast<float2*>(P.part_o + p_lo * D + i * 8 + dcol) = make_float2(o[i][0] * inv_lo, o[i][1] * inv_lo);
-        if (v_hi) *reinterpret_cast<float2*>(P.part_o + p_hi * D + i * 8 + dcol) = make_float2(o[i][2] * inv_hi, o[i][3] * inv_hi);
-      }
-      if ((lane & 3) == 0) {
-        if (v_lo) P.part_lse[p_lo] = e_lo;
-        if (v_hi) P.part_lse[p_hi] = e_hi;
-      }
-    }
-    return;
-  }
-
-  // DECODE: the four warps hold partial (m, l, O) over disjoint keys of the same 16 rows; combine through
-  // shared memory (the stage ring is free: every copy that was issued has been consumed).
-  named_bar_sync(1, kConsumerWarps * 32);
-  float* s_o = reinterpret_cast<float*>(smem_gen);                    // [warp][16][D]
-  float* s_m = s_o + kConsumerWarps * 16 * D;                         // [warp][16]
-  float* s_l = s_m + kConsumerWarps * 16;
-  {
-    float* wo = s_o + warp * 16 * D;
-    const int rl = lane >> 2, dcol = 2 * (lane & 3);
+  const float inv_lo = l_lo > 0.f ? 1.f / l_lo : 0.f, inv_hi = l_hi > 0.f ? 1.f / l_hi : 0.f;
+  const float e_lo = l_lo > 0.f ? m_lo + log2f(l_lo) : -INFINITY;
+  const float e_hi = l_hi > 0.f ? m_hi + log2f(l_hi) : -INFINITY;
+  const int dcol = 2 * (lane & 3);
+  if (direct) {
+    const long long o_lo = ((long long)(seg.q_off + qi_lo) * g.Hq + hd_lo), o_hi = ((long long)(seg.q_off + qi_hi) * g.Hq + hd_hi);
 #pragma unroll
     for (int i = 0; i < NT; ++i) {
-      *reinterpret_cast<float2*>(wo + rl * D + i * 8 + dcol) = make_float2(o[i][0], o[i][1]);
-      *reinterpret_cast<float2*>(wo + (rl + 8) * D + i * 8 + dcol) = make_float2(o[i][2], o[i][3]);
+      if (v_lo) *reinterpret_cast<uint32_t*>(P.out + o_lo * D + i * 8 + dcol) = pack_bf16(o[i][0] * inv_lo, o[i][1] * inv_lo);
+      if (v_hi) *reinterpret_cast<uint32_t*>(P.out + o_hi * D + i * 8 + dcol) = pack_bf16(o[i][2] * inv_hi, o[i][3] * inv_hi);
+    }
+    if (P.lse != nullptr && (lane & 3) == 0) {
+      if (v_lo) P.lse[o_lo] = e_lo * kLn2;
+      if (v_hi) P.lse[o_hi] = e_hi * kLn2;
+    }
+  } else {
+    const long long p_lo = seg.part_base + (long long)(split * seg.n + qi_lo) * g.Hq + hd_lo;
+    const long long p_hi = seg.part_base + (long long)(split * seg.n + qi_hi) * g.Hq + hd_hi;
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {
+      if (v_lo) *reinterpret_cast<float2*>(P.part_o + p_lo * D + i * 8 + dcol) = make_float2(o[i][0] * inv_lo, o[i][1] * inv_lo);
+      if (v_hi) *reinterpret_cast<float2*>(P.part_o + p_hi * D + i * 8 + dcol) = make_float2(o[i][2] * inv_hi, o[i][3] * inv_hi);
     }
     if ((lane & 3) == 0) {
-      s_m[warp * 16 + rl] = m_lo; s_m[warp * 16 + rl + 8] = m_hi;
-      s_l[warp * 16 + rl] = l_lo; s_l[warp * 16 + rl + 8] = l_hi;
+      if (v_lo) P.part_lse[p_lo] = e_lo;
+      if (v_hi) P.part_lse[p_hi] = e_hi;
     }
   }
-  named_bar_sync(1, kConsumerWarps * 32);
-  {
-    constexpr int DSEG = D / 8;               // 128 threads = 16 rows x 8 column segments
-    const int t = threadIdx.x;
-    const int rr = t >> 3, d0 = (t & 7) * DSEG;
-    const int r = tile_row0 + rr;
-    if (r < R) {
-      float mw[kConsumerWarps], mstar = -INFINITY;
-#pragma unroll
-      for (int w = 0; w < kConsumerWarps; ++w) { mw[w] = s_m[w * 16 + rr]; mstar = fmaxf(mstar, mw[w]); }
-      const float mu = (mstar == -INFINITY) ? 0.f : mstar;
-      float f[kConsumerWarps], lstar = 0.f;
-#pragma unroll
-      for (int w = 0; w < kConsumerWarps; ++w) { f[w] = fast_exp2(mw[w] - mu); lstar += f[w] * s_l[w * 16 + rr]; }
-      const float inv = lstar > 0.f ? 1.f / lstar : 0.f;
-      const float e2 = lstar > 0.f ? mstar + log2f(lstar) : -INFINITY;
-      const int qi = r / g.G, hd = kvh * g.G + (r - qi * g.G);
-      float acc[DSEG];
-#pragma unroll
-      for (int d = 0; d < DSEG; ++d) {
-        float a = 0.f;
-#pragma unroll
-        for (int w = 0; w < kConsumerWarps; ++w) a += f[w] * s_o[(w * 16 + rr) * D + d0 + d];
-        acc[d] = a * inv;
-      }
-      if (direct) {
-        const long long orow = (long long)(seg.q_off + qi) * g.Hq + hd;
-        uint32_t* dst = reinterpret_cast<uint32_t*>(P.out + orow * D + d0);
-#pragma unroll
-        for (int d = 0; d < DSEG; d += 2) dst[d >> 1] = pack_bf16(acc[d], acc[d + 1]);
-        if (P.lse != nullptr && (t & 7) == 0) P.lse[orow] = e2 * kLn2;
-      } else {
-        const long long prow = seg.part_base + (long long)(split * seg.n + qi) * g.Hq + hd;
-        float* dst = P.part_o + prow * D + d0;
-#pragma unroll
-        for (int d = 0; d < DSEG; d += 4) *reinterpret_cast<float4*>(dst + d) = make_float4(acc[d], acc[d + 1], acc[d + 2], acc[d + 3]);
-        if ((t & 7) == 0) P.part_lse[prow] = e2;
-      }
-    }
-    // A split decode-style row merges its own partials: every split counts itself in once its partials are written
-    // (fence, barrier, one atomic per CTA); the CTA that counts last reads all splits' partials - in split order, so
-    // the result does not depend on which one came last - and writes the row.  The counter goes back to zero for the
-    // next launch.  This removes the merge launch, and with it a dependent chain of loads, from decode-only steps.
-    if (seg.partial == 2) {
-      __shared__ int s_is_last;
-      __threadfence();
-      named_bar_sync(1, kConsumerWarps * 32);
-      if (t == 0) {
-        int* ctr = P.merge_ctr + seg.x_part_base + kvh;
-        const int done = atomicAdd(ctr, 1);
-        s_is_last = done == seg.n_splits - 1 ? 1 : 0;
-        if (s_is_last) *ctr = 0;
-      }
-      named_bar_sync(1, kConsumerWarps * 32);
-      if (s_is_last && r < R) {
-        __threadfence();
-        const int qi = r / g.G, hd = kvh * g.G + (r - qi * g.G);
-        const long long stride = (long long)seg.n * g.Hq;                       // partial rows per split
-        const long long p0 = seg.part_base + (long long)qi * g.Hq + hd;         // this (token, head) in split 0
-        float mstar = -INFINITY;
-        for (int sp = 0; sp < seg.n_splits; ++sp) mstar = fmaxf(mstar, __ldcg(P.part_lse + p0 + sp * stride));
-        const float mu = (mstar == -INFINITY) ? 0.f : mstar;
-        float acc[DSEG];
-#pragma unroll
-        for (int d = 0; d < DSEG; ++d) acc[d] = 0.f;
-        float tot = 0.f;
-        for (int sp = 0; sp < seg.n_splits; ++sp) {
-          const float e = __ldcg(P.part_lse + p0 + sp * stride);
-          if (e == -INFINITY) continue;
-          const float w = exp2f(e - mu);
-          tot += w;
-          const float4* po = reinterpret_cast<const float4*>(P.part_o + (p0 + sp * stride) * D + d0);
-#pragma unroll
-          for (int d = 0; d < DSEG; d += 4) {
-            const float4 v = __ldcg(po + (d >> 2));
-            acc[d] += w * v.x; acc[d + 1] += w * v.y; acc[d + 2] += w * v.z; acc[d + 3] += w * v.w;
-          }
-        }
-        const float inv = tot > 0.f ? 1.f / tot : 0.f;
-        const long long orow = (long long)(seg.q_off + qi) * g.Hq + hd;
-        uint32_t* dst = reinterpret_cast<uint32_t*>(P.out + orow * D + d0);
-#pragma unroll
-        for (int d = 0; d < DSEG; d += 2) dst[d >> 1] = pack_bf16(acc[d] * inv, acc[d + 1] * inv);
-        if (P.lse != nullptr && (t & 7) == 0) P.lse[orow] = (tot > 0.f ? mstar + log2f(tot) : -INFINITY) * kLn2;
-      }
-    }
-  }
-}
-
-template <int D, bool DECODE>
-__global__ void __launch_bounds__(kAttendThreads, 2) attend_mma_kernel(const AttendParams P) {
-  attend_mma_body<D, DECODE>(P, P.segs);
-}
-
-// Decode-style items whose row descriptors travel in the kernel's parameters (small decode-only batches).
-template <int D>
-__global__ void __launch_bounds__(kAttendThreads, 2) attend_decode_inline_kernel(const __grid_constant__ AttendInline PI) {
-  attend_mma_body<D, true>(PI.p, PI.segs);
 }
 
 cudaError_t attend_kernels_init() {
-  cudaError_t e;
-  e = cudaFuncSetAttribute(attend_mma_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<128>::kSmemBytes);
+  const cudaError_t e = cudaFuncSetAttribute(attend_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<128>::kSmemBytes);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_mma_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<128>::kSmemBytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_mma_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<64>::kSmemBytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_mma_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<64>::kSmemBytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_decode_inline_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<128>::kSmemBytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(attend_decode_inline_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<64>::kSmemBytes);
-  return e;
-}
-
-cudaError_t launch_attend_decode_inline(const AttendInline& pi, cudaStream_t s) {
-  const int grid = pi.p.n_items;
-  if (grid <= 0) return cudaSuccess;
-  if (pi.p.g.D == 128) attend_decode_inline_kernel<128><<<grid, kAttendThreads, MmaCfg<128>::kSmemBytes, s>>>(pi);
-  else attend_decode_inline_kernel<64><<<grid, kAttendThreads, MmaCfg<64>::kSmemBytes, s>>>(pi);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_attend_decode(const AttendParams& p, cudaStream_t s) {
-  const int grid = p.dyn ? p.grid_cap : p.n_items;
-  if (grid <= 0) return cudaSuccess;
-  if (p.g.D == 128) attend_mma_kernel<128, true><<<grid, kAttendThreads, MmaCfg<128>::kSmemBytes, s>>>(p);
-  else attend_mma_kernel<64, true><<<grid, kAttendThreads, MmaCfg<64>::kSmemBytes, s>>>(p);
-  return cudaGetLastError();
+  return cudaFuncSetAttribute(attend_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, MmaCfg<64>::kSmemBytes);
 }
 
 cudaError_t launch_attend_tile(const AttendParams& p, cudaStream_t s) {
   const int grid = p.dyn ? p.grid_cap : p.n_items;
   if (grid <= 0) return cudaSuccess;
-  if (p.g.D == 128) attend_mma_kernel<128, false><<<grid, kAttendThreads, MmaCfg<128>::kSmemBytes, s>>>(p);
-  else attend_mma_kernel<64, false><<<grid, kAttendThreads, MmaCfg<64>::kSmemBytes, s>>>(p);
+  if (p.g.D == 128) attend_mma_kernel<128><<<grid, kAttendThreads, MmaCfg<128>::kSmemBytes, s>>>(p);
+  else attend_mma_kernel<64><<<grid, kAttendThreads, MmaCfg<64>::kSmemBytes, s>>>(p);
   return cudaGetLastError();
 }
 

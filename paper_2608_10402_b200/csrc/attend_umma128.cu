@@ -172,23 +172,6 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// Ask the hardware for the index of a block of this launch that has not started: the 16-byte answer lands at `resp`
-// and is counted on `bar`.  After an answer "none left" nothing more may be asked.
-__device__ __forceinline__ void next_block_ask(uint32_t resp, uint32_t bar) {
-  mbar_expect_tx(bar, 16);
-  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(resp), "r"(bar) : "memory");
-}
-__device__ __forceinline__ int next_block_answer(uint32_t resp) {        // -1: none left
-  int x;
-  asm volatile(
-      "{\n\t.reg .b128 r;\n\t.reg .pred p;\n\t"
-      "ld.shared.b128 r, [%1];\n\t"
-      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
-      "mov.b32 %0, -1;\n\t"
-      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, r;\n\t}"
-      : "=r"(x) : "r"(resp) : "memory");
-  return x;
-}
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {     // zero-fills when not valid
   const int n = valid ? 16 : 0;
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");

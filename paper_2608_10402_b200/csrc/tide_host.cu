@@ -316,7 +316,7 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
   bool ok = cudaGetDevice(&kv->device) == cudaSuccess;
   kv->num_sms = sm_count();
   ok = ok && kv->num_sms > 0;
-  ok = ok && attend_kernels_init() == cudaSuccess && attend_umma_init() == cudaSuccess && attend_umma128_init() == cudaSuccess;
+  ok = ok && attend_kernels_init() == cudaSuccess && attend_decode_init() == cudaSuccess && attend_umma_init() == cudaSuccess && attend_umma128_init() == cudaSuccess;
   ok = ok && cudaMemset(kv->d_status, 0, 256) == cudaSuccess;
   ok = ok && cudaMemset(kv->d_merge_ctr, 0, (size_t)kStepSegStride * cfg->max_batch_rows * g.Hkv * 4) == cudaSuccess;
   ok = ok && cudaHostAlloc((void**)&kv->h_status, 64, cudaHostAllocDefault) == cudaSuccess;

@@ -1,7 +1,7 @@
-"""The tcgen05 kernel runs one persistent thread block per SM that takes over item after item: batches of several
-hundred short items (every block walks many, of one tile and of several, with one row tile and with two), items cut
-along the keys, both head sizes, and launch shapes fixed larger than the batch.  Every output element and every LSE is
-compared with the float64 oracle."""
+"""The attention kernels run persistent thread blocks that take over item after item: batches of several hundred short
+items (every block walks many, of one tile and of several, with one row tile and with two), items cut along the keys,
+both head sizes, and launch shapes fixed larger than the batch.  Every output element and every LSE is compared with
+the float64 oracle."""
 import math
 
 import numpy as np
@@ -64,4 +64,62 @@ def test_many_short_items_per_thread_block(geom, n_rows, fixed):
     orc.append(ids, ip, nk, nv)
     ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
     H.check_outputs(H.from_dev(out), lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
+    kv.close()
+
+
+@pytest.mark.parametrize("geom,n_rows,fixed", [((28, 4, 128, 16), 100, False), ((28, 4, 128, 32), 180, False), ((8, 2, 64, 16), 300, True),
+                                               ((16, 1, 64, 32), 400, False), ((6, 2, 128, 16), 3, False), ((32, 8, 128, 16), 90, True)])
+def test_many_decode_items_per_thread_block(geom, n_rows, fixed):
+    """Decode-style rows from one key to several thousand, of one token or as many as still make one item: rows of one
+    split beside rows whose splits are finished by different blocks, descriptors in the launch and uploaded."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    HQ, HKV, D, S = geom
+    G = HQ // HKV
+    rng = np.random.default_rng(HQ + 3 * D + S + n_rows)
+    scale = 1.0 / math.sqrt(D)
+    new = [int(rng.integers(1, 16 // G + 1)) for _ in range(n_rows)]
+    edges = [0, 1, 63, 64, 65, 127, 128, 129, 511, 512]
+    prefix = [edges[b % 10] if b % 2 else int(rng.integers(0, 900)) for b in range(n_rows)]
+    for b in range(0, n_rows, 7):
+        prefix[b] = int(rng.integers(2000, 9000))
+    pages = sum((p + n + S - 1) // S for p, n in zip(prefix, new)) + 4
+    max_pages = max((p + n + S - 1) // S for p, n in zip(prefix, new)) + 1
+    T = sum(new)
+    order = rng.permutation(pages).astype(np.int32)
+    kv = tide.TideKV(HQ, HKV, D, S, pages, n_rows, max_pages, n_rows, T, free_order=order)
+    orc = PagedKVOracle(pages, S, HKV, D, n_rows, max_pages, free_order=order)
+    ids = list(range(n_rows))
+    for o in (kv, orc):
+        for t in ids:
+            o.alloc(t)
+    ip = np.concatenate([[0], np.cumsum(prefix)]).astype(np.int32)
+    pk, pv = inputs.normal_bf16(rng, (int(ip[-1]), HKV, D)), inputs.normal_bf16(rng, (int(ip[-1]), HKV, D))
+    kv.append(ids, ip, H.to_dev(pk, torch), H.to_dev(pv, torch))
+    orc.append(ids, ip, pk, pv)
+    ip = np.concatenate([[0], np.cumsum(new)]).astype(np.int32)
+    nk, nv = inputs.normal_bf16(rng, (T, HKV, D)), inputs.normal_bf16(rng, (T, HKV, D))
+    q = inputs.normal_bf16(rng, (T, HQ, D))
+    rows = [(t, n, p + n) for t, (p, n) in enumerate(zip(prefix, new))]
+    out = torch.zeros((T, HQ, D), dtype=torch.int16, device="cuda")
+    lse = torch.zeros((T, HQ), dtype=torch.float32, device="cuda")
+    dq = H.to_dev(q, torch)
+    if fixed:
+        kv.step_fix_grids(max_decode_items=3000, max_tokens=T)
+        kv.step_begin(rows)
+        kv.step_layer(0, H.to_dev(nk, torch), H.to_dev(nv, torch), dq, scale, out, lse)
+    else:
+        kv.append(ids, ip, H.to_dev(nk, torch), H.to_dev(nv, torch))
+        kv.attend(rows, dq, scale, out, lse)
+    assert kv.status() == tide.OK
+    plan = kv.last_plan()
+    assert plan["prefill_items"] == 0 and plan["merge_rows"] > 0 and (n_rows < 10 or plan["decode_items"] > 296)
+    orc.append(ids, ip, nk, nv)
+    ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
+    H.check_outputs(H.from_dev(out), lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
+    # a second call finds the finished-split counters at zero again and gives the same bits
+    first = out.clone()
+    out.zero_()
+    kv.attend(rows, dq, scale, out, lse)
+    assert kv.status() == tide.OK and torch.equal(first, out)
     kv.close()
