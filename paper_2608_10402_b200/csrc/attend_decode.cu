@@ -139,19 +139,13 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
   __shared__ __align__(16) uint4 s_next;
   __shared__ Item items[kItemSlots];
   __shared__ float s_m[kConsumerWarps * 16], s_l[kConsumerWarps * 16];
-  __shared__ int s_abort, s_skip, s_is_last;
+  __shared__ int s_abort, s_is_last;
 
   const uint32_t ring = smem_u32(smem_raw);
   float* s_o = reinterpret_cast<float*>(smem_raw + NS * C::kStageBytes);     // [warp][8 rows][D]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Geom& g = P.g;
-  const int n_items = P.dyn ? P.dyn[0] : P.n_items;      // fixed grid: the batch's counts live in device memory
-  if ((int)blockIdx.x >= n_items) return;
-
-  // The status word is set when a bounded wait runs out and stays set until tide_status clears it.  While it is
-  // set no block starts work, so outputs are undefined from the time-out until the caller has read the status.
   if (threadIdx.x == 0) {
-    s_skip = *reinterpret_cast<volatile int*>(P.status);
     s_abort = 0;
     for (int i = 0; i < NS; ++i) {
       mbar_init(smem_u32(&s_full[i]), 1);
@@ -166,8 +160,14 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     mbar_init(smem_u32(&s_part_done), 1);
     mbar_fence_init();
   }
+  if (!P.overlapped) grid_dep_wait();
+  grid_dep_launch();
+  const int n_items = P.dyn ? __ldcg(P.dyn) : P.n_items;     // fixed grid: the batch's counts live in device memory
   __syncthreads();
-  if (s_skip != 0) return;
+  if ((int)blockIdx.x >= n_items) {
+    if (P.overlapped) grid_dep_wait();
+    return;
+  }
   volatile int* abort_flag = &s_abort;
   auto wait = [&](uint64_t& bar, int parity) -> bool {
     return mbar_wait(smem_u32(&bar), (uint32_t)parity, abort_flag, P.status, P.wait_limit_ns);
@@ -194,7 +194,7 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
       const int lp0 = kv_begin / g.S, lp_last = (kv_end - 1) / g.S;
       auto load_ids = [&](int grp) -> int {
         const int lp = lp0 + grp * 32 + lane;
-        return lp <= lp_last ? trow[lp] : 0;
+        return lp <= lp_last ? __ldcg(trow + lp) : 0;
       };
       int ids_cur = load_ids(0), ids_nxt = load_ids(1), cur_grp = 0;
       const int ask_at = max(0, n_st - 2);
@@ -231,7 +231,7 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
   }
   if (warp == kConsumerWarps + 1) {
     // ================= scheduler warp: hands out the items =================
-    const int n_segs = P.dyn ? P.dyn[1] : P.n_segs;
+    const int n_segs = P.dyn ? __ldcg(P.dyn + 1) : P.n_segs;
     int item = (int)blockIdx.x, asks = 0, done = 0;
     int merge = 0;                                           // lane 0: the last item but one completed its row
     bool fused_before = false, open = false;                                       // a question without an answer yet
@@ -239,6 +239,8 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
       const int slot = it % kItemSlots;
       if (it >= kItemSlots && !wait_all(s_item_empty[slot], (it / kItemSlots - 1) & 1)) break;
       Item& w = items[slot];
+      // The status word is set when a bounded wait runs out and stays set until tide_status clears it.  While it is set
+      // no item is started, so outputs are undefined from the time-out until the caller has read the status.
       if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(P.status), 0) != 0) item = -1;
       if (item < 0) {
         if (lane == 0) { w.run = 0; w.merge = merge; mbar_arrive(smem_u32(&s_item_full[slot])); }
@@ -255,14 +257,14 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const int i = i0 + k * 32 + lane;
-            le[k] = i < n_segs && segs[i].item_base <= item;
+            le[k] = i < n_segs && __ldcg(&segs[i].item_base) <= item;
           }
 #pragma unroll
           for (int k = 0; k < 4; ++k) si += __popc(__ballot_sync(0xffffffffu, le[k]));
           if (si + 1 < i0 + 128) break;
         }
       }
-      const Segment seg = segs[si];
+      const Segment seg = INLINE ? segs[si] : load_segment(segs + si);
       if (lane == 0) {
         const int local = item - seg.item_base;
         const int split = local % seg.n_splits, kvh = local / seg.n_splits;
@@ -335,10 +337,10 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     const uint16_t* q_hi = P.q + ((long long)w.q_row0 + qi_hi * g.Hq + (r_hi - qi_hi * g.G)) * D + 2 * (lane & 3);
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      qa[ks][0] = v_lo ? *reinterpret_cast<const uint32_t*>(q_lo + ks * 16) : 0u;
-      qa[ks][1] = v_hi ? *reinterpret_cast<const uint32_t*>(q_hi + ks * 16) : 0u;
-      qa[ks][2] = v_lo ? *reinterpret_cast<const uint32_t*>(q_lo + ks * 16 + 8) : 0u;
-      qa[ks][3] = v_hi ? *reinterpret_cast<const uint32_t*>(q_hi + ks * 16 + 8) : 0u;
+      qa[ks][0] = v_lo ? __ldcg(reinterpret_cast<const uint32_t*>(q_lo + ks * 16)) : 0u;
+      qa[ks][1] = v_hi ? __ldcg(reinterpret_cast<const uint32_t*>(q_hi + ks * 16)) : 0u;
+      qa[ks][2] = v_lo ? __ldcg(reinterpret_cast<const uint32_t*>(q_lo + ks * 16 + 8)) : 0u;
+      qa[ks][3] = v_hi ? __ldcg(reinterpret_cast<const uint32_t*>(q_hi + ks * 16 + 8)) : 0u;
     }
   };
   int slot = 0, use = 0;
@@ -535,6 +537,7 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
       if (lane == 0) mbar_arrive(smem_u32(&s_item_empty[before]));
     }
   }
+  if (P.overlapped) grid_dep_wait();
 }
 
 template <int D>
@@ -565,17 +568,15 @@ cudaError_t attend_decode_init() {
 cudaError_t launch_attend_decode_inline(const AttendInline& pi, cudaStream_t s) {
   const int grid = pi.p.n_items;
   if (grid <= 0) return cudaSuccess;
-  if (pi.p.g.D == 128) decode::attend_decode_inline_kernel<128><<<grid, decode::kThreads, decode::Cfg<128>::kSmemBytes, s>>>(pi);
-  else decode::attend_decode_inline_kernel<64><<<grid, decode::kThreads, decode::Cfg<64>::kSmemBytes, s>>>(pi);
-  return cudaGetLastError();
+  if (pi.p.g.D == 128) return launch_dep(decode::attend_decode_inline_kernel<128>, grid, decode::kThreads, decode::Cfg<128>::kSmemBytes, s, pi);
+  return launch_dep(decode::attend_decode_inline_kernel<64>, grid, decode::kThreads, decode::Cfg<64>::kSmemBytes, s, pi);
 }
 
 cudaError_t launch_attend_decode(const AttendParams& p, cudaStream_t s) {
   const int grid = p.dyn ? p.grid_cap : p.n_items;
   if (grid <= 0) return cudaSuccess;
-  if (p.g.D == 128) decode::attend_decode_kernel<128><<<grid, decode::kThreads, decode::Cfg<128>::kSmemBytes, s>>>(p);
-  else decode::attend_decode_kernel<64><<<grid, decode::kThreads, decode::Cfg<64>::kSmemBytes, s>>>(p);
-  return cudaGetLastError();
+  if (p.g.D == 128) return launch_dep(decode::attend_decode_kernel<128>, grid, decode::kThreads, decode::Cfg<128>::kSmemBytes, s, p);
+  return launch_dep(decode::attend_decode_kernel<64>, grid, decode::kThreads, decode::Cfg<64>::kSmemBytes, s, p);
 }
 
 }  // namespace tide

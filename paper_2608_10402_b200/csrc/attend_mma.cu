@@ -46,6 +46,8 @@ __global__ void __launch_bounds__(kAttendThreads, 2) attend_mma_kernel(const Att
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Geom& g = P.g;
   const Segment* __restrict__ segs = P.segs;
+  grid_dep_wait();
+  grid_dep_launch();
 
   // ---- which item ----
   const int item = blockIdx.x;
@@ -331,9 +333,8 @@ cudaError_t attend_kernels_init() {
 cudaError_t launch_attend_tile(const AttendParams& p, cudaStream_t s) {
   const int grid = p.dyn ? p.grid_cap : p.n_items;
   if (grid <= 0) return cudaSuccess;
-  if (p.g.D == 128) attend_mma_kernel<128><<<grid, kAttendThreads, MmaCfg<128>::kSmemBytes, s>>>(p);
-  else attend_mma_kernel<64><<<grid, kAttendThreads, MmaCfg<64>::kSmemBytes, s>>>(p);
-  return cudaGetLastError();
+  if (p.g.D == 128) return launch_dep(attend_mma_kernel<128>, grid, kAttendThreads, MmaCfg<128>::kSmemBytes, s, p);
+  return launch_dep(attend_mma_kernel<64>, grid, kAttendThreads, MmaCfg<64>::kSmemBytes, s, p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -342,13 +343,15 @@ cudaError_t launch_attend_tile(const AttendParams& p, cudaStream_t s) {
 // The kernel is a chain of dependent loads if written naively (one split after the other), so the partial LSEs
 // are fetched side by side, one per lane, and the partial outputs four splits at a time; the order in which the
 // terms are added is still the order of the splits.
-__global__ void __launch_bounds__(256) merge_kernel(const MergeParams P) {
+__device__ __forceinline__ void merge_body(const MergeParams& P, const Segment* __restrict__ segs) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int n_rows = P.dyn ? P.dyn[0] : P.n_rows, n_segs = P.dyn ? P.dyn[1] : P.n_segs;
   if (row >= n_rows) return;
-  const int si = find_segment(n_segs, row, [&](int i) { return P.segs[i].merge_base; });
-  const Segment seg = P.segs[si];
+  const int si = find_segment(n_segs, row, [&](int i) { return segs[i].merge_base; });
+  const Segment seg = segs[si];
   const int local = row - seg.merge_base;                 // token * Hq + head inside the segment
   const long long stride = (long long)seg.n * P.Hq;       // partial rows per split
   const long long p0 = seg.part_base + local;
@@ -416,12 +419,19 @@ __global__ void __launch_bounds__(256) merge_kernel(const MergeParams P) {
   if (P.lse != nullptr && lane == 0) P.lse[orow] = (tot > 0.f ? mstar + log2f(tot) : -INFINITY) * 0.6931471805599453f;
 }
 
+__global__ void __launch_bounds__(256) merge_kernel(const MergeParams P) { merge_body(P, P.segs); }
+__global__ void __launch_bounds__(256) merge_inline_kernel(const __grid_constant__ MergeInline PI) { merge_body(PI.p, PI.segs); }
+
+cudaError_t launch_merge_inline(const MergeInline& pi, cudaStream_t s) {
+  if (pi.p.n_rows <= 0) return cudaSuccess;
+  return launch_dep(merge_inline_kernel, (unsigned)((pi.p.n_rows + 7) / 8), 256, 0, s, pi);
+}
+
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t s) {
   const int rows = p.dyn ? p.grid_cap_rows : p.n_rows;
   if (rows <= 0) return cudaSuccess;
   const int blocks = (rows + 7) / 8;
-  merge_kernel<<<blocks, 256, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_dep(merge_kernel, (unsigned)blocks, 256, 0, s, p);
 }
 
 }  // namespace tide

@@ -224,8 +224,8 @@ struct Bars {
 };
 constexpr int kItemReaders = 3 + 8;   // K producer, V producer, MMA warp, eight softmax warps: one arrival each
 
-template <int D>
-__global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const AttendParams P) {
+template <int D, bool INLINE>
+__device__ __forceinline__ void attend_umma128_body(const AttendParams& P, const Segment* __restrict__ segs) {
   using C = Cfg<D>;
   // The swizzled operand layouts need their tiles on 1-KB boundaries; there is no room for alignment slack, so the
   // dynamic part is declared with that alignment (and checked below).
@@ -241,18 +241,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
   uint8_t* ring_gen = smem_raw + C::kQBytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Geom& g = P.g;
-  const int n_items = P.dyn ? P.dyn[0] : P.n_items;                // fixed grid: the batch's counts live in device memory
-  if ((int)blockIdx.x >= n_items) return;
-
-  // The status word is set when a bounded wait runs out and stays set until tide_status clears it; while it is set
-  // no block starts work, so outputs are undefined from the time-out until the caller has read the status.
-  __shared__ int s_skip;
   if (threadIdx.x == 0) {
-    s_skip = *reinterpret_cast<volatile int*>(P.status);
-    if ((smem_q & 1023u) != 0) {             // cannot happen with the declared alignment; refuse rather than compute garbage
-      atomicExch(P.status, (int)TIDE_ERR_CUDA);
-      s_skip = 1;
-    }
+    if ((smem_q & 1023u) != 0) atomicExch(P.status, (int)TIDE_ERR_CUDA);   // cannot happen with the declared alignment; refuse rather than compute garbage
     s_abort = 0;
     for (int i = 0; i < C::kNumUnits; ++i) { mbar_init(smem_u32(&bars.kv_full[i]), 1); mbar_init(smem_u32(&bars.kv_empty[i]), 1); }
     for (int t = 0; t < 2; ++t) {
@@ -269,13 +259,14 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
     mbar_init(smem_u32(&bars.mma_done), 1);
     mbar_fence_init();
   }
-  __syncthreads();
-  if (s_skip != 0) return;
   if (warp == 9) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  if (!P.overlapped) grid_dep_wait();
+  grid_dep_launch();
+  const int n_items = P.dyn ? __ldcg(P.dyn) : P.n_items;           // fixed grid: the batch's counts live in device memory
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem_base;
@@ -313,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
         const int lp0 = kv_begin / g.S;
         auto load_ids = [&](int grp) -> int {
           const int lp = lp0 + grp * 32 + lane;
-          return lp < g.max_pages_per_task ? trow[lp] : 0;
+          return lp < g.max_pages_per_task ? __ldcg(trow + lp) : 0;
         };
         int ids_cur = load_ids(0), ids_nxt = load_ids(1), cur_grp = 0;
         for (int j = 0; j < n_tiles; ++j) {
@@ -456,26 +447,28 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
       }
     } else {
       // ================= warp 11: hands out the items and copies their queries =================
-      const int n_segs = P.dyn ? P.dyn[1] : P.n_segs;
+      const int n_segs = P.dyn ? __ldcg(P.dyn + 1) : P.n_segs;
       // copies of Q: lane -> row (mod 8) and 16-byte chunk (mod 4); eight rows on is dq tokens and dg heads on
       const int my_row = lane >> 2, my_chunk = lane & 3;
       const uint32_t my_swz0 = (uint32_t)((my_chunk ^ my_row) << 4), my_swz1 = (uint32_t)(((my_chunk + 4) ^ my_row) << 4);
       const int dq = 8 / g.G, dg = 8 - dq * g.G;
       const int src_step = (dq * g.Hq + dg) * D * 2, src_wrap = (g.Hq - g.G) * D * 2;
       int n_q[2] = {0, 0};
-      int item = (int)blockIdx.x, asks = 0;
+      int item = (int)blockIdx.x < n_items ? (int)blockIdx.x : -1, asks = 0;
       bool open = false;                                           // a question without an answer yet
       for (int it = 0; ; ++it) {
         const int slot = it % kItemSlots;
         if (it >= kItemSlots && !wait_all(bars.item_empty[slot], (it / kItemSlots - 1) & 1)) break;
         Item& w = items[slot];
+        // The status word is set when a bounded wait runs out and stays set until tide_status clears it.  While it is set
+        // no item is started, so outputs are undefined from the time-out until the caller has read the status.
         if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(P.status), 0) != 0) item = -1;
         if (item < 0) {
           if (lane == 0) { w.run = 0; mbar_arrive(smem_u32(&bars.item_full[slot])); }
           break;
         }
-        const int si = find_segment(n_segs, item, [&](int i) { return P.segs[i].item_base; });
-        const Segment seg = P.segs[si];
+        const int si = find_segment(n_segs, item, [&](int i) { return INLINE ? segs[i].item_base : __ldcg(&segs[i].item_base); });
+        const Segment seg = INLINE ? segs[si] : load_segment(segs + si);
         int local = item - seg.item_base;
         const int m_tile = local % seg.n_mtiles;
         local /= seg.n_mtiles;
@@ -770,13 +763,27 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const Atten
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }
+  if (P.overlapped) grid_dep_wait();
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1) attend_umma128_kernel(const AttendParams P) {
+  attend_umma128_body<D, false>(P, P.segs);
+}
+// Items whose row descriptors travel in the kernel's parameters (small batches).
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1) attend_umma128_inline_kernel(const __grid_constant__ AttendInline PI) {
+  attend_umma128_body<D, true>(PI.p, PI.segs);
 }
 
 }  // namespace umma128
 
 template <int D>
 static cudaError_t init_one() {
-  return cudaFuncSetAttribute(umma128::attend_umma128_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, umma128::Cfg<D>::kSmemBytes);
+  const cudaError_t e =
+      cudaFuncSetAttribute(umma128::attend_umma128_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, umma128::Cfg<D>::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(umma128::attend_umma128_inline_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, umma128::Cfg<D>::kSmemBytes);
 }
 cudaError_t attend_umma128_init() {
   const cudaError_t e = init_one<128>();
@@ -786,9 +793,15 @@ cudaError_t attend_umma128_init() {
 cudaError_t launch_attend_umma128(const AttendParams& p, cudaStream_t s) {
   const int grid = p.dyn ? p.grid_cap : p.n_items;
   if (grid <= 0) return cudaSuccess;
-  if (p.g.D == 128) umma128::attend_umma128_kernel<128><<<grid, umma128::kThreads, umma128::Cfg<128>::kSmemBytes, s>>>(p);
-  else umma128::attend_umma128_kernel<64><<<grid, umma128::kThreads, umma128::Cfg<64>::kSmemBytes, s>>>(p);
-  return cudaGetLastError();
+  if (p.g.D == 128) return launch_dep(umma128::attend_umma128_kernel<128>, grid, umma128::kThreads, umma128::Cfg<128>::kSmemBytes, s, p);
+  return launch_dep(umma128::attend_umma128_kernel<64>, grid, umma128::kThreads, umma128::Cfg<64>::kSmemBytes, s, p);
+}
+
+cudaError_t launch_attend_umma128_inline(const AttendInline& pi, cudaStream_t s) {
+  if (pi.p.n_items <= 0) return cudaSuccess;
+  if (pi.p.g.D == 128)
+    return launch_dep(umma128::attend_umma128_inline_kernel<128>, pi.p.n_items, umma128::kThreads, umma128::Cfg<128>::kSmemBytes, s, pi);
+  return launch_dep(umma128::attend_umma128_inline_kernel<64>, pi.p.n_items, umma128::kThreads, umma128::Cfg<64>::kSmemBytes, s, pi);
 }
 
 }  // namespace tide

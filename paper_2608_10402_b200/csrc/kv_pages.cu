@@ -25,6 +25,8 @@ cudaError_t launch_table_update(int32_t* table, const int32_t* idx, const int32_
 // Small host-to-device upload done by the SMs: src is pinned host memory mapped into the device's address space.
 // Unlike a copy-engine transfer it does not queue behind large copies that other streams have in flight.
 __global__ void upload_kernel(uint32_t* __restrict__ dst, const uint32_t* __restrict__ src, size_t n_words) {
+  grid_dep_wait();
+  grid_dep_launch();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_words; i += (size_t)gridDim.x * blockDim.x)
     dst[i] = src[i];
 }
@@ -33,8 +35,7 @@ cudaError_t launch_upload(void* dst, const void* src_mapped_host, size_t bytes, 
   if (bytes == 0) return cudaSuccess;
   const size_t n = bytes / 4;
   const unsigned blocks = (unsigned)std::min<size_t>((n + 255) / 256, 64);
-  upload_kernel<<<blocks, 256, 0, s>>>((uint32_t*)dst, (const uint32_t*)src_mapped_host, n);
-  return cudaGetLastError();
+  return launch_dep(upload_kernel, blocks, 256, 0, s, (uint32_t*)dst, (const uint32_t*)src_mapped_host, n);
 }
 
 constexpr int kAppendThreads = 256;
@@ -57,6 +58,8 @@ template <int SLABS>
 __device__ __forceinline__ void append_scatter_body(const AppendParams& P, const AppendRec* __restrict__ recs,
                                                   const int32_t* __restrict__ upd_idx, const int32_t* __restrict__ upd_val) {
   __shared__ int32_t s_grp0[kAppendMaxRecsSmem];
+  grid_dep_wait();
+  grid_dep_launch();
   const int n_recs = P.dyn ? P.dyn[0] : P.n_recs;
   for (int i = blockIdx.x * kAppendThreads + threadIdx.x; i < P.n_upd; i += gridDim.x * kAppendThreads)
     P.table_rw[upd_idx[i]] = upd_val[i];
@@ -139,18 +142,13 @@ static unsigned append_grid(const AppendParams& p) {
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s) {
   const int tokens = p.dyn ? p.grid_cap_tokens : p.n_tokens;
   if (tokens <= 0 && p.n_upd <= 0) return cudaSuccess;
-  const dim3 grid(append_grid(p));
-  if (p.g.D == 128) append_scatter_kernel<2><<<grid, kAppendThreads, 0, s>>>(p);
-  else append_scatter_kernel<1><<<grid, kAppendThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_dep(p.g.D == 128 ? append_scatter_kernel<2> : append_scatter_kernel<1>, append_grid(p), kAppendThreads, 0, s, p);
 }
 
 cudaError_t launch_append_inline(const AppendInline& pi, cudaStream_t s) {
   if (pi.p.n_tokens <= 0 && pi.p.n_upd <= 0) return cudaSuccess;
-  const dim3 grid(append_grid(pi.p));
-  if (pi.p.g.D == 128) append_scatter_inline_kernel<2><<<grid, kAppendThreads, 0, s>>>(pi);
-  else append_scatter_inline_kernel<1><<<grid, kAppendThreads, 0, s>>>(pi);
-  return cudaGetLastError();
+  return launch_dep(pi.p.g.D == 128 ? append_scatter_inline_kernel<2> : append_scatter_inline_kernel<1>, append_grid(pi.p), kAppendThreads, 0,
+                    s, pi);
 }
 
 // Whole-page copies dst[i] <- src[i] (the private copy a forked task gets of a partial last page, and the copy an

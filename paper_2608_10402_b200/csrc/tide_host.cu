@@ -91,6 +91,7 @@ struct tide_kv {
   float* d_part_lse = nullptr;
   AppendInline append_inline;   // host images of the launches that carry their descriptors
   AttendInline attend_inline;
+  MergeInline merge_inline;
   int* d_merge_ctr = nullptr;   // finished-split counters of the segments whose last split merges (zero between launches)
   Slot slots[kSlots];
   int next_slot = 0;
@@ -1183,8 +1184,9 @@ static PlanDev pack_plan(const PlanHost& P, Segment* h, const Segment* d, size_t
 }
 
 // The attention launches of one planned batch on one layer: kernel launches only (and, with `events`, the phase
-// time stamps), so a caller may capture them in a CUDA graph.
-static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const int32_t* page_table, const void* q, float scale,
+// time stamps), so a caller may capture them in a CUDA graph.  With `inl` the row descriptors come from that plan and
+// travel in the launches' parameters; otherwise they are on the device, where `d` says.
+static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanHost* inl, const int32_t* page_table, const void* q, float scale,
                        void* out, float* lse, cudaStream_t st, bool events, int64_t* n_launches, const int32_t* dyn) {
   AttendParams ap;
   ap.pool = kv->layer_pool(layer);
@@ -1203,28 +1205,45 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const int32
   kv->drop_first_stage_once = false;
   int64_t launches = 0;
   // dyn != nullptr: fixed launch shapes; the counts of the batch are read on the device (header of the step area)
-  if (events) cudaEventRecord(kv->ev_attend[0], st);
-  if (dyn ? kv->cap_dec > 0 : d.items_dec > 0) {
+  const bool dec = dyn ? kv->cap_dec > 0 : d.items_dec > 0, tile = dyn ? kv->cap_tile > 0 : d.items_tile > 0;
+  const bool umma = dyn ? kv->cap_umma > 0 : d.items_umma > 0, merge = dyn ? kv->cap_merge_rows > 0 : d.merge_rows > 0;
+  auto inline_segs = [&](const std::vector<Segment>& v) -> AttendInline& {
+    AttendInline& pi = kv->attend_inline;
+    std::copy(v.begin(), v.end(), pi.segs);
+    pi.p = ap;
+    return pi;
+  };
+  auto launch_dec = [&](bool overlapped) -> cudaError_t {
     ap.segs = d.seg_dec; ap.n_segs = (int)d.n_dec; ap.n_items = (int)d.items_dec;
-    ap.dyn = dyn ? dyn + kHdrDecItems : nullptr; ap.grid_cap = kv->cap_dec;
-    if (launch_attend_decode(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
+    ap.dyn = dyn ? dyn + kHdrDecItems : nullptr; ap.grid_cap = kv->cap_dec; ap.overlapped = overlapped ? 1 : 0;
     ++launches;
-  }
-  if (events) cudaEventRecord(kv->ev_attend[1], st);
-  if (dyn ? kv->cap_tile > 0 : d.items_tile > 0) {
-    ap.segs = d.seg_tile; ap.n_segs = (int)d.n_tile; ap.n_items = (int)d.items_tile;
-    ap.dyn = dyn ? dyn + kHdrTileItems : nullptr; ap.grid_cap = kv->cap_tile;
-    if (launch_attend_tile(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
-    ++launches;
-  }
-  if (dyn ? kv->cap_umma > 0 : d.items_umma > 0) {
+    return inl ? launch_attend_decode_inline(inline_segs(inl->seg_dec), st) : launch_attend_decode(ap, st);
+  };
+  auto launch_umma = [&]() -> cudaError_t {
     ap.segs = d.seg_umma; ap.n_segs = (int)d.n_umma; ap.n_items = (int)d.items_umma;
-    ap.dyn = dyn ? dyn + kHdrUmmaItems : nullptr; ap.grid_cap = kv->cap_umma;
-    if ((kv->umma_tile_keys == 128 ? launch_attend_umma128(ap, st) : launch_attend_umma(ap, st)) != cudaSuccess) return TIDE_ERR_CUDA;
+    ap.dyn = dyn ? dyn + kHdrUmmaItems : nullptr; ap.grid_cap = kv->cap_umma; ap.overlapped = 0;
     ++launches;
+    if (kv->umma_tile_keys != 128) return launch_attend_umma(ap, st);
+    return inl ? launch_attend_umma128_inline(inline_segs(inl->seg_umma), st) : launch_attend_umma128(ap, st);
+  };
+  if (events) cudaEventRecord(kv->ev_attend[0], st);
+  if (dec && umma && !tile && kv->umma_tile_keys == 128 && !events) {
+    // The two kernels do not depend on each other.  The tensor-bound one goes first; the decode blocks start on SMs that
+    // it leaves idle (a small batch) or as its last items end.
+    if (launch_umma() != cudaSuccess || launch_dec(true) != cudaSuccess) return TIDE_ERR_CUDA;
+  } else {
+    if (dec && launch_dec(false) != cudaSuccess) return TIDE_ERR_CUDA;
+    if (events) cudaEventRecord(kv->ev_attend[1], st);
+    if (tile) {
+      ap.segs = d.seg_tile; ap.n_segs = (int)d.n_tile; ap.n_items = (int)d.items_tile;
+      ap.dyn = dyn ? dyn + kHdrTileItems : nullptr; ap.grid_cap = kv->cap_tile; ap.overlapped = 0;
+      if (launch_attend_tile(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
+      ++launches;
+    }
+    if (umma && launch_umma() != cudaSuccess) return TIDE_ERR_CUDA;
   }
   if (events) cudaEventRecord(kv->ev_attend[2], st);
-  if (dyn ? kv->cap_merge_rows > 0 : d.merge_rows > 0) {
+  if (merge) {
     MergeParams mp;
     mp.segs = d.seg_merge;
     mp.n_segs = (int)d.n_merge;
@@ -1232,7 +1251,14 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const int32
     mp.part_o = kv->d_part_o; mp.part_lse = kv->d_part_lse;
     mp.out = (uint16_t*)out; mp.lse = lse; mp.Hq = kv->g.Hq; mp.D = kv->g.D;
     mp.dyn = dyn ? dyn + kHdrMergeRows : nullptr; mp.grid_cap_rows = kv->cap_merge_rows;
-    if (launch_merge(mp, st) != cudaSuccess) return TIDE_ERR_CUDA;
+    cudaError_t e;
+    if (inl) {
+      MergeInline& mi = kv->merge_inline;
+      std::copy(inl->seg_merge.begin(), inl->seg_merge.end(), mi.segs);
+      mi.p = mp;
+      e = launch_merge_inline(mi, st);
+    } else e = launch_merge(mp, st);
+    if (e != cudaSuccess) return TIDE_ERR_CUDA;
     ++launches;
   }
   if (events) {
@@ -1257,50 +1283,23 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
   if (P.n_all() * sizeof(Segment) + 256 > kv->lay.slot_bytes) return TIDE_ERR_WORKSPACE;
 
   cudaStream_t st = (cudaStream_t)stream;
-  if (kv->inline_descriptors && P.seg_tile.empty() && P.seg_umma.empty() && P.seg_merge.empty() &&
-      P.seg_dec.size() <= (size_t)kInlineSegs) {
-    // A small decode-only batch: the row descriptors travel in the decode launch's own parameters (no upload).
-    AttendInline& pi = kv->attend_inline;
-    std::copy(P.seg_dec.begin(), P.seg_dec.end(), pi.segs);
-    AttendParams& ap = pi.p;
-    ap = AttendParams();
-    ap.pool = kv->layer_pool(layer);
-    ap.table = page_table ? page_table : kv->d_table;
-    ap.n_segs = (int)P.seg_dec.size();
-    ap.n_items = (int)P.items_dec;
-    ap.q = (const uint16_t*)q;
-    ap.out = (uint16_t*)out;
-    ap.lse = lse;
-    ap.part_o = kv->d_part_o;
-    ap.part_lse = kv->d_part_lse;
-    ap.scale_log2e = scale * 1.4426950408889634f;
-    ap.status = kv->d_status;
-    ap.g = kv->g;
-    ap.merge_ctr = kv->d_merge_ctr;
-    ap.wait_limit_ns = kv->wait_limit_ns;
-    ap.debug_drop_first_stage = kv->drop_first_stage_once ? 1 : 0;
-    kv->drop_first_stage_once = false;
-    if (kv->profiling) cudaEventRecord(kv->ev_attend[0], st);
-    if (launch_attend_decode_inline(pi, st) != cudaSuccess) return TIDE_ERR_CUDA;
-    if (kv->profiling) {
-      for (int i = 1; i <= 3; ++i) cudaEventRecord(kv->ev_attend[i], st);
-      kv->have_attend_times = true;
-    }
-    kv->last_decode_items = P.items_dec;
-    kv->last_prefill_items = 0;
-    kv->last_merge_rows = P.fused_rows;
-    kv->last_launches = 1 + kv->append_launches;
-    kv->append_launches = 0;
-    return TIDE_OK;
-  }
-  Slot* slot;
-  if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
-  const PlanDev pd = pack_plan(P, (Segment*)(slot->host + 256), (const Segment*)(slot->dev + 256), 0);
-  if (upload(kv, slot->dev + 256, slot->host + 256, P.n_all() * sizeof(Segment), st) != cudaSuccess)
-    return TIDE_ERR_CUDA;
   int64_t launches = 0;
-  if ((rc = launch_plan(kv, layer, pd, page_table, q, scale, out, lse, st, kv->profiling, &launches, nullptr)) != TIDE_OK) return rc;
-  if ((rc = release_slot(slot, st)) != TIDE_OK) return rc;
+  PlanDev pd;
+  if (kv->inline_descriptors && P.seg_tile.empty() && (P.seg_umma.empty() || kv->umma_tile_keys == 128) &&
+      P.seg_dec.size() <= (size_t)kInlineSegs && P.seg_umma.size() <= (size_t)kInlineSegs && P.seg_merge.size() <= (size_t)kInlineSegs) {
+    // a small batch: the row descriptors travel in the launches' own parameters (no upload)
+    pd.n_dec = P.seg_dec.size(); pd.n_umma = P.seg_umma.size(); pd.n_merge = P.seg_merge.size();
+    pd.items_dec = P.items_dec; pd.items_umma = P.items_umma; pd.merge_rows = P.merge_rows;
+    if ((rc = launch_plan(kv, layer, pd, &P, page_table, q, scale, out, lse, st, kv->profiling, &launches, nullptr)) != TIDE_OK) return rc;
+  } else {
+    Slot* slot;
+    if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
+    pd = pack_plan(P, (Segment*)(slot->host + 256), (const Segment*)(slot->dev + 256), 0);
+    if (upload(kv, slot->dev + 256, slot->host + 256, P.n_all() * sizeof(Segment), st) != cudaSuccess)
+      return TIDE_ERR_CUDA;
+    if ((rc = launch_plan(kv, layer, pd, nullptr, page_table, q, scale, out, lse, st, kv->profiling, &launches, nullptr)) != TIDE_OK) return rc;
+    if ((rc = release_slot(slot, st)) != TIDE_OK) return rc;
+  }
   kv->last_decode_items = pd.items_dec;
   kv->last_prefill_items = pd.items_tile + pd.items_umma;
   kv->last_merge_rows = pd.merge_rows + P.fused_rows;
@@ -1421,7 +1420,7 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   ap.g = kv->g;
   if (launch_append(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
   int64_t launches = 0;
-  const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, q, scale, out, lse, st, false, &launches, dyn);
+  const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, nullptr, q, scale, out, lse, st, false, &launches, dyn);
   if (rc != TIDE_OK) return rc;
   kv->last_launches = launches + 1;
   return TIDE_OK;

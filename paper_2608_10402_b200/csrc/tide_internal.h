@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "../../include/tide.h"
 
 namespace tide {
@@ -87,6 +89,7 @@ struct AttendParams {
   int grid_cap = 0;
   int* merge_ctr = nullptr;   // per (segment with partial == 2, kv head): splits finished so far; zero between launches
   long long wait_limit_ns = kWaitLimitNsDefault;   // bound of every wait inside the kernel
+  int overlapped = 0;         // the kernel before this one in the stream is the other attention kernel of the same batch (see grid_dep_wait)
   // Test hook for the bounded waits (never set in normal use): in work item 0 the producer leaves out its part
   // of the first stage, so the consumers' wait for that stage runs out and the time-out path executes.
   int debug_drop_first_stage = 0;
@@ -138,14 +141,19 @@ struct AppendParams {
   int n_upd = 0;
 };
 
-// Small batches carry their descriptors in the launch itself: a decode-only batch of up to kInlineSegs rows, and an
-// append of up to kInlineRecs records with up to kInlineUpd new page-table entries, need no upload before the kernel
-// (the kernels read them from their own parameter space), which takes one launch each out of a decode step.
+// Small batches carry their descriptors in the launches themselves: an attention call whose kernels have up to kInlineSegs
+// row descriptors each, and an append of up to kInlineRecs records with up to kInlineUpd new page-table entries, need no
+// upload before the kernels (these read them from their own parameter space), which takes one launch each out of a step.
+// A launch with 8.6 KB of parameters costs the host 1.9 us, one with 64 bytes 1.8.
 constexpr int kInlineSegs = 128;
 constexpr int kInlineRecs = 128;
 constexpr int kInlineUpd = 256;
 struct AttendInline {
   AttendParams p;                  // p.segs is not used
+  Segment segs[kInlineSegs];
+};
+struct MergeInline {
+  MergeParams p;                   // p.segs is not used
   Segment segs[kInlineSegs];
 };
 struct AppendInline {
@@ -178,15 +186,47 @@ cudaError_t launch_attend_decode_inline(const AttendInline& p, cudaStream_t s); 
 cudaError_t launch_append_inline(const AppendInline& p, cudaStream_t s);
 cudaError_t launch_attend_tile(const AttendParams& p, cudaStream_t s);
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t s);
+cudaError_t launch_merge_inline(const MergeInline& p, cudaStream_t s);
 cudaError_t launch_attend_umma(const AttendParams& p, cudaStream_t s);
 cudaError_t attend_kernels_init();
 cudaError_t attend_decode_init();
 cudaError_t attend_umma_init();
 cudaError_t launch_attend_umma128(const AttendParams& p, cudaStream_t s);
+cudaError_t launch_attend_umma128_inline(const AttendInline& p, cudaStream_t s);
 cudaError_t attend_umma128_init();
 int sm_count();   // multiprocessors of the current device (looked up once per device)
 
 #ifdef __CUDACC__
+// ---------------------------------------------------------------------------------------------
+// Launches of one stream overlap at their edges (programmatic dependent launch): a kernel may start while the one before
+// it still runs, once every block of that one has called grid_dep_launch (or left), and calls grid_dep_wait before it
+// touches anything that earlier work of the stream reads or writes.  A kernel boundary without it costs 1 to 2.5 us of
+// launch latency, and the blocks' set-up on top.
+// Measured (with the descriptors in the launches): four-task step 34.4 to 21.7 us, forked groups 103 to 90 us, eight layers
+// of decode rows 584 to 569 us, a prune-and-resume turn 1294 to 1215 us; nothing at 64 decode rows and above.
+// The rule that keeps the chain of dependencies whole: every kernel calls grid_dep_wait before it ends, and calls
+// grid_dep_launch only after everything that the NEXT kernel may rely on without waiting is complete.  The two attention
+// kernels of one batch do not depend on each other: the second one (AttendParams::overlapped) starts without waiting -
+// the first has waited for all earlier work before it let the second one start - and waits when it is done, so that what
+// follows it in the stream still follows both.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
+template <typename... A>
+cudaError_t launch_dep(void (*kernel)(A...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, const std::common_type_t<A>&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  void* ptrs[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), ptrs);
+}
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------------------------
 // device helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -319,6 +359,12 @@ __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+__device__ __forceinline__ Segment load_segment(const Segment* p) {      // through L2
+  Segment s;
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(Segment) / 16); ++i) reinterpret_cast<uint4*>(&s)[i] = __ldcg(reinterpret_cast<const uint4*>(p) + i);
+  return s;
 }
 // Locate the segment that owns work index `idx` (segments sorted by the base returned by `base_of`).
 template <typename F>

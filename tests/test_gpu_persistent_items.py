@@ -123,3 +123,60 @@ def test_many_decode_items_per_thread_block(geom, n_rows, fixed):
     kv.attend(rows, dq, scale, out, lse)
     assert kv.status() == tide.OK and torch.equal(first, out)
     kv.close()
+
+
+@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (12, 4, 64, 16)])
+@pytest.mark.parametrize("layers", [1, 2])
+def test_steps_queued_without_waiting_follow_one_another(geom, layers):
+    """Kernels of one stream overlap at their edges: steps queued back to back (decode rows, resume rows and split rows
+    in one batch; their own output buffers) each see the tokens of the steps before them and nothing of those after."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    from oracle.layers import LayeredKVOracle
+    HQ, HKV, D, S = geom
+    rng = np.random.default_rng(HQ + D + layers)
+    scale = 1.0 / math.sqrt(D)
+    B, steps = 9, 12
+    prefix = [0, 15, 16, 130, 700, 1500, 2500, 60, 300]
+    cnt = [[1 if (b + s) % 3 else int(rng.integers(1, 70)) for b in range(B)] for s in range(steps)]
+    pages = sum((p + sum(c[b] for c in cnt) + S - 1) // S for b, p in enumerate(prefix)) + 4
+    T = max(sum(c) for c in cnt)
+    kv = tide.TideKV(HQ, HKV, D, S, pages, B, pages, B, max(T, 128), num_layers=layers)
+    orc = LayeredKVOracle(layers, num_pages=pages, page_size=S, num_kv_heads=HKV, head_dim=D, max_tasks=B, max_pages_per_task=pages)
+    ids = list(range(B))
+    queue = []
+    for s in range(-1, steps):
+        n = prefix if s < 0 else cnt[s]
+        ip = np.concatenate([[0], np.cumsum(n)]).astype(np.int32)
+        shape = lambda h: (layers, int(ip[-1]), h, D)
+        k, v, q = (inputs.normal_bf16(rng, shape(h)) for h in (HKV, HKV, HQ))
+        queue.append((ip, k, v, q, *(H.to_dev(x, torch) for x in (k, v, q)), torch.zeros(shape(HQ), dtype=torch.int16, device="cuda"),
+                      torch.zeros(shape(HQ)[:3], dtype=torch.float32, device="cuda")))
+    for t in ids:
+        kv.alloc(t)
+        orc.alloc(t)
+    ip, _, _, _, dk, dv, *_ = queue[0]
+    kv.extend(ids, ip)
+    for l in range(layers):
+        kv.write(l, ids, ip, dk[l], dv[l])
+    torch.cuda.synchronize()
+    length = list(prefix)
+    for ip, _, _, _, dk, dv, dq, out, lse in queue[1:]:
+        length = [a + int(b) for a, b in zip(length, np.diff(ip))]
+        rows = [(t, int(ip[t + 1] - ip[t]), length[t]) for t in ids]
+        if layers > 1:
+            kv.step_begin(rows)
+            for l in range(layers):
+                kv.step_layer(l, dk[l], dv[l], dq[l], scale, out[l], lse[l])
+        else:
+            kv.append(ids, ip, dk[0], dv[0])
+            kv.attend(rows, dq[0], scale, out[0], lse[0])
+    assert kv.status() == tide.OK
+    orc.append(ids, *queue[0][:3])
+    for s, (ip, k, v, q, _, _, _, out, lse) in enumerate(queue[1:]):
+        orc.append(ids, ip, k, v)
+        rows = [(t, int(ip[t + 1] - ip[t]), orc.task_len(t)) for t in ids]
+        for l in range(layers):
+            ref_o, ref_l = cbuild.attend_paged(orc.layer(l), rows, q[l], scale)
+            H.check_outputs(H.from_dev(out[l]), lse[l].cpu().numpy(), ref_o, ref_l, f"step {s}, layer {l}")
+    kv.close()
