@@ -107,7 +107,7 @@ __device__ __forceinline__ void append_scatter_body(const AppendParams& P, const
         const int slab = e >> 6, row = (e >> 3) & 7, c = (e & 7) ^ row;
         v[k][i] = make_uint4(0, 0, 0, 0);
         if (hh < heads2 && row >= lo && row < hi)
-          v[k][i] = __ldg(reinterpret_cast<const uint4*>(src + (long long)row * g.Hkv * g.D + (slab * 8 + c) * 8));
+          v[k][i] = __ldcg(reinterpret_cast<const uint4*>(src + (long long)row * g.Hkv * g.D + (slab * 8 + c) * 8));
       }
     }
 #pragma unroll
@@ -166,6 +166,127 @@ cudaError_t launch_copy_pages(uint8_t* pool, const int32_t* src, const int32_t* 
   dim3 grid(8, (unsigned)n);
   copy_pages_kernel<<<grid, 256, 0, s>>>(pool, src, dst, page_bytes);
   return cudaGetLastError();
+}
+
+// Sliding-window pruning in place: positions [to, to + n) of a task take the content of [to + shift, to + shift + n), on
+// every layer.  The task keeps its pages, so this is a move inside its own page list by a distance that need not be a
+// multiple of anything, bound by memory: 2 * Hkv * D * 2 bytes read and as many written per token.  (Staged through the
+// workspace - table update, gather, scatter and two uploads per chunk of max_batch_tokens - eight tasks with tails of 4k
+// to 16k tokens took 390 us, mostly launches; this way they take about 100.)  The moves of different tasks do not depend on
+// each other: one that directly follows another (`overlapped`) runs beside it.
+//
+// Large shifts: position d depends only on d + shift, so the positions of one residue modulo the shift form a chain that
+// one thread walks front to back, always reading ahead of what it writes; chains are independent of one another.
+constexpr int kMoveLinks = 4;
+constexpr int kMoveChainsFrom = 64;   // shift from which chains are faster than runs (4 KV heads, D = 128, tail of 4000 / 16000 tokens: shift 32
+                                      // 43 / 156 us by chains and 29 / 90 by runs, 64 27 / 80 and 33 / 90, 128 16 / 45 and 33 / 90, 512 12 / 20 and 33 / 94)
+template <int SLABS>
+__global__ void __launch_bounds__(256) move_chains_kernel(uint8_t* pool0, size_t layer_stride, const int32_t* __restrict__ table_row, int to,
+                                                          int shift, int n, int overlapped, const Geom g) {
+  constexpr int CPR = SLABS * 8;                              // 16-byte chunks of a row: that many neighbouring lanes move one
+  if (!overlapped) grid_dep_wait();
+  grid_dep_launch();
+  uint8_t* const pool = pool0 + (size_t)blockIdx.y * layer_stride;
+  const int chains = min(shift, n);
+  // rows of one (kv, head) whose chains start at neighbouring positions go to neighbouring lanes: whole lines of an atom
+  const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CPR;
+  const int c = threadIdx.x % CPR;
+  const int hh = (int)(row / chains), first = (int)(row - (long long)hh * chains);
+  const int kv = hh >= g.Hkv ? 1 : 0;
+  const long long head = (long long)(hh - kv * g.Hkv) * g.head_bytes;
+  auto at = [&](long long pos) -> uint4* {
+    const int lp = (int)pos / g.S;
+    return reinterpret_cast<uint4*>(pool + (long long)__ldcg(table_row + lp) * g.page_bytes + head + blk_offset(g, (int)pos - lp * g.S, kv, c));
+  };
+  const long long end = hh < 2 * g.Hkv ? (long long)to + n : 0;
+  // kMoveLinks links from position d on: the address of the first target is known, a[i + 1] is link i's source and the
+  // target of link i + 1.  The next links are loaded before these are stored.
+  uint4 *a0[kMoveLinks + 1], *a1[kMoveLinks + 1];
+  uint4 v0[kMoveLinks], v1[kMoveLinks];
+  auto load = [&](long long d, uint4* target, uint4* (&a)[kMoveLinks + 1], uint4 (&v)[kMoveLinks]) {
+    a[0] = target;
+#pragma unroll
+    for (int i = 0; i < kMoveLinks; ++i) a[i + 1] = d + (long long)i * shift < end ? at(d + (i + 1ll) * shift) : target;
+#pragma unroll
+    for (int i = 0; i < kMoveLinks; ++i) v[i] = __ldcg(a[i + 1]);
+  };
+  auto store = [&](long long d, uint4* const (&a)[kMoveLinks + 1], const uint4 (&v)[kMoveLinks]) {
+#pragma unroll
+    for (int i = 0; i < kMoveLinks; ++i)
+      if (d + (long long)i * shift < end) *a[i] = v[i];
+  };
+  const long long step = (long long)kMoveLinks * shift;
+  long long d = to + first;
+  if (d < end) load(d, at(d), a0, v0);
+  while (d < end) {
+    if (d + step < end) load(d + step, a0[kMoveLinks], a1, v1);
+    store(d, a0, v0);
+    d += step;
+    if (d >= end) break;
+    if (d + step < end) load(d + step, a1[kMoveLinks], a0, v0);
+    store(d, a1, v1);
+    d += step;
+  }
+  if (overlapped) grid_dep_wait();
+}
+
+// Small shifts have few chains.  One block per (layer, kv, head, 64-element slab) moves a run of rows at a time, front to
+// back: the whole run is in registers before its first row is stored (the run's last sources lie behind its targets, so
+// no later run is touched), and the next run is loaded before this one is stored.
+constexpr int kMoveThreads = 512, kMoveRows = 8;              // 16-byte chunks per thread and run: 512 rows of 128 bytes
+template <int SLABS>
+__global__ void __launch_bounds__(kMoveThreads) move_runs_kernel(uint8_t* pool0, size_t layer_stride, const int32_t* __restrict__ table_row, int to,
+                                                                 int shift, int n, int overlapped, const Geom g) {
+  if (!overlapped) grid_dep_wait();
+  grid_dep_launch();
+  uint8_t* const pool = pool0 + (size_t)blockIdx.y * layer_stride;
+  const int slab = blockIdx.x % SLABS, hh = blockIdx.x / SLABS, kv = hh >= g.Hkv ? 1 : 0;
+  const long long head = (long long)(hh - kv * g.Hkv) * g.head_bytes;
+  const int c = slab * 8 + threadIdx.x % 8, r0 = threadIdx.x / 8;
+  constexpr int kRun = kMoveThreads / 8 * kMoveRows, kStep = kMoveThreads / 8;
+  auto at = [&](int pos) -> uint4* {
+    const int lp = pos / g.S;
+    return reinterpret_cast<uint4*>(pool + (long long)__ldcg(table_row + lp) * g.page_bytes + head + blk_offset(g, pos - lp * g.S, kv, c));
+  };
+  uint4 v[2][kMoveRows];
+  auto load = [&](int run, uint4 (&x)[kMoveRows]) {
+#pragma unroll
+    for (int i = 0; i < kMoveRows; ++i) {
+      x[i] = __ldcg(at(to + shift + min(run + r0 + i * kStep, n - 1)));   // (no branch: the loads go out side by side)
+    }
+  };
+  auto store = [&](int run, const uint4 (&x)[kMoveRows]) {
+#pragma unroll
+    for (int i = 0; i < kMoveRows; ++i) {
+      const int r = run + r0 + i * kStep;
+      uint4* const dst = at(to + min(r, n - 1));
+      if (r < n) *dst = x[i];
+    }
+  };
+  load(0, v[0]);
+  for (int run = 0; run < n; run += 2 * kRun) {
+    __syncthreads();                                          // every thread has loaded run `run`
+    load(run + kRun, v[1]);
+    store(run, v[0]);
+    __syncthreads();
+    load(run + 2 * kRun, v[0]);
+    store(run + kRun, v[1]);
+  }
+  if (overlapped) grid_dep_wait();
+}
+
+cudaError_t launch_move(uint8_t* pool, size_t layer_stride, int layers, const int32_t* table_row, int to, int shift, int n, bool overlapped,
+                        const Geom& g, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (shift >= kMoveChainsFrom) {
+    const long long threads = (long long)std::min(shift, n) * 2 * g.Hkv * (g.D / 8);
+    const dim3 grid((unsigned)((threads + 255) / 256), (unsigned)layers);
+    return launch_dep(g.D == 128 ? move_chains_kernel<2> : move_chains_kernel<1>, grid, 256, 0, s, pool, layer_stride, table_row, to, shift, n,
+                      overlapped ? 1 : 0, g);
+  }
+  const dim3 grid((unsigned)(2 * g.Hkv * (g.D / 64)), (unsigned)layers);
+  return launch_dep(g.D == 128 ? move_runs_kernel<2> : move_runs_kernel<1>, grid, kMoveThreads, 0, s, pool, layer_stride, table_row, to, shift, n,
+                      overlapped ? 1 : 0, g);
 }
 
 // Logical content of one task -> contiguous [len, Hkv, D]; inverse of the scatter above.

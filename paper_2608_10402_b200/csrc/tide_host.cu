@@ -105,6 +105,11 @@ struct tide_kv {
   ExtendOut ext;              // result of the most recent extension
   std::vector<int32_t> mark;  // scratch for duplicate detection
   int32_t mark_gen = 0;
+  // moves of pruned tasks launched one after the other on one stream, with no other device work of this handle between
+  bool moves_open = false;
+  cudaStream_t moves_stream = nullptr;
+  std::vector<int64_t> move_mark;   // per task: the series (move_gen) it was last moved in
+  int64_t move_gen = 0;
   int64_t used_tokens = 0;
   // last plan
   int64_t last_decode_items = 0, last_prefill_items = 0, last_merge_rows = 0, last_launches = 0;
@@ -342,6 +347,7 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
   kv->len.assign((size_t)cfg->max_tasks, 0);
   kv->pages.resize((size_t)cfg->max_tasks);
   kv->mark.assign((size_t)cfg->max_tasks, 0);
+  kv->move_mark.assign((size_t)cfg->max_tasks, 0);
   kv->refcnt.assign((size_t)cfg->num_pages, 0);
   prime_free_stack(kv, cfg->free_order);
   *out = kv;
@@ -491,6 +497,7 @@ static int extend_bookkeeping(tide_kv* kv, int32_t n_tasks, const int32_t* task_
   if (rc != TIDE_OK) return rc;
   // ---- mutation ----
   kv->step_valid = false;
+  kv->moves_open = false;
   ExtendOut& x = kv->ext;
   x.clear();
   for (int j = 0; j < n_tasks; ++j) {
@@ -592,6 +599,7 @@ static int write_tasks(tide_kv* kv, int32_t layer, int32_t n_tasks, const int32_
   const Geom& g = kv->g;
   int j = 0;
   int rc = TIDE_OK;
+  kv->moves_open = false;
   while (j < n_tasks) {
     Slot* slot;
     if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
@@ -762,6 +770,7 @@ int tide_kv_read(tide_kv_t* kv, int32_t layer, int32_t task, void* out_k, void* 
   if (kv->len[task] == 0) return TIDE_OK;
   if (out_k == nullptr || out_v == nullptr || ((uintptr_t)out_k & 15) || ((uintptr_t)out_v & 15)) return TIDE_ERR_INVALID_ARG;
   const int32_t* row = kv->d_table + (size_t)task * kv->g.max_pages_per_task;
+  kv->moves_open = false;
   if (launch_read(kv->layer_pool(layer), row, 0, kv->len[task], (uint16_t*)out_k, (uint16_t*)out_v, kv->g, (cudaStream_t)stream) != cudaSuccess)
     return TIDE_ERR_CUDA;
   return TIDE_OK;
@@ -777,6 +786,7 @@ int tide_kv_fork(tide_kv_t* kv, int32_t layer, int32_t parent, int32_t child, vo
   const bool partial = L % g.S != 0;
   if (partial && kv->free_stack.empty()) return TIDE_ERR_NO_PAGES;
   cudaStream_t st = (cudaStream_t)stream;
+  kv->moves_open = false;
   // ---- bookkeeping: share the full pages, take one fresh page for the copy of the partial one ----
   auto& cp = kv->pages[child];
   cp.assign(kv->pages[parent].begin(), kv->pages[parent].begin() + n_full);
@@ -879,8 +889,8 @@ int tide_kv_prune(tide_kv_t* kv, int32_t layer, int32_t task, int32_t keep_prefi
   if (tail > 0 && keep_prefix % g.S != 0 && kv->refcnt[(size_t)pg[(size_t)first]] > 1) ++need;
   if (need > (long long)kv->free_stack.size() + freed) return TIDE_ERR_NO_PAGES;
   const int chunk_cap = (int)std::min<int64_t>(kv->cfg.max_batch_tokens, 0x7fffffff);
-  // A task that shares none of these pages gets the same pages back in the same places, so its tail can move in
-  // place, chunk by chunk.  Otherwise its new pages differ from the old ones and may be old ones in other places:
+  // A task that shares none of these pages gets the same pages back in the same places, so its tail moves in place and
+  // the device table stays as it is.  Otherwise its new pages differ from the old ones and may be old ones in other places:
   // the whole tail of a layer has to sit in the staging area before anything of that layer is written.
   if (shared_any && tail > chunk_cap) return TIDE_ERR_WORKSPACE;
 
@@ -891,18 +901,17 @@ int tide_kv_prune(tide_kv_t* kv, int32_t layer, int32_t task, int32_t keep_prefi
   const int L = kv->cfg.num_layers;
   int rc;
   if (!shared_any) {
-    if ((rc = tide_kv_truncate(kv, task, keep_prefix)) != TIDE_OK) return rc;
-    // front to back: a chunk is written below the positions the next one reads
-    for (int done = 0; done < tail; done += chunk_cap) {
-      const int n = std::min(chunk_cap, tail - done);
-      const int32_t ip[2] = {0, n};
-      if ((rc = extend_tasks(kv, 1, &task, ip, st, nullptr)) != TIDE_OK) return rc;
-      for (int l = 0; l < L; ++l) {
-        if (launch_read(kv->layer_pool(l), row, tail_begin + done, n, sk, sv, g, st) != cudaSuccess) return TIDE_ERR_CUDA;
-        if ((rc = write_tasks(kv, l, 1, &task, ip, sk, sv, st)) != TIDE_OK) return rc;
-      }
+    // a move right behind other tasks' moves on the same stream need not wait for them
+    const bool overlapped = kv->moves_open && kv->moves_stream == st && kv->move_mark[(size_t)task] != kv->move_gen;
+    if (!overlapped) ++kv->move_gen;
+    if (tail > 0 && launch_move(kv->pool, kv->layer_stride, L, row, keep_prefix, tail_begin - keep_prefix, tail, overlapped, g, st) != cudaSuccess)
+      return TIDE_ERR_CUDA;
+    if (tail > 0) {
+      kv->moves_open = true;
+      kv->moves_stream = st;
+      kv->move_mark[(size_t)task] = kv->move_gen;
     }
-    return TIDE_OK;
+    return tide_kv_truncate(kv, task, keep_prefix + tail);
   }
   // keep the row as it is now: the tail is read through it after the table has changed
   if (cudaMemcpyAsync(kv->d_old_row, row, pg.size() * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return TIDE_ERR_CUDA;
@@ -1188,6 +1197,7 @@ static PlanDev pack_plan(const PlanHost& P, Segment* h, const Segment* d, size_t
 // travel in the launches' parameters; otherwise they are on the device, where `d` says.
 static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanHost* inl, const int32_t* page_table, const void* q, float scale,
                        void* out, float* lse, cudaStream_t st, bool events, int64_t* n_launches, const int32_t* dyn) {
+  kv->moves_open = false;
   AttendParams ap;
   ap.pool = kv->layer_pool(layer);
   ap.table = page_table ? page_table : kv->d_table;
@@ -1654,6 +1664,7 @@ int tide_tune(tide_kv_t* kv, int knob, int64_t value) {
 // Read-only view of a handle for attend_static.cu (not part of the public header).
 int tide_internal_view(tide_kv_t* kv, tide::StaticView* v) {
   if (kv == nullptr || v == nullptr) return TIDE_ERR_INVALID_ARG;
+  kv->moves_open = false;
   v->g = kv->g;
   v->pool = kv->pool;
   v->table = kv->d_table;

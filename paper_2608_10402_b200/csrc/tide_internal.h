@@ -178,6 +178,9 @@ struct StaticView {
 cudaError_t launch_table_update(int32_t* table, const int32_t* idx, const int32_t* val, int n, cudaStream_t s);
 cudaError_t launch_upload(void* dst, const void* src_mapped_host, size_t bytes, cudaStream_t s);   // bytes % 4 == 0
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s);
+// positions [to, to + n) of the task <- positions [to + shift, to + shift + n), in place, on every layer
+cudaError_t launch_move(uint8_t* pool, size_t layer_stride, int layers, const int32_t* table_row, int to, int shift, int n, bool overlapped,
+                        const Geom& g, cudaStream_t s);
 cudaError_t launch_copy_pages(uint8_t* pool, const int32_t* src, const int32_t* dst, int n, long long page_bytes, cudaStream_t s);
 cudaError_t launch_read(const uint8_t* pool, const int32_t* table_row, int pos0, int len, uint16_t* out_k,
                         uint16_t* out_v, const Geom& g, cudaStream_t s);
@@ -208,11 +211,11 @@ int sm_count();   // multiprocessors of the current device (looked up once per d
 // grid_dep_launch only after everything that the NEXT kernel may rely on without waiting is complete.  The two attention
 // kernels of one batch do not depend on each other: the second one (AttendParams::overlapped) starts without waiting -
 // the first has waited for all earlier work before it let the second one start - and waits when it is done, so that what
-// follows it in the stream still follows both.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
+// follows it in the stream still follows both.  The same goes for the moves of several tasks that are pruned in a row.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
 template <typename... A>
-cudaError_t launch_dep(void (*kernel)(A...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, const std::common_type_t<A>&... args) {
+cudaError_t launch_dep(void (*kernel)(A...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, const std::common_type_t<A>&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
