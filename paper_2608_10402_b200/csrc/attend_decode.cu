@@ -50,6 +50,7 @@ struct __align__(16) Item {
   int part_row0;             // the same in the partials of this split
   int n, n_splits, part_base, merge_ctr;   // for the block that merges the splits
   int mode;                  // 0: one split, results go to out / lse; 1: partials; 2: partials, the last split merges
+  int live_from;             // first key that the kernel before this one may still be writing
   int drop;                  // test hook: the first stage never arrives
   int merge;                 // the item two before this one finished its row: its splits are to be merged
 };
@@ -160,12 +161,13 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     mbar_init(smem_u32(&s_part_done), 1);
     mbar_fence_init();
   }
-  if (!P.overlapped) grid_dep_wait();
-  grid_dep_launch();
-  const int n_items = P.dyn ? __ldcg(P.dyn) : P.n_items;     // fixed grid: the batch's counts live in device memory
   __syncthreads();
+  const bool early = P.run_ahead != 0 && warp >= kConsumerWarps;   // these warps touch only what earlier work has finished with
+  if (!P.overlapped && !early) grid_dep_wait();
+  if (!early) grid_dep_launch();
+  const int n_items = P.dyn ? __ldcg(P.dyn) : P.n_items;     // fixed grid: the batch's counts live in device memory
   if ((int)blockIdx.x >= n_items) {
-    if (P.overlapped) grid_dep_wait();
+    if (P.overlapped || early) grid_dep_wait();
     return;
   }
   volatile int* abort_flag = &s_abort;
@@ -179,12 +181,12 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     // ================= producer warp =================
     const int pages_per_stage = kStageKeys / g.S, stages_per_group = 32 / pages_per_stage;
     int slot = 0, use = 0, issued = 0;
-    bool ok = true;
+    bool ok = true, ahead = early;
     for (int it = 0; ok; ++it) {
       if (!wait_all(s_item_full[it % kItemSlots], (it / kItemSlots) & 1)) break;
       const Item& w = items[it % kItemSlots];
       if (!w.run) break;
-      const int kv_begin = w.kv_begin, kv_end = w.kv_end, drop = w.drop;
+      const int kv_begin = w.kv_begin, kv_end = w.kv_end, drop = w.drop, live_from = w.live_from;
       const int32_t* trow = P.table + w.table_off;
       const uint8_t* head_base = P.pool + (long long)w.kvh * g.head_bytes;
       __syncwarp();
@@ -207,6 +209,13 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
         ++issued;
         const int key0 = kv_begin + st * kStageKeys;
         const int npages = min(pages_per_stage, (kv_end - key0 + g.S - 1) / g.S);
+        if (ahead && key0 + npages * g.S > live_from) {
+          // from here on pages, and page numbers, may belong to the kernel before this one
+          grid_dep_wait();
+          ahead = false;
+          ids_cur = load_ids(cur_grp);
+          ids_nxt = load_ids(cur_grp + 1);
+        }
         const uint32_t bar = smem_u32(&s_full[slot]);
         const long long page = __shfl_sync(0xffffffffu, ids_cur, ((st % stages_per_group) * pages_per_stage + lane) & 31);
         if (!(drop != 0 && st == 0)) {                       // test hook: this stage never arrives
@@ -234,7 +243,7 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     const int n_segs = P.dyn ? __ldcg(P.dyn + 1) : P.n_segs;
     int item = (int)blockIdx.x, asks = 0, done = 0;
     int merge = 0;                                           // lane 0: the last item but one completed its row
-    bool fused_before = false, open = false;                                       // a question without an answer yet
+    bool fused_before = false, open = false;                 // a question without an answer yet
     for (int it = 0; ; ++it) {
       const int slot = it % kItemSlots;
       if (it >= kItemSlots && !wait_all(s_item_empty[slot], (it / kItemSlots - 1) & 1)) break;
@@ -273,7 +282,7 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
         w.table_off = seg.table_off; w.kvh = kvh;
         w.kv_begin = seg.origin + split * seg.chunk;
         w.kv_end = max(w.kv_begin, min(w.kv_begin + seg.chunk, seg.p + (seg.n - 1) * seg.causal + 1));
-        w.R = R; w.p = seg.p; w.causal = seg.causal;
+        w.R = R; w.p = seg.p; w.causal = seg.causal; w.live_from = seg.live_from;
         w.q_row0 = seg.q_off * g.Hq + kvh * g.G;
         w.part_row0 = seg.part_base + split * seg.n * g.Hq + kvh * g.G;
         w.n = seg.n; w.n_splits = seg.n_splits; w.part_base = seg.part_base;

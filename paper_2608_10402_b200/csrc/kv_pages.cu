@@ -38,6 +38,22 @@ cudaError_t launch_upload(void* dst, const void* src_mapped_host, size_t bytes, 
   return launch_dep(upload_kernel, blocks, 256, 0, s, (uint32_t*)dst, (const uint32_t*)src_mapped_host, n);
 }
 
+__global__ void upload_set_kernel(const __grid_constant__ UploadSet u) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = first; i < (size_t)u.n_upd; i += step) u.table[u.idx[i]] = u.val[i];
+  for (int p = 0; p < u.n_parts; ++p)
+    for (size_t i = first; i < u.part[p].words; i += step) u.part[p].dst[i] = u.part[p].src[i];
+}
+
+cudaError_t launch_upload_set(const UploadSet& u, cudaStream_t s) {
+  size_t most = (size_t)u.n_upd;
+  for (int p = 0; p < u.n_parts; ++p) most = std::max(most, u.part[p].words);
+  if (most == 0) return cudaSuccess;
+  return launch_dep(upload_set_kernel, (unsigned)std::min<size_t>((most + 255) / 256, 64), 256, 0, s, u);
+}
+
 constexpr int kAppendThreads = 256;
 constexpr int kAppendWarps = kAppendThreads / 32;
 constexpr int kAppendMaxRecsSmem = 1024;

@@ -12,6 +12,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "tide_internal.h"
@@ -105,6 +106,12 @@ struct tide_kv {
   ExtendOut ext;              // result of the most recent extension
   std::vector<int32_t> mark;  // scratch for duplicate detection
   int32_t mark_gen = 0;
+  // what the most recent append, write or series of moves may still be writing while the kernel behind it starts: keys
+  // from live_from[t] on (a page boundary) of the tasks of that generation
+  std::vector<int64_t> live_gen_of;
+  std::vector<int32_t> live_from;
+  int64_t live_gen = 0;
+  cudaStream_t live_stream = nullptr;
   // moves of pruned tasks launched one after the other on one stream, with no other device work of this handle between
   bool moves_open = false;
   cudaStream_t moves_stream = nullptr;
@@ -243,6 +250,19 @@ bool last_page_shared(const tide_kv* kv, int32_t task) {
 
 bool task_in_range(const tide_kv* kv, int32_t t) { return t >= 0 && t < kv->cfg.max_tasks; }
 
+// A kernel that writes keys is about to be launched on `st`; mark_live says which.  It waits for the one before it on its
+// stream, whose keys are then no longer live; the keys of kernels on other streams stay so.
+void begin_live(tide_kv* kv, cudaStream_t st) {
+  if (kv->live_stream == st) ++kv->live_gen;
+  kv->live_stream = st;
+}
+void mark_live(tide_kv* kv, int32_t task, int32_t from) {
+  from -= from % kv->g.S;
+  int32_t& f = kv->live_from[(size_t)task];
+  f = kv->live_gen_of[(size_t)task] == kv->live_gen ? std::min(f, from) : from;
+  kv->live_gen_of[(size_t)task] = kv->live_gen;
+}
+
 // Takes the next staging slot, waiting until the device work that last used it has finished.
 int acquire_slot(tide_kv* kv, Slot** out) {
   Slot& s = kv->slots[kv->next_slot];
@@ -326,7 +346,7 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
   ok = ok && cudaMemset(kv->d_status, 0, 256) == cudaSuccess;
   ok = ok && cudaMemset(kv->d_merge_ctr, 0, (size_t)kStepSegStride * cfg->max_batch_rows * g.Hkv * 4) == cudaSuccess;
   ok = ok && cudaHostAlloc((void**)&kv->h_status, 64, cudaHostAllocDefault) == cudaSuccess;
-  ok = ok && cudaHostAlloc((void**)&kv->h_step, lay.step_bytes, cudaHostAllocDefault) == cudaSuccess;
+  ok = ok && cudaHostAlloc((void**)&kv->h_step, lay.step_bytes, cudaHostAllocMapped) == cudaSuccess;
   ok = ok && cudaEventCreateWithFlags(&kv->ev_step, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; ok && i < kSlots; ++i) {
     ok = cudaHostAlloc((void**)&kv->slots[i].host, lay.slot_bytes, cudaHostAllocMapped) == cudaSuccess;
@@ -348,6 +368,8 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
   kv->pages.resize((size_t)cfg->max_tasks);
   kv->mark.assign((size_t)cfg->max_tasks, 0);
   kv->move_mark.assign((size_t)cfg->max_tasks, 0);
+  kv->live_gen_of.assign((size_t)cfg->max_tasks, 0);
+  kv->live_from.assign((size_t)cfg->max_tasks, 0);
   kv->refcnt.assign((size_t)cfg->num_pages, 0);
   prime_free_stack(kv, cfg->free_order);
   *out = kv;
@@ -600,6 +622,9 @@ static int write_tasks(tide_kv* kv, int32_t layer, int32_t n_tasks, const int32_
   int j = 0;
   int rc = TIDE_OK;
   kv->moves_open = false;
+  if (indptr[n_tasks] > 0) begin_live(kv, st);
+  for (int i = 0; i < n_tasks; ++i)
+    if (indptr[i + 1] > indptr[i]) mark_live(kv, task_ids[i], kv->len[task_ids[i]] - (indptr[i + 1] - indptr[i]));
   while (j < n_tasks) {
     Slot* slot;
     if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
@@ -685,7 +710,13 @@ int tide_kv_append(tide_kv_t* kv, int32_t layer, int32_t n_tasks, const int32_t*
   if ((rc = extend_bookkeeping(kv, n_tasks, task_ids, indptr)) != TIDE_OK) return rc;
   if ((rc = upload_cow_copies(kv, st)) != TIDE_OK) return rc;     // a copied page must be in place before it is written
   int n_recs = 0;
-  for (int j = 0; j < n_tasks; ++j) n_recs += indptr[j + 1] > indptr[j] ? 1 : 0;
+  if (indptr[n_tasks] > 0) begin_live(kv, st);
+  for (int j = 0; j < n_tasks; ++j) {
+    const int c = indptr[j + 1] - indptr[j];
+    if (c == 0) continue;
+    ++n_recs;
+    mark_live(kv, task_ids[j], kv->len[task_ids[j]] - c);
+  }
   const ExtendOut& x = kv->ext;
   auto fill_recs = [&](AppendRec* recs) {
     int r = 0, grp_cursor = 0;
@@ -903,7 +934,10 @@ int tide_kv_prune(tide_kv_t* kv, int32_t layer, int32_t task, int32_t keep_prefi
   if (!shared_any) {
     // a move right behind other tasks' moves on the same stream need not wait for them
     const bool overlapped = kv->moves_open && kv->moves_stream == st && kv->move_mark[(size_t)task] != kv->move_gen;
-    if (!overlapped) ++kv->move_gen;
+    if (tail > 0) {
+      if (!overlapped) { ++kv->move_gen; begin_live(kv, st); }
+      mark_live(kv, task, keep_prefix);
+    }
     if (tail > 0 && launch_move(kv->pool, kv->layer_stride, L, row, keep_prefix, tail_begin - keep_prefix, tail, overlapped, g, st) != cudaSuccess)
       return TIDE_ERR_CUDA;
     if (tail > 0) {
@@ -1024,8 +1058,9 @@ static bool umma_takes(const tide_kv* kv) { return kv->g.D == 128 || kv->umma_ti
 // tcgen05-style; long contexts are split along the keys so that the grid has about items_per_sm items per SM.
 // A group of rows that share their first pages gets one more segment for the shared range (its tokens are the
 // members' queries, all seeing the same keys); the members' own segments start behind it and their merge takes both.
-// The plan depends on the rows and the page tables only, so every layer of a step can use it.
-static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool umma_ok, bool allow_groups, PlanHost& P) {
+// The plan depends on the rows and the page tables only, so every layer of a step can use it.  `step`: the kernel in front
+// of the attention kernels is the append of exactly these rows (tide_step_layer).
+static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool umma_ok, bool allow_groups, bool step, PlanHost& P) {
   const Geom& g = kv->g;
   enum { kDec = 0, kTile = 1, kUmma = 2 };
   struct RowPlan { int kind; int n_mtiles; long long items; };
@@ -1084,6 +1119,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
         s.n_mtiles = mtiles_of(kind, sg.m * g.G);
         cut(true, sg.pages * g.S, s.n_splits, s.chunk);
         s.causal = 0;
+        s.live_from = INT_MAX;                               // full pages that several tasks hold: nothing writes them
         s.partial = 1;
         s.x_part_base = gi;
         s.x_n_splits = -2;                                   // marks the shared range until the links are resolved
@@ -1097,6 +1133,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
       s.p = r.ctx_len - r.q_len;
       s.n_mtiles = p.n_mtiles;
       s.causal = 1;
+      s.live_from = step ? s.p : kv->live_gen_of[(size_t)r.task] == kv->live_gen ? kv->live_from[(size_t)r.task] : INT_MAX;
       if (gi >= 0) {
         s.origin = groups[(size_t)gi].pages * g.S;
         s.partial = 1;
@@ -1126,7 +1163,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
   P.fused_rows = 0;
   long long part_cursor = 0;
   int32_t ctr_cursor = 0;
-  std::vector<Segment*> merged;                              // segments with rows to merge, in merge_base order
+  std::vector<std::pair<const Segment*, int32_t>> merged;    // segments with rows to merge, and the first of these rows
   for (auto* v : {&P.seg_dec, &P.seg_tile, &P.seg_umma}) {
     long long base = 0;
     for (Segment& s : *v) {
@@ -1146,9 +1183,8 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
           ctr_cursor += g.Hkv;
           P.fused_rows += (long long)s.n * g.Hq;
         } else {
-          s.merge_base = (int32_t)P.merge_rows;
+          merged.emplace_back(&s, (int32_t)P.merge_rows);
           P.merge_rows += (long long)s.n * g.Hq;
-          merged.push_back(&s);
         }
       }
     }
@@ -1168,7 +1204,10 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
         s.x_n_splits = 0;
       }
     }
-  for (const Segment* s : merged) P.seg_merge.push_back(*s);
+  for (const auto& [s, base] : merged) {
+    P.seg_merge.push_back(*s);
+    P.seg_merge.back().merge_base = base;
+  }
   kv->last_groups = (int64_t)groups.size();
   kv->last_grouped_rows = 0;
   for (const ShareGroup& sg : groups) kv->last_grouped_rows += sg.m;
@@ -1195,8 +1234,8 @@ static PlanDev pack_plan(const PlanHost& P, Segment* h, const Segment* d, size_t
 // The attention launches of one planned batch on one layer: kernel launches only (and, with `events`, the phase
 // time stamps), so a caller may capture them in a CUDA graph.  With `inl` the row descriptors come from that plan and
 // travel in the launches' parameters; otherwise they are on the device, where `d` says.
-static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanHost* inl, const int32_t* page_table, const void* q, float scale,
-                       void* out, float* lse, cudaStream_t st, bool events, int64_t* n_launches, const int32_t* dyn) {
+static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanHost* inl, bool step, const int32_t* page_table, const void* q,
+                       float scale, void* out, float* lse, cudaStream_t st, bool events, int64_t* n_launches, const int32_t* dyn) {
   kv->moves_open = false;
   AttendParams ap;
   ap.pool = kv->layer_pool(layer);
@@ -1217,6 +1256,9 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   // dyn != nullptr: fixed launch shapes; the counts of the batch are read on the device (header of the step area)
   const bool dec = dyn ? kv->cap_dec > 0 : d.items_dec > 0, tile = dyn ? kv->cap_tile > 0 : d.items_tile > 0;
   const bool umma = dyn ? kv->cap_umma > 0 : d.items_umma > 0, merge = dyn ? kv->cap_merge_rows > 0 : d.merge_rows > 0;
+  // The decode kernel's producers may run ahead of the append when their row descriptors do not come from an upload right
+  // in front of it (they are in the launch, or in the step area), and the page table is the handle's own.
+  const bool run_ahead = (inl != nullptr || step) && page_table == nullptr && !tile && !events;
   auto inline_segs = [&](const std::vector<Segment>& v) -> AttendInline& {
     AttendInline& pi = kv->attend_inline;
     std::copy(v.begin(), v.end(), pi.segs);
@@ -1226,6 +1268,7 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   auto launch_dec = [&](bool overlapped) -> cudaError_t {
     ap.segs = d.seg_dec; ap.n_segs = (int)d.n_dec; ap.n_items = (int)d.items_dec;
     ap.dyn = dyn ? dyn + kHdrDecItems : nullptr; ap.grid_cap = kv->cap_dec; ap.overlapped = overlapped ? 1 : 0;
+    ap.run_ahead = run_ahead && !overlapped ? 1 : 0;
     ++launches;
     return inl ? launch_attend_decode_inline(inline_segs(inl->seg_dec), st) : launch_attend_decode(ap, st);
   };
@@ -1289,7 +1332,7 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
   int rc = check_rows(kv, n_rows, rows);
   if (rc != TIDE_OK) return rc;
   PlanHost P;
-  if ((rc = build_plan(kv, n_rows, rows, umma_takes(kv) && scale > 0.f, page_table == nullptr, P)) != TIDE_OK) return rc;
+  if ((rc = build_plan(kv, n_rows, rows, umma_takes(kv) && scale > 0.f, page_table == nullptr, false, P)) != TIDE_OK) return rc;
   if (P.n_all() * sizeof(Segment) + 256 > kv->lay.slot_bytes) return TIDE_ERR_WORKSPACE;
 
   cudaStream_t st = (cudaStream_t)stream;
@@ -1300,14 +1343,14 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
     // a small batch: the row descriptors travel in the launches' own parameters (no upload)
     pd.n_dec = P.seg_dec.size(); pd.n_umma = P.seg_umma.size(); pd.n_merge = P.seg_merge.size();
     pd.items_dec = P.items_dec; pd.items_umma = P.items_umma; pd.merge_rows = P.merge_rows;
-    if ((rc = launch_plan(kv, layer, pd, &P, page_table, q, scale, out, lse, st, kv->profiling, &launches, nullptr)) != TIDE_OK) return rc;
+    if ((rc = launch_plan(kv, layer, pd, &P, false, page_table, q, scale, out, lse, st, kv->profiling, &launches, nullptr)) != TIDE_OK) return rc;
   } else {
     Slot* slot;
     if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
     pd = pack_plan(P, (Segment*)(slot->host + 256), (const Segment*)(slot->dev + 256), 0);
     if (upload(kv, slot->dev + 256, slot->host + 256, P.n_all() * sizeof(Segment), st) != cudaSuccess)
       return TIDE_ERR_CUDA;
-    if ((rc = launch_plan(kv, layer, pd, nullptr, page_table, q, scale, out, lse, st, kv->profiling, &launches, nullptr)) != TIDE_OK) return rc;
+    if ((rc = launch_plan(kv, layer, pd, nullptr, false, page_table, q, scale, out, lse, st, kv->profiling, &launches, nullptr)) != TIDE_OK) return rc;
     if ((rc = release_slot(slot, st)) != TIDE_OK) return rc;
   }
   kv->last_decode_items = pd.items_dec;
@@ -1355,16 +1398,30 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   PlanHost P;
   // Launch shapes fixed without tcgen05 items (or with too few): head size 64 has the warp-MMA tile kernel as well.
   bool umma = umma_takes(kv) && !(kv->fixed_grids && g.D == 64 && kv->cap_umma == 0);
-  if ((rc = build_plan(kv, n_rows, rows, umma, true, P)) != TIDE_OK) return rc;
+  if ((rc = build_plan(kv, n_rows, rows, umma, true, true, P)) != TIDE_OK) return rc;
   if (umma && kv->fixed_grids && g.D == 64 && P.items_umma > kv->cap_umma &&
-      (rc = build_plan(kv, n_rows, rows, false, true, P)) != TIDE_OK) return rc;
+      (rc = build_plan(kv, n_rows, rows, false, true, true, P)) != TIDE_OK) return rc;
   if (kv->fixed_grids && (P.items_dec > kv->cap_dec || P.items_tile > kv->cap_tile || P.items_umma > kv->cap_umma ||
                           P.merge_rows > kv->cap_merge_rows || indptr[(size_t)n_rows] > kv->cap_tokens))
     return TIDE_ERR_WORKSPACE;   // the step does not fit the launch shapes that were fixed
   cudaStream_t st = (cudaStream_t)stream;
   kv->append_launches = 0;
-  if ((rc = extend_tasks(kv, n_rows, ids.data(), indptr.data(), st, nullptr)) != TIDE_OK) return rc;
-  // one upload: the write records of the rows, then the segments
+  if ((rc = extend_bookkeeping(kv, n_rows, ids.data(), indptr.data())) != TIDE_OK) return rc;
+  // Header, write records, segments and page-table delta travel in one launch that reads the pinned buffers (as a table
+  // update with its upload and two copies they took 27 us of a step).  Large deltas, and the copy engine, take the
+  // steps one by one.
+  const ExtendOut& x = kv->ext;
+  const bool one_launch = kv->slots_mapped && (kv->upload_by_kernel || kv->always_upload_by_kernel) && x.idx.size() <= kSlotPageIds;
+  Slot* slot = nullptr;
+  UploadSet up;
+  if (one_launch && !x.idx.empty()) {
+    if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
+    int32_t* h = (int32_t*)(slot->host + 256);
+    std::memcpy(h, x.idx.data(), x.idx.size() * 4);
+    std::memcpy(h + x.idx.size(), x.val.data(), x.idx.size() * 4);
+    up.table = kv->d_table; up.idx = h; up.val = h + x.idx.size(); up.n_upd = (int)x.idx.size();
+  } else if (!one_launch && (rc = upload_table_delta(kv, st)) != TIDE_OK) return rc;
+  if ((rc = upload_cow_copies(kv, st)) != TIDE_OK) return rc;
   if (kv->step_upload_pending && cudaEventSynchronize(kv->ev_step) != cudaSuccess) return TIDE_ERR_CUDA;
   int32_t* hdr = (int32_t*)kv->h_step;
   hdr[kHdrRecs] = n_rows; hdr[kHdrRecs + 1] = indptr[(size_t)n_rows];
@@ -1387,15 +1444,20 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   uint8_t* d_step = kv->ws + kv->lay.off_step;
   const size_t stride = (size_t)kStepSegStride * (size_t)kv->cfg.max_batch_rows;
   kv->step_plan = pack_plan(P, (Segment*)(kv->h_step + kv->lay.step_seg_off), (const Segment*)(d_step + kv->lay.step_seg_off), stride);
-  // header and records in one copy, then each segment array that is not empty (their places are fixed)
-  if (cudaMemcpyAsync(d_step, kv->h_step, 256 + (size_t)n_rows * sizeof(AppendRec), cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return TIDE_ERR_CUDA;
+  // header and records, then each segment array that is not empty (their places are fixed)
+  auto put = [&](size_t off, size_t bytes) -> cudaError_t {
+    if (!one_launch) return cudaMemcpyAsync(d_step + off, kv->h_step + off, bytes, cudaMemcpyHostToDevice, st);
+    up.part[up.n_parts++] = {(uint32_t*)(d_step + off), (const uint32_t*)(kv->h_step + off), bytes / 4};
+    return cudaSuccess;
+  };
+  if (put(0, 256 + (size_t)n_rows * sizeof(AppendRec)) != cudaSuccess) return TIDE_ERR_CUDA;
   const size_t counts[4] = {P.seg_dec.size(), P.seg_tile.size(), P.seg_umma.size(), P.seg_merge.size()};
-  for (int a = 0; a < 4; ++a) {
-    const size_t off = kv->lay.step_seg_off + (size_t)a * stride * sizeof(Segment);
-    if (counts[a] > 0 &&
-        cudaMemcpyAsync(d_step + off, kv->h_step + off, counts[a] * sizeof(Segment), cudaMemcpyHostToDevice, st) != cudaSuccess)
+  for (int a = 0; a < 4; ++a)
+    if (counts[a] > 0 && put(kv->lay.step_seg_off + (size_t)a * stride * sizeof(Segment), counts[a] * sizeof(Segment)) != cudaSuccess)
       return TIDE_ERR_CUDA;
+  if (one_launch) {
+    if (launch_upload_set(up, st) != cudaSuccess) return TIDE_ERR_CUDA;
+    if (slot != nullptr && (rc = release_slot(slot, st)) != TIDE_OK) return rc;
   }
   if (cudaEventRecord(kv->ev_step, st) != cudaSuccess) return TIDE_ERR_CUDA;
   kv->step_upload_pending = true;
@@ -1430,7 +1492,7 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   ap.g = kv->g;
   if (launch_append(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
   int64_t launches = 0;
-  const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, nullptr, q, scale, out, lse, st, false, &launches, dyn);
+  const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, true, nullptr, q, scale, out, lse, st, false, &launches, dyn);
   if (rc != TIDE_OK) return rc;
   kv->last_launches = launches + 1;
   return TIDE_OK;

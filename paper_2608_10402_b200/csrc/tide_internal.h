@@ -54,7 +54,10 @@ struct __align__(16) Segment {
   int32_t n_splits;
   int32_t chunk;       // keys per split, a multiple of kStageKeys
   int32_t part_base;   // first partial row ((split * n + token) * Hq + head) when the item writes partials
-  int32_t merge_base;  // first row of this segment in the merge launch
+  union {
+    int32_t merge_base;  // in the merge launch's list: first row of this segment
+    int32_t live_from;   // in the decode launch's list: first key that the kernel before it may still be writing (run_ahead)
+  };
   // Rows of one batch whose tasks share their first pages (forked tasks) read those pages once: the shared range
   // is one segment whose `n` tokens are the member rows' queries and all see the same keys (causal = 0), each
   // member's own range starts behind it (origin), both write partials, and the member's merge takes both.
@@ -89,6 +92,7 @@ struct AttendParams {
   int grid_cap = 0;
   int* merge_ctr = nullptr;   // per (segment with partial == 2, kv head): splits finished so far; zero between launches
   long long wait_limit_ns = kWaitLimitNsDefault;   // bound of every wait inside the kernel
+  int run_ahead = 0;          // decode: the producers may read keys below Segment::live_from before earlier work is complete
   int overlapped = 0;         // the kernel before this one in the stream is the other attention kernel of the same batch (see grid_dep_wait)
   // Test hook for the bounded waits (never set in normal use): in work item 0 the producer leaves out its part
   // of the first stage, so the consumers' wait for that stage runs out and the time-out path executes.
@@ -162,6 +166,16 @@ struct AppendInline {
   int32_t upd[2 * kInlineUpd];     // p.n_upd table indices, then p.n_upd values
 };
 
+// Several small host-to-device uploads and a page-table delta in one launch; sources are pinned and mapped.
+struct UploadSet {
+  struct Part { uint32_t* dst; const uint32_t* src; size_t words; };
+  Part part[5];
+  int n_parts = 0;
+  int32_t* table = nullptr;
+  const int32_t *idx = nullptr, *val = nullptr;
+  int n_upd = 0;
+};
+
 // What tide_attend_decode_static needs of a handle (filled by tide_internal_view in tide_host.cu).
 struct StaticView {
   Geom g;
@@ -177,6 +191,7 @@ struct StaticView {
 
 cudaError_t launch_table_update(int32_t* table, const int32_t* idx, const int32_t* val, int n, cudaStream_t s);
 cudaError_t launch_upload(void* dst, const void* src_mapped_host, size_t bytes, cudaStream_t s);   // bytes % 4 == 0
+cudaError_t launch_upload_set(const UploadSet& u, cudaStream_t s);
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s);
 // positions [to, to + n) of the task <- positions [to + shift, to + shift + n), in place, on every layer
 cudaError_t launch_move(uint8_t* pool, size_t layer_stride, int layers, const int32_t* table_row, int to, int shift, int n, bool overlapped,
@@ -211,7 +226,9 @@ int sm_count();   // multiprocessors of the current device (looked up once per d
 // grid_dep_launch only after everything that the NEXT kernel may rely on without waiting is complete.  The two attention
 // kernels of one batch do not depend on each other: the second one (AttendParams::overlapped) starts without waiting -
 // the first has waited for all earlier work before it let the second one start - and waits when it is done, so that what
-// follows it in the stream still follows both.  The same goes for the moves of several tasks that are pruned in a row.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
+// follows it in the stream still follows both.  Nor do the keys that a decode row saw in the step before depend on the
+// append in front of the decode kernel, which waits for everything earlier: the decode kernel's producers stream those
+// pages (AttendParams::run_ahead, Segment::live_from) while the append runs.  The same goes for the moves of several tasks that are pruned in a row.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
 template <typename... A>
 cudaError_t launch_dep(void (*kernel)(A...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, const std::common_type_t<A>&... args) {
   cudaLaunchConfig_t cfg = {};
