@@ -48,7 +48,8 @@ struct __align__(16) Item {
   int p, causal;             // query q_index sees keys [0, p + q_index * causal]
   int q_row0;                // (token, head) row of packed row 0 in q (and out)
   int part_row0;             // the same in the partials of this split
-  int n, n_splits, part_base, merge_ctr;   // for the block that merges the splits
+  int n, n_splits, part_base, merge_ctr;   // for the block that merges the splits ...
+  int x_n_splits, x_part_row0, x_stride;   // ... with those of the shared range in front of them
   int mode;                  // 0: one split, results go to out / lse; 1: partials; 2: partials, the last split merges
   int live_from;             // first key that the kernel before this one may still be writing
   int drop;                  // test hook: the first stage never arrives
@@ -73,16 +74,20 @@ template <int D>
 __device__ __forceinline__ void merge_splits(const AttendParams& P, const Item& w, int row0, int d0) {
   constexpr int CW = D / 16;
   const Geom& g = P.g;
-  const int n_splits = w.n_splits, R = w.R;
+  const int own = w.n_splits, n_splits = own + w.x_n_splits, R = w.R;
   const long long stride = (long long)w.n * g.Hq;              // partial rows per split
+  if (w.x_n_splits > 0) grid_dep_wait();                       // the shared range's partials are complete
   for (int rr = row0; rr < R; rr += 8) {
     const int qi = rr / g.G, gi = rr - qi * g.G;
     const long long p0 = (long long)w.part_base + w.kvh * g.G + (long long)qi * g.Hq + gi;   // this (token, head) in split 0
+    auto src_row = [&](int sp) -> long long {
+      return sp < own ? p0 + sp * stride : (long long)w.x_part_row0 + gi + (long long)(sp - own) * w.x_stride;
+    };
     float mstar = -INFINITY;
     for (int sp0 = 0; sp0 < n_splits; sp0 += 16) {
       float e[16];
 #pragma unroll
-      for (int x = 0; x < 16; ++x) e[x] = sp0 + x < n_splits ? __ldcg(P.part_lse + p0 + (sp0 + x) * stride) : -INFINITY;
+      for (int x = 0; x < 16; ++x) e[x] = sp0 + x < n_splits ? __ldcg(P.part_lse + src_row(sp0 + x)) : -INFINITY;
 #pragma unroll
       for (int x = 0; x < 16; ++x) mstar = fmaxf(mstar, e[x]);
     }
@@ -96,7 +101,7 @@ __device__ __forceinline__ void merge_splits(const AttendParams& P, const Item& 
 #pragma unroll
       for (int x = 0; x < kMergeBatch; ++x) {
         const bool there = sp0 + x < n_splits;
-        const long long row = p0 + (there ? sp0 + x : sp0) * stride;
+        const long long row = src_row(there ? sp0 + x : sp0);
         e[x] = there ? __ldcg(P.part_lse + row) : -INFINITY;
         const float* src = P.part_o + row * D + d0;
 #pragma unroll
@@ -286,7 +291,8 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
         w.q_row0 = seg.q_off * g.Hq + kvh * g.G;
         w.part_row0 = seg.part_base + split * seg.n * g.Hq + kvh * g.G;
         w.n = seg.n; w.n_splits = seg.n_splits; w.part_base = seg.part_base;
-        w.merge_ctr = seg.x_part_base + kvh;
+        w.merge_ctr = seg.merge_ctr + kvh;
+        w.x_n_splits = seg.x_n_splits; w.x_part_row0 = seg.x_part_base + kvh * g.G; w.x_stride = seg.x_stride;
         w.mode = seg.partial == 2 ? 2 : (seg.n_splits == 1 && seg.partial == 0) ? 0 : 1;
         w.drop = P.debug_drop_first_stage != 0 && item == 0;
         mbar_arrive(smem_u32(&s_item_full[slot]));

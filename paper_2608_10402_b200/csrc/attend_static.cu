@@ -72,6 +72,7 @@ __global__ void static_plan_kernel(const StaticPlanArgs a, Segment* __restrict__
     s.x_part_base = 0;
     s.x_n_splits = 0;
     s.x_stride = 0;
+    s.merge_ctr = s.pad[0] = s.pad[1] = s.pad[2] = 0;
     items += a.Hkv * r.n_splits;
     if (r.n_splits > 1) {
       s.part_base = part;

@@ -70,16 +70,28 @@ constexpr int kAppendLoadsInFlight = 8;    // 16-byte loads a lane has in flight
 // the page-table delta of the append, if it is given one; the pages that delta brings are then taken from the delta
 // itself, not from the table (no ordering between thread blocks is needed).
 // AppendRec::grp0 = number of 8-slot groups that the records before this one touch.
+// What does not depend on earlier kernels - finding the first round's record, when the records are in the launch or were
+// complete before (AppendParams::early) - happens before the wait for them.
 template <int SLABS>
 __device__ __forceinline__ void append_scatter_body(const AppendParams& P, const AppendRec* __restrict__ recs,
-                                                  const int32_t* __restrict__ upd_idx, const int32_t* __restrict__ upd_val) {
+                                                  const int32_t* __restrict__ upd_idx, const int32_t* __restrict__ upd_val,
+                                                  const bool early) {
   __shared__ int32_t s_grp0[kAppendMaxRecsSmem];
-  grid_dep_wait();
-  grid_dep_launch();
-  const int n_recs = P.dyn ? P.dyn[0] : P.n_recs;
-  for (int i = blockIdx.x * kAppendThreads + threadIdx.x; i < P.n_upd; i += gridDim.x * kAppendThreads)
-    P.table_rw[upd_idx[i]] = upd_val[i];
-  if (n_recs <= 0) return;
+  bool waited = false;
+  auto wait = [&] {
+    if (waited) return;
+    waited = true;
+    grid_dep_wait();
+    grid_dep_launch();
+    for (int i = blockIdx.x * kAppendThreads + threadIdx.x; i < P.n_upd; i += gridDim.x * kAppendThreads)
+      P.table_rw[upd_idx[i]] = upd_val[i];
+  };
+  if (!early) wait();
+  const int n_recs = P.dyn ? __ldcg(P.dyn) : P.n_recs;
+  if (n_recs <= 0) {
+    wait();
+    return;
+  }
   const bool in_smem = n_recs <= kAppendMaxRecsSmem;
   if (in_smem) {
     for (int i = threadIdx.x; i < n_recs; i += blockDim.x) s_grp0[i] = recs[i].grp0;
@@ -106,6 +118,7 @@ __device__ __forceinline__ void append_scatter_body(const AppendParams& P, const
     if (in_smem) r = find_segment(n_recs, grp, [&](int i) { return s_grp0[i]; });
     else r = find_segment(n_recs, grp, [&](int i) { return recs[i].grp0; });
     const AppendRec rec = recs[r];
+    wait();
     const int g_pos0 = (rec.pos0 & ~7) + (grp - rec.grp0) * 8;                 // first slot position of the group
     const int lp = g_pos0 / g.S;
     const long long page = lp >= rec.new_lp0 ? upd_val[rec.new_off + (lp - rec.new_lp0)] : P.table[rec.table_off + lp];
@@ -137,15 +150,16 @@ __device__ __forceinline__ void append_scatter_body(const AppendParams& P, const
       }
     }
   }
+  wait();
 }
 
 template <int SLABS>
 __global__ void __launch_bounds__(kAppendThreads, 3) append_scatter_kernel(const AppendParams P) {
-  append_scatter_body<SLABS>(P, P.recs, P.upd_idx, P.upd_val);
+  append_scatter_body<SLABS>(P, P.recs, P.upd_idx, P.upd_val, P.early != 0);
 }
 template <int SLABS>
 __global__ void __launch_bounds__(kAppendThreads, 3) append_scatter_inline_kernel(const __grid_constant__ AppendInline PI) {
-  append_scatter_body<SLABS>(PI.p, PI.recs, PI.upd, PI.upd + PI.p.n_upd);
+  append_scatter_body<SLABS>(PI.p, PI.recs, PI.upd, PI.upd + PI.p.n_upd, true);
 }
 
 static unsigned append_grid(const AppendParams& p) {

@@ -141,7 +141,8 @@ struct tide_kv {
   cudaEvent_t ev_step = nullptr;
   bool step_upload_pending = false, step_valid = false;
   PlanDev step_plan;
-  int step_recs = 0, step_tokens = 0;
+  int step_recs = 0, step_tokens = 0, step_layers = 0;   // step_layers: calls of tide_step_layer since tide_step_begin
+  cudaStream_t step_stream = nullptr;
   // fixed launch shapes for tide_step_layer (0 = off): most work items / rows / tokens a step may plan
   bool fixed_grids = false;
   int cap_dec = 0, cap_tile = 0, cap_umma = 0, cap_merge_rows = 0, cap_tokens = 0;
@@ -1176,10 +1177,11 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
         if (s.x_n_splits == -2) {                            // a shared range: it has no output rows of its own
           groups[(size_t)s.x_part_base].part_base = s.part_base;
           groups[(size_t)s.x_part_base].n_splits = s.n_splits;
-        } else if (v == &P.seg_dec && s.partial == 0 && s.x_n_splits == 0) {
-          // a plain split decode-style row: the split that finishes last merges the partials inside the decode kernel
+        } else if (v == &P.seg_dec && (s.partial == 0 || shared_kind(groups[(size_t)s.x_part_base].m * g.G) == kUmma)) {
+          // a split decode-style row, or a member of a group whose shared range runs in the tcgen05 kernel (the decode kernel
+          // follows it): the split that finishes last merges the partials inside the decode kernel
           s.partial = 2;
-          s.x_part_base = ctr_cursor;
+          s.merge_ctr = ctr_cursor;
           ctr_cursor += g.Hkv;
           P.fused_rows += (long long)s.n * g.Hq;
         } else {
@@ -1279,22 +1281,18 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
     if (kv->umma_tile_keys != 128) return launch_attend_umma(ap, st);
     return inl ? launch_attend_umma128_inline(inline_segs(inl->seg_umma), st) : launch_attend_umma128(ap, st);
   };
+  // The decode kernel goes last: it merges the partials of shared ranges too.  It does not depend on the tcgen05 kernel
+  // otherwise: its blocks start on SMs that the tensor-bound kernel leaves idle (a small batch) or as its last items end.
   if (events) cudaEventRecord(kv->ev_attend[0], st);
-  if (dec && umma && !tile && kv->umma_tile_keys == 128 && !events) {
-    // The two kernels do not depend on each other.  The tensor-bound one goes first; the decode blocks start on SMs that
-    // it leaves idle (a small batch) or as its last items end.
-    if (launch_umma() != cudaSuccess || launch_dec(true) != cudaSuccess) return TIDE_ERR_CUDA;
-  } else {
-    if (dec && launch_dec(false) != cudaSuccess) return TIDE_ERR_CUDA;
-    if (events) cudaEventRecord(kv->ev_attend[1], st);
-    if (tile) {
-      ap.segs = d.seg_tile; ap.n_segs = (int)d.n_tile; ap.n_items = (int)d.items_tile;
-      ap.dyn = dyn ? dyn + kHdrTileItems : nullptr; ap.grid_cap = kv->cap_tile; ap.overlapped = 0;
-      if (launch_attend_tile(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
-      ++launches;
-    }
-    if (umma && launch_umma() != cudaSuccess) return TIDE_ERR_CUDA;
+  if (tile) {
+    ap.segs = d.seg_tile; ap.n_segs = (int)d.n_tile; ap.n_items = (int)d.items_tile;
+    ap.dyn = dyn ? dyn + kHdrTileItems : nullptr; ap.grid_cap = kv->cap_tile; ap.overlapped = 0;
+    if (launch_attend_tile(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
+    ++launches;
   }
+  if (umma && launch_umma() != cudaSuccess) return TIDE_ERR_CUDA;
+  if (events) cudaEventRecord(kv->ev_attend[1], st);
+  if (dec && launch_dec(umma && kv->umma_tile_keys == 128 && !events) != cudaSuccess) return TIDE_ERR_CUDA;
   if (events) cudaEventRecord(kv->ev_attend[2], st);
   if (merge) {
     MergeParams mp;
@@ -1464,6 +1462,7 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   kv->step_recs = n_rows;
   kv->step_tokens = indptr[(size_t)n_rows];
   kv->step_valid = true;
+  kv->step_layers = 0;
   kv->last_decode_items = P.items_dec;
   kv->last_prefill_items = P.items_tile + P.items_umma;
   kv->last_merge_rows = P.merge_rows + P.fused_rows;
@@ -1490,6 +1489,9 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   ap.new_k = (const uint16_t*)new_k;
   ap.new_v = (const uint16_t*)new_v;
   ap.g = kv->g;
+  ap.early = kv->step_layers > 0 && kv->step_stream == st ? 1 : 0;   // behind another layer, whose kernels waited for the upload
+  kv->step_stream = st;
+  ++kv->step_layers;
   if (launch_append(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
   int64_t launches = 0;
   const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, true, nullptr, q, scale, out, lse, st, false, &launches, dyn);
@@ -1673,8 +1675,8 @@ int tide_phase_ms(tide_kv_t* kv, float* append_ms, float* decode_ms, float* tile
   }
   if (kv->have_attend_times) {
     if (cudaEventSynchronize(kv->ev_attend[3]) != cudaSuccess) return TIDE_ERR_CUDA;
-    if (cudaEventElapsedTime(&d, kv->ev_attend[0], kv->ev_attend[1]) != cudaSuccess) return TIDE_ERR_CUDA;
-    if (cudaEventElapsedTime(&t, kv->ev_attend[1], kv->ev_attend[2]) != cudaSuccess) return TIDE_ERR_CUDA;
+    if (cudaEventElapsedTime(&t, kv->ev_attend[0], kv->ev_attend[1]) != cudaSuccess) return TIDE_ERR_CUDA;
+    if (cudaEventElapsedTime(&d, kv->ev_attend[1], kv->ev_attend[2]) != cudaSuccess) return TIDE_ERR_CUDA;
     if (cudaEventElapsedTime(&m, kv->ev_attend[2], kv->ev_attend[3]) != cudaSuccess) return TIDE_ERR_CUDA;
   }
   if (append_ms) *append_ms = a;

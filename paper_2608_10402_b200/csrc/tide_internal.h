@@ -64,13 +64,16 @@ struct __align__(16) Segment {
   int32_t causal;      // query i sees keys [0, p + i * causal + 1): 1 for a task's own tokens, 0 for a shared range
   int32_t origin;      // first key of the range this segment covers (split s starts at origin + s * chunk)
   int32_t partial;     // 1: write partials even when n_splits == 1 (another segment contributes to the same rows);
-                       // 2: a split decode-style segment whose last-finishing split merges the partials itself
-                       //    (AttendParams::merge_ctr[x_part_base + kv_head] counts the finished splits)
+                       // 2: a decode-style segment whose last-finishing split merges the partials itself
+                       //    (AttendParams::merge_ctr[merge_ctr + kv_head] counts the finished splits); a shared range's
+                       //    partials among them come from the tcgen05 kernel, which the decode kernel follows
   int32_t x_part_base; // the other contribution to this segment's rows: first partial row of token 0's head 0 ...
   int32_t x_n_splits;  // ... its number of splits (0 = none) ...
   int32_t x_stride;    // ... and the distance in rows between its consecutive splits
+  int32_t merge_ctr;
+  int32_t pad[3];
 };
-static_assert(sizeof(Segment) == 64, "Segment layout");
+static_assert(sizeof(Segment) == 80, "Segment layout");
 
 struct AttendParams {
   const uint8_t* pool;
@@ -143,6 +146,7 @@ struct AppendParams {
   const int32_t* upd_idx = nullptr;
   const int32_t* upd_val = nullptr;
   int n_upd = 0;
+  int early = 0;                  // the records were on the device before the kernel in front of this one started
 };
 
 // Small batches carry their descriptors in the launches themselves: an attention call whose kernels have up to kInlineSegs
