@@ -1084,18 +1084,20 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
     if (p.kind == kDec) w_dec += (long long)g.Hkv * own;
     else { w_tile += p.items * own; items_tile_nosplit += p.items; }
   }
-  // A shared range is streaming work like a decode row (few rows against many keys), so it is cut as finely as
-  // decode rows are, whichever kernel its packed rows call for.
+  // A shared range is streaming work like a decode row (few rows against many keys) and is cut like one, whichever kernel
+  // its packed rows call for.
   auto shared_kind = [&](int R) { return kind_of(R); };
   for (const ShareGroup& sg : groups) w_dec += (long long)g.Hkv * sg.pages * g.S;
-  const long long target = (long long)kv->num_sms * kv->items_per_sm;
+  // With groups in the batch a third fewer items, and a shared range on the tcgen05 kernel in pieces twice as long (one block
+  // of it fills an SM): 8 groups of 8, 6149 shared and 900 to 3100 own tokens, 78.2 us against 87.6 with the cut of a
+  // batch without groups; 4 of 4 38.9 and 41.8, 12 of 12 with 2000 shared 81.3 and 83.1, 2 of 8 with 11000 34.2 and 39.2.
+  const long long target = std::max<long long>(1, (long long)kv->num_sms * kv->items_per_sm * (groups.empty() ? 3 : 2) / 3);
   long long chunk_dec = std::max<long long>(256, align_up((size_t)(w_dec / target + 1), kStageKeys));
   long long chunk_tile = (items_tile_nosplit >= target / 2)
                              ? (1LL << 30)
                              : std::max<long long>(2048, align_up((size_t)(w_tile / target + 1), kStageKeys));
-  // a range of `len` keys cut for the given kind
-  auto cut = [&](bool streaming, int len, int& n_splits, int& chunk) {
-    const long long chunk_target = streaming ? chunk_dec : chunk_tile;
+  // a range of `len` keys cut into pieces of about chunk_target
+  auto cut = [&](long long chunk_target, int len, int& n_splits, int& chunk) {
     n_splits = (int)std::min<long long>(kMaxSplits, ((long long)len + chunk_target - 1) / chunk_target);
     n_splits = std::max(1, n_splits);
     chunk = (int)align_up((size_t)std::max(1, ceil_div(len, n_splits)), 2 * kStageKeys);
@@ -1118,7 +1120,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
         s.n = sg.m;
         s.p = sg.pages * g.S - 1;
         s.n_mtiles = mtiles_of(kind, sg.m * g.G);
-        cut(true, sg.pages * g.S, s.n_splits, s.chunk);
+        cut(kind == kUmma ? 2 * chunk_dec : chunk_dec, sg.pages * g.S, s.n_splits, s.chunk);
         s.causal = 0;
         s.live_from = INT_MAX;                               // full pages that several tasks hold: nothing writes them
         s.partial = 1;
@@ -1142,7 +1144,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
         s.x_n_splits = -1;                                   // marks a member until the links are resolved
         s.x_stride = b - groups[(size_t)gi].first;           // member index, for now
       }
-      cut(p.kind == kDec, r.ctx_len - s.origin, s.n_splits, s.chunk);
+      cut(p.kind == kDec ? chunk_dec : chunk_tile, r.ctx_len - s.origin, s.n_splits, s.chunk);
       if (s.n_splits > 1 || s.partial) part_rows += (long long)s.n_splits * r.q_len * g.Hq;
       (p.kind == kDec ? P.seg_dec : p.kind == kTile ? P.seg_tile : P.seg_umma).push_back(s);
       qoff += r.q_len;
