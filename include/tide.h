@@ -142,7 +142,7 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
  * the copies to be asynchronous.  The call returns after the results have arrived.  A small step (up to
  * 2 MiB in all) whose buffers are pinned and addressable by the device is not copied at all: the kernels
  * read the inputs and write the results across PCIe themselves.  A large step is cut
- * into groups of consecutive rows whose copies (on two streams the library owns) run beside the kernels
+ * into groups of consecutive tokens whose copies (on streams the library owns) run beside the kernels
  * of other groups; pages, cache contents and results do not depend on the cut.  The whole step is checked
  * (rows, duplicates, pages) before anything is copied or changed.  Takes layer 0 only. */
 int tide_step_host(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* rows /*host*/,
@@ -247,7 +247,7 @@ typedef enum {
   TIDE_TUNE_ITEMS_PER_SM = 0,     /* work items per SM the KV-split planner aims for, 1..64 (default 3)            */
   TIDE_TUNE_GROUPING = 1,         /* 0: never plan forked rows as groups that read shared pages once (default 1)   */
   TIDE_TUNE_MIN_SAVED_BYTES = 2,  /* KV bytes a batch must save before groups are used (default 64 MiB)            */
-  TIDE_TUNE_HOST_STEP_CHUNKS = 3, /* row groups of tide_step_host, 1..8; 0 = chosen by transfer size (default)     */
+  TIDE_TUNE_HOST_STEP_CHUNKS = 3, /* token groups of tide_step_host, 1..8; 0 = chosen by transfer size (default)   */
   TIDE_TUNE_UMMA_MIN_ROWS = 4,    /* packed rows (q_len * Hq/Hkv) from which a head_dim-128 row runs on the        */
                                   /* tcgen05 kernel, >= 17 (default 17)                                            */
   TIDE_TUNE_WAIT_LIMIT_US = 5,    /* time limit of every wait inside a kernel, microseconds (default 2 000 000)    */

@@ -31,7 +31,17 @@ constexpr int kStepSegStride = 2;   // each segment array of the step area holds
 // header of the step area (int32 words): counts a fixed-shape launch reads on the device, as (count, segments) pairs
 constexpr int kHdrRecs = 0, kHdrDecItems = 2, kHdrTileItems = 4, kHdrUmmaItems = 6, kHdrMergeRows = 8;
 constexpr int kMaxHostChunks = 8;                 // most row groups of one host-buffer step
-constexpr size_t kHostChunkBytes = 64u << 20;      // transfer bytes per group from which cutting a step pays
+constexpr int kHostEvents = 3 * kMaxHostChunks + 2;
+constexpr double kHostFirstShare = 0.5, kHostLastShare = 0.5;   // of an equal share
+// Groups of a host-buffer step by its transfer bytes, in and out.  Both directions together run at about 70 GB/s, so groups
+// only have to hide the kernels and one direction behind the other; every group costs copies and a tail of its kernels.
+// us with 1 / 3 / 4 / 5 / 6 / 8 groups: 8 MB 599 / 433 / 426 / 444 / 458 / 493, 28 MB 857 / 611 / 590 / 593 / 625 / 631,
+// 102 MB 2713 / 1818 / 1770 / 2000 / 1874 / 1899, 253 MB 6458 / 4452 / 4222 / 3958 / 4097 / 4106, 539 MB 13053 / 9164 / 8047 /
+// 7622 / 7439 / 7444.
+int host_chunks(size_t bytes) {
+  const size_t mb = bytes >> 20;
+  return mb < 4 ? 1 : mb < 12 ? 3 : mb < 120 ? 4 : mb < 400 ? 5 : 6;
+}
 constexpr size_t kZeroCopyBytes = 2u << 20;        // a host-buffer step up to this size is read and written in place (no copies)
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -96,7 +106,8 @@ struct tide_kv {
   int* d_merge_ctr = nullptr;   // finished-split counters of the segments whose last split merges (zero between launches)
   Slot slots[kSlots];
   int next_slot = 0;
-  int* h_status = nullptr;  // pinned
+  uint8_t* h_pinned = nullptr;   // pinned, mapped: the slots' host side, h_step, h_status
+  int* h_status = nullptr;
   // bookkeeping
   std::vector<int32_t> free_stack;  // back() is the next page handed out
   std::vector<uint8_t> live;
@@ -137,7 +148,7 @@ struct tide_kv {
   int umma_tile_keys = 128;              // key-tile size of the tcgen05 kernel: 64 (Q in TMEM) or 128 (Q in shared memory)
   bool drop_first_stage_once = false;    // test hook: armed by tide_tune, consumed by the next attention launch set
   // multi-layer step held between tide_step_begin and the tide_step_layer calls
-  uint8_t* h_step = nullptr;   // pinned staging of the step area
+  uint8_t* h_step = nullptr;   // staging of the step area
   cudaEvent_t ev_step = nullptr;
   bool step_upload_pending = false, step_valid = false;
   PlanDev step_plan;
@@ -148,7 +159,11 @@ struct tide_kv {
   int cap_dec = 0, cap_tile = 0, cap_umma = 0, cap_merge_rows = 0, cap_tokens = 0;
   // host-buffer steps: copy streams and the events that order them against the caller's stream
   cudaStream_t st_in = nullptr, st_out = nullptr;
-  cudaEvent_t ev_host[2 * kMaxHostChunks + 2] = {};   // copies-in done, kernels done (per group); start, end
+  cudaStream_t st_even = nullptr;                     // kernels of every other row group (the rest run on the caller's stream)
+  cudaEvent_t ev_host[kHostEvents] = {};              // copies-in done, append done, kernels done (per group); start, end
+  // the part of the partials and of the finished-split counters that a plan may use (two row groups run at a time)
+  long long part_row0 = 0, part_rows = 0;
+  int32_t merge_ctr0 = 0;
   int host_step_chunks = 0;   // 0 = by size
   bool slots_mapped = false;     // the staging slots' host addresses are valid on the device too
   bool upload_by_kernel = false;
@@ -339,6 +354,7 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
   kv->d_old_row = (int32_t*)(kv->ws + lay.off_old_row);
   kv->d_part_o = (float*)(kv->ws + lay.off_part_o);
   kv->d_part_lse = (float*)(kv->ws + lay.off_part_lse);
+  kv->part_rows = lay.part_rows;
   kv->d_merge_ctr = (int*)(kv->ws + lay.off_merge_ctr);
   bool ok = cudaGetDevice(&kv->device) == cudaSuccess;
   kv->num_sms = sm_count();
@@ -346,20 +362,25 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
   ok = ok && attend_kernels_init() == cudaSuccess && attend_decode_init() == cudaSuccess && attend_umma_init() == cudaSuccess && attend_umma128_init() == cudaSuccess;
   ok = ok && cudaMemset(kv->d_status, 0, 256) == cudaSuccess;
   ok = ok && cudaMemset(kv->d_merge_ctr, 0, (size_t)kStepSegStride * cfg->max_batch_rows * g.Hkv * 4) == cudaSuccess;
-  ok = ok && cudaHostAlloc((void**)&kv->h_status, 64, cudaHostAllocDefault) == cudaSuccess;
-  ok = ok && cudaHostAlloc((void**)&kv->h_step, lay.step_bytes, cudaHostAllocMapped) == cudaSuccess;
+  // one pinned, mapped allocation: staging slots, step area, status word (ten of them took most of this call's time)
+  const size_t pinned = (size_t)kSlots * lay.slot_bytes + lay.step_bytes + 256;
+  ok = ok && cudaHostAlloc((void**)&kv->h_pinned, pinned, cudaHostAllocMapped) == cudaSuccess;
+  if (ok) {
+    void* on_device = nullptr;
+    kv->slots_mapped = cudaHostGetDevicePointer(&on_device, kv->h_pinned, 0) == cudaSuccess && on_device == (void*)kv->h_pinned;
+    if (!kv->slots_mapped) cudaGetLastError();   // no unified addressing: uploads stay copy-engine transfers
+    kv->h_step = kv->h_pinned + (size_t)kSlots * lay.slot_bytes;
+    kv->h_status = (int*)(kv->h_step + lay.step_bytes);
+  }
   ok = ok && cudaEventCreateWithFlags(&kv->ev_step, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; ok && i < kSlots; ++i) {
-    ok = cudaHostAlloc((void**)&kv->slots[i].host, lay.slot_bytes, cudaHostAllocMapped) == cudaSuccess;
-    void* on_device = nullptr;
-    if (ok && i == 0) kv->slots_mapped = true;
-    if (ok && (cudaHostGetDevicePointer(&on_device, kv->slots[i].host, 0) != cudaSuccess || on_device != (void*)kv->slots[i].host)) {
-      kv->slots_mapped = false;   // no unified addressing: uploads stay copy-engine transfers
-      cudaGetLastError();
-    }
-    ok = ok && cudaEventCreateWithFlags(&kv->slots[i].ev, cudaEventDisableTiming) == cudaSuccess;
+    kv->slots[i].host = kv->h_pinned + (size_t)i * lay.slot_bytes;
     kv->slots[i].dev = kv->ws + lay.off_meta + (size_t)i * lay.slot_bytes;
+    ok = cudaEventCreateWithFlags(&kv->slots[i].ev, cudaEventDisableTiming) == cudaSuccess;
   }
+  // streams and events of large host-buffer steps: here, not in the first of these steps (200 us)
+  for (cudaStream_t* x : {&kv->st_in, &kv->st_out, &kv->st_even}) ok = ok && cudaStreamCreateWithFlags(x, cudaStreamNonBlocking) == cudaSuccess;
+  for (int i = 0; ok && i < kHostEvents; ++i) ok = cudaEventCreateWithFlags(&kv->ev_host[i], cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
     tide_kv_destroy(kv);
     return TIDE_ERR_CUDA;
@@ -380,15 +401,13 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
 int tide_kv_destroy(tide_kv_t* kv) {
   if (kv == nullptr) return TIDE_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
-  for (int i = 0; i < kSlots; ++i) {
-    if (kv->slots[i].host) cudaFreeHost(kv->slots[i].host);
+  for (int i = 0; i < kSlots; ++i)
     if (kv->slots[i].ev) cudaEventDestroy(kv->slots[i].ev);
-  }
-  if (kv->h_status) cudaFreeHost(kv->h_status);
-  if (kv->h_step) cudaFreeHost(kv->h_step);
+  if (kv->h_pinned) cudaFreeHost(kv->h_pinned);
   if (kv->ev_step) cudaEventDestroy(kv->ev_step);
   if (kv->st_in) cudaStreamDestroy(kv->st_in);
   if (kv->st_out) cudaStreamDestroy(kv->st_out);
+  if (kv->st_even) cudaStreamDestroy(kv->st_even);
   for (cudaEvent_t e : kv->ev_host) if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : kv->ev_append) if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : kv->ev_attend) if (e) cudaEventDestroy(e);
@@ -1149,7 +1168,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
       (p.kind == kDec ? P.seg_dec : p.kind == kTile ? P.seg_tile : P.seg_umma).push_back(s);
       qoff += r.q_len;
     }
-    if (part_rows <= kv->lay.part_rows) break;
+    if (part_rows <= kv->part_rows) break;
     chunk_dec *= 2;
     chunk_tile = std::min<long long>(chunk_tile * 2, 1LL << 30);
     if (attempt == 39) return TIDE_ERR_WORKSPACE;
@@ -1164,8 +1183,8 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
   P.seg_merge.clear();
   P.merge_rows = 0;
   P.fused_rows = 0;
-  long long part_cursor = 0;
-  int32_t ctr_cursor = 0;
+  long long part_cursor = kv->part_row0;
+  int32_t ctr_cursor = kv->merge_ctr0;
   std::vector<std::pair<const Segment*, int32_t>> merged;    // segments with rows to merge, and the first of these rows
   for (auto* v : {&P.seg_dec, &P.seg_tile, &P.seg_umma}) {
     long long base = 0;
@@ -1532,12 +1551,13 @@ int tide_step_host(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_
   uint8_t* dout = kv->ws + kv->lay.off_stage_out;
   float* dlse = (float*)(kv->ws + kv->lay.off_stage_lse);
   const size_t kv_row = (size_t)g.Hkv * g.D * 2, q_row = (size_t)g.Hq * g.D * 2, lse_row = (size_t)g.Hq * 4;
-  // Large steps are cut into groups of consecutive rows, each with its own copies in, append, attention and copies
+  // Large steps are cut into groups of consecutive tokens, each with its own copies in, append, attention and copies
   // out, so that the transfers of one group run beside the kernels of another (copy engines in both directions
-  // and the SMs all busy).  Appending the groups in row order takes the same pages as one append of all rows.
+  // and the SMs all busy).  A long row may be cut as well: its later tokens are a row of their own whose context holds the
+  // earlier ones.  Appending the groups in order takes the same pages as one append of all rows.
   const size_t bytes = T * (2 * kv_row + 2 * q_row + (lse ? lse_row : 0));
-  int n_chunks = kv->host_step_chunks > 0 ? kv->host_step_chunks : (int)std::min<size_t>(kMaxHostChunks, bytes / kHostChunkBytes);
-  n_chunks = std::max(1, std::min(std::min(n_chunks, kMaxHostChunks), n_rows));
+  int n_chunks = kv->host_step_chunks > 0 ? kv->host_step_chunks : host_chunks(bytes);
+  n_chunks = std::max(1, std::min(n_chunks, kMaxHostChunks));
   // A small step from pinned host buffers that the device can address is not copied at all: the append kernel reads
   // new_k / new_v, and the attention kernels read q and write out / lse, straight across PCIe.  Five copies of a few
   // hundred KB cost more in engine hand-overs than the bytes do (a 64-row decode step: 0.22 -> 0.20 ms, a tiny one
@@ -1560,52 +1580,80 @@ int tide_step_host(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_
       return TIDE_OK;
     }
   }
-  if (n_chunks > 1 && kv->st_in == nullptr) {
-    bool ok = cudaStreamCreateWithFlags(&kv->st_in, cudaStreamNonBlocking) == cudaSuccess;
-    ok = ok && cudaStreamCreateWithFlags(&kv->st_out, cudaStreamNonBlocking) == cudaSuccess;
-    for (int i = 0; ok && i < 2 * kMaxHostChunks + 2; ++i)
-      ok = cudaEventCreateWithFlags(&kv->ev_host[i], cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) return TIDE_ERR_CUDA;
+  // the groups: rows (parts of rows) with their tokens [t0, t0 + tn)
+  struct Group {
+    std::vector<int32_t> ids, ip;
+    std::vector<tide_row_t> rows;
+    size_t t0 = 0, tn = 0;
+  };
+  std::vector<Group> groups;
+  {
+    // Shares are equal but for the first and the last: nothing overlaps the first group's copies in, nor what follows the
+    // last copy in - that group's kernels and its copy out - so these are kept short.
+    double share[kMaxHostChunks], sum = 0.0, acc = 0.0;
+    for (int c = 0; c < n_chunks; ++c) {
+      share[c] = n_chunks < 3 ? 1.0 : c == 0 ? kHostFirstShare : c == n_chunks - 1 ? kHostLastShare : 1.0;
+      sum += share[c];
+    }
+    const int tile = std::max(1, 2 * kUmmaTileRows / g.G);                // tokens of a tcgen05 work item
+    int b = 0, used = 0;                                                  // next row, tokens of it taken already
+    size_t t = 0;
+    for (int c = 0; c < n_chunks && b < n_rows; ++c) {
+      acc += share[c];
+      const size_t goal = c == n_chunks - 1 ? T : (size_t)((double)T * acc / sum);
+      Group gr;
+      gr.t0 = t;
+      gr.ip.push_back(0);
+      while (b < n_rows && (t < goal || c == n_chunks - 1)) {
+        const int rem = rows[b].q_len - used;
+        int take = rem;
+        if (c < n_chunks - 1 && t + (size_t)rem > goal) {
+          const int want = (int)(goal - t) / tile * tile;
+          if (want >= 2 * tile && rem - want >= 2 * tile) take = want;
+          else if ((goal - t) * 2 < (size_t)rem && !gr.rows.empty()) break;    // most of it belongs to the next group
+        }
+        used += take;
+        t += (size_t)take;
+        gr.rows.push_back(tide_row_t{rows[b].task, take, rows[b].ctx_len - rows[b].q_len + used});
+        gr.ids.push_back(rows[b].task);
+        gr.ip.push_back((int32_t)(t - gr.t0));
+        if (used == rows[b].q_len) { ++b; used = 0; }
+        else break;
+      }
+      gr.tn = t - gr.t0;
+      if (gr.tn > 0) groups.push_back(std::move(gr));
+    }
+    n_chunks = (int)groups.size();
   }
   cudaStream_t s_in = n_chunks > 1 ? kv->st_in : st, s_out = n_chunks > 1 ? kv->st_out : st;
-  struct UploadMode {   // planning uploads bypass the copy engine while this step's large copies are in flight
+  struct GroupMode {   // planning uploads bypass the copy engine while this step's large copies are in flight
     tide_kv* kv;
-    ~UploadMode() { kv->upload_by_kernel = false; }
-  } upload_mode{kv};
+    ~GroupMode() {
+      kv->upload_by_kernel = false;
+      kv->part_row0 = 0;
+      kv->part_rows = kv->lay.part_rows;
+      kv->merge_ctr0 = 0;
+    }
+  } group_mode{kv};
   kv->upload_by_kernel = n_chunks > 1 && kv->slots_mapped;
-  cudaEvent_t ev_start = kv->ev_host[2 * kMaxHostChunks], ev_end = kv->ev_host[2 * kMaxHostChunks + 1];
+  cudaEvent_t *ev_in = kv->ev_host, *ev_app = ev_in + kMaxHostChunks, *ev_done = ev_app + kMaxHostChunks;
+  cudaEvent_t ev_start = kv->ev_host[3 * kMaxHostChunks], ev_end = kv->ev_host[3 * kMaxHostChunks + 1];
   if (n_chunks > 1) {
     // the copies in may not overtake work already queued on the caller's stream that still uses the staging area
-    if (cudaEventRecord(ev_start, st) != cudaSuccess || cudaStreamWaitEvent(s_in, ev_start, 0) != cudaSuccess) return TIDE_ERR_CUDA;
-    if (cudaStreamWaitEvent(s_out, ev_start, 0) != cudaSuccess) return TIDE_ERR_CUDA;
-  }
-  // rows [cut[c], cut[c+1]): up to the c+1-th share of the tokens, at least one row each.  The shares are equal but for
-  // the last two groups, which are a half and a fifth of a share: what follows the last copy in - that group's kernels
-  // and its copy out - is the part of the step that nothing overlaps, so it is kept short.
-  int cut[kMaxHostChunks + 1];
-  cut[0] = 0;
-  double share[kMaxHostChunks], share_sum = 0.0, share_acc = 0.0;
-  for (int c = 0; c < n_chunks; ++c) {
-    share[c] = (n_chunks >= 4 && c == n_chunks - 1) ? 0.2 : (n_chunks >= 4 && c == n_chunks - 2) ? 0.5 : 1.0;
-    share_sum += share[c];
-  }
-  for (int c = 0; c < n_chunks; ++c) {
-    int r1 = cut[c] + 1;
-    share_acc += share[c];
-    const long long goal = (long long)((double)T * share_acc / share_sum);
-    while (r1 < n_rows && indptr[(size_t)r1 + 1] <= goal && n_rows - r1 > n_chunks - 1 - c) ++r1;
-    cut[c + 1] = c == n_chunks - 1 ? n_rows : r1;
+    if (cudaEventRecord(ev_start, st) != cudaSuccess) return TIDE_ERR_CUDA;
+    for (cudaStream_t x : {s_in, s_out, kv->st_even})
+      if (cudaStreamWaitEvent(x, ev_start, 0) != cudaSuccess) return TIDE_ERR_CUDA;
   }
   // The copy engine works through its queue in order.  If the small uploads that every append and attention call
   // makes (records, plan) go through the same queue, the copies in of group c+1 are queued right AFTER the calls
   // of group c: queued earlier they would hold those uploads, and with them the kernels, back.
   auto copy_in = [&](int c) -> int {
-    const size_t t0 = (size_t)indptr[(size_t)cut[c]], tn = (size_t)indptr[(size_t)cut[c + 1]] - t0;
+    const size_t t0 = groups[(size_t)c].t0, tn = groups[(size_t)c].tn;
     if (cudaMemcpyAsync(dk + t0 * kv_row, (const uint8_t*)new_k + t0 * kv_row, tn * kv_row, cudaMemcpyHostToDevice, s_in) != cudaSuccess ||
         cudaMemcpyAsync(dv + t0 * kv_row, (const uint8_t*)new_v + t0 * kv_row, tn * kv_row, cudaMemcpyHostToDevice, s_in) != cudaSuccess ||
         cudaMemcpyAsync(dq + t0 * q_row, (const uint8_t*)q + t0 * q_row, tn * q_row, cudaMemcpyHostToDevice, s_in) != cudaSuccess)
       return TIDE_ERR_CUDA;
-    if (n_chunks > 1 && cudaEventRecord(kv->ev_host[c], s_in) != cudaSuccess) return TIDE_ERR_CUDA;
+    if (n_chunks > 1 && cudaEventRecord(ev_in[c], s_in) != cudaSuccess) return TIDE_ERR_CUDA;
     return TIDE_OK;
   };
   // With kernel uploads nothing of the calls goes through the copy engine, and every copy in can be queued at once.
@@ -1613,25 +1661,34 @@ int tide_step_host(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_
   for (int c = 0; c < (all_first ? n_chunks : 1); ++c)
     if ((rc = copy_in(c)) != TIDE_OK) return rc;
   int64_t launches = 0, dec_items = 0, pre_items = 0, mrg_rows = 0;
-  std::vector<int32_t> ip;
   for (int c = 0; c < n_chunks; ++c) {
-    const int r0 = cut[c], r1 = cut[c + 1];
-    const size_t t0 = (size_t)indptr[(size_t)r0], tn = (size_t)indptr[(size_t)r1] - t0;
-    cudaEvent_t ev_done = kv->ev_host[kMaxHostChunks + c];
-    if (n_chunks > 1 && cudaStreamWaitEvent(st, kv->ev_host[c], 0) != cudaSuccess) return TIDE_ERR_CUDA;
-    ip.assign((size_t)(r1 - r0) + 1, 0);
-    for (int b = r0; b <= r1; ++b) ip[(size_t)(b - r0)] = indptr[(size_t)b] - (int32_t)t0;
-    rc = tide_kv_append(kv, layer, r1 - r0, ids.data() + r0, ip.data(), dk + t0 * kv_row, dv + t0 * kv_row, stream);
+    const Group& gr = groups[(size_t)c];
+    const int rows_c = (int)gr.rows.size();
+    // Groups take turns on two streams, so that the kernels of one start on the SMs that the last blocks of the one before
+    // leave idle; their appends stay in order, and each has its own half of the partials and its own counters.
+    cudaStream_t s_k = st;
+    if (n_chunks > 1) {
+      s_k = c % 2 == 0 ? kv->st_even : st;
+      kv->part_rows = kv->lay.part_rows / 2;
+      kv->part_row0 = (c % 2) * kv->part_rows;
+      kv->merge_ctr0 = (c % 2) * kv->cfg.max_batch_rows * g.Hkv;
+      if (cudaStreamWaitEvent(s_k, ev_in[c], 0) != cudaSuccess) return TIDE_ERR_CUDA;
+      if (c > 0 && cudaStreamWaitEvent(s_k, ev_app[c - 1], 0) != cudaSuccess) return TIDE_ERR_CUDA;
+    }
+    rc = tide_kv_append(kv, layer, rows_c, gr.ids.data(), gr.ip.data(), dk + gr.t0 * kv_row, dv + gr.t0 * kv_row, s_k);
     if (rc != TIDE_OK) return rc;
-    rc = tide_attend(kv, layer, r1 - r0, rows + r0, nullptr, dq + t0 * q_row, scale, dout + t0 * q_row,
-                     lse ? dlse + t0 * g.Hq : nullptr, stream);
+    if (n_chunks > 1 && cudaEventRecord(ev_app[c], s_k) != cudaSuccess) return TIDE_ERR_CUDA;
+    rc = tide_attend(kv, layer, rows_c, gr.rows.data(), nullptr, dq + gr.t0 * q_row, scale, dout + gr.t0 * q_row,
+                     lse ? dlse + gr.t0 * g.Hq : nullptr, s_k);
     if (rc != TIDE_OK) return rc;
     launches += kv->last_launches; dec_items += kv->last_decode_items; pre_items += kv->last_prefill_items; mrg_rows += kv->last_merge_rows;
     if (!all_first && c + 1 < n_chunks && (rc = copy_in(c + 1)) != TIDE_OK) return rc;
-    if (n_chunks > 1 && (cudaEventRecord(ev_done, st) != cudaSuccess || cudaStreamWaitEvent(s_out, ev_done, 0) != cudaSuccess))
+    if (n_chunks > 1 && (cudaEventRecord(ev_done[c], s_k) != cudaSuccess || cudaStreamWaitEvent(s_out, ev_done[c], 0) != cudaSuccess))
       return TIDE_ERR_CUDA;
-    if (cudaMemcpyAsync((uint8_t*)out + t0 * q_row, dout + t0 * q_row, tn * q_row, cudaMemcpyDeviceToHost, s_out) != cudaSuccess) return TIDE_ERR_CUDA;
-    if (lse && cudaMemcpyAsync(lse + t0 * g.Hq, dlse + t0 * g.Hq, tn * lse_row, cudaMemcpyDeviceToHost, s_out) != cudaSuccess) return TIDE_ERR_CUDA;
+    if (cudaMemcpyAsync((uint8_t*)out + gr.t0 * q_row, dout + gr.t0 * q_row, gr.tn * q_row, cudaMemcpyDeviceToHost, s_out) != cudaSuccess)
+      return TIDE_ERR_CUDA;
+    if (lse && cudaMemcpyAsync(lse + gr.t0 * g.Hq, dlse + gr.t0 * g.Hq, gr.tn * lse_row, cudaMemcpyDeviceToHost, s_out) != cudaSuccess)
+      return TIDE_ERR_CUDA;
   }
   kv->last_launches = launches; kv->last_decode_items = dec_items; kv->last_prefill_items = pre_items; kv->last_merge_rows = mrg_rows;
   if (n_chunks > 1) {
