@@ -4,11 +4,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtide.so")
 SOURCES = ["tide_host.cu", "kv_pages.cu", "attend_decode.cu", "attend_mma.cu", "attend_umma.cu", "attend_umma128.cu", "attend_static.cu"]
+BINDING = os.path.join(HERE, "_binding.so")      # CPython module of the hot calls, linked against libtide.so
+BINDING_SOURCE = os.path.join(CSRC, "binding.cpp")
 HEADERS = ["tide_internal.h", os.path.join("..", "..", "include", "tide.h")]
 
 
@@ -24,15 +27,15 @@ def sources():
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + [os.path.join(CSRC, h) for h in HEADERS]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
+    deps = sources() + [BINDING_SOURCE] + [os.path.join(CSRC, h) for h in HEADERS]
     return any(os.path.getmtime(d) > t for d in deps if os.path.exists(d))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every kernel for sm_100a and link libtide.so next to this file."""
+    """Compile every kernel for sm_100a and link libtide.so next to this file, then the CPython module beside it."""
     if not force and not is_stale():
         return LIB
     os.makedirs(os.path.join(HERE, "build"), exist_ok=True)
@@ -56,6 +59,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.check_call([_nvcc(), "-arch=sm_100a", "-shared", "-o", tmp] + objs + ["-lcudart_static", "-lpthread", "-ldl", "-lrt"])
     os.replace(tmp, LIB)
+    tmp = BINDING + f".tmp{os.getpid()}"
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wall", "-I", sysconfig.get_paths()["include"], BINDING_SOURCE,
+                           "-o", tmp, "-L", HERE, "-l:libtide.so", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, BINDING)
     return LIB
 
 

@@ -63,7 +63,20 @@ struct PlanDev {
   long long items_dec = 0, items_tile = 0, items_umma = 0, merge_rows = 0;
 };
 
+struct RowPlan { int kind; int n_mtiles; long long items; };
+
+// Rows of one batch whose tasks hold the same first pages (forked tasks of a GRPO group, Section 2.1) are planned as
+// a group: consecutive decode rows of distinct tasks whose page lists agree on at least kMinSharedTokens tokens of
+// full pages that every member's context covers.
+struct ShareGroup {
+  int first = 0, m = 0, pages = 0;       // first member row, members, shared pages
+  int32_t part_base = 0, n_splits = 0;   // of the shared range's segment, known once it has been placed
+};
+
 struct PlanHost {
+  std::vector<RowPlan> row_plan;
+  std::vector<ShareGroup> groups;
+  std::vector<int> group_of;             // per row: its group or -1
   std::vector<Segment> seg_dec, seg_tile, seg_umma, seg_merge;
   long long items_dec = 0, items_tile = 0, items_umma = 0, merge_rows = 0;
   long long fused_rows = 0;   // rows whose partials are merged by the decode kernel itself (not part of merge_rows)
@@ -101,6 +114,7 @@ struct tide_kv {
   float* d_part_o = nullptr;
   float* d_part_lse = nullptr;
   AppendInline append_inline;   // host images of the launches that carry their descriptors
+  PlanHost plan;                // scratch of build_plan and its callers; its arrays keep their capacity from call to call
   AttendInline attend_inline;
   MergeInline merge_inline;
   int* d_merge_ctr = nullptr;   // finished-split counters of the segments whose last split merges (zero between launches)
@@ -1005,13 +1019,6 @@ static int check_rows(tide_kv* kv, int32_t n_rows, const tide_row_t* rows) {
   return TIDE_OK;
 }
 
-// Rows of one batch whose tasks hold the same first pages (forked tasks of a GRPO group, Section 2.1) are planned as
-// a group: consecutive decode rows of distinct tasks whose page lists agree on at least kMinSharedTokens tokens of
-// full pages that every member's context covers.
-struct ShareGroup {
-  int first = 0, m = 0, pages = 0;       // first member row, members, shared pages
-  int32_t part_base = 0, n_splits = 0;   // of the shared range's segment, known once it has been placed
-};
 constexpr int kMinSharedTokens = 256;
 
 constexpr int kMaxGroupRows = 64;        // packed rows of a shared range (one 64-row tile of the warp-MMA kernel, a quarter of a tcgen05 item)
@@ -1083,14 +1090,15 @@ static bool umma_takes(const tide_kv* kv) { return kv->g.D == 128 || kv->umma_ti
 static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool umma_ok, bool allow_groups, bool step, PlanHost& P) {
   const Geom& g = kv->g;
   enum { kDec = 0, kTile = 1, kUmma = 2 };
-  struct RowPlan { int kind; int n_mtiles; long long items; };
   auto kind_of = [&](int R) { return R <= kDecodeTileRows ? kDec : (umma_ok && R >= kv->umma_min_rows ? kUmma : kTile); };
   auto mtiles_of = [&](int kind, int R) { return kind == kDec ? 1 : ceil_div(R, kind == kUmma ? 2 * kUmmaTileRows : kMmaTileRows); };
-  std::vector<ShareGroup> groups;
-  std::vector<int> group_of;
+  std::vector<ShareGroup>& groups = P.groups;
+  std::vector<int>& group_of = P.group_of;
+  groups.clear();
   if (allow_groups) find_share_groups(kv, n_rows, rows, groups, group_of);
   else group_of.assign((size_t)n_rows, -1);
-  std::vector<RowPlan> plan((size_t)n_rows);
+  std::vector<RowPlan>& plan = P.row_plan;
+  plan.resize((size_t)n_rows);
   long long w_dec = 0, w_tile = 0, items_tile_nosplit = 0;
   for (int b = 0; b < n_rows; ++b) {
     const tide_row_t& r = rows[b];
@@ -1177,9 +1185,9 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
   auto heavier = [](const Segment& a, const Segment& b) {
     return std::min(a.chunk, a.p + a.n - a.origin) > std::min(b.chunk, b.p + b.n - b.origin);
   };
-  std::stable_sort(P.seg_dec.begin(), P.seg_dec.end(), heavier);
-  std::stable_sort(P.seg_tile.begin(), P.seg_tile.end(), heavier);
-  std::stable_sort(P.seg_umma.begin(), P.seg_umma.end(), heavier);
+  if (P.seg_dec.size() > 1) std::stable_sort(P.seg_dec.begin(), P.seg_dec.end(), heavier);
+  if (P.seg_tile.size() > 1) std::stable_sort(P.seg_tile.begin(), P.seg_tile.end(), heavier);
+  if (P.seg_umma.size() > 1) std::stable_sort(P.seg_umma.begin(), P.seg_umma.end(), heavier);
   P.seg_merge.clear();
   P.merge_rows = 0;
   P.fused_rows = 0;
@@ -1350,7 +1358,7 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
   if (!(scale == scale)) return TIDE_ERR_INVALID_ARG;
   int rc = check_rows(kv, n_rows, rows);
   if (rc != TIDE_OK) return rc;
-  PlanHost P;
+  PlanHost& P = kv->plan;
   if ((rc = build_plan(kv, n_rows, rows, umma_takes(kv) && scale > 0.f, page_table == nullptr, false, P)) != TIDE_OK) return rc;
   if (P.n_all() * sizeof(Segment) + 256 > kv->lay.slot_bytes) return TIDE_ERR_WORKSPACE;
 
@@ -1414,7 +1422,7 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   if (rc != TIDE_OK) return rc;
   // The plan needs the lengths after the step only through ctx_len, which the rows already carry, so it is built
   // (and can still be refused) before anything changes.
-  PlanHost P;
+  PlanHost& P = kv->plan;
   // Launch shapes fixed without tcgen05 items (or with too few): head size 64 has the warp-MMA tile kernel as well.
   bool umma = umma_takes(kv) && !(kv->fixed_grids && g.D == 64 && kv->cap_umma == 0);
   if ((rc = build_plan(kv, n_rows, rows, umma, true, true, P)) != TIDE_OK) return rc;

@@ -1,7 +1,8 @@
-"""ctypes binding of libtide.so: the same names as include/tide.h, argument marshalling only.
+"""Binding of libtide.so: the same names as include/tide.h, argument marshalling only.
 
 Every step of the path runs inside the CUDA library; this module only turns torch tensors / numpy
-arrays into pointers.  There is no fallback: if libtide.so is missing or cannot be loaded the import
+arrays into pointers: through the CPython module _binding for the calls of an engine step, through ctypes
+for the others.  There is no fallback: if one of the two libraries is missing or cannot be loaded the import
 of this module raises.
 """
 from __future__ import annotations
@@ -58,6 +59,7 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2608_10402_b200.build` "
                       "(there is no fallback path)")
 lib = ctypes.CDLL(LIB_PATH)
+from . import _binding as _b  # noqa: E402  (after the message above: it is linked against libtide.so)
 lib.tide_strerror.restype = ctypes.c_char_p
 lib.tide_strerror.argtypes = [ctypes.c_int]
 for _name in EXPORTS[1:]:
@@ -88,19 +90,28 @@ def _ptr(x):
     return ctypes.c_void_p(x.data_ptr())
 
 
-def _raw_stream():
-    """The current stream's handle.  torch.cuda.current_stream() builds a Stream object on every call (3.2 us, twice in a
-    decode step whose kernels take 17 us); the raw handle costs 0.2 us."""
+_ready = False
+
+
+def _prepare_binding():
+    """Gives _binding the accessors of torch's current stream.  (torch.cuda.current_stream() builds a Stream object on every
+    call, 3.2 us; the raw handle costs 0.2.)"""
+    global _ready
+    if _ready:
+        return
     import torch
     raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    if raw is None or not torch.cuda.is_initialized():
-        return torch.cuda.current_stream().cuda_stream
-    return raw(torch._C._cuda_getDevice())
+    if raw is not None:
+        _b.use(torch._C._cuda_getDevice, raw, _i32)
+    else:
+        _b.use(torch.cuda.current_device, lambda device: torch.cuda.current_stream(device).cuda_stream, _i32)
+    _ready = True
 
 
 def _stream(stream):
     if stream is None:
-        return ctypes.c_void_p(_raw_stream())
+        import torch
+        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
     return ctypes.c_void_p(stream.cuda_stream)
@@ -150,12 +161,16 @@ class TideKV:
         self.cfg.free_order = None if free_order is None else self._free_order.ctypes.data
         self.Hq, self.Hkv, self.D, self.S = int(Hq), int(Hkv), int(D), int(S)
         self.handle = ctypes.c_void_p(0)
+        self._h = 0
         _check(lib.tide_kv_create(ctypes.byref(self.cfg), ctypes.byref(self.handle)), "tide_kv_create")
+        self._h = self.handle.value
+        _prepare_binding()
 
     def close(self):
         if self.handle:
             lib.tide_kv_destroy(self.handle)
             self.handle = ctypes.c_void_p(0)
+            self._h = 0
 
     def __del__(self):
         try:
@@ -189,32 +204,34 @@ class TideKV:
         _check(lib.tide_kv_release_many(self.handle, ctypes.c_int32(ids.shape[0]), _ptr(ids)), "tide_kv_release_many")
 
     def prune(self, task, keep_prefix, tail_begin, stream=None):
-        _check(lib.tide_kv_prune(self.handle, ctypes.c_int32(0), ctypes.c_int32(task), ctypes.c_int32(keep_prefix),
-                                 ctypes.c_int32(tail_begin), _stream(stream)), "tide_kv_prune")
+        rc = _b.prune(self._h, task, keep_prefix, tail_begin, stream)
+        if rc:
+            raise TideError(rc, "tide_kv_prune")
 
     def truncate(self, task, new_len):
-        _check(lib.tide_kv_truncate(self.handle, ctypes.c_int32(task), ctypes.c_int32(new_len)), "tide_kv_truncate")
+        rc = _b.truncate(self._h, task, new_len)
+        if rc:
+            raise TideError(rc, "tide_kv_truncate")
 
     def append(self, task_ids, indptr, new_k, new_v, stream=None):
-        ids, ip = _i32(task_ids), _i32(indptr)
-        assert ip.shape[0] == ids.shape[0] + 1
-        _check(lib.tide_kv_append(self.handle, ctypes.c_int32(0), ctypes.c_int32(ids.shape[0]), _ptr(ids), _ptr(ip),
-                                  _ptr(new_k), _ptr(new_v), _stream(stream)), "tide_kv_append")
+        rc = _b.append(self._h, task_ids, indptr, new_k, new_v, stream)
+        if rc:
+            raise TideError(rc, "tide_kv_append")
 
     def extend(self, task_ids, indptr, stream=None):
-        ids, ip = _i32(task_ids), _i32(indptr)
-        assert ip.shape[0] == ids.shape[0] + 1
-        _check(lib.tide_kv_extend(self.handle, ctypes.c_int32(ids.shape[0]), _ptr(ids), _ptr(ip), _stream(stream)), "tide_kv_extend")
+        rc = _b.extend(self._h, task_ids, indptr, stream)
+        if rc:
+            raise TideError(rc, "tide_kv_extend")
 
     def write(self, layer, task_ids, indptr, new_k, new_v, stream=None):
-        ids, ip = _i32(task_ids), _i32(indptr)
-        assert ip.shape[0] == ids.shape[0] + 1
-        _check(lib.tide_kv_write(self.handle, ctypes.c_int32(layer), ctypes.c_int32(ids.shape[0]), _ptr(ids), _ptr(ip),
-                                 _ptr(new_k), _ptr(new_v), _stream(stream)), "tide_kv_write")
+        rc = _b.write(self._h, layer, task_ids, indptr, new_k, new_v, stream)
+        if rc:
+            raise TideError(rc, "tide_kv_write")
 
     def step_begin(self, rows, stream=None):
-        arr = rows if not isinstance(rows, (list, tuple)) else rows_array(rows)
-        _check(lib.tide_step_begin(self.handle, ctypes.c_int32(len(arr)), arr, _stream(stream)), "tide_step_begin")
+        rc = _b.step_begin(self._h, rows_array(rows) if isinstance(rows, (list, tuple)) else rows, stream)
+        if rc:
+            raise TideError(rc, "tide_step_begin")
 
     def step_fix_grids(self, max_decode_items=0, max_tile_items=0, max_umma_items=0, max_merge_rows=0, max_tokens=0):
         _check(lib.tide_step_fix_grids(self.handle, ctypes.c_int32(max_decode_items), ctypes.c_int32(max_tile_items),
@@ -222,13 +239,14 @@ class TideKV:
                                        ctypes.c_int32(max_tokens)), "tide_step_fix_grids")
 
     def step_layer(self, layer, new_k, new_v, q, scale, out, lse=None, stream=None):
-        _check(lib.tide_step_layer(self.handle, ctypes.c_int32(layer), _ptr(new_k), _ptr(new_v), _ptr(q),
-                                   ctypes.c_float(scale), _ptr(out), _ptr(lse), _stream(stream)), "tide_step_layer")
+        rc = _b.step_layer(self._h, layer, new_k, new_v, q, scale, out, lse, stream)
+        if rc:
+            raise TideError(rc, "tide_step_layer")
 
     def attend(self, rows, q, scale, out, lse=None, page_table=None, stream=None, layer=0):
-        arr = rows if not isinstance(rows, (list, tuple)) else rows_array(rows)
-        _check(lib.tide_attend(self.handle, ctypes.c_int32(layer), ctypes.c_int32(len(arr)), arr, _ptr(page_table), _ptr(q),
-                               ctypes.c_float(scale), _ptr(out), _ptr(lse), _stream(stream)), "tide_attend")
+        rc = _b.attend(self._h, layer, rows_array(rows) if isinstance(rows, (list, tuple)) else rows, page_table, q, scale, out, lse, stream)
+        if rc:
+            raise TideError(rc, "tide_attend")
 
     def attend_decode_static(self, rows, q, scale, out, lse=None, stream=None):
         """tide_attend_decode_static: decode-style rows only, scratch in the library's fixed device array."""
@@ -237,9 +255,9 @@ class TideKV:
                                              _ptr(out), _ptr(lse), _stream(stream)), "tide_attend_decode_static")
 
     def step_host(self, rows, new_k, new_v, q, scale, out, lse=None, stream=None):
-        arr = rows if not isinstance(rows, (list, tuple)) else rows_array(rows)
-        _check(lib.tide_step_host(self.handle, ctypes.c_int32(0), ctypes.c_int32(len(arr)), arr, _ptr(new_k), _ptr(new_v),
-                                  _ptr(q), ctypes.c_float(scale), _ptr(out), _ptr(lse), _stream(stream)), "tide_step_host")
+        rc = _b.step_host(self._h, rows_array(rows) if isinstance(rows, (list, tuple)) else rows, new_k, new_v, q, scale, out, lse, stream)
+        if rc:
+            raise TideError(rc, "tide_step_host")
 
     # ---- introspection ----
     def task_len(self, task):
