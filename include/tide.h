@@ -244,7 +244,8 @@ int tide_last_plan(tide_kv_t* kv, int64_t* decode_items, int64_t* prefill_items,
  * environment.  Changing a setting closes an open step (tide_step_begin must be called again).
  * TIDE_ERR_INVALID_ARG for an unknown knob or a value outside its range. */
 typedef enum {
-  TIDE_TUNE_ITEMS_PER_SM = 0,     /* work items per SM the KV-split planner aims for, 1..64 (default 3)            */
+  TIDE_TUNE_ITEMS_PER_SM = 0,     /* work items per SM the KV-split planner aims for, 1..64 (default: for decode    */
+                                  /* rows chosen by the batch, 3 otherwise)                                        */
   TIDE_TUNE_GROUPING = 1,         /* 0: never plan forked rows as groups that read shared pages once (default 1)   */
   TIDE_TUNE_MIN_SAVED_BYTES = 2,  /* KV bytes a batch must save before groups are used (default 64 MiB)            */
   TIDE_TUNE_HOST_STEP_CHUNKS = 3, /* token groups of tide_step_host, 1..8; 0 = chosen by transfer size (default)   */

@@ -157,6 +157,7 @@ struct tide_kv {
   int umma_min_rows = kDecodeTileRows + 1;  // packed rows from which a resume row takes the tcgen05 path (measured:
                                             // it beats the warp-MMA tile path from the first row beyond a decode item)
   int items_per_sm = kTargetItemsPerSm;  // work items the planner aims for per SM
+  bool items_per_sm_set = false;         // by the caller: decode rows are then cut for it as well
   int num_sms = 0;                       // multiprocessors of the handle's device
   long long wait_limit_ns = kWaitLimitNsDefault;   // bound of every wait inside a kernel
   int umma_tile_keys = 128;              // key-tile size of the tcgen05 kernel: 64 (Q in TMEM) or 128 (Q in shared memory)
@@ -1120,6 +1121,29 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
   // batch without groups; 4 of 4 38.9 and 41.8, 12 of 12 with 2000 shared 81.3 and 83.1, 2 of 8 with 11000 34.2 and 39.2.
   const long long target = std::max<long long>(1, (long long)kv->num_sms * kv->items_per_sm * (groups.empty() ? 3 : 2) / 3);
   long long chunk_dec = std::max<long long>(256, align_up((size_t)(w_dec / target + 1), kStageKeys));
+  if (groups.empty() && !kv->items_per_sm_set && w_dec > 0) {
+    // Decode rows: the launch holds 2 blocks per SM at a time, and what is left over when their number is exceeded by a few
+    // runs alone.  So rows are cut as finely as ONE round of blocks allows when a block then reads up to 1.6 MB, and as two
+    // rounds allow otherwise (or as many as there are rows and KV heads).  us with the cut that leaves n items: 20 rows of
+    // 1k to 32k keys 55.5 (296), 60.6 (464); 48 rows of eight layers 521 (308), 537 (540); 100 rows of one KV head 55.2 (244),
+    // 58.4 (493); 130 rows of 300 to 8k keys 96.9 (568), 100.3 (740); 64 rows of 64-wide heads 152.5 (584), 158.5 (744);
+    // 64 rows of 1k to 32k keys 133.0 (408), 130.1 (556), 137.8 (660).
+    const long long blocks = 2LL * kv->num_sms;
+    long long dec_rows = 0;
+    for (const RowPlan& p : plan) dec_rows += p.kind == kDec;
+    const long long rounds = std::max<long long>(w_dec * g.D * 4 / blocks <= (1600ll << 10) ? 1 : 2, (dec_rows * g.Hkv + blocks - 1) / blocks);
+    double target_keys = std::max(256.0, (double)w_dec / (double)(blocks * rounds));
+    for (int step = 0; step < 6; ++step) {
+      long long items = 0;
+      const double inv = 1.0 / target_keys;
+      for (int b = 0; b < n_rows; ++b)
+        if (plan[(size_t)b].kind == kDec) items += (long long)((double)(rows[b].ctx_len - 1) * inv) + 1;
+      items *= g.Hkv;
+      if (items <= blocks * rounds) break;
+      target_keys *= std::max(1.02, (double)items / (double)(blocks * rounds));
+    }
+    chunk_dec = align_up((size_t)target_keys, 2 * kStageKeys);
+  }
   long long chunk_tile = (items_tile_nosplit >= target / 2)
                              ? (1LL << 30)
                              : std::max<long long>(2048, align_up((size_t)(w_tile / target + 1), kStageKeys));
@@ -1760,6 +1784,7 @@ int tide_tune(tide_kv_t* kv, int knob, int64_t value) {
     case TIDE_TUNE_ITEMS_PER_SM:
       if (value < 1 || value > 64) return TIDE_ERR_INVALID_ARG;
       kv->items_per_sm = (int)value;
+      kv->items_per_sm_set = true;
       break;
     case TIDE_TUNE_GROUPING: kv->no_grouping = value == 0; break;
     case TIDE_TUNE_MIN_SAVED_BYTES:
