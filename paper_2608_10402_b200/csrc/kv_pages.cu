@@ -38,6 +38,21 @@ cudaError_t launch_upload(void* dst, const void* src_mapped_host, size_t bytes, 
   return launch_dep(upload_kernel, blocks, 256, 0, s, (uint32_t*)dst, (const uint32_t*)src_mapped_host, n);
 }
 
+// Queries of a small host-buffer step: each byte crosses PCIe once, 16 at a time, while the append in front of this launch
+// runs (the destination is idle: the step before has been waited for).  Read in place by the decode kernel they crossed it
+// once per work item and consumer warp, 32 bytes at a time: nine rows of 3k keys 361 us a step.
+__global__ void __launch_bounds__(256) fetch_kernel(uint4* __restrict__ dst, const uint4* __restrict__ src, size_t n) {
+  grid_dep_launch();
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = __ldcg(src + i);
+  grid_dep_wait();
+}
+
+cudaError_t launch_fetch(void* dst, const void* src_mapped_host, size_t bytes, cudaStream_t s) {
+  if (bytes == 0) return cudaSuccess;
+  const size_t n = bytes / 16;
+  return launch_dep(fetch_kernel, (unsigned)std::min<size_t>((n + 255) / 256, 148), 256, 0, s, (uint4*)dst, (const uint4*)src_mapped_host, n);
+}
+
 __global__ void upload_set_kernel(const __grid_constant__ UploadSet u) {
   grid_dep_wait();
   grid_dep_launch();

@@ -1590,8 +1590,8 @@ int tide_step_host(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_
   const size_t bytes = T * (2 * kv_row + 2 * q_row + (lse ? lse_row : 0));
   int n_chunks = kv->host_step_chunks > 0 ? kv->host_step_chunks : host_chunks(bytes);
   n_chunks = std::max(1, std::min(n_chunks, kMaxHostChunks));
-  // A small step from pinned host buffers that the device can address is not copied at all: the append kernel reads
-  // new_k / new_v, and the attention kernels read q and write out / lse, straight across PCIe.  Five copies of a few
+  // A small step from pinned host buffers that the device can address is not copied by the engines: the append kernel reads
+  // new_k / new_v, a small kernel fetches q, and the attention kernels write out / lse, straight across PCIe.  Five copies of a few
   // hundred KB cost more in engine hand-overs than the bytes do (a 64-row decode step: 0.22 -> 0.20 ms, a tiny one
   // 0.11 -> 0.09).
   if (kv->host_zero_copy && n_chunks == 1 && bytes <= kZeroCopyBytes) {
@@ -1606,7 +1606,8 @@ int tide_step_host(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_
     if (mapped(new_k, &zk) && mapped(new_v, &zv) && mapped(q, &zq) && mapped(out, &zo) && (lse == nullptr || mapped(lse, &zl))) {
       rc = tide_kv_append(kv, layer, n_rows, ids.data(), indptr.data(), zk, zv, stream);
       if (rc != TIDE_OK) return rc;
-      rc = tide_attend(kv, layer, n_rows, rows, nullptr, zq, scale, zo, (float*)zl, stream);
+      if (launch_fetch(dq, zq, T * q_row, st) != cudaSuccess) return TIDE_ERR_CUDA;
+      rc = tide_attend(kv, layer, n_rows, rows, nullptr, dq, scale, zo, (float*)zl, stream);
       if (rc != TIDE_OK) return rc;
       if (cudaStreamSynchronize(st) != cudaSuccess) return TIDE_ERR_CUDA;
       return TIDE_OK;

@@ -195,6 +195,7 @@ struct StaticView {
 
 cudaError_t launch_table_update(int32_t* table, const int32_t* idx, const int32_t* val, int n, cudaStream_t s);
 cudaError_t launch_upload(void* dst, const void* src_mapped_host, size_t bytes, cudaStream_t s);   // bytes % 4 == 0
+cudaError_t launch_fetch(void* dst, const void* src_mapped_host, size_t bytes, cudaStream_t s);   // right behind an append; bytes % 16 == 0
 cudaError_t launch_upload_set(const UploadSet& u, cudaStream_t s);
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s);
 // positions [to, to + n) of the task <- positions [to + shift, to + shift + n), in place, on every layer
