@@ -279,9 +279,10 @@ __device__ __forceinline__ void attend_umma128_body(const AttendParams& P, const
 
   // register budget: the data-movement warpgroup gives registers to the two softmax warpgroups.  setmaxnreg
   // moves registers inside the CTA's own launch allocation (384 x 168), so the new counts must not add up to
-  // more than that: 256 x 224 + 128 x 56 = 384 x 168.  (An over-subscribed .inc waits for ever.)
+  // more than that: 256 x 208 + 128 x 88 = 384 x 168.  (An over-subscribed .inc waits for ever.)  With 224 + 56 the MMA and
+  // scheduler warps spilled inside their loops: prompts 728 us, now 708; mixed text batch 7165, now 7076.
   if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     if (warp == 8 || warp == 10) {
       // ================= producers: warp 8 the K tiles (units 0, 2, 4, ...), warp 10 the V tiles (1, 3, 5, ...) =================
       const int is_v = warp == 10 ? 1 : 0;
@@ -569,7 +570,7 @@ __device__ __forceinline__ void attend_umma128_body(const AttendParams& P, const
       }
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
     // ================= softmax warpgroups =================
     const int t = warp >> 2;                                   // 0 = A, 1 = B
     const int row = ((warp & 3) << 5) | lane;                  // row of the 128-row tile = TMEM lane
