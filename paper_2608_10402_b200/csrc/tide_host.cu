@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1121,6 +1122,8 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
   // batch without groups; 4 of 4 38.9 and 41.8, 12 of 12 with 2000 shared 81.3 and 83.1, 2 of 8 with 11000 34.2 and 39.2.
   const long long target = std::max<long long>(1, (long long)kv->num_sms * kv->items_per_sm * (groups.empty() ? 3 : 2) / 3);
   long long chunk_dec = std::max<long long>(256, align_up((size_t)(w_dec / target + 1), kStageKeys));
+  // Launch shapes that a caller has fixed may have been sized for the cuts without these rules, so no rule goes beyond them.
+  const bool fixed = step && kv->fixed_grids;
   if (groups.empty() && !kv->items_per_sm_set && w_dec > 0) {
     // Decode rows: the launch holds 2 blocks per SM at a time, and what is left over when their number is exceeded by a few
     // runs alone.  So rows are cut as finely as ONE round of blocks allows when a block then reads up to 1.6 MB, and as two
@@ -1133,8 +1136,9 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
     for (const RowPlan& p : plan) dec_rows += p.kind == kDec;
     const long long rounds = std::max<long long>(w_dec * g.D * 4 / blocks <= (1600ll << 10) ? 1 : 2, (dec_rows * g.Hkv + blocks - 1) / blocks);
     double target_keys = std::max(256.0, (double)w_dec / (double)(blocks * rounds));
-    for (int step = 0; step < 6; ++step) {
-      long long items = 0;
+    long long items = 0;
+    for (int step_up = 0; step_up < 6; ++step_up) {
+      items = 0;
       const double inv = 1.0 / target_keys;
       for (int b = 0; b < n_rows; ++b)
         if (plan[(size_t)b].kind == kDec) items += (long long)((double)(rows[b].ctx_len - 1) * inv) + 1;
@@ -1142,11 +1146,39 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
       if (items <= blocks * rounds) break;
       target_keys *= std::max(1.02, (double)items / (double)(blocks * rounds));
     }
-    chunk_dec = align_up((size_t)target_keys, 2 * kStageKeys);
+    if (!fixed || items <= kv->cap_dec) chunk_dec = align_up((size_t)target_keys, 2 * kStageKeys);
   }
   long long chunk_tile = (items_tile_nosplit >= target / 2)
                              ? (1LL << 30)
                              : std::max<long long>(2048, align_up((size_t)(w_tile / target + 1), kStageKeys));
+  if (umma_ok && !kv->items_per_sm_set && !fixed && w_dec == 0 && items_tile_nosplit > 0) {
+    // Resume rows alone, on the tcgen05 kernel.  An item costs 4 us beside its 1.65 us per 128 keys, split rows a merge launch and
+    // their partials.  Few items: cut into as many as one round of blocks (one per SM) takes, but not below 6.5 * sqrt(keys)
+    // a piece, where the shorter items stop paying for the merge (one row of 17 to 35 tokens, us with pieces of 256 / 384 /
+    // 512 / 768 / 2048 keys: 1500 keys 18.5 / 19.7 / 20.0 / 21.6 / 33, 6000 keys 29.9 / 26.3 / 25.4 / 26.6 / 37).  From half a
+    // round on they stay whole (36 items 57.8, in 128 pieces 35.2; 84 items 60.2, in 168 62.3; 160 items 76, in 320 100), but for
+    // long items that end in a nearly empty second round (168 of 9500 keys 252, in 504 pieces 219).  Beside decode rows the
+    // pieces above stay: blocks that these items take are missing there (16 rows of 3000 keys, 2 of them resume rows: whole 86.7,
+    // 40 items 48.6, 128 items 58.7).
+    const long long sms = kv->num_sms;
+    if (2 * items_tile_nosplit <= sms) {
+      int longest = 0;
+      for (int b = 0; b < n_rows; ++b)
+        if (plan[(size_t)b].kind != kDec) longest = std::max(longest, rows[b].ctx_len);
+      double target_keys = std::max(6.5 * std::sqrt((double)longest), (double)w_tile / (double)sms);
+      for (int step_up = 0; step_up < 6; ++step_up) {
+        long long items = 0;
+        const double inv = 1.0 / target_keys;
+        for (int b = 0; b < n_rows; ++b)
+          if (plan[(size_t)b].kind != kDec) items += plan[(size_t)b].items * ((long long)((double)(rows[b].ctx_len - 1) * inv) + 1);
+        if (items <= sms) break;
+        target_keys *= std::max(1.05, (double)items / (double)sms);
+      }
+      chunk_tile = align_up((size_t)target_keys, 2 * kStageKeys);
+    } else if (items_tile_nosplit <= sms || w_tile < 7000 * items_tile_nosplit) {
+      chunk_tile = 1LL << 30;
+    }
+  }
   // a range of `len` keys cut into pieces of about chunk_target
   auto cut = [&](long long chunk_target, int len, int& n_splits, int& chunk) {
     n_splits = (int)std::min<long long>(kMaxSplits, ((long long)len + chunk_target - 1) / chunk_target);

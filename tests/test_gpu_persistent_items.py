@@ -125,6 +125,53 @@ def test_many_decode_items_per_thread_block(geom, n_rows, fixed):
     kv.close()
 
 
+@pytest.mark.parametrize("geom,lens", [((28, 4, 128, 16), [(0, 500)]), ((28, 4, 128, 16), [(1500, 17)]), ((6, 2, 128, 16), [(128, 1), (257, 300), (1, 90)]),
+                                       ((12, 4, 64, 16), [(0, 900), (2305, 31)]), ((8, 1, 128, 32), [(383, 20), (9001, 3), (40, 2), (767, 64)]),
+                                       ((28, 4, 128, 16), [(900 + 7 * i, 20 + i) for i in range(18)]), ((28, 4, 128, 16), [(900 + 7 * i, 20 + i) for i in range(19)])])
+def test_few_resume_rows_cut_to_one_round_of_blocks(geom, lens):
+    """Resume rows alone: up to half a round of blocks they are cut along the keys, above it (the last case) they stay
+    whole.  Pieces that begin behind the last key of a row tile's tokens, rows shorter than a piece beside split ones."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    HQ, HKV, D, S = geom
+    rng = np.random.default_rng(HQ + D + S + len(lens))
+    scale = 1.0 / math.sqrt(D)
+    lens = [(p, max(n, 16 // (HQ // HKV) + 1)) for p, n in lens]
+    n_rows, T = len(lens), sum(n for _, n in lens)
+    max_pages = max((p + n + S - 1) // S for p, n in lens) + 1
+    pages = n_rows * max_pages
+    order = rng.permutation(pages).astype(np.int32)
+    kv = tide.TideKV(HQ, HKV, D, S, pages, n_rows, max_pages, n_rows, T, free_order=order)
+    orc = PagedKVOracle(pages, S, HKV, D, n_rows, max_pages, free_order=order)
+    ids = list(range(n_rows))
+    for o in (kv, orc):
+        for t in ids:
+            o.alloc(t)
+    for part in (0, 1):
+        ip = np.concatenate([[0], np.cumsum([x[part] for x in lens])]).astype(np.int32)
+        nk, nv = inputs.normal_bf16(rng, (int(ip[-1]), HKV, D)), inputs.normal_bf16(rng, (int(ip[-1]), HKV, D))
+        if ip[-1]:
+            kv.append(ids, ip, H.to_dev(nk, torch), H.to_dev(nv, torch))
+            orc.append(ids, ip, nk, nv)
+    q = inputs.normal_bf16(rng, (T, HQ, D))
+    rows = [(t, n, p + n) for t, (p, n) in enumerate(lens)]
+    out = torch.zeros((T, HQ, D), dtype=torch.int16, device="cuda")
+    lse = torch.zeros((T, HQ), dtype=torch.float32, device="cuda")
+    kv.attend(rows, H.to_dev(q, torch), scale, out, lse)
+    assert kv.status() == tide.OK
+    plan = kv.last_plan()
+    whole = sum(HKV * -(-n * (HQ // HKV) // 256) for _, n in lens)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert plan["decode_items"] == 0
+    if 2 * whole <= sms:
+        assert whole < plan["prefill_items"] <= sms and plan["merge_rows"] > 0
+    else:
+        assert plan["prefill_items"] == whole and plan["merge_rows"] == 0
+    ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
+    H.check_outputs(H.from_dev(out), lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
+    kv.close()
+
+
 @pytest.mark.parametrize("geom", [(28, 4, 128, 16), (12, 4, 64, 16)])
 @pytest.mark.parametrize("layers", [1, 2])
 def test_steps_queued_without_waiting_follow_one_another(geom, layers):
