@@ -1131,22 +1131,39 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
     // 1k to 32k keys 55.5 (296), 60.6 (464); 48 rows of eight layers 521 (308), 537 (540); 100 rows of one KV head 55.2 (244),
     // 58.4 (493); 130 rows of 300 to 8k keys 96.9 (568), 100.3 (740); 64 rows of 64-wide heads 152.5 (584), 158.5 (744);
     // 64 rows of 1k to 32k keys 133.0 (408), 130.1 (556), 137.8 (660).
-    const long long blocks = 2LL * kv->num_sms;
-    long long dec_rows = 0;
-    for (const RowPlan& p : plan) dec_rows += p.kind == kDec;
-    const long long rounds = std::max<long long>(w_dec * g.D * 4 / blocks <= (1600ll << 10) ? 1 : 2, (dec_rows * g.Hkv + blocks - 1) / blocks);
-    double target_keys = std::max(256.0, (double)w_dec / (double)(blocks * rounds));
-    long long items = 0;
-    for (int step_up = 0; step_up < 6; ++step_up) {
-      items = 0;
-      const double inv = 1.0 / target_keys;
-      for (int b = 0; b < n_rows; ++b)
-        if (plan[(size_t)b].kind == kDec) items += (long long)((double)(rows[b].ctx_len - 1) * inv) + 1;
-      items *= g.Hkv;
-      if (items <= blocks * rounds) break;
-      target_keys *= std::max(1.02, (double)items / (double)(blocks * rounds));
+    // Small batches: a piece costs its block 0.63 us per 64 keys, and the block that merges a row 0.8 us per 8 pieces, so a
+    // row of n keys is cut into pieces of at least some 3.5 * sqrt(n) keys, and up to 32k in some 32 at most (one row of 16k keys, us with pieces of
+    // 256 / 512 / 1024: 20.8 / 16.3 / 18.6; of 32k 42.9 / 27.8 / 23.4; of 4k 10.9 / 12.2 / 17.0).  128-wide heads: one block per
+    // SM is enough where its piece is no longer than 640 keys (four rows of 4k: 256 pieces 14.1, 128 pieces 12.8; six layers of
+    // six rows of 3k: 288 pieces 105.7, 120 pieces 99.0; but 16 rows of 250 to 4k: 228 pieces 13.9, 128 pieces 15.3).
+    long long dec_rows = 0, items = 0;
+    int longest = 0;
+    for (int b = 0; b < n_rows; ++b)
+      if (plan[(size_t)b].kind == kDec) {
+        ++dec_rows;
+        longest = std::max(longest, rows[b].ctx_len);
+      }
+    const bool few = 2 * dec_rows * g.Hkv <= kv->num_sms;      // with more rows a merge runs beside the others' pieces
+    const double shortest = !few ? 256.0 : 128.0 * std::max(2.0, std::floor(std::max(3.5 * std::sqrt((double)longest), std::min(1024.0, longest / 32.0)) / 128.0 + 0.5));
+    double target_keys = 0.0;
+    for (int per_sm = g.D == 128 ? 1 : 2; per_sm <= 2; ++per_sm) {
+      const long long blocks = (long long)per_sm * kv->num_sms;
+      const long long rounds = per_sm == 1 ? 1 : std::max<long long>(w_dec * g.D * 4 / blocks <= (1600ll << 10) ? 1 : 2, (dec_rows * g.Hkv + blocks - 1) / blocks);
+      target_keys = std::max(shortest, (double)w_dec / (double)(blocks * rounds));
+      for (int step_up = 0; step_up < 6; ++step_up) {
+        items = 0;
+        const double inv = 1.0 / target_keys;
+        for (int b = 0; b < n_rows; ++b) {
+          const double pieces = (double)(rows[b].ctx_len - 1) * inv;
+          if (plan[(size_t)b].kind == kDec && pieces >= 0.125) items += (long long)pieces + 1;   // shorter ones hold no block up
+        }
+        items *= g.Hkv;
+        if (items <= blocks * rounds || (per_sm == 1 && target_keys > 640.0)) break;
+        target_keys *= std::max(1.02, (double)items / (double)(blocks * rounds));
+      }
+      if (target_keys <= 640.0) break;
     }
-    if (!fixed || items <= kv->cap_dec) chunk_dec = align_up((size_t)target_keys, 2 * kStageKeys);
+    if (!fixed || items + dec_rows * g.Hkv <= kv->cap_dec) chunk_dec = align_up((size_t)target_keys, 2 * kStageKeys);
   }
   long long chunk_tile = (items_tile_nosplit >= target / 2)
                              ? (1LL << 30)

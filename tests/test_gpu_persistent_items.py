@@ -172,6 +172,37 @@ def test_few_resume_rows_cut_to_one_round_of_blocks(geom, lens):
     kv.close()
 
 
+@pytest.mark.parametrize("geom,ctx", [((28, 4, 128, 16), [1024]), ((28, 4, 128, 16), [16000]), ((28, 4, 128, 32), [4000] * 4), ((16, 1, 128, 16), [40001, 130]),
+                                      ((12, 4, 64, 16), [9000, 2047, 1]), ((6, 2, 128, 16), [70000]), ((28, 4, 128, 16), [250 + 250 * i for i in range(16)])])
+def test_few_decode_rows_and_their_merge(geom, ctx):
+    """Decode rows that are cut for the merge of their pieces: up to eight pieces, whole and ragged batches of eight, more
+    than thirty-two; one block per SM and two."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    HQ, HKV, D, S = geom
+    rng = np.random.default_rng(HQ + D + len(ctx) + ctx[0])
+    scale, n = 1.0 / math.sqrt(D), len(ctx)
+    max_pages = (max(ctx) + S) // S + 1
+    pages = sum((c + S) // S + 1 for c in ctx)
+    order = rng.permutation(pages).astype(np.int32)
+    kv = tide.TideKV(HQ, HKV, D, S, pages, n, max_pages, n, max(ctx), free_order=order)
+    orc = PagedKVOracle(pages, S, HKV, D, n, max_pages, free_order=order)
+    for t, c in enumerate(ctx):
+        nk, nv = inputs.normal_bf16(rng, (c, HKV, D)), inputs.normal_bf16(rng, (c, HKV, D))
+        for o, k, v in ((kv, H.to_dev(nk, torch), H.to_dev(nv, torch)), (orc, nk, nv)):
+            o.alloc(t)
+            o.append([t], [0, c], k, v)
+    q = inputs.normal_bf16(rng, (n, HQ, D))
+    rows = [(t, 1, c) for t, c in enumerate(ctx)]
+    out = torch.zeros((n, HQ, D), dtype=torch.int16, device="cuda")
+    lse = torch.zeros((n, HQ), dtype=torch.float32, device="cuda")
+    kv.attend(rows, H.to_dev(q, torch), scale, out, lse)
+    assert kv.status() == tide.OK
+    ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
+    H.check_outputs(H.from_dev(out), lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
+    kv.close()
+
+
 @pytest.mark.parametrize("geom", [(28, 4, 128, 16), (12, 4, 64, 16)])
 @pytest.mark.parametrize("layers", [1, 2])
 def test_steps_queued_without_waiting_follow_one_another(geom, layers):
