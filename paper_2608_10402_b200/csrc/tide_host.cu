@@ -1379,6 +1379,7 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   auto launch_umma = [&]() -> cudaError_t {
     ap.segs = d.seg_umma; ap.n_segs = (int)d.n_umma; ap.n_items = (int)d.items_umma;
     ap.dyn = dyn ? dyn + kHdrUmmaItems : nullptr; ap.grid_cap = kv->cap_umma; ap.overlapped = 0;
+    ap.run_ahead = run_ahead ? 1 : 0;
     ++launches;
     if (kv->umma_tile_keys != 128) return launch_attend_umma(ap, st);
     return inl ? launch_attend_umma128_inline(inline_segs(inl->seg_umma), st) : launch_attend_umma128(ap, st);

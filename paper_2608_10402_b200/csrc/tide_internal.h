@@ -56,7 +56,7 @@ struct __align__(16) Segment {
   int32_t part_base;   // first partial row ((split * n + token) * Hq + head) when the item writes partials
   union {
     int32_t merge_base;  // in the merge launch's list: first row of this segment
-    int32_t live_from;   // in the decode launch's list: first key that the kernel before it may still be writing (run_ahead)
+    int32_t live_from;   // in the decode and tcgen05 launches' lists: first key that the kernel before it may still be writing (run_ahead)
   };
   // Rows of one batch whose tasks share their first pages (forked tasks) read those pages once: the shared range
   // is one segment whose `n` tokens are the member rows' queries and all see the same keys (causal = 0), each
@@ -95,7 +95,7 @@ struct AttendParams {
   int grid_cap = 0;
   int* merge_ctr = nullptr;   // per (segment with partial == 2, kv head): splits finished so far; zero between launches
   long long wait_limit_ns = kWaitLimitNsDefault;   // bound of every wait inside the kernel
-  int run_ahead = 0;          // decode: the producers may read keys below Segment::live_from before earlier work is complete
+  int run_ahead = 0;          // decode, 128-key tcgen05: the producers may read keys below Segment::live_from before earlier work is complete
   int overlapped = 0;         // the kernel before this one in the stream is the other attention kernel of the same batch (see grid_dep_wait)
   // Test hook for the bounded waits (never set in normal use): in work item 0 the producer leaves out its part
   // of the first stage, so the consumers' wait for that stage runs out and the time-out path executes.
@@ -232,8 +232,9 @@ int sm_count();   // multiprocessors of the current device (looked up once per d
 // kernels of one batch do not depend on each other: the second one (AttendParams::overlapped) starts without waiting -
 // the first has waited for all earlier work before it let the second one start - and waits when it is done, so that what
 // follows it in the stream still follows both.  Nor do the keys that a decode row saw in the step before depend on the
-// append in front of the decode kernel, which waits for everything earlier: the decode kernel's producers stream those
-// pages (AttendParams::run_ahead, Segment::live_from) while the append runs.  The same goes for the moves of several tasks that are pruned in a row.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
+// append in front of the attention kernels, which waits for everything earlier: the producers of the first of them stream
+// those pages (AttendParams::run_ahead, Segment::live_from) while the append runs.  The same goes for the moves of several
+// tasks that are pruned in a row.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
 template <typename... A>
 cudaError_t launch_dep(void (*kernel)(A...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, const std::common_type_t<A>&... args) {
   cudaLaunchConfig_t cfg = {};
