@@ -340,16 +340,21 @@ cudaError_t launch_attend_tile(const AttendParams& p, cudaStream_t s) {
 // ---------------------------------------------------------------------------------------------
 // Log-sum-exp merge of the split partials: one warp per (token, head) row.
 //   LSE = log2 sum_i 2^{LSE_i},  O = sum_i 2^{LSE_i - LSE} O_i;  fixed order, no atomics.
-// The kernel is a chain of dependent loads if written naively (one split after the other), so the partial LSEs
-// are fetched side by side, one per lane, and the partial outputs four splits at a time; the order in which the
-// terms are added is still the order of the splits.
+// Bound by latency (a chain of dependent loads if written naively), so the partial LSEs are fetched side by side, one per
+// lane, the partial outputs four splits at a time, the first four beside the LSEs, and the row's segment is looked up
+// before the wait; the order in which the terms are added is still the order of the splits.
+// (All LSEs of up to 256 contributions in eight registers a lane, picked by index, and the outputs behind them: one row of
+// 17 to 35 tokens behind 1500 / 16000 keys 18.0 / 33.2 us with its append, now 16.0 / 27.0; 16 rows, two of them resumed,
+// 44.8, now 41.8; eight splits at a time spill, 15.7 / 26.5 / 42.8.)
 __device__ __forceinline__ void merge_body(const MergeParams& P, const Segment* __restrict__ segs) {
-  grid_dep_wait();
-  grid_dep_launch();
+  // the descriptors were complete before the attention kernels started: the look-up needs no wait
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int n_rows = P.dyn ? P.dyn[0] : P.n_rows, n_segs = P.dyn ? P.dyn[1] : P.n_segs;
-  if (row >= n_rows) return;
+  if (row >= n_rows) {
+    grid_dep_wait();
+    return;
+  }
   const int si = find_segment(n_segs, row, [&](int i) { return segs[i].merge_base; });
   const Segment seg = segs[si];
   const int local = row - seg.merge_base;                 // token * Hq + head inside the segment
@@ -361,47 +366,44 @@ __device__ __forceinline__ void merge_body(const MergeParams& P, const Segment* 
   auto src_row = [&](int s) -> long long {
     return s < seg.n_splits ? p0 + s * stride : (long long)seg.x_part_base + local + (long long)(s - seg.n_splits) * seg.x_stride;
   };
-  // lane i holds the LSEs of contributions i, i + 32, ... (at most 2 * kMaxSplits = 256 of them)
-  constexpr int kPerLane = 2 * kMaxSplits / 32;
-  float e[kPerLane];
-  float mstar = -INFINITY;
-#pragma unroll
-  for (int k = 0; k < kPerLane; ++k) {
-    const int s = k * 32 + lane;
-    e[k] = s < n_src ? P.part_lse[src_row(s)] : -INFINITY;
-    mstar = fmaxf(mstar, e[k]);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mstar = fmaxf(mstar, __shfl_xor_sync(0xffffffffu, mstar, o));
-  const float mu = (mstar == -INFINITY) ? 0.f : mstar;
-#pragma unroll
-  for (int k = 0; k < kPerLane; ++k) e[k] = e[k] == -INFINITY ? 0.f : exp2f(e[k] - mu);   // the contribution's weight
   const int per = P.D / 32;                               // 2 or 4 floats per lane
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  float tot = 0.f;
-  for (int s0 = 0; s0 < n_src; s0 += 4) {
-    float4 v[4];
-    float w[4];
+  constexpr int kBatch = 4;
+  float4 v[kBatch];
+  auto fetch = [&](int s0) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int s = s0 + u;
-      // weight of contribution s: held by lane s % 32 in its slot s / 32 (kPerLane is small: select, then shuffle)
-      float mine = 0.f;
-#pragma unroll
-      for (int k = 0; k < kPerLane; ++k) if ((s >> 5) == k) mine = e[k];
-      w[u] = s < n_src ? __shfl_sync(0xffffffffu, mine, s & 31) : 0.f;
-      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (w[u] != 0.f) {
-        const float* po = P.part_o + src_row(s) * P.D + lane * per;
-        if (per == 4) v[u] = *reinterpret_cast<const float4*>(po);
-        else { const float2 t = *reinterpret_cast<const float2*>(po); v[u].x = t.x; v[u].y = t.y; }
-      }
+    for (int u = 0; u < kBatch; ++u) {
+      if (s0 + u >= n_src) continue;
+      const float* po = P.part_o + src_row(s0 + u) * P.D + lane * per;
+      if (per == 4) v[u] = __ldcg(reinterpret_cast<const float4*>(po));
+      else { const float2 t = __ldcg(reinterpret_cast<const float2*>(po)); v[u] = make_float4(t.x, t.y, 0.f, 0.f); }
     }
+  };
+  grid_dep_wait();
+  grid_dep_launch();
+  fetch(0);
+  float mstar = -INFINITY, tot = 0.f;
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int c0 = 0; c0 < n_src; c0 += 32) {                // 32 contributions: lane i holds the LSE, then the weight, of c0 + i
+    const float e = c0 + lane < n_src ? __ldcg(P.part_lse + src_row(c0 + lane)) : -INFINITY;
+    float m_new = e;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (w[u] != 0.f) {
-        tot += w[u];
-        acc[0] += w[u] * v[u].x; acc[1] += w[u] * v[u].y; acc[2] += w[u] * v[u].z; acc[3] += w[u] * v[u].w;
+    for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
+    m_new = fmaxf(mstar, m_new);
+    const float mu = (m_new == -INFINITY) ? 0.f : m_new, keep = exp2f(mstar - mu), mine = exp2f(e - mu);   // -inf: 0
+    mstar = m_new;
+    tot *= keep;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) acc[d] *= keep;
+    const int n_here = min(32, n_src - c0);
+    for (int s0 = 0; s0 < n_here; s0 += kBatch) {
+      if (c0 + s0 > 0) fetch(c0 + s0);
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const float w = __shfl_sync(0xffffffffu, mine, s0 + u);
+        if (w != 0.f) {
+          tot += w;
+          acc[0] += w * v[u].x; acc[1] += w * v[u].y; acc[2] += w * v[u].z; acc[3] += w * v[u].w;
+        }
       }
     }
   }
