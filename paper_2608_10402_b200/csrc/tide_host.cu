@@ -1087,6 +1087,58 @@ static bool umma_takes(const tide_kv* kv) { return kv->g.D == 128 || kv->umma_ti
 // tcgen05-style; long contexts are split along the keys so that the grid has about items_per_sm items per SM.
 // A group of rows that share their first pages gets one more segment for the shared range (its tokens are the
 // members' queries, all seeing the same keys); the members' own segments start behind it and their merge takes both.
+// Into pieces of how many keys the resume rows of a batch are cut when their items (256 packed rows on an SM each) are few:
+// the candidate with the least estimated time, in us.  An item takes 4 + 0.0129 a key (0.0085 with one row tile; 64-wide heads
+// a tenth less); up to one item per SM the longest one counts and the decode rows beside it stream at full rate while some
+// 60 % of the SMs are free, beyond that the sum counts, and half of the longest item or the decode rows fill the end;
+// rows that are cut cost a merge launch, 0.4 ns a row and their partials.  us as estimated (without the append) and as measured with pieces
+// of n keys: one row of 17 to 35 tokens behind 16000 keys 768 15 (25.7), 2048 36 (37.7), whole 209 (248); 2 rows of 200 to 500
+// behind 12000 3072 147 (148), 2048 152 (155), whole 197 (196); 24 of 17 to 60 behind 3000 whole 70 (74), 3072 81 (81); 14
+// decode rows and two of 30 and 40 tokens 2048 35 (55), 1024 26 (46), 512 30 (48), 384 35 (56).
+static long long resume_chunk(const tide_kv* kv, int32_t n_rows, const tide_row_t* rows, const std::vector<RowPlan>& plan, long long w_dec) {
+  const Geom& g = kv->g;
+  const double sms = kv->num_sms, per_key = g.D == 128 ? 0.0129 : 0.0116, part_row = g.D * 8.0 / 5.0e6;
+  const double t_dec = (double)w_dec * g.D * 4.0 / 6.5e6;
+  static const int kKeys[] = {INT_MAX, 24576, 16384, 12288, 8192, 6144, 5120, 4096, 3072, 2560, 2048, 1536, 1280, 1024, 768, 640, 512, 384, 256};
+  long long best_keys = 1LL << 30;
+  double best = 0.0;
+  int longest_ctx = 0;
+  for (int b = 0; b < n_rows; ++b)
+    if (plan[(size_t)b].kind != 0) longest_ctx = std::max(longest_ctx, rows[b].ctx_len);
+  for (const int keys : kKeys) {
+    if (keys != INT_MAX && keys >= longest_ctx) continue;      // cuts nothing
+    double sum = 0.0, longest = 0.0, items = 0.0, part_rows = 0.0, merge_rows = 0.0;
+    int tile_rows = 0;
+    for (int b = 0; b < n_rows; ++b) {
+      const RowPlan& p = plan[(size_t)b];
+      if (p.kind == 0) continue;
+      const int ctx = rows[b].ctx_len, pieces = std::min(kMaxSplits, (ctx - 1) / keys + 1);
+      const double each = per_key * (rows[b].q_len * g.G <= kUmmaTileRows ? 0.66 : 1.0) * ((ctx - 1) / pieces + 1);
+      ++tile_rows;
+      items += (double)p.items * pieces;
+      sum += (double)p.items * (each + 4.0) * pieces;
+      longest = std::max(longest, each + 4.0);
+      if (pieces > 1) {
+        merge_rows += (double)rows[b].q_len * g.Hq;
+        part_rows += (double)pieces * rows[b].q_len * g.Hq;
+      }
+    }
+    double t;
+    if (items <= sms) t = longest + std::max(0.0, t_dec - longest * std::min(1.0, (sms - items) / (0.6 * sms)));
+    else if (tile_rows == 1) t = std::ceil(items / sms) * longest + t_dec;
+    else t = sum / sms + std::max(t_dec, 0.5 * longest);
+    if (merge_rows > 0.0) t += 3.0 + merge_rows * 0.0004 + part_rows * part_row;
+    // (the end of several rounds of unequal items is the least certain part of the estimate)
+    if (keys == INT_MAX || t < (items <= sms || tile_rows == 1 ? 0.97 : 0.85) * best) {
+      best = t;
+      best_keys = keys == INT_MAX ? 1LL << 30 : keys;
+    } else if (t > 1.3 * best) {
+      break;
+    }
+  }
+  return best_keys;
+}
+
 // The plan depends on the rows and the page tables only, so every layer of a step can use it.  `step`: the kernel in front
 // of the attention kernels is the append of exactly these rows (tide_step_layer).
 static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool umma_ok, bool allow_groups, bool step, PlanHost& P) {
@@ -1168,34 +1220,8 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
   long long chunk_tile = (items_tile_nosplit >= target / 2)
                              ? (1LL << 30)
                              : std::max<long long>(2048, align_up((size_t)(w_tile / target + 1), kStageKeys));
-  if (umma_ok && !kv->items_per_sm_set && !fixed && w_dec == 0 && items_tile_nosplit > 0) {
-    // Resume rows alone, on the tcgen05 kernel.  An item costs 4 us beside its 1.65 us per 128 keys, split rows a merge launch and
-    // their partials.  Few items: cut into as many as one round of blocks (one per SM) takes, but not below 6.5 * sqrt(keys)
-    // a piece, where the shorter items stop paying for the merge (one row of 17 to 35 tokens, us with pieces of 256 / 384 /
-    // 512 / 768 / 2048 keys: 1500 keys 18.5 / 19.7 / 20.0 / 21.6 / 33, 6000 keys 29.9 / 26.3 / 25.4 / 26.6 / 37).  From half a
-    // round on they stay whole (36 items 57.8, in 128 pieces 35.2; 84 items 60.2, in 168 62.3; 160 items 76, in 320 100), but for
-    // long items that end in a nearly empty second round (168 of 9500 keys 252, in 504 pieces 219).  Beside decode rows the
-    // pieces above stay: blocks that these items take are missing there (16 rows of 3000 keys, 2 of them resume rows: whole 86.7,
-    // 40 items 48.6, 128 items 58.7).
-    const long long sms = kv->num_sms;
-    if (2 * items_tile_nosplit <= sms) {
-      int longest = 0;
-      for (int b = 0; b < n_rows; ++b)
-        if (plan[(size_t)b].kind != kDec) longest = std::max(longest, rows[b].ctx_len);
-      double target_keys = std::max(6.5 * std::sqrt((double)longest), (double)w_tile / (double)sms);
-      for (int step_up = 0; step_up < 6; ++step_up) {
-        long long items = 0;
-        const double inv = 1.0 / target_keys;
-        for (int b = 0; b < n_rows; ++b)
-          if (plan[(size_t)b].kind != kDec) items += plan[(size_t)b].items * ((long long)((double)(rows[b].ctx_len - 1) * inv) + 1);
-        if (items <= sms) break;
-        target_keys *= std::max(1.05, (double)items / (double)sms);
-      }
-      chunk_tile = align_up((size_t)target_keys, 2 * kStageKeys);
-    } else if (items_tile_nosplit <= sms || w_tile < 7000 * items_tile_nosplit) {
-      chunk_tile = 1LL << 30;
-    }
-  }
+  if (umma_ok && !kv->items_per_sm_set && !fixed && groups.empty() && items_tile_nosplit > 0 && items_tile_nosplit <= 2LL * kv->num_sms)
+    chunk_tile = resume_chunk(kv, n_rows, rows, plan, w_dec);
   // a range of `len` keys cut into pieces of about chunk_target
   auto cut = [&](long long chunk_target, int len, int& n_splits, int& chunk) {
     n_splits = (int)std::min<long long>(kMaxSplits, ((long long)len + chunk_target - 1) / chunk_target);
