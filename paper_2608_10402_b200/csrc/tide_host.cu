@@ -1217,6 +1217,8 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
     }
     if (!fixed || items + dec_rows * g.Hkv <= kv->cap_dec) chunk_dec = align_up((size_t)target_keys, 2 * kStageKeys);
   }
+  // Resume rows: whole when there are many items; few of them by estimate (resume_chunk), or where something else is laid out
+  // for it - shared ranges, launch shapes or item counts that a caller has fixed - in pieces of 2048 keys and more.
   long long chunk_tile = (items_tile_nosplit >= target / 2)
                              ? (1LL << 30)
                              : std::max<long long>(2048, align_up((size_t)(w_tile / target + 1), kStageKeys));
