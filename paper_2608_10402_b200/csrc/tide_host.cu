@@ -99,6 +99,74 @@ struct Slot {
   bool used = false;
 };
 
+// Keys that work of a stream may still be writing while the kernel behind it starts: for every stream the positions, from
+// a page boundary on, that its most recent writer (append, write, series of moves) touches.  A writer waits for all
+// earlier work of its stream before the next launch may start, so its predecessors' keys on that stream are complete.
+// Writers of other streams say nothing about this one: a stream has a record of its own.  Keys that another stream writes
+// are ordered by an event, which a launch waits for in full; until that stream's next writer they count as live all the
+// same, unless the reading stream has written the task since.
+// Launches on a stream that is not among the kMostStreams last written read nothing ahead.
+class LiveKeys {
+ public:
+  void init(int max_tasks, int page_size) {
+    max_tasks_ = max_tasks;
+    page_ = page_size;
+  }
+  // A kernel that writes keys is about to be launched on `st` (and will wait for the work in front of it).
+  void begin(cudaStream_t st) {
+    cur_ = find(st);
+    if (cur_ < 0) {
+      if (n_ < kMostStreams) cur_ = n_++;
+      else {
+        cur_ = 0;
+        for (int i = 1; i < n_; ++i) if (w_[i].seq < w_[cur_].seq) cur_ = i;
+        forgotten_ = true;
+      }
+      w_[cur_].stream = st;
+      w_[cur_].seq_of.assign((size_t)max_tasks_, 0);
+      w_[cur_].from.assign((size_t)max_tasks_, 0);
+    }
+    w_[cur_].seq = ++seq_;
+  }
+  // ... and writes `task` from position `from` on.
+  void mark(int task, int from) {
+    Writer& w = w_[cur_];
+    from -= from % page_;
+    int32_t& f = w.from[(size_t)task];
+    f = w.seq_of[(size_t)task] == w.seq ? std::min(f, (int32_t)from) : from;
+    w.seq_of[(size_t)task] = w.seq;
+  }
+  // First live key of `task` for a launch on `st`.
+  int32_t from(int task, cudaStream_t st) const {
+    const int own = find(st);
+    if (own < 0 && forgotten_) return 0;
+    const int64_t own_seq = own < 0 ? 0 : w_[own].seq_of[(size_t)task];
+    int32_t f = INT_MAX;
+    for (int i = 0; i < n_; ++i) {
+      const Writer& w = w_[i];
+      if (w.seq_of[(size_t)task] == w.seq && w.seq >= own_seq) f = std::min(f, w.from[(size_t)task]);
+    }
+    return f;
+  }
+
+ private:
+  static constexpr int kMostStreams = 8;
+  struct Writer {
+    cudaStream_t stream;
+    int64_t seq;                       // of the most recent writer of the stream, over all streams
+    std::vector<int64_t> seq_of;       // per task: the last writer of this stream that wrote it ...
+    std::vector<int32_t> from;         // ... and from where on
+  };
+  int find(cudaStream_t st) const {
+    for (int i = 0; i < n_; ++i) if (w_[i].stream == st) return i;
+    return -1;
+  }
+  Writer w_[kMostStreams];
+  int n_ = 0, cur_ = 0, max_tasks_ = 0, page_ = 1;
+  int64_t seq_ = 0;
+  bool forgotten_ = false;             // a stream's record has made room for another's
+};
+
 }  // namespace
 
 struct tide_kv {
@@ -132,12 +200,7 @@ struct tide_kv {
   ExtendOut ext;              // result of the most recent extension
   std::vector<int32_t> mark;  // scratch for duplicate detection
   int32_t mark_gen = 0;
-  // what the most recent append, write or series of moves may still be writing while the kernel behind it starts: keys
-  // from live_from[t] on (a page boundary) of the tasks of that generation
-  std::vector<int64_t> live_gen_of;
-  std::vector<int32_t> live_from;
-  int64_t live_gen = 0;
-  cudaStream_t live_stream = nullptr;
+  LiveKeys live_keys;
   // moves of pruned tasks launched one after the other on one stream, with no other device work of this handle between
   bool moves_open = false;
   cudaStream_t moves_stream = nullptr;
@@ -282,19 +345,6 @@ bool last_page_shared(const tide_kv* kv, int32_t task) {
 
 bool task_in_range(const tide_kv* kv, int32_t t) { return t >= 0 && t < kv->cfg.max_tasks; }
 
-// A kernel that writes keys is about to be launched on `st`; mark_live says which.  It waits for the one before it on its
-// stream, whose keys are then no longer live; the keys of kernels on other streams stay so.
-void begin_live(tide_kv* kv, cudaStream_t st) {
-  if (kv->live_stream == st) ++kv->live_gen;
-  kv->live_stream = st;
-}
-void mark_live(tide_kv* kv, int32_t task, int32_t from) {
-  from -= from % kv->g.S;
-  int32_t& f = kv->live_from[(size_t)task];
-  f = kv->live_gen_of[(size_t)task] == kv->live_gen ? std::min(f, from) : from;
-  kv->live_gen_of[(size_t)task] = kv->live_gen;
-}
-
 // Takes the next staging slot, waiting until the device work that last used it has finished.
 int acquire_slot(tide_kv* kv, Slot** out) {
   Slot& s = kv->slots[kv->next_slot];
@@ -406,8 +456,7 @@ int tide_kv_create(const tide_kv_config_t* cfg, tide_kv_t** out) {
   kv->pages.resize((size_t)cfg->max_tasks);
   kv->mark.assign((size_t)cfg->max_tasks, 0);
   kv->move_mark.assign((size_t)cfg->max_tasks, 0);
-  kv->live_gen_of.assign((size_t)cfg->max_tasks, 0);
-  kv->live_from.assign((size_t)cfg->max_tasks, 0);
+  kv->live_keys.init(cfg->max_tasks, g.S);
   kv->refcnt.assign((size_t)cfg->num_pages, 0);
   prime_free_stack(kv, cfg->free_order);
   *out = kv;
@@ -658,9 +707,9 @@ static int write_tasks(tide_kv* kv, int32_t layer, int32_t n_tasks, const int32_
   int j = 0;
   int rc = TIDE_OK;
   kv->moves_open = false;
-  if (indptr[n_tasks] > 0) begin_live(kv, st);
+  if (indptr[n_tasks] > 0) kv->live_keys.begin(st);
   for (int i = 0; i < n_tasks; ++i)
-    if (indptr[i + 1] > indptr[i]) mark_live(kv, task_ids[i], kv->len[task_ids[i]] - (indptr[i + 1] - indptr[i]));
+    if (indptr[i + 1] > indptr[i]) kv->live_keys.mark(task_ids[i], kv->len[task_ids[i]] - (indptr[i + 1] - indptr[i]));
   while (j < n_tasks) {
     Slot* slot;
     if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
@@ -746,12 +795,12 @@ int tide_kv_append(tide_kv_t* kv, int32_t layer, int32_t n_tasks, const int32_t*
   if ((rc = extend_bookkeeping(kv, n_tasks, task_ids, indptr)) != TIDE_OK) return rc;
   if ((rc = upload_cow_copies(kv, st)) != TIDE_OK) return rc;     // a copied page must be in place before it is written
   int n_recs = 0;
-  if (indptr[n_tasks] > 0) begin_live(kv, st);
+  if (indptr[n_tasks] > 0) kv->live_keys.begin(st);
   for (int j = 0; j < n_tasks; ++j) {
     const int c = indptr[j + 1] - indptr[j];
     if (c == 0) continue;
     ++n_recs;
-    mark_live(kv, task_ids[j], kv->len[task_ids[j]] - c);
+    kv->live_keys.mark(task_ids[j], kv->len[task_ids[j]] - c);
   }
   const ExtendOut& x = kv->ext;
   auto fill_recs = [&](AppendRec* recs) {
@@ -971,8 +1020,8 @@ int tide_kv_prune(tide_kv_t* kv, int32_t layer, int32_t task, int32_t keep_prefi
     // a move right behind other tasks' moves on the same stream need not wait for them
     const bool overlapped = kv->moves_open && kv->moves_stream == st && kv->move_mark[(size_t)task] != kv->move_gen;
     if (tail > 0) {
-      if (!overlapped) { ++kv->move_gen; begin_live(kv, st); }
-      mark_live(kv, task, keep_prefix);
+      if (!overlapped) { ++kv->move_gen; kv->live_keys.begin(st); }
+      kv->live_keys.mark(task, keep_prefix);
     }
     if (tail > 0 && launch_move(kv->pool, kv->layer_stride, L, row, keep_prefix, tail_begin - keep_prefix, tail, overlapped, g, st) != cudaSuccess)
       return TIDE_ERR_CUDA;
@@ -1140,8 +1189,9 @@ static long long resume_chunk(const tide_kv* kv, int32_t n_rows, const tide_row_
 }
 
 // The plan depends on the rows and the page tables only, so every layer of a step can use it.  `step`: the kernel in front
-// of the attention kernels is the append of exactly these rows (tide_step_layer).
-static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool umma_ok, bool allow_groups, bool step, PlanHost& P) {
+// of the attention kernels is the append of exactly these rows (tide_step_layer); otherwise they go to stream `st`.
+static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool umma_ok, bool allow_groups, bool step, cudaStream_t st,
+                      PlanHost& P) {
   const Geom& g = kv->g;
   enum { kDec = 0, kTile = 1, kUmma = 2 };
   auto kind_of = [&](int R) { return R <= kDecodeTileRows ? kDec : (umma_ok && R >= kv->umma_min_rows ? kUmma : kTile); };
@@ -1264,7 +1314,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
       s.p = r.ctx_len - r.q_len;
       s.n_mtiles = p.n_mtiles;
       s.causal = 1;
-      s.live_from = step ? s.p : kv->live_gen_of[(size_t)r.task] == kv->live_gen ? kv->live_from[(size_t)r.task] : INT_MAX;
+      s.live_from = step ? s.p : kv->live_keys.from(r.task, st);
       if (gi >= 0) {
         s.origin = groups[(size_t)gi].pages * g.S;
         s.partial = 1;
@@ -1461,7 +1511,7 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
   int rc = check_rows(kv, n_rows, rows);
   if (rc != TIDE_OK) return rc;
   PlanHost& P = kv->plan;
-  if ((rc = build_plan(kv, n_rows, rows, umma_takes(kv) && scale > 0.f, page_table == nullptr, false, P)) != TIDE_OK) return rc;
+  if ((rc = build_plan(kv, n_rows, rows, umma_takes(kv) && scale > 0.f, page_table == nullptr, false, (cudaStream_t)stream, P)) != TIDE_OK) return rc;
   if (P.n_all() * sizeof(Segment) + 256 > kv->lay.slot_bytes) return TIDE_ERR_WORKSPACE;
 
   cudaStream_t st = (cudaStream_t)stream;
@@ -1527,9 +1577,9 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   PlanHost& P = kv->plan;
   // Launch shapes fixed without tcgen05 items (or with too few): head size 64 has the warp-MMA tile kernel as well.
   bool umma = umma_takes(kv) && !(kv->fixed_grids && g.D == 64 && kv->cap_umma == 0);
-  if ((rc = build_plan(kv, n_rows, rows, umma, true, true, P)) != TIDE_OK) return rc;
+  if ((rc = build_plan(kv, n_rows, rows, umma, true, true, (cudaStream_t)stream, P)) != TIDE_OK) return rc;
   if (umma && kv->fixed_grids && g.D == 64 && P.items_umma > kv->cap_umma &&
-      (rc = build_plan(kv, n_rows, rows, false, true, true, P)) != TIDE_OK) return rc;
+      (rc = build_plan(kv, n_rows, rows, false, true, true, (cudaStream_t)stream, P)) != TIDE_OK) return rc;
   if (kv->fixed_grids && (P.items_dec > kv->cap_dec || P.items_tile > kv->cap_tile || P.items_umma > kv->cap_umma ||
                           P.merge_rows > kv->cap_merge_rows || indptr[(size_t)n_rows] > kv->cap_tokens))
     return TIDE_ERR_WORKSPACE;   // the step does not fit the launch shapes that were fixed
