@@ -100,8 +100,10 @@ struct Slot {
 };
 
 // Keys that work of a stream may still be writing while the kernel behind it starts: for every stream the positions, from
-// a page boundary on, that its most recent writer (append, write, series of moves) touches.  A writer waits for all
-// earlier work of its stream before the next launch may start, so its predecessors' keys on that stream are complete.
+// a page boundary on, that its most recent writer (append, write, series of moves) touches, or whose pages or page-table
+// entries it puts in place (extend, fork, the begin of a step).  A writer waits for all earlier work of its stream before
+// the next launch may start - or is an ordinary launch, which starts behind all of it - so its predecessors' keys on that
+// stream are complete.  Whatever changes the pool or the table on the device is a writer; a call that launches nothing is not.
 // Writers of other streams say nothing about this one: a stream has a record of its own.  Keys that another stream writes
 // are ordered by an event, which a launch waits for in full; until that stream's next writer they count as live all the
 // same, unless the reading stream has written the task since.
@@ -112,7 +114,7 @@ class LiveKeys {
     max_tasks_ = max_tasks;
     page_ = page_size;
   }
-  // A kernel that writes keys is about to be launched on `st` (and will wait for the work in front of it).
+  // Work that writes keys or table entries is about to be launched on `st` (behind all work in front of it).
   void begin(cudaStream_t st) {
     cur_ = find(st);
     if (cur_ < 0) {
@@ -637,6 +639,16 @@ static int extend_bookkeeping(tide_kv* kv, int32_t n_tasks, const int32_t* task_
   return TIDE_OK;
 }
 
+// The last indptr[j+1]-indptr[j] positions of task_ids[j] are about to be written on `st` - new entries of the table row,
+// the private copy of a last page, the rows themselves.
+static void mark_grown(tide_kv* kv, int32_t n_tasks, const int32_t* task_ids, const int32_t* indptr, cudaStream_t st) {
+  kv->live_keys.begin(st);
+  for (int j = 0; j < n_tasks; ++j) {
+    const int c = indptr[j + 1] - indptr[j];
+    if (c > 0) kv->live_keys.mark(task_ids[j], kv->len[task_ids[j]] - c);
+  }
+}
+
 // The private page copies of kv->ext on every layer, in uploads of bounded size.
 static int upload_cow_copies(tide_kv* kv, cudaStream_t st) {
   const ExtendOut& x = kv->ext;
@@ -688,6 +700,7 @@ static int extend_tasks(tide_kv* kv, int32_t n_tasks, const int32_t* task_ids, c
                         std::vector<int32_t>* cow_out) {
   int rc = extend_bookkeeping(kv, n_tasks, task_ids, indptr);
   if (rc != TIDE_OK) return rc;
+  if (!kv->ext.idx.empty()) mark_grown(kv, n_tasks, task_ids, indptr, st);
   if ((rc = upload_table_delta(kv, st)) != TIDE_OK) return rc;
   if (cow_out != nullptr) {
     for (size_t i = 0; i < kv->ext.cpy_src.size(); ++i) {
@@ -707,9 +720,7 @@ static int write_tasks(tide_kv* kv, int32_t layer, int32_t n_tasks, const int32_
   int j = 0;
   int rc = TIDE_OK;
   kv->moves_open = false;
-  if (indptr[n_tasks] > 0) kv->live_keys.begin(st);
-  for (int i = 0; i < n_tasks; ++i)
-    if (indptr[i + 1] > indptr[i]) kv->live_keys.mark(task_ids[i], kv->len[task_ids[i]] - (indptr[i + 1] - indptr[i]));
+  if (indptr[n_tasks] > 0) mark_grown(kv, n_tasks, task_ids, indptr, st);
   while (j < n_tasks) {
     Slot* slot;
     if ((rc = acquire_slot(kv, &slot)) != TIDE_OK) return rc;
@@ -795,13 +806,8 @@ int tide_kv_append(tide_kv_t* kv, int32_t layer, int32_t n_tasks, const int32_t*
   if ((rc = extend_bookkeeping(kv, n_tasks, task_ids, indptr)) != TIDE_OK) return rc;
   if ((rc = upload_cow_copies(kv, st)) != TIDE_OK) return rc;     // a copied page must be in place before it is written
   int n_recs = 0;
-  if (indptr[n_tasks] > 0) kv->live_keys.begin(st);
-  for (int j = 0; j < n_tasks; ++j) {
-    const int c = indptr[j + 1] - indptr[j];
-    if (c == 0) continue;
-    ++n_recs;
-    kv->live_keys.mark(task_ids[j], kv->len[task_ids[j]] - c);
-  }
+  if (indptr[n_tasks] > 0) mark_grown(kv, n_tasks, task_ids, indptr, st);
+  for (int j = 0; j < n_tasks; ++j) n_recs += indptr[j + 1] > indptr[j] ? 1 : 0;
   const ExtendOut& x = kv->ext;
   auto fill_recs = [&](AppendRec* recs) {
     int r = 0, grp_cursor = 0;
@@ -916,6 +922,10 @@ int tide_kv_fork(tide_kv_t* kv, int32_t layer, int32_t parent, int32_t child, vo
   kv->live[child] = 1;
   kv->len[child] = L;
   kv->used_tokens += L;
+  if (L > 0) {
+    kv->live_keys.begin(st);
+    kv->live_keys.mark(child, 0);
+  }
   // ---- device: the child's page-table row, then the page copy ----
   for (size_t done = 0; done < cp.size();) {
     Slot* slot;
@@ -1281,6 +1291,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
     chunk = (int)align_up((size_t)std::max(1, ceil_div(len, n_splits)), 2 * kStageKeys);
     n_splits = std::max(1, ceil_div(len, chunk));
   };
+  auto live_from = [&](const tide_row_t& r) -> int32_t { return step ? r.ctx_len - r.q_len : kv->live_keys.from(r.task, st); };
   for (int attempt = 0; attempt < 40; ++attempt) {
     P.seg_dec.clear(); P.seg_tile.clear(); P.seg_umma.clear();
     long long part_rows = 0, qoff = 0;
@@ -1300,7 +1311,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
         s.n_mtiles = mtiles_of(kind, sg.m * g.G);
         cut(kind == kUmma ? 2 * chunk_dec : chunk_dec, sg.pages * g.S, s.n_splits, s.chunk);
         s.causal = 0;
-        s.live_from = INT_MAX;                               // full pages that several tasks hold: nothing writes them
+        s.live_from = live_from(r);                          // (the pages are read through this row's page table)
         s.partial = 1;
         s.x_part_base = gi;
         s.x_n_splits = -2;                                   // marks the shared range until the links are resolved
@@ -1314,7 +1325,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
       s.p = r.ctx_len - r.q_len;
       s.n_mtiles = p.n_mtiles;
       s.causal = 1;
-      s.live_from = step ? s.p : kv->live_keys.from(r.task, st);
+      s.live_from = live_from(r);
       if (gi >= 0) {
         s.origin = groups[(size_t)gi].pages * g.S;
         s.partial = 1;
@@ -1438,8 +1449,9 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   // dyn != nullptr: fixed launch shapes; the counts of the batch are read on the device (header of the step area)
   const bool dec = dyn ? kv->cap_dec > 0 : d.items_dec > 0, tile = dyn ? kv->cap_tile > 0 : d.items_tile > 0;
   const bool umma = dyn ? kv->cap_umma > 0 : d.items_umma > 0, merge = dyn ? kv->cap_merge_rows > 0 : d.merge_rows > 0;
-  // The decode kernel's producers may run ahead of the append when their row descriptors do not come from an upload right
-  // in front of it (they are in the launch, or in the step area), and the page table is the handle's own.
+  // The producers of the first attention kernel may run ahead of the work in front of it when their row descriptors do not
+  // come from an upload right there (they are in the launch, or in the step area), and the page table is the handle's own,
+  // so that all that may still be written is in LiveKeys.
   const bool run_ahead = (inl != nullptr || step) && page_table == nullptr && !tile && !events;
   auto inline_segs = [&](const std::vector<Segment>& v) -> AttendInline& {
     AttendInline& pi = kv->attend_inline;
@@ -1586,6 +1598,7 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   cudaStream_t st = (cudaStream_t)stream;
   kv->append_launches = 0;
   if ((rc = extend_bookkeeping(kv, n_rows, ids.data(), indptr.data())) != TIDE_OK) return rc;
+  mark_grown(kv, n_rows, ids.data(), indptr.data(), st);
   // Header, write records, segments and page-table delta travel in one launch that reads the pinned buffers (as a table
   // update with its upload and two copies they took 27 us of a step).  Large deltas, and the copy engine, take the
   // steps one by one.

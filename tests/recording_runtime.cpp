@@ -83,6 +83,7 @@ cudaError_t launch_upload_set(const UploadSet& u, cudaStream_t s) {
   return note(kUpload, s);
 }
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s) {
+  if (p.n_tokens <= 0 && p.n_upd <= 0) return cudaSuccess;
   g_log.push_back({kAppend, 0, 0, p.n_tokens, p.early, (void*)s, {}});
   return cudaSuccess;
 }

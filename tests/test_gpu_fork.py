@@ -250,3 +250,42 @@ def test_step_planned_before_its_append_does_not_share_a_page_that_is_about_to_b
     ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
     H.check_outputs(H.from_dev(out), lse.cpu().numpy(), ref_o, ref_l, "step over a rolled-back group")
     kv.close()
+
+
+@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 32)])
+@pytest.mark.parametrize("fresh", [1, 30])
+def test_children_are_attended_right_behind_their_fork(geom, fresh):
+    """Fork at a length inside a page, then attention of the child with nothing between the two; the child is released and
+    forked again, from parents of other lengths, so its table row and its copied page change every time."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    Hq, Hkv, d, s = geom
+    rng = np.random.default_rng(Hq + d + fresh)
+    scale, lens = 1.0 / math.sqrt(d), [1007, 33, 2500, 1007, 640]
+    n = len(lens)
+    pages = sum((c + s - 1) // s for c in lens) + 16
+    order = rng.permutation(pages).astype(np.int32)
+    kv = tide.TideKV(Hq, Hkv, d, s, pages, n + 1, pages, 4, 4096, free_order=order)
+    orc = PagedKVOracle(pages, s, Hkv, d, n + 1, pages, free_order=order)
+    for t, c in enumerate(lens):
+        k, v = inputs.normal_bf16(rng, (c, Hkv, d)), inputs.normal_bf16(rng, (c, Hkv, d))
+        for o, a, b in ((kv, H.to_dev(k, torch), H.to_dev(v, torch)), (orc, k, v)):
+            o.alloc(t)
+            o.append([t], [0, c], a, b)
+    q = inputs.normal_bf16(rng, (fresh, Hq, d))
+    dq = H.to_dev(q, torch)
+    turns = list(range(n)) * 3
+    out = torch.zeros((len(turns), fresh, Hq, d), dtype=torch.int16, device="cuda")
+    lse = torch.zeros((len(turns), fresh, Hq), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    for i, parent in enumerate(turns):
+        kv.fork(parent, n)
+        kv.attend([(n, fresh, lens[parent])], dq, scale, out[i], lse[i])
+        kv.release(n)
+    assert kv.status() == tide.OK
+    for i, parent in enumerate(turns):
+        orc.fork(parent, n)
+        ref_o, ref_l = cbuild.attend_paged(orc, [(n, fresh, lens[parent])], q, scale)
+        H.check_outputs(H.from_dev(out[i]), lse[i].cpu().numpy(), ref_o, ref_l, f"child {i}")
+        orc.release(n)
+    kv.close()

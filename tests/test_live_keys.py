@@ -67,3 +67,70 @@ def test_a_series_of_moves(kv):
     assert kv.live([(0, 1, n0), (1, 1, n1)], A) == {0: 64, 1: 32}
     assert kv.prune(2, 64, 100, A) == 0                        # an attention call came between: a series of its own
     assert kv.live([(0, 1, n0), (1, 1, n1), (2, 1, 1002 - 36)], A) == {0: hp.INT_MAX, 1: hp.INT_MAX, 2: 64}
+
+
+def test_a_forked_child_is_live_as_a_whole(kv):
+    """Its page-table row and the copy of its last page are written by the launches in front."""
+    kv.alloc(9)
+    assert kv.append({9: 1}, A) == 0                           # nothing of the parent is in flight any more
+    assert kv.fork(0, 5, A) == 0
+    assert kv.live([(5, 1, 1000), (0, 1, 1000)], A) == {5: 0, 0: hp.INT_MAX}
+    assert kv.append({5: 1}, A) == 0
+    assert kv.live([(5, 1, 1001), (0, 1, 1000)], A) == {5: 992, 0: hp.INT_MAX}
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_a_shared_range_is_as_live_as_the_row_it_is_read_through(lib, D):
+    kv = hp.Handle(lib, D=D, Hq=8, Hkv=2)
+    kv.tune(2, 0)                                              # groups however little they save
+    kv.alloc(0)
+    assert kv.append({0: 1003}, A) == 0
+    for c in range(1, 8):
+        assert kv.fork(0, c, A) == 0
+    kv.forget()
+    assert kv.attend([(c, 1, 1003) for c in (7, 6, 5, 4, 3, 2, 1, 0)], A) == 0
+    found = {}
+    for l in kv.launches():
+        if l["kind"] in (hp.DECODE, hp.UMMA) and l["run_ahead"]:
+            for s in l["segs"]:
+                found.setdefault("own" if s["causal"] else "shared", []).append(s["live_from"])
+    assert found["shared"] == [0]
+    kv.close()
+
+
+def test_extended_tasks_are_live_from_their_last_page_on(kv):
+    """A page that the growth replaces by a private copy, and new entries of the page table, are being written."""
+    assert kv.fork(0, 5, A) == 0 and kv.fork(0, 6, A) == 0
+    assert kv.truncate(6, 500) == 0                            # inside a page that the others hold
+    assert kv.append({1: 1}, A) == 0
+    assert kv.extend({6: 1, 2: 40}, A) == 0
+    assert kv.live([(6, 1, 500), (2, 1, 1002), (5, 1, 1000)], A) == {6: 496, 2: 992, 5: hp.INT_MAX}
+
+
+def test_growth_that_tells_the_device_nothing_leaves_everything_live(kv):
+    assert kv.append({1: 5}, A) == 0
+    kv.forget()
+    assert kv.extend({0: 1}, A) == 0 and kv.launches() == []   # inside its last page
+    assert kv.append({0: 0, 2: 0}, A) == 0 and kv.launches() == []
+    assert kv.truncate(2, 0) == 0 and kv.fork(2, 5, A) == 0 and kv.launches() == []
+    assert kv.live([(1, 1, 1006)], A) == {1: 992}
+
+
+def test_a_step_that_has_begun(kv):
+    assert kv.fork(0, 6, A) == 0 and kv.truncate(6, 500) == 0
+    assert kv.append({1: 1}, A) == 0
+    assert kv.step_begin([(6, 1, 501), (2, 40, 1042)], A) == 0
+    assert kv.live([(6, 1, 500), (2, 1, 1002), (3, 1, 1003)], A) == {6: 496, 2: 992, 3: hp.INT_MAX}
+    kv.forget()
+    assert kv.step_layer(0, A) == 0                            # behind its own append, which waits for all that
+    launches = [l for l in kv.launches() if l["kind"] in (hp.DECODE, hp.UMMA)]
+    assert [(l["kind"], l["run_ahead"], l["overlapped"]) for l in launches] == [(hp.UMMA, 1, 0), (hp.DECODE, 0, 1)]
+    live = {s["task"]: s["live_from"] for l in launches for s in l["segs"]}
+    assert live == {6: 500, 2: 1002}
+
+
+def test_a_prune_that_goes_through_the_staging_area(kv):
+    assert kv.fork(0, 5, A) == 0
+    assert kv.append({1: 1}, A) == 0
+    assert kv.prune(5, 100, 300, A) == 0                       # shares its pages: a new table row, a copied page, an append
+    assert kv.live([(5, 1, 800), (0, 1, 1000)], A) == {5: 96, 0: hp.INT_MAX}
