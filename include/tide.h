@@ -251,7 +251,8 @@ typedef enum {
   TIDE_TUNE_HOST_STEP_CHUNKS = 3, /* token groups of tide_step_host, 1..8; 0 = chosen by transfer size (default)   */
   TIDE_TUNE_UMMA_MIN_ROWS = 4,    /* packed rows (q_len * Hq/Hkv) from which a head_dim-128 row runs on the        */
                                   /* tcgen05 kernel, >= 17 (default 17)                                            */
-  TIDE_TUNE_WAIT_LIMIT_US = 5,    /* time limit of every wait inside a kernel, microseconds (default 2 000 000)    */
+  TIDE_TUNE_WAIT_LIMIT_US = 5,    /* time limit of every wait inside a kernel, microseconds (default 2 000 000);   */
+                                  /* earlier work of the stream that a kernel has started beside does not count    */
   TIDE_TUNE_UMMA_TILE_KEYS = 7,   /* key-tile size of the tcgen05 kernel: 64 or 128                                */
   TIDE_TUNE_UPLOAD_BY_KERNEL = 8, /* the small planning uploads of every call are done by a kernel that reads the   */
                                   /* pinned, device-mapped staging slot (default 1) or by the copy engine (0)       */

@@ -181,7 +181,7 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
   }
   volatile int* abort_flag = &s_abort;
   auto wait = [&](uint64_t& bar, int parity) -> bool {
-    return mbar_wait(smem_u32(&bar), (uint32_t)parity, abort_flag, P.status, P.wait_limit_ns);
+    return mbar_wait(smem_u32(&bar), (uint32_t)parity, abort_flag, P.status, P.wait_limit_ns, (P.run_ahead | P.overlapped) != 0);
   };
   // where a warp branches on the outcome: its lanes stay together
   auto wait_all = [&](uint64_t& bar, int parity) -> bool { return __all_sync(0xffffffffu, wait(bar, parity)) != 0; };

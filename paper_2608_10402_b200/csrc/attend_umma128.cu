@@ -300,6 +300,10 @@ __device__ __forceinline__ void attend_umma128_body(const AttendParams& P, const
       int issued = 0;                                          // tiles this warp has issued its copies of
       bool ok = true, ahead = early;
       for (int it = 0; ok; ++it) {
+        if (ahead && it > 0) {                                 // the scheduler publishes no second item before that either
+          grid_dep_wait();
+          ahead = false;
+        }
         if (!wait_all(bars.item_full[it % kItemSlots], (it / kItemSlots) & 1)) break;
         const Item& w = items[it % kItemSlots];
         if (!w.run) break;

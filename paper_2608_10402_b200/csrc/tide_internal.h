@@ -301,16 +301,24 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait.  `abort_flag` lives in shared memory: once any thread of the CTA has given up, every
 // later wait returns at once so that the CTA still walks its normal control flow to the end.
+// `beside`: the kernel may have started before the one in front of it was complete.  What it waits for can then depend on
+// warps that are held up until that one is, however long that takes: a limit that runs out is counted anew from there.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
-                                          long long limit_ns) {
+                                          long long limit_ns, bool beside = false) {
   if (mbar_try(bar, parity)) return true;
   if (*abort_flag) return false;
-  const long long t0 = global_ns();
+  long long t0 = global_ns();
   int spins = 0;
   while (!mbar_try(bar, parity)) {
     if ((++spins & 255) == 0) {
       if (*abort_flag) return false;
       if (global_ns() - t0 > limit_ns) {
+        if (beside) {
+          grid_dep_wait();
+          beside = false;
+          t0 = global_ns();
+          continue;
+        }
         *abort_flag = 1;
         atomicExch(status, (int)TIDE_ERR_DEVICE_TIMEOUT);
         return false;
