@@ -443,13 +443,15 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
         // ---- O += P.V ----
         if (key0 + 16 > kv_end) {
           // slots past the end of the item hold whatever the page held before: clear V there so that
-          // weight 0 times stale bits cannot produce NaN
+          // weight 0 times stale bits cannot produce NaN.  The stage is filled again for the next item by bulk copies, which
+          // are ordered behind these stores only by the fence.
           const int koff = warp * 16, first = kv_end - key0;           // 1..15
           uint8_t* vgen = smem_raw + slot * C::kStageBytes + (koff / g.S) * g.head_bytes;
           for (int idx = lane; idx < (16 - first) * (D / 8); idx += 32) {
             const int rr = koff % g.S + first + idx / (D / 8), c = idx % (D / 8);
             *reinterpret_cast<uint4*>(vgen + blk_offset(g, rr, 1, c)) = make_uint4(0, 0, 0, 0);
           }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
         }
         uint32_t pa[4];

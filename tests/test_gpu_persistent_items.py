@@ -258,3 +258,38 @@ def test_steps_queued_without_waiting_follow_one_another(geom, layers):
             ref_o, ref_l = cbuild.attend_paged(orc.layer(l), rows, q[l], scale)
             H.check_outputs(H.from_dev(out[l]), lse[l].cpu().numpy(), ref_o, ref_l, f"step {s}, layer {l}")
     kv.close()
+
+
+@pytest.mark.parametrize("geom", [(16, 16, 128, 16), (16, 16, 128, 32), (32, 16, 64, 16), (16, 16, 64, 32)])
+def test_ragged_ends_leave_the_next_item_alone(geom):
+    """Every item ends inside a 16-key block, whose unused V slots its consumers clear; the stage is filled again at once
+    for the block's next item.  Few keys and large values: a slot lost to the item before shows far above the tolerance."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    HQ, HKV, D, S = geom
+    rng = np.random.default_rng(HQ + D + S)
+    scale, n = 1.0 / math.sqrt(D), 120
+    ctx = [16 * int(rng.integers(0, 13)) + int(rng.integers(1, 16)) for _ in range(n)]
+    pages, max_pages = sum((c + S - 1) // S for c in ctx) + 1, 208 // S + 1
+    order = rng.permutation(pages).astype(np.int32)
+    kv = tide.TideKV(HQ, HKV, D, S, pages, n, max_pages, n, sum(ctx), free_order=order)
+    orc = PagedKVOracle(pages, S, HKV, D, n, max_pages, free_order=order)
+    ip = np.concatenate([[0], np.cumsum(ctx)]).astype(np.int32)
+    k = inputs.normal_bf16(rng, (int(ip[-1]), HKV, D))
+    v = inputs.f32_to_bf16_bits(8.0 + 8.0 * rng.random((int(ip[-1]), HKV, D)).astype(np.float32))
+    for o in (kv, orc):
+        for t in range(n):
+            o.alloc(t)
+    kv.append(list(range(n)), ip, H.to_dev(k, torch), H.to_dev(v, torch))
+    orc.append(list(range(n)), ip, k, v)
+    q = inputs.normal_bf16(rng, (n, HQ, D))
+    dq, rows = H.to_dev(q, torch), [(t, 1, c) for t, c in enumerate(ctx)]
+    outs = [torch.zeros((n, HQ, D), dtype=torch.int16, device="cuda") for _ in range(20)]
+    lse = torch.zeros((n, HQ), dtype=torch.float32, device="cuda")
+    for out in outs:
+        kv.attend(rows, dq, scale, out, lse)
+    assert kv.status() == tide.OK and kv.last_plan()["decode_items"] == n * HKV
+    ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
+    H.check_outputs(H.from_dev(outs[0]), lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
+    kv.close()
