@@ -1587,13 +1587,16 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   // The plan needs the lengths after the step only through ctx_len, which the rows already carry, so it is built
   // (and can still be refused) before anything changes.
   PlanHost& P = kv->plan;
-  // Launch shapes fixed without tcgen05 items (or with too few): head size 64 has the warp-MMA tile kernel as well.
-  bool umma = umma_takes(kv) && !(kv->fixed_grids && g.D == 64 && kv->cap_umma == 0);
+  // Launch shapes that do not hold the plan with tcgen05 items may hold the one without: 64-wide heads have the warp-MMA
+  // tile kernel as well, whose rows are cut (and then merged) less.
+  auto fits = [&]() -> bool {
+    return !kv->fixed_grids || (P.items_dec <= kv->cap_dec && P.items_tile <= kv->cap_tile && P.items_umma <= kv->cap_umma &&
+                                P.merge_rows <= kv->cap_merge_rows && indptr[(size_t)n_rows] <= kv->cap_tokens);
+  };
+  const bool umma = umma_takes(kv) && !(kv->fixed_grids && g.D == 64 && kv->cap_umma == 0);
   if ((rc = build_plan(kv, n_rows, rows, umma, true, true, (cudaStream_t)stream, P)) != TIDE_OK) return rc;
-  if (umma && kv->fixed_grids && g.D == 64 && P.items_umma > kv->cap_umma &&
-      (rc = build_plan(kv, n_rows, rows, false, true, true, (cudaStream_t)stream, P)) != TIDE_OK) return rc;
-  if (kv->fixed_grids && (P.items_dec > kv->cap_dec || P.items_tile > kv->cap_tile || P.items_umma > kv->cap_umma ||
-                          P.merge_rows > kv->cap_merge_rows || indptr[(size_t)n_rows] > kv->cap_tokens))
+  if (!fits() && umma && g.D == 64 && (rc = build_plan(kv, n_rows, rows, false, true, true, (cudaStream_t)stream, P)) != TIDE_OK) return rc;
+  if (!fits())
     return TIDE_ERR_WORKSPACE;   // the step does not fit the launch shapes that were fixed
   cudaStream_t st = (cudaStream_t)stream;
   kv->append_launches = 0;
