@@ -93,14 +93,19 @@ __device__ __forceinline__ void merge_splits(const AttendParams& P, const Item& 
       float e[kMergeBatch], v[kMergeBatch][CW];
 #pragma unroll
       for (int x = 0; x < kMergeBatch; ++x) {
-        const bool there = sp0 + x < n_splits;
-        const long long row = src_row(there ? sp0 + x : sp0);
-        e[x] = there ? __ldcg(P.part_lse + row) : -INFINITY;
-        const float* src = P.part_o + row * D + d0;
+        if (sp0 + x < n_splits) {
+          const long long row = src_row(sp0 + x);
+          e[x] = __ldcg(P.part_lse + row);
+          const float* src = P.part_o + row * D + d0;
 #pragma unroll
-        for (int d = 0; d < CW; d += 4) {
-          const float4 t = __ldcg(reinterpret_cast<const float4*>(src + d));
-          v[x][d] = t.x; v[x][d + 1] = t.y; v[x][d + 2] = t.z; v[x][d + 3] = t.w;
+          for (int d = 0; d < CW; d += 4) {
+            const float4 t = __ldcg(reinterpret_cast<const float4*>(src + d));
+            v[x][d] = t.x; v[x][d + 1] = t.y; v[x][d + 2] = t.z; v[x][d + 3] = t.w;
+          }
+        } else {                                             // (another piece in its place, weight 0, would make NaN of infinities)
+          e[x] = -INFINITY;
+#pragma unroll
+          for (int d = 0; d < CW; ++d) v[x][d] = 0.f;
         }
       }
       float m_new = mstar;
@@ -537,6 +542,10 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
           }
 #pragma unroll
         for (int d = 0; d < CW; ++d) acc[d] *= inv;
+        if (mode != 0 && lstar == 0.f) {                     // no key of this piece is visible: weight 0 in the merge, and
+#pragma unroll
+          for (int d = 0; d < CW; ++d) acc[d] = 0.f;         // nothing of the values, which may be infinite, in its rows
+        }
         const int qi = rr / g.G;
         emit(mode == 0, qi, rr - qi * g.G, acc, e2);
       }
