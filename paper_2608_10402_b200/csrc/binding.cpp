@@ -8,6 +8,7 @@
 #include <Python.h>
 
 #include <cstdint>
+#include <cstring>
 
 #include "../../include/tide.h"
 
@@ -15,9 +16,11 @@ namespace {
 
 PyObject *g_data_ptr, *g_cuda_stream;                      // names
 PyObject *g_get_device, *g_raw_stream, *g_as_int32;         // torch's two accessors, and what makes an int32 array of a sequence
+PyObject* g_ndarray;                                        // numpy's array type
 
-// A pointer argument: None, an address, something with data_ptr() (a tensor), or a buffer (numpy, ctypes).  Buffers are
-// held until the call has returned.
+// A pointer argument: None, an address, a numpy array (the address of its first element) or something with data_ptr() (a
+// tensor); arrays are held until the call has returned.  Other objects that export a buffer are not taken for pointers: a
+// numpy integer, for one, may BE an address.
 class Pointer {
  public:
   ~Pointer() { if (view_.obj != nullptr) PyBuffer_Release(&view_); }
@@ -27,19 +30,20 @@ class Pointer {
       p = PyLong_AsVoidPtr(x);
       return !PyErr_Occurred();
     }
-    if (PyObject_CheckBuffer(x)) return buffer(x);
+    if (PyType_Check(g_ndarray) && PyObject_TypeCheck(x, reinterpret_cast<PyTypeObject*>(g_ndarray))) return buffer(x, PyBUF_STRIDES);
     PyObject* v = PyObject_CallMethodNoArgs(x, g_data_ptr);
     if (v == nullptr) return false;
     p = PyLong_AsVoidPtr(v);
     Py_DECREF(v);
     return !PyErr_Occurred();
   }
-  bool buffer(PyObject* x) {
-    if (PyObject_GetBuffer(x, &view_, PyBUF_SIMPLE) != 0) return false;    // C-contiguous or an error
+  bool buffer(PyObject* x, int flags) {
+    if (PyObject_GetBuffer(x, &view_, flags) != 0) return false;
     p = view_.buf;
     bytes = view_.len;
     return true;
   }
+  const Py_buffer& view() const { return view_; }
   // int32 values: a contiguous buffer of that type, or whatever converts to one
   bool ints(PyObject* x) {
     if (PyObject_CheckBuffer(x) && PyObject_GetBuffer(x, &view_, PyBUF_ND | PyBUF_FORMAT) == 0) {
@@ -54,7 +58,7 @@ class Pointer {
     PyErr_Clear();
     PyObject* made = PyObject_CallOneArg(g_as_int32, x);
     if (made == nullptr) return false;
-    const bool ok = buffer(made);                             // the view keeps the array
+    const bool ok = buffer(made, PyBUF_SIMPLE);               // the view keeps the array
     Py_DECREF(made);
     return ok;
   }
@@ -123,13 +127,37 @@ struct TaskList {
     return false;
   }
 };
+// tide_row_t records (of ctypes or numpy), or int32 values in rows of three
 struct Rows {
   Pointer rows;
   int32_t n = 0;
   bool from(PyObject* a) {
-    if (!rows.buffer(a)) return false;
-    n = static_cast<int32_t>(rows.bytes / static_cast<Py_ssize_t>(sizeof(tide_row_t)));
-    return true;
+    if (rows.buffer(a, PyBUF_ND | PyBUF_FORMAT)) {
+      const Py_buffer& v = rows.view();
+      char kind[8] = "";
+      types(v.format, kind, sizeof(kind));
+      const bool records = std::strcmp(kind, "T{iii}") == 0 && v.itemsize == static_cast<Py_ssize_t>(sizeof(tide_row_t));
+      const bool triples = std::strcmp(kind, "i") == 0 && v.itemsize == 4 && v.ndim == 2 && v.shape[1] == 3;
+      if (records || triples) {
+        n = static_cast<int32_t>(v.len / static_cast<Py_ssize_t>(sizeof(tide_row_t)));
+        return true;
+      }
+    }
+    PyErr_SetString(PyExc_TypeError, "rows are tide_row_t records or int32 values in rows of three");
+    return false;
+  }
+  // a format without field names and native byte orders; `out` stays short of one that is too long
+  static void types(const char* f, char* out, size_t cap) {
+    size_t k = 0;
+    for (; f != nullptr && *f != 0 && k + 1 < cap; ++f) {
+      if (*f == ':') {
+        for (++f; *f != 0 && *f != ':'; ++f) {}
+        if (*f == 0) break;
+      } else if (*f != '<' && *f != '=' && *f != '@') {
+        out[k++] = *f;
+      }
+    }
+    out[k] = 0;
   }
 };
 #define I32(x) static_cast<const int32_t*>((x).p)
@@ -220,12 +248,13 @@ PyObject* py_step_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return call([&] { return tide_step_host(kv, 0, r.n, ROWS(r), k.p, v.p, q.p, scale, out.p, static_cast<float*>(lse.p), st); });
 }
 
-// use(get_device, raw_stream, as_int32)
+// use(get_device, raw_stream, as_int32, ndarray)
 PyObject* py_use(PyObject*, PyObject* const* a, Py_ssize_t n) {
-  if (!arity(n, 3)) return nullptr;
+  if (!arity(n, 4)) return nullptr;
   Py_XSETREF(g_get_device, Py_NewRef(a[0]));
   Py_XSETREF(g_raw_stream, Py_NewRef(a[1]));
   Py_XSETREF(g_as_int32, Py_NewRef(a[2]));
+  Py_XSETREF(g_ndarray, Py_NewRef(a[3]));
   Py_RETURN_NONE;
 }
 
@@ -242,6 +271,7 @@ PyMODINIT_FUNC PyInit__binding() {
   g_get_device = Py_NewRef(Py_None);
   g_raw_stream = Py_NewRef(Py_None);
   g_as_int32 = Py_NewRef(Py_None);
+  g_ndarray = Py_NewRef(Py_None);
   if (g_data_ptr == nullptr || g_cuda_stream == nullptr) return nullptr;
   return PyModule_Create(&module);
 }

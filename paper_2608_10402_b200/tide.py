@@ -102,9 +102,9 @@ def _prepare_binding():
     import torch
     raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
     if raw is not None:
-        _b.use(torch._C._cuda_getDevice, raw, _i32)
+        _b.use(torch._C._cuda_getDevice, raw, _i32, np.ndarray)
     else:
-        _b.use(torch.cuda.current_device, lambda device: torch.cuda.current_stream(device).cuda_stream, _i32)
+        _b.use(torch.cuda.current_device, lambda device: torch.cuda.current_stream(device).cuda_stream, _i32, np.ndarray)
     _ready = True
 
 

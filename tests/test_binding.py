@@ -37,3 +37,34 @@ def test_pointers_rows_and_numbers(tide):
                 lambda: tide._b.append(0, [1]), lambda: tide._b.attend(0, 0, rows, None, x, "a", x, None, 0)):
         with pytest.raises(TypeError):
             bad()
+
+
+def test_rows_are_records_or_triples_of_int32(tide):
+    x = np.zeros(4)
+    call = lambda rows: (tide._b.attend(0, 0, rows, None, x, 0.5, x, None, 0), tide._b.step_begin(0, rows, 0),
+                         tide._b.step_host(0, rows, x, x, x, 0.5, x, None, 0))
+    record = np.dtype([("task", np.int32), ("q_len", np.int32), ("ctx_len", np.int32)])
+    for good in (tide.rows_array([(0, 1, 5), (1, 2, 7)]), tide.rows_array([]), np.zeros((5, 3), np.int32), np.zeros((0, 3), np.int32), np.zeros(5, record)):
+        assert call(good) == (tide.ERR_INVALID_ARG,) * 3
+    for bad in (np.zeros((5, 3), np.int64), np.zeros((5, 3), np.float32), np.zeros((5, 3), np.uint32), np.zeros((5, 3), ">i4"), np.zeros(15, np.int32),
+                np.zeros((3, 5), np.int32), np.zeros((5, 4), np.int32), np.zeros((4, 2, 3), np.int32), bytes(24), bytearray(7), np.zeros(5, "V12"),
+                np.zeros(5, [("a", np.int32), ("b", np.float32), ("c", np.int32)]), (tide.ctypes.c_int32 * 6)()):
+        for f in (lambda: tide._b.attend(0, 0, bad, None, x, 0.5, x, None, 0), lambda: tide._b.step_begin(0, bad, 0),
+                  lambda: tide._b.step_host(0, bad, x, x, x, 0.5, x, None, 0)):
+            with pytest.raises(TypeError):
+                f()
+
+
+def test_pointers_are_numbers_arrays_and_tensors(tide):
+    """numpy arrays by the address of their first element, whatever their strides and type; nothing else that happens to
+    export a buffer - a numpy integer that holds an address is not the address of that integer."""
+    import torch
+    rows = tide.rows_array([(0, 1, 5)])
+    call = lambda p: tide._b.attend(0, 0, rows, None, p, 0.5, p, p, 0)
+    a = np.zeros((4, 4))
+    for good in (None, 4096, a, a[:, :2], a[::-1], a.T, np.zeros(()), np.zeros(0), np.zeros(3, "M8[s]"), np.frombuffer(b"1234", np.int32),
+                 torch.zeros(3), torch.zeros((3, 3), dtype=torch.bfloat16).t()):
+        assert call(good) == tide.ERR_INVALID_ARG
+    for bad in (np.int64(4096), b"1234", bytearray(4), memoryview(b"1234"), (tide.ctypes.c_int32 * 6)(), tide.ctypes.c_void_p(4096), 4096.0, "a"):
+        with pytest.raises((TypeError, AttributeError)):
+            call(bad)
