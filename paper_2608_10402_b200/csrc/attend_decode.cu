@@ -118,8 +118,7 @@ __device__ __forceinline__ void merge_splits(const AttendParams& P, const Item& 
       for (int d = 0; d < CW; ++d) acc[d] *= keep;
 #pragma unroll
       for (int x = 0; x < kMergeBatch; ++x) {
-        if (e[x] == -INFINITY) continue;                     // no key of this piece is visible; what it holds may be NaN
-        const float wgt = exp2f(e[x] - mu);
+        const float wgt = exp2f(e[x] - mu);                                           // -inf: 0
         tot += wgt;
 #pragma unroll
         for (int d = 0; d < CW; ++d) acc[d] += wgt * v[x][d];

@@ -44,7 +44,6 @@ def test_an_infinite_value_behind_a_query_in_a_piece_of_its_own(geom, n, front, 
     ref_o, ref_l = cbuild.attend_paged(orc, [(0, n, L)], q, scale)
     H.check_outputs(H.from_dev(out)[:1], lse.cpu().numpy()[:1], ref_o[:1], ref_l[:1], f"{geom}")
     kv.close()
-<<<<<<< Updated upstream
 
 
 @pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 32)])
@@ -80,5 +79,3 @@ def test_an_infinite_value_that_is_visible_stays_infinite(geom, ctx):
     ref_o[0, G:2 * G, 5], ref_o[0, :G, D - 1] = 0, 0
     H.check_outputs(bits, lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
     kv.close()
-=======
->>>>>>> Stashed changes
