@@ -272,7 +272,7 @@ __device__ __forceinline__ void attend_umma128_body(const AttendParams& P, const
   // with one of 46 to 463 tokens 21.9 to 19.3, groups 76.2 to 74.4, prompts 698 to 692.
   const bool early = P.run_ahead != 0 && warp >= 8;
   if (!early) {
-    if (!P.overlapped) grid_dep_wait();
+    grid_dep_wait();
     grid_dep_launch();
   }
   const int n_items = P.dyn ? __ldcg(P.dyn) : P.n_items;           // fixed grid: the batch's counts live in device memory
@@ -785,7 +785,6 @@ __device__ __forceinline__ void attend_umma128_body(const AttendParams& P, const
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }
-  if (P.overlapped) grid_dep_wait();
 }
 
 template <int D>

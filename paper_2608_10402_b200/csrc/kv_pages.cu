@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) fetch_kernel(uint4* __restrict__ dst, con
 cudaError_t launch_fetch(void* dst, const void* src_mapped_host, size_t bytes, cudaStream_t s) {
   if (bytes == 0) return cudaSuccess;
   const size_t n = bytes / 16;
-  return launch_dep(fetch_kernel, (unsigned)std::min<size_t>((n + 255) / 256, 148), 256, 0, s, (uint4*)dst, (const uint4*)src_mapped_host, n);
+  return launch_dep(fetch_kernel, (unsigned)std::min<size_t>((n + 255) / 256, (size_t)sm_count()), 256, 0, s, (uint4*)dst, (const uint4*)src_mapped_host, n);
 }
 
 __global__ void upload_set_kernel(const __grid_constant__ UploadSet u) {

@@ -1227,7 +1227,6 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
   }
   // A shared range is streaming work like a decode row (few rows against many keys) and is cut like one, whichever kernel
   // its packed rows call for.
-  auto shared_kind = [&](int R) { return kind_of(R); };
   for (const ShareGroup& sg : groups) w_dec += (long long)g.Hkv * sg.pages * g.S;
   // With groups in the batch a third fewer items, and a shared range on the tcgen05 kernel in pieces twice as long (one block
   // of it fills an SM): 8 groups of 8, 6149 shared and 900 to 3100 own tokens, 78.2 us against 87.6 with the cut of a
@@ -1302,7 +1301,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
       if (gi >= 0 && groups[(size_t)gi].first == b) {
         // the shared range of the group that starts at this row
         const ShareGroup& sg = groups[(size_t)gi];
-        const int kind = shared_kind(sg.m * g.G);
+        const int kind = kind_of(sg.m * g.G);
         Segment s{};
         s.table_off = r.task * g.max_pages_per_task;
         s.q_off = (int32_t)qoff;
@@ -1368,7 +1367,7 @@ static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool 
         if (s.x_n_splits == -2) {                            // a shared range: it has no output rows of its own
           groups[(size_t)s.x_part_base].part_base = s.part_base;
           groups[(size_t)s.x_part_base].n_splits = s.n_splits;
-        } else if (v == &P.seg_dec && (s.partial == 0 || shared_kind(groups[(size_t)s.x_part_base].m * g.G) == kUmma)) {
+        } else if (v == &P.seg_dec && (s.partial == 0 || kind_of(groups[(size_t)s.x_part_base].m * g.G) == kUmma)) {
           // a split decode-style row, or a member of a group whose shared range runs in the tcgen05 kernel (the decode kernel
           // follows it): the split that finishes last merges the partials inside the decode kernel
           s.partial = 2;
@@ -1468,7 +1467,7 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   };
   auto launch_umma = [&]() -> cudaError_t {
     ap.segs = d.seg_umma; ap.n_segs = (int)d.n_umma; ap.n_items = (int)d.items_umma;
-    ap.dyn = dyn ? dyn + kHdrUmmaItems : nullptr; ap.grid_cap = kv->cap_umma; ap.overlapped = 0;
+    ap.dyn = dyn ? dyn + kHdrUmmaItems : nullptr; ap.grid_cap = kv->cap_umma;
     ap.run_ahead = run_ahead ? 1 : 0;
     ++launches;
     if (kv->umma_tile_keys != 128) return launch_attend_umma(ap, st);
@@ -1479,7 +1478,7 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   if (events) cudaEventRecord(kv->ev_attend[0], st);
   if (tile) {
     ap.segs = d.seg_tile; ap.n_segs = (int)d.n_tile; ap.n_items = (int)d.items_tile;
-    ap.dyn = dyn ? dyn + kHdrTileItems : nullptr; ap.grid_cap = kv->cap_tile; ap.overlapped = 0;
+    ap.dyn = dyn ? dyn + kHdrTileItems : nullptr; ap.grid_cap = kv->cap_tile;
     if (launch_attend_tile(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
     ++launches;
   }

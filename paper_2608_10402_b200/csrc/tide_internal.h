@@ -96,7 +96,7 @@ struct AttendParams {
   int* merge_ctr = nullptr;   // per (segment with partial == 2, kv head): splits finished so far; zero between launches
   long long wait_limit_ns = kWaitLimitNsDefault;   // bound of every wait inside the kernel
   int run_ahead = 0;          // decode, 128-key tcgen05: the producers may read keys below Segment::live_from before earlier work is complete
-  int overlapped = 0;         // the kernel before this one in the stream is the other attention kernel of the same batch (see grid_dep_wait)
+  int overlapped = 0;         // decode: the kernel before this one in the stream is the tcgen05 kernel of the same batch (see grid_dep_wait)
   // Test hook for the bounded waits (never set in normal use): in work item 0 the producer leaves out its part
   // of the first stage, so the consumers' wait for that stage runs out and the time-out path executes.
   int debug_drop_first_stage = 0;
@@ -281,18 +281,6 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Whether the phase is complete, without waiting.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.b32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
