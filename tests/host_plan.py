@@ -39,7 +39,7 @@ class Handle:
         cfg.workspace, cfg.workspace_bytes = (self._ws.ctypes.data + 255) // 256 * 256, wb.value
         self.h = ctypes.c_void_p(0)
         assert lib.tide_kv_create(ctypes.byref(cfg), ctypes.byref(self.h)) == 0
-        self.mp = max_pages
+        self.cfg, self.mp = cfg, max_pages
 
     def close(self):
         self.lib.tide_kv_destroy(self.h)
@@ -83,6 +83,14 @@ class Handle:
     def step_layer(self, layer, stream=0):
         p = ctypes.c_void_p(4096)
         return self.lib.tide_step_layer(self.h, layer, p, p, p, ctypes.c_float(0.125), p, None, ctypes.c_void_p(stream))
+
+    def step_host(self, rows):
+        """A host-buffer step on stream 0 with (empty) host buffers."""
+        kv_row, q_row = 2 * self.cfg.num_kv_heads * self.cfg.head_dim, 2 * self.cfg.num_q_heads * self.cfg.head_dim
+        tokens = sum(n for _, n, _ in rows)
+        k, q, o = (np.zeros(tokens * b, np.uint8) for b in (kv_row, q_row, q_row))
+        a = lambda x: x.ctypes.data_as(ctypes.c_void_p)
+        return self.lib.tide_step_host(self.h, 0, len(rows), tide.rows_array(rows), a(k), a(k), a(q), ctypes.c_float(0.125), a(o), None, None)
 
     def fix_grids(self, *caps):
         return self.lib.tide_step_fix_grids(self.h, *caps)

@@ -172,9 +172,11 @@ def test_few_resume_rows_cut_along_their_keys(geom, lens, cut):
     kv.close()
 
 
-@pytest.mark.parametrize("geom,ctx", [((28, 4, 128, 16), [1024]), ((28, 4, 128, 16), [16000]), ((28, 4, 128, 32), [4000] * 4), ((16, 1, 128, 16), [40001, 130]),
-                                      ((12, 4, 64, 16), [9000, 2047, 1]), ((6, 2, 128, 16), [70000]), ((28, 4, 128, 16), [250 + 250 * i for i in range(16)])])
-def test_few_decode_rows_and_their_merge(geom, ctx):
+@pytest.mark.parametrize("geom,ctx,pieces", [((28, 4, 128, 16), [1024], [4]), ((28, 4, 128, 16), [16000], [32]), ((28, 4, 128, 32), [4000] * 4, [8] * 4),
+                                             ((16, 1, 128, 16), [40001, 130], [40, 1]), ((12, 4, 64, 16), [9000, 2047, 1], [24, 6, 1]),
+                                             ((6, 2, 128, 16), [70000], [69]),
+                                             ((28, 4, 128, 16), [250 + 250 * i for i in range(16)], [1, 1] + [2 + i // 2 for i in range(14)])])
+def test_few_decode_rows_and_their_merge(geom, ctx, pieces):
     """Decode rows that are cut for the merge of their pieces: up to eight pieces, whole and ragged batches of eight, more
     than thirty-two; one block per SM and two."""
     import torch
@@ -198,6 +200,8 @@ def test_few_decode_rows_and_their_merge(geom, ctx):
     lse = torch.zeros((n, HQ), dtype=torch.float32, device="cuda")
     kv.attend(rows, H.to_dev(q, torch), scale, out, lse)
     assert kv.status() == tide.OK
+    plan = kv.last_plan()
+    assert plan["decode_items"] == HKV * sum(pieces) and plan["merge_rows"] == HQ * sum(p > 1 for p in pieces)
     ref_o, ref_l = cbuild.attend_paged(orc, rows, q, scale)
     H.check_outputs(H.from_dev(out), lse.cpu().numpy(), ref_o, ref_l, f"{geom}")
     kv.close()

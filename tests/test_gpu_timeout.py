@@ -19,6 +19,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("kind,geom,p,n", [("warp-MMA decode kernel", (8, 2, 64, 16), 300, 1),
                                            ("warp-MMA decode kernel, head size 128", (28, 4, 128, 16), 700, 1),
                                            ("warp-MMA tile kernel", (8, 2, 64, 16), 150, 40),
+                                           ("tcgen05 kernel, head size 64", (8, 2, 64, 16), 150, 40),
                                            ("tcgen05 kernel", (28, 4, 128, 16), 200, 40)])
 def test_a_wait_that_runs_out_is_reported_once_and_the_handle_stays_usable(kind, geom, p, n):
     import torch
@@ -28,6 +29,8 @@ def test_a_wait_that_runs_out_is_reported_once_and_the_handle_stays_usable(kind,
     L = p + n
     pages = (L + S - 1) // S + 2
     kv = tide.TideKV(HQ, HKV, D, S, pages, 2, pages, 2, max(n, 4))
+    if kind == "warp-MMA tile kernel":
+        kv.tune(tide.TUNE_UMMA_TILE_KEYS, 64)                 # the tcgen05 kernel with these takes no 64-wide heads
     orc = PagedKVOracle(pages, S, HKV, D, 2, pages)
     k, v = inputs.normal_bf16(rng, (L, HKV, D)), inputs.normal_bf16(rng, (L, HKV, D))
     for o in (kv, orc):
@@ -50,6 +53,7 @@ def test_a_wait_that_runs_out_is_reported_once_and_the_handle_stays_usable(kind,
     elapsed = time.perf_counter() - t0
     assert st == tide.ERR_DEVICE_TIMEOUT, f"{kind}: status {st}"
     assert elapsed < 2.0, f"{kind}: {elapsed:.3f} s for waits bounded at 2 ms"
+    assert (kv.last_plan()["prefill_items"] == HKV * -(-n * (HQ // HKV) // (64 if "tile" in kind else 256))) == (n > 1)
     assert kv.status() == tide.OK                             # reported once, then cleared
 
     kv.tune(tide.TUNE_WAIT_LIMIT_US, 2_000_000)

@@ -1,6 +1,7 @@
 """What the library's host side plans and launches, recorded without a GPU."""
 import pytest
 
+from paper_2608_10402_b200 import tide
 from tests import host_plan as hp
 
 
@@ -35,4 +36,37 @@ def test_fixed_launch_shapes_that_hold_neither_plan_are_refused(lib):
         assert kv.fix_grids(*caps) == 0
         assert kv.step_begin([(0, 2000, 11000)]) == -8
         assert kv.attend([(0, 1, 9000)]) == 0 and kv.attend([(0, 1, 9001)]) == -7      # nothing has changed
+    kv.close()
+
+
+@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (16, 1, 64, 32)])
+@pytest.mark.parametrize("groups", [1, 2, 4, 7])
+def test_a_host_step_is_cut_between_and_inside_rows(lib, geom, groups):
+    """Every token of every row is attended once, in order, its context ending with it; long rows are cut between groups at
+    whole tcgen05 items; the groups take turns on two streams, each behind its own append."""
+    kv = hp.Handle(lib, *geom)
+    kv.tune(tide.TUNE_HOST_STEP_CHUNKS, groups)
+    kv.tune(tide.TUNE_HOST_ZERO_COPY, 0)
+    prefix, new = [0, 700, 15, 2500, 3000, 1, 64, 900], [1400, 1, 1, 1, 733, 1, 160, 17]
+    kv.alloc(*range(8))
+    assert kv.append(dict(enumerate(prefix))) == 0
+    kv.forget()
+    assert kv.step_host([(t, n, p + n) for t, (p, n) in enumerate(zip(prefix, new))]) == 0
+    launches = kv.launches()
+    appends = [l for l in launches if l["kind"] == hp.APPEND]
+    assert sum(l["items"] for l in appends) == sum(new) and (groups == 1) == (len(appends) == 1) and len(appends) <= groups
+    if groups > 1:
+        assert all(a["stream"] != b["stream"] for a, b in zip(appends, appends[1:])) and {a["stream"] for a in appends} == {a["stream"] for a in appends[:2]}
+    seen, parts, stream = dict(enumerate(prefix)), dict.fromkeys(range(8), 0), None
+    for l in launches:
+        if l["kind"] == hp.APPEND:
+            stream = l["stream"]
+        if l["kind"] in (hp.DECODE, hp.UMMA):
+            assert l["stream"] == stream
+            for s in l["segs"]:
+                assert s["p"] == seen[s["task"]]
+                seen[s["task"]] += s["n"]
+                parts[s["task"]] += 1
+    assert seen == {t: p + n for t, (p, n) in enumerate(zip(prefix, new))}
+    assert (parts[0] > 1) == (groups > 1) and all(parts[t] == 1 for t in (1, 2, 3, 5, 7))
     kv.close()
