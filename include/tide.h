@@ -140,8 +140,8 @@ int tide_attend(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_t* 
  * after the append), attends, and copies out / lse back.  new_k, new_v: host bf16 [sum q_len, Hkv, D];
  * q, out: host bf16 [sum q_len, Hq, D]; lse: host fp32 or NULL.  Host buffers should be pinned for
  * the copies to be asynchronous.  The call returns after the results have arrived.  A small step (up to
- * 2 MiB in all) whose buffers are pinned and addressable by the device is not copied at all: the kernels
- * read the inputs and write the results across PCIe themselves.  A large step is cut
+ * 2 MiB in all) whose buffers are pinned and addressable by the device is not copied by the copy engines: kernels
+ * read new_k / new_v, fetch q and write the results across PCIe themselves.  A large step is cut
  * into groups of consecutive tokens whose copies (on streams the library owns) run beside the kernels
  * of other groups; pages, cache contents and results do not depend on the cut.  The whole step is checked
  * (rows, duplicates, pages) before anything is copied or changed.  Takes layer 0 only. */
@@ -200,8 +200,9 @@ int tide_kv_release_many(tide_kv_t* kv, int32_t n_tasks, const int32_t* task_ids
 /* Sliding-window pruning of old observations (Appendix C.2: only the most recent images are kept, which splits
  * the trajectory): the task keeps tokens [0, keep_prefix) and [tail_begin, len); the tokens in between are
  * dropped and the tail moves down to start at keep_prefix.  Equivalent, page table included, to reading the
- * tail, tide_kv_truncate(task, keep_prefix) and appending the tail again; the move runs on `stream` through
- * the workspace staging area and covers every layer (`layer` must be 0).  Requires
+ * tail, tide_kv_truncate(task, keep_prefix) and appending the tail again; the move runs on `stream` inside the
+ * task's own pages (through the workspace staging area where it shares pages from keep_prefix on) and covers every
+ * layer (`layer` must be 0).  Requires
  * 0 <= keep_prefix <= tail_begin <= len.  All-or-nothing: TIDE_ERR_NO_PAGES if the shorter task could not get
  * its pages (only possible when it shares pages, which do not come back to the free stack);
  * TIDE_ERR_WORKSPACE if the task shares a page from position keep_prefix on and its tail is longer than
@@ -249,18 +250,19 @@ typedef enum {
   TIDE_TUNE_GROUPING = 1,         /* 0: never plan forked rows as groups that read shared pages once (default 1)   */
   TIDE_TUNE_MIN_SAVED_BYTES = 2,  /* KV bytes a batch must save before groups are used (default 64 MiB)            */
   TIDE_TUNE_HOST_STEP_CHUNKS = 3, /* token groups of tide_step_host, 1..8; 0 = chosen by transfer size (default)   */
-  TIDE_TUNE_UMMA_MIN_ROWS = 4,    /* packed rows (q_len * Hq/Hkv) from which a head_dim-128 row runs on the        */
-                                  /* tcgen05 kernel, >= 17 (default 17)                                            */
+  TIDE_TUNE_UMMA_MIN_ROWS = 4,    /* packed rows (q_len * Hq/Hkv) from which a row runs on the tcgen05 kernel,     */
+                                  /* >= 17 (default 17)                                                            */
   TIDE_TUNE_WAIT_LIMIT_US = 5,    /* time limit of every wait inside a kernel, microseconds (default 2 000 000);   */
                                   /* earlier work of the stream that a kernel has started beside does not count    */
-  TIDE_TUNE_UMMA_TILE_KEYS = 7,   /* key-tile size of the tcgen05 kernel: 64 or 128                                */
+  TIDE_TUNE_UMMA_TILE_KEYS = 7,   /* key-tile size of the tcgen05 kernel: 128 (default) or 64 (head_dim 128 only;  */
+                                  /* 64-wide heads then run on the warp-MMA tile kernel)                           */
   TIDE_TUNE_UPLOAD_BY_KERNEL = 8, /* the small planning uploads of every call are done by a kernel that reads the   */
                                   /* pinned, device-mapped staging slot (default 1) or by the copy engine (0)       */
-  TIDE_TUNE_INLINE_DESCRIPTORS = 9, /* small appends (<= 128 rows, <= 256 new pages) and decode-only batches of up  */
-                                  /* to 128 rows carry their descriptors in the launch's own parameters, so that  */
-                                  /* nothing is uploaded before the kernel (default 1); 0: always upload           */
+  TIDE_TUNE_INLINE_DESCRIPTORS = 9, /* small appends (<= 128 rows, <= 256 new pages) and batches of up to 128 decode */
+                                  /* and 128 resume rows carry their descriptors in the launches' own parameters,  */
+                                  /* so that nothing is uploaded before the kernels (default 1); 0: always upload  */
   TIDE_TUNE_HOST_ZERO_COPY = 10,  /* tide_step_host: a step of up to 2 MiB whose host buffers are pinned and mapped   */
-                                  /* is not copied; the kernels read and write the host buffers themselves         */
+                                  /* bypasses the copy engines; kernels read and write the host buffers themselves */
                                   /* (default 1); 0: always copy                                                  */
   TIDE_TUNE_DROP_FIRST_STAGE = 6  /* test hook, non-zero arms it for the NEXT attention call only: in work item 0   */
                                   /* of each attention kernel of that call the K/V producer leaves out (its part   */

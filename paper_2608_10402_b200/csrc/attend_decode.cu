@@ -12,13 +12,14 @@
 // blocks with ldmatrix (the G query heads are the M rows); a scheduler warp takes over the index of a block of this
 // launch that has not started (clusterlaunchcontrol.try_cancel) shortly before the producer runs out of stages, looks
 // up the item and publishes it.  So the ring stays full across items: while the consumers merge their four partials of
-// one item, the next item's pages are already on their way.  With one block per item every item began with an empty ring
-// and 3 to 5 us of set-up (segment search, page ids, first stage) and ended with 2 us in which it read nothing: decode
-// step of 64 rows (0.82 GB of KV) 137.8 us, now 134.8 (6.66 TB/s between the first and the last time stamp of the kernel);
-// eight layers of 48 shorter rows 594 us, now 584.
-// Work items: about three per SM (TIDE_TUNE_ITEMS_PER_SM).  More, shorter items even out the end of the launch but pay
-// more partials and merges (4 / 6 / 8 per SM: 139 / 142 / 141 us on the 64 rows, 606 / 632 / 654 on the layers); so did
-// rows cut into a few large items first in the launch and small ones behind them (136 to 142 us).
+// one item, the next item's pages are already on their way.  With one block per item every item begins with an empty ring
+// and 3 to 5 us of set-up (segment search, page ids, first stage) and ends with 2 us in which it reads nothing: with three
+// items per SM a decode step of 64 rows (0.82 GB of KV) took 137.8 us that way and 134.8 with persistent blocks (6.66 TB/s
+// between the first and the last time stamp of the kernel), eight layers of 48 shorter rows 594 and 584.
+// Work items: one or two rounds of the resident blocks (build_plan in tide_host.cu, with the figures), or what
+// TIDE_TUNE_ITEMS_PER_SM says.  More, shorter items even out the end of the launch but pay more partials and merges (3 / 4 /
+// 6 / 8 per SM: 135 / 139 / 142 / 141 us on the 64 rows, 584 / 606 / 632 / 654 on the layers); so did rows cut into a few
+// large items first in the launch and small ones behind them (136 to 142 us).
 #include <cfloat>
 #include <climits>
 
@@ -69,9 +70,11 @@ __device__ __forceinline__ int count_in(int* ctr, int n_splits) {
 
 // D / 16 columns, from d0 on, of the item's rows row0, row0 + 8, ...: the splits are added in split order, so the result
 // does not depend on which one came last.  Bound by the latency of its loads: the partials of kMergeBatch splits and their
-// LSEs are fetched side by side, in ONE pass with a running maximum.  (All LSEs first and the rows behind them: a lone row
-// of 4k keys 12.1 us, now 10.8; of 16k keys 24.0, now 20.5; eight layers of eight 1k rows 99.4, now 95.8.  12 splits at a
-// time 11.5, 21.5; 16 spill.)
+// LSEs are fetched side by side, in ONE pass with a running maximum.  (A step of a lone row
+// of 4k keys 10.8 us, of 16k keys 20.5, eight layers of eight 1k rows 95.8; all LSEs first and the rows behind them 12.1, 24.0
+// and 99.4; 12 splits at a time 11.5, 21.5; 16 spill.)  A piece without a visible key has the weight 0 and holds zeros, and
+// absent pieces of the last batch are not loaded: 0 times an infinite value would be NaN.  (As a branch on the LSE beside
+// every piece's sum the same costs the lone row 0.4 us.)
 template <int D>
 __device__ __forceinline__ void merge_splits(const AttendParams& P, const Item& w, int row0, int d0) {
   constexpr int CW = D / 16;

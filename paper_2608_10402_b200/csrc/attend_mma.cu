@@ -343,9 +343,9 @@ cudaError_t launch_attend_tile(const AttendParams& p, cudaStream_t s) {
 // Bound by latency (a chain of dependent loads if written naively), so the partial LSEs are fetched side by side, one per
 // lane, the partial outputs four splits at a time, the first four beside the LSEs, and the row's segment is looked up
 // before the wait; the order in which the terms are added is still the order of the splits.
-// (All LSEs of up to 256 contributions in eight registers a lane, picked by index, and the outputs behind them: one row of
-// 17 to 35 tokens behind 1500 / 16000 keys 18.0 / 33.2 us with its append, now 16.0 / 27.0; 16 rows, two of them resumed,
-// 44.8, now 41.8; eight splits at a time spill, 15.7 / 26.5 / 42.8.)
+// (One row of 17 to 35 tokens behind 1500 / 16000 keys with its append 16.0 / 27.0 us, 16 rows, two of them resumed, 41.8;
+// with all LSEs of up to 256 contributions in eight registers a lane, picked by index, and the outputs behind them 18.0 /
+// 33.2 and 44.8; eight splits at a time spill, 15.7 / 26.5 and 42.8.)
 __device__ __forceinline__ void merge_body(const MergeParams& P, const Segment* __restrict__ segs) {
   // the descriptors were complete before the attention kernels started: the look-up needs no wait
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -288,7 +288,7 @@ __device__ __forceinline__ void attend_umma128_body(const AttendParams& P, const
   // register budget: the data-movement warpgroup gives registers to the two softmax warpgroups.  setmaxnreg
   // moves registers inside the CTA's own launch allocation (384 x 168), so the new counts must not add up to
   // more than that: 256 x 208 + 128 x 88 = 384 x 168.  (An over-subscribed .inc waits for ever.)  With 224 + 56 the MMA and
-  // scheduler warps spilled inside their loops: prompts 728 us, now 708; mixed text batch 7165, now 7076.
+  // scheduler warps spill inside their loops: prompts 728 us against 708, mixed text batch 7165 against 7076.
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
     if (warp == 8 || warp == 10) {

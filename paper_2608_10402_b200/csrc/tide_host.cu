@@ -1142,10 +1142,6 @@ static void find_share_groups(const tide_kv* kv, int32_t n_rows, const tide_row_
 // Head sizes the selected tcgen05 kernel is built for: 64-key tiles only 128, 128-key tiles both.
 static bool umma_takes(const tide_kv* kv) { return kv->g.D == 128 || kv->umma_tile_keys == 128; }
 
-// The work plan of one batch: one segment per row, decode-style (<= 16 packed rows), warp-MMA tile-style or
-// tcgen05-style; long contexts are split along the keys so that the grid has about items_per_sm items per SM.
-// A group of rows that share their first pages gets one more segment for the shared range (its tokens are the
-// members' queries, all seeing the same keys); the members' own segments start behind it and their merge takes both.
 // Into pieces of how many keys the resume rows of a batch are cut when their items (256 packed rows on an SM each) are few:
 // the candidate with the least estimated time, in us.  An item takes 4 + 0.0129 a key (0.0085 with one row tile; 64-wide heads
 // a tenth less); up to one item per SM the longest one counts and the decode rows beside it stream at full rate while some
@@ -1198,6 +1194,11 @@ static long long resume_chunk(const tide_kv* kv, int32_t n_rows, const tide_row_
   return best_keys;
 }
 
+// The work plan of one batch: one segment per row, decode-style (<= 16 packed rows), warp-MMA tile-style or
+// tcgen05-style; long contexts are split along the keys, decode rows to fill rounds of resident blocks, few resume rows by
+// an estimate of their time.
+// A group of rows that share their first pages gets one more segment for the shared range (its tokens are the
+// members' queries, all seeing the same keys); the members' own segments start behind it and their merge takes both.
 // The plan depends on the rows and the page tables only, so every layer of a step can use it.  `step`: the kernel in front
 // of the attention kernels is the append of exactly these rows (tide_step_layer); otherwise they go to stream `st`.
 static int build_plan(tide_kv* kv, int32_t n_rows, const tide_row_t* rows, bool umma_ok, bool allow_groups, bool step, cudaStream_t st,

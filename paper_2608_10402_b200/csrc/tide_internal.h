@@ -26,7 +26,8 @@ constexpr int kDecodeTileRows = 16;  // packed (query, head) rows per decode-sty
 constexpr int kMmaTileRows = 64;     // packed rows per work item of the warp-MMA tile path
 constexpr int kUmmaTileRows = 128;   // packed rows per work item of the tcgen05 path
 constexpr long long kWaitLimitNsDefault = 2000000000LL;  // bound of every in-kernel wait unless the handle says otherwise
-constexpr int kTargetItemsPerSm = 3;   // measured: fewer, longer items beat finer balance (per-item set-up dominates)
+constexpr int kTargetItemsPerSm = 3;   // work items per SM where no rule of the planner says otherwise: batches with groups (two thirds of it), tile
+                                       // rows, fixed launch shapes.  More even out the end but cost partials and merges (attend_decode.cu)
 
 struct Geom {
   int Hq, Hkv, D, S, G;
@@ -225,16 +226,18 @@ int sm_count();   // multiprocessors of the current device (looked up once per d
 // it still runs, once every block of that one has called grid_dep_launch (or left), and calls grid_dep_wait before it
 // touches anything that earlier work of the stream reads or writes.  A kernel boundary without it costs 1 to 2.5 us of
 // launch latency, and the blocks' set-up on top.
-// Measured (with the descriptors in the launches): four-task step 34.4 to 21.7 us, forked groups 103 to 90 us, eight layers
-// of decode rows 584 to 569 us, a prune-and-resume turn 1294 to 1215 us; nothing at 64 decode rows and above.
+// Worth, with the descriptors in the launches: four-task step 21.7 us against 34.4, forked groups 90 against 103, eight layers
+// of decode rows 569 against 584, a prune-and-resume turn 1215 against 1294; nothing at 64 decode rows and above.
 // The rule that keeps the chain of dependencies whole: every kernel calls grid_dep_wait before it ends, and calls
 // grid_dep_launch only after everything that the NEXT kernel may rely on without waiting is complete.  The two attention
 // kernels of one batch do not depend on each other: the second one (AttendParams::overlapped) starts without waiting -
 // the first has waited for all earlier work before it let the second one start - and waits when it is done, so that what
 // follows it in the stream still follows both.  Nor do the keys that a decode row saw in the step before depend on the
 // append in front of the attention kernels, which waits for everything earlier: the producers of the first of them stream
-// those pages (AttendParams::run_ahead, Segment::live_from) while the append runs.  The same goes for the moves of several
-// tasks that are pruned in a row.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
+// those pages (AttendParams::run_ahead, Segment::live_from) while the append runs; whatever writes keys or page-table
+// entries - append, move, fork, extend - has marked them live (LiveKeys in tide_host.cu).  Nor do the moves of several tasks
+// that are pruned in a row depend on each other.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
+// A wait limit does not count the time that the work in front still takes (mbar_wait).
 template <typename... A>
 cudaError_t launch_dep(void (*kernel)(A...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, const std::common_type_t<A>&... args) {
   cudaLaunchConfig_t cfg = {};
