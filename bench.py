@@ -31,8 +31,8 @@ METRIC = "mixed resume batch: KV-read GB/s vs HBM peak; append-prefill TFLOP/s v
 # DRAM traffic per unit of algorithmic work, from the ncu captures summarised under profiles/ (reduced cases,
 # scaled by the units one launch processes): decode kernel dram bytes / algorithmic KV bytes; tcgen05 kernel
 # dram bytes / algorithmic bytes of its launch (K and V of every resume row once + Q + O).
-NCU_DECODE_TRAFFIC_RATIO = 1.012
-NCU_UMMA_TRAFFIC_RATIO = 1155.1e6 / 1153.2e6     # one-pass capture of the full-size mixed batch
+NCU_DECODE_TRAFFIC_RATIO = 1.013
+NCU_UMMA_TRAFFIC_RATIO = 1150.8e6 / 1153.2e6     # one-pass capture of the full-size mixed batch
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
