@@ -220,62 +220,76 @@ cudaError_t launch_copy_pages(uint8_t* pool, const int32_t* src, const int32_t* 
 // to 16k tokens took 390 us, mostly launches; this way they take about 100.)  The moves of different tasks do not depend on
 // each other: one that directly follows another (`overlapped`) runs beside it.
 //
-// Large shifts: position d depends only on d + shift, so the positions of one residue modulo the shift form a chain that
-// one thread walks front to back, always reading ahead of what it writes; chains are independent of one another.
+// Position d depends only on d + shift, so the positions of one residue modulo the shift form a chain, and chains are
+// independent of one another.  A chain is cut into segments of a few links, all of them in one block, a thread moving 16
+// bytes of each link of its segment front to back, always reading ahead of what it writes.  Only the source of a segment's
+// last link is written by another thread (it is the first target of the next segment): every thread loads that one, and
+// its first kMoveLinks links, ahead of the block's barrier and stores nothing before it.
 constexpr int kMoveLinks = 4;
-constexpr int kMoveChainsFrom = 64;   // shift from which chains are faster than runs (4 KV heads, D = 128, tail of 4000 / 16000 tokens: shift 32
-                                      // 43 / 156 us by chains and 29 / 90 by runs, 64 27 / 80 and 33 / 90, 128 16 / 45 and 33 / 90, 512 12 / 20 and 33 / 94)
+// Bound by latency - two dependent loads, page number and data, for every kMoveLinks links of a thread - until the blocks fill
+// the chip, where it is memory; so a chain is cut no further than that.  us, a thread per chain or, for shifts below 64, runs / this
+// (4 KV heads, D = 128, tail of 1500 / 4000 / 16000 tokens): shift 8 18.4 28.7 90.1 / 8.2 11.2 24.6, shift 64 14.3 24.6 81.9 / 8.2 12.3
+// 22.5, shift 128 10.2 16.4 43.0 / 8.2 12.3 22.6, shift 512 8.2 10.2 20.5 / 8.2 10.2 18.4; eleven tails of 3500 tokens by 107 in a
+// row, with their append and attention, 109 / 59.
+constexpr int kMovePairsLog2 = 5, kMoveChainThreads = 8 << kMovePairsLog2;   // 32 (segment, chain) pairs of eight lanes, 128 bytes of a row
 template <int SLABS>
-__global__ void __launch_bounds__(256) move_chains_kernel(uint8_t* pool0, size_t layer_stride, const int32_t* __restrict__ table_row, int to,
-                                                          int shift, int n, int overlapped, const Geom g) {
-  constexpr int CPR = SLABS * 8;                              // 16-byte chunks of a row: that many neighbouring lanes move one
+__global__ void __launch_bounds__(kMoveChainThreads, 3) move_chains_kernel(uint8_t* pool0, size_t layer_stride, const int32_t* __restrict__ table_row, int to,
+                                                                           int shift, int n, int segs_log2, int seg_links, int overlapped,
+                                                                           const Geom g) {
   if (!overlapped) grid_dep_wait();
   grid_dep_launch();
   uint8_t* const pool = pool0 + (size_t)blockIdx.y * layer_stride;
-  const int chains = min(shift, n);
-  // rows of one (kv, head) whose chains start at neighbouring positions go to neighbouring lanes: whole lines of an atom
-  const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / CPR;
-  const int c = threadIdx.x % CPR;
-  const int hh = (int)(row / chains), first = (int)(row - (long long)hh * chains);
-  const int kv = hh >= g.Hkv ? 1 : 0;
+  // neighbouring chains, whose rows are neighbours in the pages' atoms, go to neighbouring lanes
+  const int chains = min(shift, n), chains_log2 = kMovePairsLog2 - segs_log2;
+  const int groups = (chains + (1 << chains_log2) - 1) >> chains_log2;
+  const int group = blockIdx.x % groups, slab = blockIdx.x / groups % SLABS, hh = blockIdx.x / groups / SLABS, kv = hh >= g.Hkv ? 1 : 0;
   const long long head = (long long)(hh - kv * g.Hkv) * g.head_bytes;
-  auto at = [&](long long pos) -> uint4* {
-    const int lp = (int)pos / g.S;
-    return reinterpret_cast<uint4*>(pool + (long long)__ldcg(table_row + lp) * g.page_bytes + head + blk_offset(g, (int)pos - lp * g.S, kv, c));
+  const int c = slab * 8 + (threadIdx.x & 7), pair = threadIdx.x >> 3;
+  const int chain = (group << chains_log2) + (pair & ((1 << chains_log2) - 1)), seg = pair >> chains_log2;
+  const int links = chain < chains ? (n - chain - 1) / shift + 1 : 0;
+  const int first = min(seg * seg_links, links), end = min(first + seg_links, links), last = end - 1;   // this segment's links
+  auto at = [&](int link) -> uint4* {                        // a link's target: the source of the link before it
+    const int pos = to + chain + link * shift, lp = pos / g.S;
+    return reinterpret_cast<uint4*>(pool + (long long)__ldcg(table_row + lp) * g.page_bytes + head + blk_offset(g, pos - lp * g.S, kv, c));
   };
-  const long long end = hh < 2 * g.Hkv ? (long long)to + n : 0;
-  // kMoveLinks links from position d on: the address of the first target is known, a[i + 1] is link i's source and the
-  // target of link i + 1.  The next links are loaded before these are stored.
   uint4 *a0[kMoveLinks + 1], *a1[kMoveLinks + 1];
   uint4 v0[kMoveLinks], v1[kMoveLinks];
-  auto load = [&](long long d, uint4* target, uint4* (&a)[kMoveLinks + 1], uint4 (&v)[kMoveLinks]) {
+  // links i, i + 1, ... of those in front of the last one; a[k + 1] is link i + k's source and the target of link i + k + 1
+  auto load = [&](int i, uint4* target, uint4* (&a)[kMoveLinks + 1], uint4 (&v)[kMoveLinks]) {
     a[0] = target;
 #pragma unroll
-    for (int i = 0; i < kMoveLinks; ++i) a[i + 1] = d + (long long)i * shift < end ? at(d + (i + 1ll) * shift) : target;
+    for (int k = 0; k < kMoveLinks; ++k) a[k + 1] = i + k < last ? at(i + k + 1) : target;
 #pragma unroll
-    for (int i = 0; i < kMoveLinks; ++i) v[i] = __ldcg(a[i + 1]);
+    for (int k = 0; k < kMoveLinks; ++k) v[k] = __ldcg(a[k + 1]);
   };
-  auto store = [&](long long d, uint4* const (&a)[kMoveLinks + 1], const uint4 (&v)[kMoveLinks]) {
+  auto store = [&](int i, uint4* const (&a)[kMoveLinks + 1], const uint4 (&v)[kMoveLinks]) {
 #pragma unroll
-    for (int i = 0; i < kMoveLinks; ++i)
-      if (d + (long long)i * shift < end) *a[i] = v[i];
+    for (int k = 0; k < kMoveLinks; ++k)
+      if (i + k < last) *a[k] = v[k];
   };
-  const long long step = (long long)kMoveLinks * shift;
-  long long d = to + first;
-  if (d < end) load(d, at(d), a0, v0);
-  while (d < end) {
-    if (d + step < end) load(d + step, a0[kMoveLinks], a1, v1);
-    store(d, a0, v0);
-    d += step;
-    if (d >= end) break;
-    if (d + step < end) load(d + step, a1[kMoveLinks], a0, v0);
-    store(d, a1, v1);
-    d += step;
+  uint4* last_target = nullptr;
+  uint4 last_value = make_uint4(0, 0, 0, 0);
+  int i = first;
+  if (first < end) {
+    last_target = at(last);
+    last_value = __ldcg(at(end));
+    if (i < last) load(i, at(i), a0, v0);
   }
+  __syncthreads();
+  while (i < last) {
+    if (i + kMoveLinks < last) load(i + kMoveLinks, a0[kMoveLinks], a1, v1);
+    store(i, a0, v0);
+    i += kMoveLinks;
+    if (i >= last) break;
+    if (i + kMoveLinks < last) load(i + kMoveLinks, a1[kMoveLinks], a0, v0);
+    store(i, a1, v1);
+    i += kMoveLinks;
+  }
+  if (first < end) *last_target = last_value;
   if (overlapped) grid_dep_wait();
 }
 
-// Small shifts have few chains.  One block per (layer, kv, head, 64-element slab) moves a run of rows at a time, front to
+// One block per (layer, kv, head, 64-element slab) moves a run of rows at a time, front to
 // back: the whole run is in registers before its first row is stored (the run's last sources lie behind its targets, so
 // no later run is touched), and the next run is loaded before this one is stored.
 constexpr int kMoveThreads = 512, kMoveRows = 8;              // 16-byte chunks per thread and run: 512 rows of 128 bytes
@@ -320,18 +334,30 @@ __global__ void __launch_bounds__(kMoveThreads) move_runs_kernel(uint8_t* pool0,
   if (overlapped) grid_dep_wait();
 }
 
+// Runs are left where a chain has more links than its threads share out well: a shift of one (tail of 1500 / 4000 / 16000 tokens 18.4 /
+// 28.7 / 88 us, by chains 20.5 / 43 / 147) and chains of thousands of links, which only tails of 100k tokens and more that move
+// by a few positions have (tests/test_gpu_timeout.py takes such a move for its long launch on few blocks).
+constexpr int kMoveMostLinks = 4096;
+
 cudaError_t launch_move(uint8_t* pool, size_t layer_stride, int layers, const int32_t* table_row, int to, int shift, int n, bool overlapped,
                         const Geom& g, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  if (shift >= kMoveChainsFrom) {
-    const long long threads = (long long)std::min(shift, n) * 2 * g.Hkv * (g.D / 8);
-    const dim3 grid((unsigned)((threads + 255) / 256), (unsigned)layers);
-    return launch_dep(g.D == 128 ? move_chains_kernel<2> : move_chains_kernel<1>, grid, 256, 0, s, pool, layer_stride, table_row, to, shift, n,
+  const int links = (n - 1) / shift + 1, slabs = g.D / 64;
+  if (shift == 1 || links > kMoveMostLinks) {
+    const dim3 grid((unsigned)(2 * g.Hkv * slabs), (unsigned)layers);
+    return launch_dep(g.D == 128 ? move_runs_kernel<2> : move_runs_kernel<1>, grid, kMoveThreads, 0, s, pool, layer_stride, table_row, to, shift, n,
                       overlapped ? 1 : 0, g);
   }
-  const dim3 grid((unsigned)(2 * g.Hkv * (g.D / 64)), (unsigned)layers);
-  return launch_dep(g.D == 128 ? move_runs_kernel<2> : move_runs_kernel<1>, grid, kMoveThreads, 0, s, pool, layer_stride, table_row, to, shift, n,
-                      overlapped ? 1 : 0, g);
+  const int chains = std::min(shift, n), fill = 3 * sm_count();        // the resident blocks
+  int segs_log2 = 0;
+  auto blocks = [&] {
+    const int per_block_log2 = kMovePairsLog2 - segs_log2;
+    return (long long)((chains + (1 << per_block_log2) - 1) >> per_block_log2) * 2 * g.Hkv * slabs;
+  };
+  while (segs_log2 < kMovePairsLog2 && (links - 1) >> segs_log2 > kMoveLinks && blocks() * layers < fill) ++segs_log2;
+  const dim3 grid((unsigned)blocks(), (unsigned)layers);
+  return launch_dep(g.D == 128 ? move_chains_kernel<2> : move_chains_kernel<1>, grid, kMoveChainThreads, 0, s, pool, layer_stride, table_row, to, shift,
+                    n, segs_log2, (links + (1 << segs_log2) - 1) >> segs_log2, overlapped ? 1 : 0, g);
 }
 
 // Logical content of one task -> contiguous [len, Hkv, D]; inverse of the scatter above.

@@ -66,3 +66,37 @@ def test_tails_move_in_place(geom, layers):
     orc.append(ids, ip, k, v)
     same()
     kv.close()
+
+
+@pytest.mark.parametrize("geom,layers", [((28, 4, 128, 16), 1), ((8, 2, 64, 32), 2)])
+def test_chains_cut_into_segments(geom, layers):
+    """Chains of as many links as a segment holds, one more and one less, of 32 segments' and of the most that are moved by
+    chains; fewer chains than a block holds, and a last block that is not full; tails that fill the chip with fewer segments."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    HQ, HKV, D, S = geom
+    rng = np.random.default_rng(7 * HQ + D)
+    shapes = [(3, 40, 40 * 5), (3, 40, 40 * 5 + 1), (0, 7, 7 * 6 - 1), (1, 2, 2 * 160), (1, 2, 2 * 160 + 1), (15, 33, 33 * 32 + 5), (2, 2, 8192), (2, 2, 8193),
+              (5, 600, 4000), (0, 31, 1), (9, 1000, 6000), (100, 65, 64 * 65)]
+    length = [sum(x) for x in shapes]
+    n, pages = len(shapes), sum((l + S - 1) // S for l in length) + 4
+    order = rng.permutation(pages).astype(np.int32)
+    kv = tide.TideKV(HQ, HKV, D, S, pages, n, pages, n, 256, free_order=order, num_layers=layers)
+    orc = LayeredKVOracle(layers, num_pages=pages, page_size=S, num_kv_heads=HKV, head_dim=D, max_tasks=n, max_pages_per_task=pages, free_order=order)
+    ids, ip = list(range(n)), np.concatenate([[0], np.cumsum(length)]).astype(np.int32)
+    k, v = (inputs.normal_bf16(rng, (layers, int(ip[-1]), HKV, D)) for _ in range(2))
+    for o in (kv, orc):
+        for t in ids:
+            o.alloc(t)
+    kv.extend(ids, ip)
+    for l in range(layers):
+        kv.write(l, ids, ip, H.to_dev(k[l], torch), H.to_dev(v[l], torch))
+    orc.append(ids, ip, k, v)
+    for t, (keep, shift, _) in enumerate(shapes):
+        kv.prune(t, keep, keep + shift)
+        orc.prune(t, keep, keep + shift)
+    for t in ids:
+        for l in range(layers):
+            (gk, gv), (ok, ov) = kv.read(t, layer=l), orc.read(l, t)
+            assert np.array_equal(H.from_dev(gk), ok) and np.array_equal(H.from_dev(gv), ov), (shapes[t], l)
+    kv.close()
