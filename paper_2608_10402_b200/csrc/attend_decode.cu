@@ -53,6 +53,7 @@ struct __align__(16) Item {
   int x_n_splits, x_part_row0, x_stride;   // ... with those of the shared range in front of them
   int mode;                  // 0: one split, results go to out / lse; 1: partials; 2: partials, the last split merges
   int live_from;             // first key that the kernel before this one may still be writing
+  int add_from, add_to, add_tok;   // AttendParams::new_k: the keys of this piece that this launch writes, the token of position 0 in new_k
   int drop;                  // test hook: the first stage never arrives
   int merge;                 // the item two before this one finished its row: its splits are to be merged
 };
@@ -139,7 +140,26 @@ __device__ __forceinline__ void merge_splits(const AttendParams& P, const Item& 
   }
 }
 
-template <int D, bool INLINE>
+// The step's new rows of positions [from, to) of an item's KV head go to their pages (AttendParams::new_k): a warp writes
+// the K and the V row of one (D = 128) or two (D = 64) tokens at a time, in the pages' swizzled layout.  The bulk copies that
+// read them next belong to another proxy, hence the fence.
+template <int D>
+__device__ __forceinline__ void put_new_rows(const AttendParams& P, int table_off, int kvh, int add_tok, int from, int to) {
+  constexpr int CPR = D / 8, TOKENS = 16 / CPR;              // 16-byte chunks of a row, tokens at a time
+  const Geom& g = P.g;
+  const int lane = threadIdx.x & 31, kv = lane / CPR & 1, c = lane % CPR;
+  for (int pos = from + lane / (2 * CPR); pos < to; pos += TOKENS) {
+    const int lp = pos / g.S;
+    const long long page = __ldcg(P.table + table_off + lp);
+    const uint4 v = __ldcg(reinterpret_cast<const uint4*>((kv ? P.new_v : P.new_k) + ((long long)(add_tok + pos) * g.Hkv + kvh) * D) + c);
+    *reinterpret_cast<uint4*>(P.pool_rw + page * g.page_bytes + (long long)kvh * g.head_bytes + blk_offset(g, pos - lp * g.S, kv, c)) = v;
+  }
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+  __syncwarp();
+}
+
+// WRITES: a layer of a step whose new rows this launch writes itself (AttendParams::new_k).
+template <int D, bool INLINE, bool WRITES>
 __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const Segment* __restrict__ segs) {
   using C = Cfg<D>;
   constexpr int KS = D / 16;                 // k-steps of Q.K^T
@@ -199,16 +219,18 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     const int pages_per_stage = kStageKeys / g.S, stages_per_group = 32 / pages_per_stage;
     int slot = 0, use = 0, issued = 0;
     bool ok = true, ahead = early;
-    for (int it = 0; ok; ++it) {
+    for (int it = 0; ok || WRITES; ++it) {                    // (after a wait gave up: only the new rows of the items handed out)
       if (!wait_all(s_item_full[it % kItemSlots], (it / kItemSlots) & 1)) break;
       const Item& w = items[it % kItemSlots];
       if (!w.run) break;
       const int kv_begin = w.kv_begin, kv_end = w.kv_end, drop = w.drop, live_from = w.live_from;
-      const int32_t* trow = P.table + w.table_off;
-      const uint8_t* head_base = P.pool + (long long)w.kvh * g.head_bytes;
+      const int kvh = w.kvh, table_off = w.table_off;
+      const int add_from = WRITES ? w.add_from : 0, add_to = WRITES ? w.add_to : 0, add_tok = WRITES ? w.add_tok : 0;
+      const int32_t* trow = P.table + table_off;
+      const uint8_t* head_base = P.pool + (long long)kvh * g.head_bytes;
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&s_item_empty[it % kItemSlots]));
-      const int n_st = (kv_end - kv_begin + kStageKeys - 1) / kStageKeys;
+      const int n_st = !WRITES || ok ? (kv_end - kv_begin + kStageKeys - 1) / kStageKeys : 0;
       // page ids are fetched 32 at a time, one per lane, a whole group ahead of their use
       const int lp0 = kv_begin / g.S, lp_last = (kv_end - 1) / g.S;
       auto load_ids = [&](int grp) -> int {
@@ -217,30 +239,43 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
       };
       int ids_cur = load_ids(0), ids_nxt = load_ids(1), cur_grp = 0;
       const int ask_at = max(0, n_st - 2);
-      for (int st = 0; st < n_st; ++st) {
-        const int grp = st / stages_per_group;
-        if (grp != cur_grp) { ids_cur = ids_nxt; ids_nxt = load_ids(grp + 1); cur_grp = grp; }
-        if (st == ask_at && lane == 0) mbar_arrive(smem_u32(&s_near_end));
-        // a wait that gave up means the ring can no longer be trusted: issue nothing more
-        if (use > 0 && !wait_all(s_empty[slot], (use - 1) & 1)) { ok = false; break; }
-        ++issued;
-        const int key0 = kv_begin + st * kStageKeys;
-        const int npages = min(pages_per_stage, (kv_end - key0 + g.S - 1) / g.S);
-        if (ahead && key0 + npages * g.S > live_from) {
-          // from here on pages, and page numbers, may belong to the kernel before this one
-          grid_dep_wait();
-          ahead = false;
-          ids_cur = load_ids(cur_grp);
-          ids_nxt = load_ids(cur_grp + 1);
+      // the stages in front of the step's own rows, then those that hold some of them (a check in every stage costs large
+      // batches of 64-wide heads 4 to 6 %)
+      const int n_plain = WRITES && add_from < add_to ? min(n_st, (add_from - kv_begin) / kStageKeys) : n_st;
+      int st = 0;
+#pragma unroll
+      for (int part = 0; part < (WRITES ? 2 : 1); ++part) {
+        if (part == 1 && !ok) break;
+        for (const int stop = part == 0 ? n_plain : n_st; st < stop; ++st) {
+          const int grp = st / stages_per_group;
+          if (grp != cur_grp) { ids_cur = ids_nxt; ids_nxt = load_ids(grp + 1); cur_grp = grp; }
+          if (st == ask_at && lane == 0) mbar_arrive(smem_u32(&s_near_end));
+          // a wait that gave up means the ring can no longer be trusted: issue nothing more
+          if (use > 0 && !wait_all(s_empty[slot], (use - 1) & 1)) { ok = false; break; }
+          ++issued;
+          const int key0 = kv_begin + st * kStageKeys;
+          const int npages = min(pages_per_stage, (kv_end - key0 + g.S - 1) / g.S);
+          if (ahead && key0 + npages * g.S > live_from) {
+            // from here on pages, and page numbers, may belong to the kernel before this one
+            grid_dep_wait();
+            ahead = false;
+            ids_cur = load_ids(cur_grp);
+            ids_nxt = load_ids(cur_grp + 1);
+          }
+          if (part == 1) put_new_rows<D>(P, table_off, kvh, add_tok, max(key0, add_from), min(key0 + kStageKeys, add_to));
+          const uint32_t bar = smem_u32(&s_full[slot]);
+          const long long page = __shfl_sync(0xffffffffu, ids_cur, ((st % stages_per_group) * pages_per_stage + lane) & 31);
+          if (!(drop != 0 && st == 0)) {                       // test hook: this stage never arrives
+            if (lane == 0) mbar_expect_tx(bar, (uint32_t)(npages * g.head_bytes));
+            __syncwarp();
+            if (lane < npages) bulk_g2s(ring + slot * C::kStageBytes + lane * g.head_bytes, head_base + page * g.page_bytes, (uint32_t)g.head_bytes, bar);
+          }
+          if (++slot == NS) { slot = 0; ++use; }
         }
-        const uint32_t bar = smem_u32(&s_full[slot]);
-        const long long page = __shfl_sync(0xffffffffu, ids_cur, ((st % stages_per_group) * pages_per_stage + lane) & 31);
-        if (!(drop != 0 && st == 0)) {                       // test hook: this stage never arrives
-          if (lane == 0) mbar_expect_tx(bar, (uint32_t)(npages * g.head_bytes));
-          __syncwarp();
-          if (lane < npages) bulk_g2s(ring + slot * C::kStageBytes + lane * g.head_bytes, head_base + page * g.page_bytes, (uint32_t)g.head_bytes, bar);
-        }
-        if (++slot == NS) { slot = 0; ++use; }
+      }
+      if (WRITES && !ok && add_from < add_to) {
+        if (ahead) { grid_dep_wait(); ahead = false; }
+        put_new_rows<D>(P, table_off, kvh, add_tok, add_from, add_to);
       }
       if (n_st == 0 && lane == 0) mbar_arrive(smem_u32(&s_near_end));
     }
@@ -259,19 +294,10 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     // ================= scheduler warp: hands out the items =================
     const int n_segs = P.dyn ? __ldcg(P.dyn + 1) : P.n_segs;
     int item = (int)blockIdx.x, asks = 0, done = 0;
+    int handed_out[kItemSlots] = {-1, -1, -1};               // the items in the slots
     int merge = 0;                                           // lane 0: the last item but one completed its row
     bool fused_before = false, open = false;                 // a question without an answer yet
-    for (int it = 0; ; ++it) {
-      const int slot = it % kItemSlots;
-      if (it >= kItemSlots && !wait_all(s_item_empty[slot], (it / kItemSlots - 1) & 1)) break;
-      Item& w = items[slot];
-      // The status word is set when a bounded wait runs out and stays set until tide_status clears it.  While it is set
-      // no item is started, so outputs are undefined from the time-out until the caller has read the status.
-      if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(P.status), 0) != 0) item = -1;
-      if (item < 0) {
-        if (lane == 0) { w.run = 0; w.merge = merge; mbar_arrive(smem_u32(&s_item_full[slot])); }
-        break;
-      }
+    auto segment_of = [&](int item) -> Segment {
       int si;
       if (INLINE) si = find_segment(n_segs, item, [&](int i) { return segs[i].item_base; });
       else {
@@ -290,7 +316,50 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
           if (si + 1 < i0 + 128) break;
         }
       }
-      const Segment seg = INLINE ? segs[si] : load_segment(segs + si);
+      return INLINE ? segs[si] : load_segment(segs + si);
+    };
+    // A launch that writes the step's rows itself writes them also where its waits run out or the status word keeps items
+    // from being started: the cache holds them whatever becomes of the results.
+    auto put_only = [&](int item) {
+      const Segment seg = segment_of(item);
+      const int local = item - seg.item_base, begin = seg.origin + local % seg.n_splits * seg.chunk;
+      put_new_rows<D>(P, seg.table_off, local / seg.n_splits, seg.q_off - seg.p, max(begin, seg.p), min(begin + seg.chunk, seg.p + seg.n));
+    };
+    auto ask = [&] {
+      if (lane == 0) next_block_ask(smem_u32(&s_next), smem_u32(&s_answer));
+      ++asks;
+      open = true;
+    };
+    auto answer = [&]() -> bool {
+      if (!wait_all(s_answer, (asks - 1) & 1)) return false;
+      open = false;
+      item = next_block_answer(smem_u32(&s_next));
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the answer has been read before the next one may land
+      __syncwarp();
+      if (item >= n_items) item = -1;                        // fixed grid: indices beyond the batch
+      return true;
+    };
+    for (int it = 0; ; ++it) {
+      const int slot = it % kItemSlots;
+      if (it >= kItemSlots && !wait_all(s_item_empty[slot], (it / kItemSlots - 1) & 1)) break;
+      Item& w = items[slot];
+      // The status word is set when a bounded wait runs out and stays set until tide_status clears it.  While it is set
+      // no item is started, so outputs are undefined from the time-out until the caller has read the status.
+      if (__shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(P.status), 0) != 0) {
+        if (WRITES && item >= 0) {
+          grid_dep_wait();
+          do {
+            put_only(item);
+            ask();
+          } while (answer() && item >= 0);
+        }
+        item = -1;
+      }
+      if (item < 0) {
+        if (lane == 0) { w.run = 0; w.merge = merge; mbar_arrive(smem_u32(&s_item_full[slot])); }
+        break;
+      }
+      const Segment seg = segment_of(item);
       if (lane == 0) {
         const int local = item - seg.item_base;
         const int split = local % seg.n_splits, kvh = local / seg.n_splits;
@@ -307,8 +376,10 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
         w.x_n_splits = seg.x_n_splits; w.x_part_row0 = seg.x_part_base + kvh * g.G; w.x_stride = seg.x_stride;
         w.mode = seg.partial == 2 ? 2 : (seg.n_splits == 1 && seg.partial == 0) ? 0 : 1;
         w.drop = P.debug_drop_first_stage != 0 && item == 0;
+        if (WRITES) { w.add_from = min(w.kv_end, max(w.kv_begin, seg.p)); w.add_to = w.kv_end; w.add_tok = seg.q_off - seg.p; }
         mbar_arrive(smem_u32(&s_item_full[slot]));
       }
+      handed_out[2] = handed_out[1]; handed_out[1] = handed_out[0]; handed_out[0] = item;
       // The split of the item before this one is counted in on the consumers' behalf, who have gone on to this one; the
       // verdict travels with the next item.
       merge = 0;
@@ -321,19 +392,22 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
       fused_before = seg.partial == 2;
       // the next item is claimed two stages before the producer runs out of this one
       if (!wait_all(s_near_end, it & 1)) break;
-      if (lane == 0) next_block_ask(smem_u32(&s_next), smem_u32(&s_answer));
-      ++asks;
-      open = true;
-      if (!wait_all(s_answer, (asks - 1) & 1)) break;
-      open = false;
-      item = next_block_answer(smem_u32(&s_next));
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the answer has been read before the next one may land
-      __syncwarp();
-      if (item >= n_items) item = -1;                        // fixed grid: indices beyond the batch
+      // (Beside a whole layer, not just an append, blocks that have started early would take items from those that start later:
+      // 32 rows of 1k keys, two KV heads, 16.7 us a layer, and 14.2 with an append in between.)
+      if (WRITES && early && it == 0) grid_dep_wait();
+      ask();
+      if (!answer()) break;
     }
     if (open) {                                              // only after a wait gave up: the answer lands before the block leaves
       const long long t0 = global_ns();
       while (!mbar_try(smem_u32(&s_answer), (asks - 1) & 1) && global_ns() - t0 < P.wait_limit_ns) {}
+      item = next_block_answer(smem_u32(&s_next));
+    }
+    if (WRITES && *abort_flag) {                             // what the producer may not have come to
+      grid_dep_wait();
+      for (int i = 0; i < kItemSlots; ++i)
+        if (handed_out[i] >= 0) put_only(handed_out[i]);
+      if (item >= 0) put_only(item);
     }
     return;
   }
@@ -580,18 +654,24 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 2) attend_decode_kernel(const AttendParams P) {
-  attend_decode_body<D, false>(P, P.segs);
+  attend_decode_body<D, false, false>(P, P.segs);
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 2) attend_decode_writes_kernel(const AttendParams P) {
+  attend_decode_body<D, false, true>(P, P.segs);
 }
 
 // Decode-style items whose row descriptors travel in the kernel's parameters (small batches).
 template <int D>
 __global__ void __launch_bounds__(kThreads, 2) attend_decode_inline_kernel(const __grid_constant__ AttendInline PI) {
-  attend_decode_body<D, true>(PI.p, PI.segs);
+  attend_decode_body<D, true, false>(PI.p, PI.segs);
 }
 
 template <int D>
 static cudaError_t init_one() {
   cudaError_t e = cudaFuncSetAttribute(attend_decode_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(attend_decode_writes_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(attend_decode_inline_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::kSmemBytes);
 }
@@ -613,8 +693,10 @@ cudaError_t launch_attend_decode_inline(const AttendInline& pi, cudaStream_t s) 
 cudaError_t launch_attend_decode(const AttendParams& p, cudaStream_t s) {
   const int grid = p.dyn ? p.grid_cap : p.n_items;
   if (grid <= 0) return cudaSuccess;
-  if (p.g.D == 128) return launch_dep(decode::attend_decode_kernel<128>, grid, decode::kThreads, decode::Cfg<128>::kSmemBytes, s, p);
-  return launch_dep(decode::attend_decode_kernel<64>, grid, decode::kThreads, decode::Cfg<64>::kSmemBytes, s, p);
+  if (p.g.D == 128)
+    return launch_dep(p.new_k ? decode::attend_decode_writes_kernel<128> : decode::attend_decode_kernel<128>, grid, decode::kThreads,
+                      decode::Cfg<128>::kSmemBytes, s, p);
+  return launch_dep(p.new_k ? decode::attend_decode_writes_kernel<64> : decode::attend_decode_kernel<64>, grid, decode::kThreads, decode::Cfg<64>::kSmemBytes, s, p);
 }
 
 }  // namespace tide

@@ -130,6 +130,7 @@ class LiveKeys {
     }
     w_[cur_].seq = ++seq_;
   }
+  int64_t seq() const { return seq_; }   // of the most recent writer of any stream
   // ... and writes `task` from position `from` on.
   void mark(int task, int from) {
     Writer& w = w_[cur_];
@@ -232,6 +233,8 @@ struct tide_kv {
   uint8_t* h_step = nullptr;   // staging of the step area
   cudaEvent_t ev_step = nullptr;
   bool step_upload_pending = false, step_valid = false;
+  int64_t step_seq = 0;        // the last writer when the step began
+  bool step_fused = false;     // the decode launches of the step write its rows themselves (AttendParams::new_k)
   PlanDev step_plan;
   int step_recs = 0, step_tokens = 0, step_layers = 0;   // step_layers: calls of tide_step_layer since tide_step_begin
   cudaStream_t step_stream = nullptr;
@@ -1428,7 +1431,8 @@ static PlanDev pack_plan(const PlanHost& P, Segment* h, const Segment* d, size_t
 // time stamps), so a caller may capture them in a CUDA graph.  With `inl` the row descriptors come from that plan and
 // travel in the launches' parameters; otherwise they are on the device, where `d` says.
 static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanHost* inl, bool step, const int32_t* page_table, const void* q,
-                       float scale, void* out, float* lse, cudaStream_t st, bool events, int64_t* n_launches, const int32_t* dyn) {
+                       float scale, void* out, float* lse, cudaStream_t st, bool events, int64_t* n_launches, const int32_t* dyn,
+                       const void* new_k = nullptr, const void* new_v = nullptr) {
   kv->moves_open = false;
   AttendParams ap;
   ap.pool = kv->layer_pool(layer);
@@ -1442,6 +1446,9 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   ap.status = kv->d_status;
   ap.g = kv->g;
   ap.merge_ctr = kv->d_merge_ctr;
+  ap.new_k = (const uint16_t*)new_k;
+  ap.new_v = (const uint16_t*)new_v;
+  ap.pool_rw = kv->layer_pool(layer);
   ap.wait_limit_ns = kv->wait_limit_ns;
   ap.debug_drop_first_stage = kv->drop_first_stage_once ? 1 : 0;
   kv->drop_first_stage_once = false;
@@ -1656,6 +1663,8 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   }
   if (cudaEventRecord(kv->ev_step, st) != cudaSuccess) return TIDE_ERR_CUDA;
   kv->step_upload_pending = true;
+  kv->step_seq = kv->live_keys.seq();
+  kv->step_fused = !kv->fixed_grids && P.items_dec > 0 && P.items_tile == 0 && P.items_umma == 0 && P.merge_rows == 0 && P.groups.empty();
   kv->step_recs = n_rows;
   kv->step_tokens = indptr[(size_t)n_rows];
   kv->step_valid = true;
@@ -1689,11 +1698,18 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   ap.early = kv->step_layers > 0 && kv->step_stream == st ? 1 : 0;   // behind another layer, whose kernels waited for the upload
   kv->step_stream = st;
   ++kv->step_layers;
-  if (launch_append(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
+  // Decode-style rows without groups: one launch a layer.  Us a layer with the append as a launch of its own and without: 28 / 4
+  // heads, D = 128, one row of 4k keys 12.8 and 10.8, 32 rows of 1k 27.5 and 24.1, 60 rows of 8k 203 and 200; 32 / 8 heads, D = 64,
+  // 32 rows of 1k 31.4 and 28.9.
+  // Not the first layer: its kernel would be the one right behind the upload of the descriptors and pages that its producers
+  // read ahead; nor behind a writer that came in between, whose keys the step's plan knows nothing of.
+  const bool fused = kv->step_fused && ap.early && kv->live_keys.seq() == kv->step_seq;
+  if (!fused && launch_append(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
   int64_t launches = 0;
-  const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, true, nullptr, q, scale, out, lse, st, false, &launches, dyn);
+  const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, true, nullptr, q, scale, out, lse, st, false, &launches, dyn,
+                             fused ? new_k : nullptr, fused ? new_v : nullptr);
   if (rc != TIDE_OK) return rc;
-  kv->last_launches = launches + 1;
+  kv->last_launches = launches + (fused ? 0 : 1);
   return TIDE_OK;
 }
 
@@ -1948,7 +1964,9 @@ int tide_tune(tide_kv_t* kv, int knob, int64_t value) {
       if (value < 1 || value > 60ll * 1000 * 1000) return TIDE_ERR_INVALID_ARG;
       kv->wait_limit_ns = value * 1000;
       break;
-    case TIDE_TUNE_DROP_FIRST_STAGE: kv->drop_first_stage_once = value != 0; break;
+    case TIDE_TUNE_DROP_FIRST_STAGE:
+      kv->drop_first_stage_once = value != 0;
+      return TIDE_OK;         // no plan depends on it: it may hit any layer of a step
     case TIDE_TUNE_UPLOAD_BY_KERNEL: kv->always_upload_by_kernel = value != 0; break;
     case TIDE_TUNE_INLINE_DESCRIPTORS: kv->inline_descriptors = value != 0; break;
     case TIDE_TUNE_HOST_ZERO_COPY: kv->host_zero_copy = value != 0; break;

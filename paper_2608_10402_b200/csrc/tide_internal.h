@@ -98,6 +98,11 @@ struct AttendParams {
   long long wait_limit_ns = kWaitLimitNsDefault;   // bound of every wait inside the kernel
   int run_ahead = 0;          // decode, 128-key tcgen05: the producers may read keys below Segment::live_from before earlier work is complete
   int overlapped = 0;         // decode: the kernel before this one in the stream is the tcgen05 kernel of the same batch (see grid_dep_wait)
+  // Decode, a layer of a step whose rows are all decode-style: the step's new rows (in the order of q), which the launch writes
+  // to their pages itself - the block that reads a page writes it first - instead of an append in front of it.
+  const uint16_t* new_k = nullptr;
+  const uint16_t* new_v = nullptr;
+  uint8_t* pool_rw = nullptr;
   // Test hook for the bounded waits (never set in normal use): in work item 0 the producer leaves out its part
   // of the first stage, so the consumers' wait for that stage runs out and the time-out path executes.
   int debug_drop_first_stage = 0;

@@ -1,0 +1,136 @@
+"""Layers of a step whose rows are all decode-style: from the second layer on the attention launch writes the step's K/V
+rows itself.  Rows of one to as many tokens as still make a decode item, new tokens across pages, stages and pieces, long rows
+cut into pieces; three steps in a row; a writer between two layers; and a wait that runs out, after which the cache must hold
+every layer's rows.  Cache bits are compared with the oracle exactly, results within its tolerance."""
+import math
+
+import numpy as np
+import pytest
+
+from oracle import cbuild
+from oracle.layers import LayeredKVOracle
+from paper_2608_10402_b200 import inputs
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+LAYERS = 3
+
+
+class Both:
+    """The library and the oracle, filled alike."""
+
+    def __init__(self, geom, prefix, room):
+        import torch
+        from paper_2608_10402_b200 import tide
+        self.torch, self.tide, self.geom = torch, tide, geom
+        HQ, HKV, D, S = geom
+        self.rng = rng = np.random.default_rng(HQ + HKV + D + S)
+        n = len(prefix)
+        pages = sum((p + room + S - 1) // S for p in prefix) + 4
+        most = max((p + room + S - 1) // S for p in prefix) + 1
+        order = rng.permutation(pages).astype(np.int32)
+        self.kv = tide.TideKV(HQ, HKV, D, S, pages, n, most, n, 4096, free_order=order, num_layers=LAYERS)
+        self.orc = LayeredKVOracle(LAYERS, num_pages=pages, page_size=S, num_kv_heads=HKV, head_dim=D, max_tasks=n, max_pages_per_task=most,
+                                   free_order=order)
+        self.ids = list(range(n))
+        for o in (self.kv, self.orc):
+            for t in self.ids:
+                o.alloc(t)
+        ip = np.concatenate([[0], np.cumsum(prefix)]).astype(np.int32)
+        k, v = self.rows(int(ip[-1])), self.rows(int(ip[-1]))
+        self.kv.extend(self.ids, ip)
+        for l in range(LAYERS):
+            self.kv.write(l, self.ids, ip, H.to_dev(k[l], torch), H.to_dev(v[l], torch))
+        self.orc.append(self.ids, ip, k, v)
+
+    def rows(self, tokens):
+        return np.stack([inputs.normal_bf16(self.rng, (tokens, self.geom[1], self.geom[2])) for _ in range(LAYERS)])
+
+    def step(self, new, between=None, check=True):
+        HQ, HKV, D, S = self.geom
+        torch, kv, orc = self.torch, self.kv, self.orc
+        ip = np.concatenate([[0], np.cumsum(new)]).astype(np.int32)
+        T = int(ip[-1])
+        k, v = self.rows(T), self.rows(T)
+        q = np.stack([inputs.normal_bf16(self.rng, (T, HQ, D)) for _ in range(LAYERS)])
+        orc.append(self.ids, ip, k, v)
+        rows = [(t, c, orc.task_len(t)) for t, c in zip(self.ids, new)]
+        out = torch.zeros((LAYERS, T, HQ, D), dtype=torch.int16, device="cuda")
+        lse = torch.zeros((LAYERS, T, HQ), dtype=torch.float32, device="cuda")
+        dk, dv, dq = H.to_dev(k, torch), H.to_dev(v, torch), H.to_dev(q, torch)
+        kv.step_begin(rows)
+        launches = []
+        for l in range(LAYERS):
+            if between:
+                between(l)
+            kv.step_layer(l, dk[l], dv[l], dq[l], 1.0 / math.sqrt(D), out[l], lse[l])
+            launches.append(kv.last_plan()["kernel_launches"])
+        if check:
+            assert kv.status() == self.tide.OK
+            for l in range(LAYERS):
+                ref_o, ref_l = cbuild.attend_paged(orc.layer(l), rows, q[l], 1.0 / math.sqrt(D))
+                H.check_outputs(H.from_dev(out[l]), lse[l].cpu().numpy(), ref_o, ref_l, f"layer {l}")
+        return launches
+
+    def same_bits(self):
+        for l in range(LAYERS):
+            for t in self.ids:
+                gk, gv = self.kv.read(t, layer=l)
+                ok, ov = self.orc.read(l, t)
+                assert np.array_equal(H.from_dev(gk), ok) and np.array_equal(H.from_dev(gv), ov), (l, t)
+
+
+@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 16), (12, 4, 64, 32), (16, 1, 128, 32), (6, 3, 64, 16)])
+def test_rows_are_written_by_the_attention_launch(geom):
+    G = geom[0] // geom[1]
+    most = 16 // G
+    prefix = [0, 1, 14, 15, 16, 31, 47, 62, 63, 64, 126, 127, 128, 129, 255, 511, 6000, 6143]
+    b = Both(geom, prefix, 3 * most)
+    for r in range(3):                                        # the last piece of a long row ends before, at or behind a boundary
+        new = [1 if r == 0 else int(b.rng.integers(1, most + 1)) for _ in prefix]
+        new[-1] = most if r else 1
+        assert b.step(new) == [2, 1, 1]
+    b.same_bits()
+    b.kv.close()
+
+
+def test_a_writer_between_two_layers_goes_in_front():
+    b = Both((8, 2, 64, 16), [300, 40, 2000], 8)
+    extra, torch = {}, b.torch
+
+    def between(l):
+        if l != 1:
+            return
+        # the last 20 rows of task 2 - 19 in front of the step's own, which its launch writes again - on every layer
+        k, v = b.rows(20), b.rows(20)
+        for x in range(LAYERS):
+            b.kv.write(x, [2], [0, 20], H.to_dev(k[x], torch), H.to_dev(v[x], torch))
+        extra["k"], extra["v"] = k, v
+
+    assert b.step([1, 1, 1], between, check=False) == [2, 2, 2]
+    assert b.kv.status() == b.tide.OK
+    for l in range(LAYERS):
+        gk, gv = (H.from_dev(x) for x in b.kv.read(2, layer=l))
+        ok, _ = b.orc.read(l, 2)
+        assert np.array_equal(gk[-20:-1], extra["k"][l][:19]) and np.array_equal(gv[-20:-1], extra["v"][l][:19])
+        assert np.array_equal(gk[-1], ok[-1] if l else extra["k"][l][19]) and np.array_equal(gk[:-20], ok[:-20])
+    b.kv.close()
+
+
+@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 16)])
+def test_rows_are_in_the_cache_when_a_wait_has_run_out(geom):
+    prefix = [5000, 3, 700, 1500, 64, 9000] + [130 + 7 * i for i in range(40)]
+    b = Both(geom, prefix, 4)
+    b.kv.tune(b.tide.TUNE_WAIT_LIMIT_US, 2000)
+
+    def between(l):
+        if l == 1:
+            b.kv.tune(b.tide.TUNE_DROP_FIRST_STAGE, 1)        # this layer's launch: one block gives up, the next layer's starts no item
+
+    b.step([1] * len(prefix), between, check=False)
+    assert b.kv.status() == b.tide.ERR_DEVICE_TIMEOUT
+    b.kv.tune(b.tide.TUNE_WAIT_LIMIT_US, 2_000_000)
+    b.same_bits()
+    b.step([2] * len(prefix))
+    b.same_bits()
+    b.kv.close()
