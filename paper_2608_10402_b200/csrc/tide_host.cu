@@ -1432,7 +1432,7 @@ static PlanDev pack_plan(const PlanHost& P, Segment* h, const Segment* d, size_t
 // travel in the launches' parameters; otherwise they are on the device, where `d` says.
 static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanHost* inl, bool step, const int32_t* page_table, const void* q,
                        float scale, void* out, float* lse, cudaStream_t st, bool events, int64_t* n_launches, const int32_t* dyn,
-                       const void* new_k = nullptr, const void* new_v = nullptr) {
+                       const void* new_k = nullptr, const void* new_v = nullptr, bool behind_layer = true) {
   kv->moves_open = false;
   AttendParams ap;
   ap.pool = kv->layer_pool(layer);
@@ -1459,7 +1459,7 @@ static int launch_plan(tide_kv* kv, int32_t layer, const PlanDev& d, const PlanH
   // The producers of the first attention kernel may run ahead of the work in front of it when their row descriptors do not
   // come from an upload right there (they are in the launch, or in the step area), and the page table is the handle's own,
   // so that all that may still be written is in LiveKeys.
-  const bool run_ahead = (inl != nullptr || step) && page_table == nullptr && !tile && !events;
+  const bool run_ahead = (inl != nullptr || step) && page_table == nullptr && !tile && !events && behind_layer;
   auto inline_segs = [&](const std::vector<Segment>& v) -> AttendInline& {
     AttendInline& pi = kv->attend_inline;
     std::copy(v.begin(), v.end(), pi.segs);
@@ -1700,14 +1700,14 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   ++kv->step_layers;
   // Decode-style rows without groups: one launch a layer.  Us a layer with the append as a launch of its own and without: 28 / 4
   // heads, D = 128, one row of 4k keys 12.8 and 10.8, 32 rows of 1k 27.5 and 24.1, 60 rows of 8k 203 and 200; 32 / 8 heads, D = 64,
-  // 32 rows of 1k 31.4 and 28.9.
-  // Not the first layer: its kernel would be the one right behind the upload of the descriptors and pages that its producers
-  // read ahead; nor behind a writer that came in between, whose keys the step's plan knows nothing of.
-  const bool fused = kv->step_fused && ap.early && kv->live_keys.seq() == kv->step_seq;
+  // 32 rows of 1k 31.4 and 28.9, 60 rows of 8k 225 and 226; a step of one layer, eight rows of 512, 20.5 and 18.2.
+  // The producers run ahead only behind another layer: not right behind the upload of the descriptors and pages that they read,
+  // nor behind a writer that came in between, whose keys the step's plan knows nothing of.
+  const bool fused = kv->step_fused, behind_layer = ap.early != 0 && kv->live_keys.seq() == kv->step_seq;
   if (!fused && launch_append(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
   int64_t launches = 0;
   const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, true, nullptr, q, scale, out, lse, st, false, &launches, dyn,
-                             fused ? new_k : nullptr, fused ? new_v : nullptr);
+                             fused ? new_k : nullptr, fused ? new_v : nullptr, !fused || behind_layer);
   if (rc != TIDE_OK) return rc;
   kv->last_launches = launches + (fused ? 0 : 1);
   return TIDE_OK;
