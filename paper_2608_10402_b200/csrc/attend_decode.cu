@@ -16,6 +16,8 @@
 // and 3 to 5 us of set-up (segment search, page ids, first stage) and ends with 2 us in which it reads nothing: with three
 // items per SM a decode step of 64 rows (0.82 GB of KV) took 137.8 us that way and 134.8 with persistent blocks (6.66 TB/s
 // between the first and the last time stamp of the kernel), eight layers of 48 shorter rows 594 and 584.
+// A layer of a planned step takes its new K/V rows along (attend_decode_writes_kernel): the block whose piece holds a new
+// position writes it to its page before it reads that page, which saves an append launch and its hand-over per layer.
 // Work items: one or two rounds of the resident blocks (build_plan in tide_host.cu, with the figures), or what
 // TIDE_TUNE_ITEMS_PER_SM says.  More, shorter items even out the end of the launch but pay more partials and merges (3 / 4 /
 // 6 / 8 per SM: 135 / 139 / 142 / 141 us on the 64 rows, 584 / 606 / 632 / 654 on the layers); so did rows cut into a few
