@@ -233,8 +233,9 @@ struct tide_kv {
   uint8_t* h_step = nullptr;   // staging of the step area
   cudaEvent_t ev_step = nullptr;
   bool step_upload_pending = false, step_valid = false;
-  int64_t step_seq = 0;        // the last writer when the step began
+  int64_t step_seq = 0;        // the last writer when the step's most recent layer had been launched (or the step begun)
   bool step_fused = false;     // the decode launches of the step write its rows themselves (AttendParams::new_k)
+  std::vector<int32_t> step_tasks, step_from;   // the step's rows: task, first new position
   PlanDev step_plan;
   int step_recs = 0, step_tokens = 0, step_layers = 0;   // step_layers: calls of tide_step_layer since tide_step_begin
   cudaStream_t step_stream = nullptr;
@@ -1664,6 +1665,12 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   if (cudaEventRecord(kv->ev_step, st) != cudaSuccess) return TIDE_ERR_CUDA;
   kv->step_upload_pending = true;
   kv->step_seq = kv->live_keys.seq();
+  kv->step_tasks.resize((size_t)n_rows);
+  kv->step_from.resize((size_t)n_rows);
+  for (int b = 0; b < n_rows; ++b) {
+    kv->step_tasks[(size_t)b] = rows[b].task;
+    kv->step_from[(size_t)b] = rows[b].ctx_len - rows[b].q_len;
+  }
   kv->step_fused = !kv->fixed_grids && P.items_dec > 0 && P.items_tile == 0 && P.items_umma == 0 && P.merge_rows == 0 && P.groups.empty();
   kv->step_recs = n_rows;
   kv->step_tokens = indptr[(size_t)n_rows];
@@ -1704,6 +1711,13 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   // The producers run ahead only behind another layer: not right behind the upload of the descriptors and pages that they read,
   // nor behind a writer that came in between, whose keys the step's plan knows nothing of.
   const bool fused = kv->step_fused, behind_layer = ap.early != 0 && kv->live_keys.seq() == kv->step_seq;
+  if (fused) {
+    // Such a launch lets the next one start before its rows are written; an append would have written them by then, since
+    // the attention kernel behind it waits for it first.
+    kv->live_keys.begin(st);
+    for (size_t b = 0; b < kv->step_tasks.size(); ++b) kv->live_keys.mark(kv->step_tasks[b], kv->step_from[b]);
+  }
+  kv->step_seq = kv->live_keys.seq();   // the layer behind this one may run ahead: this one waits for whatever came before it
   if (!fused && launch_append(ap, st) != cudaSuccess) return TIDE_ERR_CUDA;
   int64_t launches = 0;
   const int rc = launch_plan(kv, layer, kv->step_plan, nullptr, true, nullptr, q, scale, out, lse, st, false, &launches, dyn,

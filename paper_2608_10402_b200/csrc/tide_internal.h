@@ -241,8 +241,8 @@ int sm_count();   // multiprocessors of the current device (looked up once per d
 // append in front of the attention kernels, which waits for everything earlier: the producers of the first of them stream
 // those pages (AttendParams::run_ahead, Segment::live_from) while the append runs; whatever writes keys or page-table
 // entries - append, move, fork, extend - has marked them live (LiveKeys in tide_host.cu).  A decode launch that writes a layer's
-// rows itself (AttendParams::new_k) is such a writer, too: what it writes the begin of the step has marked, and it writes behind
-// its own wait for all earlier work.  Nor do the moves of several tasks
+// rows itself (AttendParams::new_k) is such a writer, too: it marks the rows in every layer, lets the next launch start ahead of
+// writing them, and writes behind its own wait for all earlier work.  Nor do the moves of several tasks
 // that are pruned in a row depend on each other.  What such a kernel reads it reads through L2 (bulk copies, __ldcg).
 // A wait limit does not count the time that the work in front still takes (mbar_wait).
 template <typename... A>

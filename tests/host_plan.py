@@ -64,6 +64,11 @@ class Handle:
         return self.lib.tide_kv_extend(self.h, len(ids), ids.ctypes.data_as(ctypes.c_void_p), ip.ctypes.data_as(ctypes.c_void_p),
                                        ctypes.c_void_p(stream))
 
+    def write(self, layer, counts, stream=0):
+        ids, ip = self._list(counts)
+        return self.lib.tide_kv_write(self.h, layer, len(ids), ids.ctypes.data_as(ctypes.c_void_p), ip.ctypes.data_as(ctypes.c_void_p),
+                                      ctypes.c_void_p(4096), ctypes.c_void_p(4096), ctypes.c_void_p(stream))
+
     def fork(self, parent, child, stream=0):
         return self.lib.tide_kv_fork(self.h, 0, parent, child, ctypes.c_void_p(stream))
 
@@ -110,14 +115,14 @@ class Handle:
         """What was launched since forget(): dicts, attention kernels with their segments' task and first live key."""
         out = []
         for i in range(self.lib.recorded()):
-            v, s = (ctypes.c_int * 6)(), (ctypes.c_int * 20)()
+            v, s = (ctypes.c_int * 7)(), (ctypes.c_int * 20)()
             stream = self.lib.launch_at(i, v)
             segs = []
             for j in range(v[5]):
                 self.lib.segment_at(i, j, s)
                 segs.append({"task": s[0] // self.mp, "n": s[2], "p": s[3], "n_splits": s[6], "chunk": s[7], "live_from": s[9], "causal": s[10],
                              "origin": s[11], "partial": s[12]})
-            out.append({"kind": v[0], "run_ahead": v[1], "overlapped": v[2], "items": v[3], "early": v[4], "stream": stream or 0, "segs": segs})
+            out.append({"kind": v[0], "run_ahead": v[1], "overlapped": v[2], "items": v[3], "early": v[4], "writes": v[6], "stream": stream or 0, "segs": segs})
         return out
 
     def live(self, rows, stream=0):

@@ -12,17 +12,17 @@ using namespace tide;
 namespace {
 enum Kind { kDecode, kTile, kUmma, kMerge, kAppend, kMove, kTable, kUpload, kCopyPages, kRead, kFetch };
 struct Launch {
-  int kind, run_ahead, overlapped, n_items, early;
+  int kind, run_ahead, overlapped, n_items, early, writes;
   void* stream;
   std::vector<Segment> segs;
 };
 std::vector<Launch> g_log;
 cudaError_t note(int kind, cudaStream_t s) {
-  g_log.push_back({kind, 0, 0, 0, 0, (void*)s, {}});
+  g_log.push_back({kind, 0, 0, 0, 0, 0, (void*)s, {}});
   return cudaSuccess;
 }
 cudaError_t note_attend(int kind, const AttendParams& p, const Segment* segs, cudaStream_t s) {
-  g_log.push_back({kind, p.run_ahead, p.overlapped, p.n_items, 0, (void*)s, std::vector<Segment>(segs, segs + p.n_segs)});
+  g_log.push_back({kind, p.run_ahead, p.overlapped, p.n_items, 0, p.new_k != nullptr, (void*)s, std::vector<Segment>(segs, segs + p.n_segs)});
   return cudaSuccess;
 }
 }  // namespace
@@ -30,10 +30,10 @@ cudaError_t note_attend(int kind, const AttendParams& p, const Segment* segs, cu
 extern "C" {
 int recorded() { return (int)g_log.size(); }
 void forget() { g_log.clear(); }
-// kind, run_ahead, overlapped, work items, early, number of segments
+// kind, run_ahead, overlapped, work items, early, number of segments, whether it writes K/V rows
 void* launch_at(int i, int* out) {
   const Launch& l = g_log[(size_t)i];
-  const int v[6] = {l.kind, l.run_ahead, l.overlapped, l.n_items, l.early, (int)l.segs.size()};
+  const int v[7] = {l.kind, l.run_ahead, l.overlapped, l.n_items, l.early, (int)l.segs.size(), l.writes};
   std::memcpy(out, v, sizeof(v));
   return l.stream;
 }
@@ -84,12 +84,12 @@ cudaError_t launch_upload_set(const UploadSet& u, cudaStream_t s) {
 }
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s) {
   if (p.n_tokens <= 0 && p.n_upd <= 0) return cudaSuccess;
-  g_log.push_back({kAppend, 0, 0, p.n_tokens, p.early, (void*)s, {}});
+  g_log.push_back({kAppend, 0, 0, p.n_tokens, p.early, 1, (void*)s, {}});
   return cudaSuccess;
 }
 cudaError_t launch_append_inline(const AppendInline& p, cudaStream_t s) { return launch_append(p.p, s); }
 cudaError_t launch_move(uint8_t*, size_t, int, const int32_t*, int, int, int, bool overlapped, const Geom&, cudaStream_t s) {
-  g_log.push_back({kMove, 0, overlapped ? 1 : 0, 0, 0, (void*)s, {}});
+  g_log.push_back({kMove, 0, overlapped ? 1 : 0, 0, 0, 1, (void*)s, {}});
   return cudaSuccess;
 }
 cudaError_t launch_copy_pages(uint8_t*, const int32_t*, const int32_t*, int, long long, cudaStream_t s) { return note(kCopyPages, s); }
@@ -100,6 +100,6 @@ cudaError_t launch_attend_tile(const AttendParams& p, cudaStream_t s) { return n
 cudaError_t launch_attend_umma(const AttendParams& p, cudaStream_t s) { return note_attend(kUmma, p, p.segs, s); }
 cudaError_t launch_attend_umma128(const AttendParams& p, cudaStream_t s) { return note_attend(kUmma, p, p.segs, s); }
 cudaError_t launch_attend_umma128_inline(const AttendInline& p, cudaStream_t s) { return note_attend(kUmma, p.p, p.segs, s); }
-cudaError_t launch_merge(const MergeParams& p, cudaStream_t s) { g_log.push_back({kMerge, 0, 0, p.n_rows, 0, (void*)s, std::vector<Segment>(p.segs, p.segs + p.n_segs)}); return cudaSuccess; }
-cudaError_t launch_merge_inline(const MergeInline& p, cudaStream_t s) { g_log.push_back({kMerge, 0, 0, p.p.n_rows, 0, (void*)s, std::vector<Segment>(p.segs, p.segs + p.p.n_segs)}); return cudaSuccess; }
+cudaError_t launch_merge(const MergeParams& p, cudaStream_t s) { g_log.push_back({kMerge, 0, 0, p.n_rows, 0, 0, (void*)s, std::vector<Segment>(p.segs, p.segs + p.n_segs)}); return cudaSuccess; }
+cudaError_t launch_merge_inline(const MergeInline& p, cudaStream_t s) { g_log.push_back({kMerge, 0, 0, p.p.n_rows, 0, 0, (void*)s, std::vector<Segment>(p.segs, p.segs + p.p.n_segs)}); return cudaSuccess; }
 }  // namespace tide

@@ -26,10 +26,10 @@ class Both:
         HQ, HKV, D, S = geom
         self.rng = rng = np.random.default_rng(HQ + HKV + D + S)
         n = len(prefix)
-        pages = sum((p + room + S - 1) // S for p in prefix) + 4
+        pages = sum((p + room + S - 1) // S for p in prefix) + 16
         most = max((p + room + S - 1) // S for p in prefix) + 1
         order = rng.permutation(pages).astype(np.int32)
-        self.kv = tide.TideKV(HQ, HKV, D, S, pages, n, most, n, 4096, free_order=order, num_layers=LAYERS)
+        self.kv = tide.TideKV(HQ, HKV, D, S, pages, n + 4, most, n, 4096, free_order=order, num_layers=LAYERS)
         self.orc = LayeredKVOracle(LAYERS, num_pages=pages, page_size=S, num_kv_heads=HKV, head_dim=D, max_tasks=n, max_pages_per_task=most,
                                    free_order=order)
         self.ids = list(range(n))
@@ -115,6 +115,61 @@ def test_a_writer_between_two_layers_goes_in_front():
         assert np.array_equal(gk[-20:-1], extra["k"][l][:19]) and np.array_equal(gv[-20:-1], extra["v"][l][:19])
         assert np.array_equal(gk[-1], ok[-1] if l else extra["k"][l][19]) and np.array_equal(gk[:-20], ok[:-20])
     b.kv.close()
+
+
+@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 32)])
+@pytest.mark.parametrize("queries", [1, 40])
+@pytest.mark.parametrize("which", ["fork", "write", "streams"])
+def test_attention_right_behind_a_layer_sees_its_rows(geom, queries, which):
+    """All queued without waiting: a step, other tasks' writers between its begin and its layers (or on the stream that the
+    layers do not run on), and behind every layer attention of the step's rows, by one query (the decode kernel) or the last 40
+    (tcgen05)."""
+    HQ, HKV, D, S = geom
+    prefix = [50 + 131 * i for i in range(40)] + [9000]
+    b = Both(geom, prefix, 4)
+    torch, kv, orc = b.torch, b.kv, b.orc
+    n, scale = len(prefix), 1.0 / math.sqrt(D)
+    sa, sb = (torch.cuda.Stream(), torch.cuda.Stream()) if which == "streams" else (None, None)
+    kv.alloc(n + 3)                                           # no task of a step
+    extra = [H.to_dev(x, torch) for x in (b.rows(700)[0], b.rows(700)[0])]
+    kv.append([n + 3], [0, 100], *extra)
+    for r in range(3):
+        k, v = b.rows(n), b.rows(n)
+        q = np.stack([inputs.normal_bf16(b.rng, (n, HQ, D)) for _ in range(LAYERS)])
+        q2 = np.stack([inputs.normal_bf16(b.rng, (n * queries, HQ, D)) for _ in range(LAYERS)])
+        ip = np.arange(n + 1, dtype=np.int32)
+        orc.append(b.ids, ip, k, v)
+        rows = [(t, 1, orc.task_len(t)) for t in b.ids]
+        rows2 = [(t, queries, orc.task_len(t)) for t in b.ids]
+        dk, dv, dq, dq2 = (H.to_dev(x, torch) for x in (k, v, q, q2))
+        out, out2 = torch.zeros_like(dq), torch.zeros_like(dq2)
+        lse, lse2 = (torch.zeros(x.shape[:3], dtype=torch.float32, device="cuda") for x in (dq, dq2))
+        torch.cuda.synchronize()
+
+        def writer():
+            if which == "fork":
+                kv.fork(0, n + r)
+            elif which == "write":
+                kv.write(1, [n + 3], [0, 90], *extra)
+            else:
+                kv.write(1, [n + 3], [0, 90], *extra, stream=sa)
+        kv.step_begin(rows, stream=sa)
+        writer()
+        if sb:
+            sb.wait_stream(sa)
+        for l in range(LAYERS):
+            kv.step_layer(l, dk[l], dv[l], dq[l], scale, out[l], lse[l], stream=sb)
+            if l == 1 and which != "fork":
+                writer()
+            kv.attend(rows2, dq2[l], scale, out2[l], lse2[l], layer=l, stream=sb)
+        torch.cuda.synchronize()
+        assert kv.status() == b.tide.OK
+        for l in range(LAYERS):
+            for got, gl, qq, rr, what in ((out, lse, q, rows, "layer"), (out2, lse2, q2, rows2, "attention behind layer")):
+                ref_o, ref_l = cbuild.attend_paged(orc.layer(l), rr, qq[l], scale)
+                H.check_outputs(H.from_dev(got[l]), gl[l].cpu().numpy(), ref_o, ref_l, f"step {r}, {what} {l}")
+    b.same_bits()
+    kv.close()
 
 
 @pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 16)])

@@ -134,3 +134,74 @@ def test_a_prune_that_goes_through_the_staging_area(kv):
     assert kv.append({1: 1}, A) == 0
     assert kv.prune(5, 100, 300, A) == 0                       # shares its pages: a new table row, a copied page, an append
     assert kv.live([(5, 1, 800), (0, 1, 1000)], A) == {5: 96, 0: hp.INT_MAX}
+
+
+@pytest.fixture
+def layered(lib):
+    h = hp.Handle(lib, layers=3)
+    h.alloc(0, 1, 2, 3)
+    for t in range(4):
+        assert h.append({t: 1000 + t}, A) == 0
+    yield h
+    h.close()
+
+
+def writer(kv, which, stream):
+    assert {"fork": lambda: kv.fork(1, 5, stream), "write": lambda: kv.write(1, {2: 20}, stream)}[which]() == 0
+
+
+# one query (the decode kernel) and 40 (the tcgen05 kernel)
+@pytest.mark.parametrize("queries", [1, 40])
+@pytest.mark.parametrize("which", ["fork", "write"])
+def test_rows_that_a_decode_launch_writes_are_live(layered, which, queries):
+    """A step of decode rows: the layers' attention launches write the step's rows, and let the next launch start before.  A
+    writer between the begin of the step and a layer changes nothing about that."""
+    kv = layered
+    assert kv.step_begin([(0, 1, 1001)], A) == 0
+    writer(kv, which, A)
+    kv.forget()
+    assert kv.step_layer(0, A) == 0
+    assert [(l["kind"], l["writes"]) for l in kv.launches()] == [(hp.DECODE, 1)]
+    assert kv.live([(0, queries, 1001)], A) == {0: 992}
+    assert kv.step_layer(1, A) == 0
+    writer(kv, "write", A)                                     # waits for the layers: their rows are complete, its own are not
+    assert kv.live([(0, queries, 1001), (2, queries, 1002)], A) == {0: hp.INT_MAX, 2: 976}
+    assert kv.step_layer(2, A) == 0
+    assert kv.live([(0, queries, 1001), (2, queries, 1002)], A) == {0: 992, 2: hp.INT_MAX}
+
+
+@pytest.mark.parametrize("queries", [1, 40])
+def test_rows_that_a_decode_launch_writes_are_live_on_its_own_stream(layered, queries):
+    kv = layered
+    assert kv.step_begin([(0, 1, 1001), (1, 1, 1002)], A) == 0
+    for l in range(3):
+        assert kv.step_layer(l, B) == 0
+    assert kv.append({2: 1}, A) == 0                           # says nothing about B
+    assert kv.live([(0, queries, 1001), (1, queries, 1002)], B) == {0: 992, 1: 992}
+    assert kv.append({3: 1}, B) == 0
+    assert kv.live([(0, queries, 1001), (1, queries, 1002)], B) == {0: hp.INT_MAX, 1: hp.INT_MAX}
+
+
+def test_layers_run_ahead_behind_a_layer(layered):
+    """Not behind the begin of the step or a writer, whose keys the step's plan does not know; again behind the layer behind it."""
+    kv = layered
+    assert kv.step_begin([(0, 1, 1001), (2, 1, 1003)], A) == 0
+    ahead = []
+
+    def layer(l, stream=A):
+        kv.forget()
+        assert kv.step_layer(l, stream) == 0
+        (launch,) = kv.launches()
+        assert launch["kind"] == hp.DECODE and launch["writes"] == 1
+        assert {s["task"]: s["live_from"] for s in launch["segs"]} == {0: 1000, 2: 1002}
+        ahead.append(launch["run_ahead"])
+
+    layer(0), layer(1), layer(2)
+    assert kv.attend([(1, 1, 1001)], A) == 0                   # a reader
+    layer(0)
+    writer(kv, "write", A)
+    layer(1), layer(2)
+    writer(kv, "fork", B)                                      # of whatever stream
+    layer(0), layer(1)
+    layer(2, B), layer(0, B)                                   # another stream: its first layer is not behind a layer
+    assert ahead == [0, 1, 1, 1, 0, 1, 0, 1, 0, 1]
