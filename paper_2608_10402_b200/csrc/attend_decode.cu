@@ -321,8 +321,10 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
       return INLINE ? segs[si] : load_segment(segs + si);
     };
     // A launch that writes the step's rows itself writes them also where its waits run out or the status word keeps items
-    // from being started: the cache holds them whatever becomes of the results.
+    // from being started: the cache holds them whatever becomes of the results.  (Only the rows of an item that the hardware
+    // has handed to this block in an answer that never landed would be missing.)
     auto put_only = [&](int item) {
+      if (item < 0 || item >= n_items) return;
       const Segment seg = segment_of(item);
       const int local = item - seg.item_base, begin = seg.origin + local % seg.n_splits * seg.chunk;
       put_new_rows<D>(P, seg.table_off, local / seg.n_splits, seg.q_off - seg.p, max(begin, seg.p), min(begin + seg.chunk, seg.p + seg.n));
@@ -335,10 +337,9 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
     auto answer = [&]() -> bool {
       if (!wait_all(s_answer, (asks - 1) & 1)) return false;
       open = false;
-      item = next_block_answer(smem_u32(&s_next));
+      item = claimed_item(true, next_block_answer(smem_u32(&s_next)), n_items);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the answer has been read before the next one may land
       __syncwarp();
-      if (item >= n_items) item = -1;                        // fixed grid: indices beyond the batch
       return true;
     };
     for (int it = 0; ; ++it) {
@@ -400,16 +401,19 @@ __device__ __forceinline__ void attend_decode_body(const AttendParams& P, const 
       ask();
       if (!answer()) break;
     }
-    if (open) {                                              // only after a wait gave up: the answer lands before the block leaves
+    if (open) {
+      // Only after a wait gave up: the answer lands before the block leaves.  The hardware always answers, in a microsecond or
+      // so, and the handle's limit may be shorter than that, hence a bound of its own.
       const long long t0 = global_ns();
-      while (!mbar_try(smem_u32(&s_answer), (asks - 1) & 1) && global_ns() - t0 < P.wait_limit_ns) {}
-      item = next_block_answer(smem_u32(&s_next));
+      bool landed = mbar_try(smem_u32(&s_answer), (asks - 1) & 1);
+      while (!landed && global_ns() - t0 < kWaitLimitNsDefault) landed = mbar_try(smem_u32(&s_answer), (asks - 1) & 1);
+      landed = __all_sync(0xffffffffu, landed) != 0;
+      item = claimed_item(landed, landed ? next_block_answer(smem_u32(&s_next)) : -1, n_items);
     }
     if (WRITES && *abort_flag) {                             // what the producer may not have come to
       grid_dep_wait();
-      for (int i = 0; i < kItemSlots; ++i)
-        if (handed_out[i] >= 0) put_only(handed_out[i]);
-      if (item >= 0) put_only(item);
+      for (int i = 0; i < kItemSlots; ++i) put_only(handed_out[i]);
+      put_only(item);
     }
     return;
   }

@@ -43,6 +43,13 @@ __host__ __device__ __forceinline__ int blk_offset(const Geom& g, int slot, int 
   return kv * g.kblock_bytes + (slot >> 3) * g.group_bytes + (c >> 3) * 1024 + (slot & 7) * 128 + (((c & 7) ^ (slot & 7)) << 4);
 }
 
+// The work item that a question to the hardware (next_block_ask) brought a block: -1 as long as the answer has not landed
+// (what the answer's place holds then is an older one, or nothing), where none was left, and where the index lies beyond the
+// batch (fixed grid).
+__host__ __device__ __forceinline__ int claimed_item(bool landed, int answer, int n_items) {
+  return landed && answer >= 0 && answer < n_items ? answer : -1;
+}
+
 // One batch row as the kernels see it.  Items of a segment are numbered
 // ((kv_head * n_splits) + split) * n_mtiles + m_tile from item_base.
 struct __align__(16) Segment {

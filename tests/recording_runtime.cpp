@@ -37,6 +37,7 @@ void* launch_at(int i, int* out) {
   std::memcpy(out, v, sizeof(v));
   return l.stream;
 }
+int claimed(int landed, int answer, int n_items) { return claimed_item(landed != 0, answer, n_items); }
 void segment_at(int i, int j, int* out) { std::memcpy(out, &g_log[(size_t)i].segs[(size_t)j], sizeof(Segment)); }
 
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }

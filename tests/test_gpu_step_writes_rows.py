@@ -133,7 +133,7 @@ def test_attention_right_behind_a_layer_sees_its_rows(geom, queries, which):
     kv.alloc(n + 3)                                           # no task of a step
     extra = [H.to_dev(x, torch) for x in (b.rows(700)[0], b.rows(700)[0])]
     kv.append([n + 3], [0, 100], *extra)
-    for r in range(3):
+    for r in range(3 if queries == 1 else 1):
         k, v = b.rows(n), b.rows(n)
         q = np.stack([inputs.normal_bf16(b.rng, (n, HQ, D)) for _ in range(LAYERS)])
         q2 = np.stack([inputs.normal_bf16(b.rng, (n * queries, HQ, D)) for _ in range(LAYERS)])
@@ -189,3 +189,47 @@ def test_rows_are_in_the_cache_when_a_wait_has_run_out(geom):
     b.step([2] * len(prefix))
     b.same_bits()
     b.kv.close()
+
+
+@pytest.mark.parametrize("geom,n,prefix", [((28, 4, 128, 16), 400, 2000), ((8, 2, 64, 32), 1200, 1000)])
+def test_the_block_that_gives_up_and_items_not_started_write_their_rows(geom, n, prefix):
+    """Every row is one piece, longer than the ring: the block that gives up (on its first item) has not come to its row's new
+    position.  The next layer finds the status word set, which keeps its items - several per resident block - from being
+    started.  Bits are compared on the device."""
+    import torch
+    from paper_2608_10402_b200 import tide
+    HQ, HKV, D, S = geom
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    rows = lambda *shape: torch.randn(shape, device="cuda", generator=gen).to(torch.bfloat16)
+    length = [prefix + i % 7 for i in range(n)]
+    most = (prefix + 10 + S - 1) // S
+    layers, pages = 2, n * most
+    kv = tide.TideKV(HQ, HKV, D, S, pages, n, most, n, 4096, free_order=np.random.default_rng(n).permutation(pages).astype(np.int32), num_layers=layers)
+    old = [(rows(prefix + 6, HKV, D), rows(prefix + 6, HKV, D)) for _ in range(layers)]     # every task begins with the same tokens
+    for t in range(n):
+        kv.alloc(t)
+        kv.extend([t], [0, length[t]])
+        for l in range(layers):
+            kv.write(l, [t], [0, length[t]], old[l][0][:length[t]], old[l][1][:length[t]])
+    new_k, new_v, q = rows(layers, n, HKV, D), rows(layers, n, HKV, D), rows(layers, n, HQ, D)
+    out = torch.zeros_like(q)
+    assert kv.status() == tide.OK
+    kv.tune(tide.TUNE_WAIT_LIMIT_US, 2000)
+    kv.step_begin([(t, 1, length[t] + 1) for t in range(n)])
+    kv.tune(tide.TUNE_DROP_FIRST_STAGE, 1)
+    for l in range(layers):
+        kv.step_layer(l, new_k[l], new_v[l], q[l], 1.0 / math.sqrt(D), out[l])
+    assert kv.last_plan()["decode_items"] == n * HKV           # one piece a row
+    assert kv.status() == tide.ERR_DEVICE_TIMEOUT
+    left_out = [int((o.view(n, HKV, -1) == 0).all(-1).sum()) for o in out]     # items that were not started
+    assert left_out[0] == 0                                    # the 2 ms are longer than the others take
+    # the second layer's blocks that start beside the first, two on an SM, may have begun one item each before the word was set
+    assert n * HKV - left_out[1] <= 2 * torch.cuda.get_device_properties(0).multi_processor_count, left_out
+    for l in range(layers):
+        for t in range(n):
+            k, v = kv.read(t, layer=l)
+            for got, before, row in ((k, old[l][0], new_k[l, t]), (v, old[l][1], new_v[l, t])):
+                got = got.view(torch.bfloat16)
+                assert torch.equal(got[-1], row) and torch.equal(got[:-1], before[:length[t]]), (l, t)
+    kv.close()

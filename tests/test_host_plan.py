@@ -70,3 +70,10 @@ def test_a_host_step_is_cut_between_and_inside_rows(lib, geom, groups):
     assert seen == {t: p + n for t, (p, n) in enumerate(zip(prefix, new))}
     assert (parts[0] > 1) == (groups > 1) and all(parts[t] == 1 for t in (1, 2, 3, 5, 7))
     kv.close()
+
+
+def test_only_an_answer_that_has_landed_is_a_work_item(lib):
+    """The place of the answer holds an older item, or nothing at all, until the hardware has written it."""
+    for stale in (-1, 0, 7, 99, 100, 2 ** 31 - 1, -2 ** 31):
+        assert lib.claimed(0, stale, 100) == -1
+    assert [lib.claimed(1, x, 100) for x in (-1, 0, 99, 100, 2 ** 31 - 1)] == [-1, 0, 99, -1, -1]
