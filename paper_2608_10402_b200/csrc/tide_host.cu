@@ -1710,7 +1710,14 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   // 32 rows of 1k 31.4 and 28.9, 60 rows of 8k 225 and 226; a step of one layer, eight rows of 512, 20.5 and 18.2.
   // The producers run ahead only behind another layer: not right behind the upload of the descriptors and pages that they read,
   // nor behind a writer that came in between, whose keys the step's plan knows nothing of.
-  const bool fused = kv->step_fused, behind_layer = ap.early != 0 && kv->live_keys.seq() == kv->step_seq;
+  // Results written over the new rows would replace rows that other blocks of such a launch have yet to read: append first.
+  const size_t T = (size_t)kv->step_tokens, row_bytes = T * kv->g.Hkv * kv->g.D * 2;
+  auto overwrites = [&](const void* dst, size_t bytes) -> bool {
+    auto meets = [&](const void* src) { return (uintptr_t)dst < (uintptr_t)src + row_bytes && (uintptr_t)src < (uintptr_t)dst + bytes; };
+    return dst != nullptr && (meets(new_k) || meets(new_v));
+  };
+  const bool fused = kv->step_fused && !overwrites(out, T * kv->g.Hq * kv->g.D * 2) && !overwrites(lse, T * kv->g.Hq * 4);
+  const bool behind_layer = ap.early != 0 && kv->live_keys.seq() == kv->step_seq;
   if (fused) {
     // Such a launch lets the next one start before its rows are written; an append would have written them by then, since
     // the attention kernel behind it waits for it first.

@@ -85,9 +85,9 @@ class Handle:
     def step_begin(self, rows, stream=0):
         return self.lib.tide_step_begin(self.h, len(rows), tide.rows_array(rows), ctypes.c_void_p(stream))
 
-    def step_layer(self, layer, stream=0):
-        p = ctypes.c_void_p(4096)
-        return self.lib.tide_step_layer(self.h, layer, p, p, p, ctypes.c_float(0.125), p, None, ctypes.c_void_p(stream))
+    def step_layer(self, layer, stream=0, new_k=1 << 30, new_v=2 << 30, q=3 << 30, out=4 << 30, lse=None):
+        p = ctypes.c_void_p
+        return self.lib.tide_step_layer(self.h, layer, p(new_k), p(new_v), p(q), ctypes.c_float(0.125), p(out), p(lse), p(stream))
 
     def step_host(self, rows):
         """A host-buffer step on stream 0 with (empty) host buffers."""

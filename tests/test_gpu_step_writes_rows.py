@@ -117,6 +117,34 @@ def test_a_writer_between_two_layers_goes_in_front():
     b.kv.close()
 
 
+@pytest.mark.parametrize("geom", [(16, 16, 128, 16), (8, 2, 64, 32)])
+@pytest.mark.parametrize("over", ["k", "v"])
+def test_results_over_the_new_rows(geom, over):
+    HQ, HKV, D, S = geom
+    b = Both(geom, [40 + 37 * i for i in range(60)], 2)
+    torch, n = b.torch, len(b.ids)
+    k, v = b.rows(n), b.rows(n)
+    q = np.stack([inputs.normal_bf16(b.rng, (n, HQ, D)) for _ in range(LAYERS)])
+    b.orc.append(b.ids, np.arange(n + 1, dtype=np.int32), k, v)
+    rows = [(t, 1, b.orc.task_len(t)) for t in b.ids]
+    dk, dv, dq = H.to_dev(k, torch), H.to_dev(v, torch), H.to_dev(q, torch)
+    b.kv.step_begin(rows)
+    outs = []
+    for l in range(LAYERS):
+        # the rows lie where the results of the first heads go
+        out = torch.zeros((n, HQ, D), dtype=torch.int16, device="cuda")
+        new = out.view(-1)[:n * HKV * D].view(n, HKV, D)
+        new.copy_((dk if over == "k" else dv)[l])
+        b.kv.step_layer(l, new if over == "k" else dk[l], new if over == "v" else dv[l], dq[l], 1.0 / math.sqrt(D), out)
+        outs.append(out)
+    assert b.kv.status() == b.tide.OK
+    for l in range(LAYERS):
+        ref_o, ref_l = cbuild.attend_paged(b.orc.layer(l), rows, q[l], 1.0 / math.sqrt(D))
+        H.check_outputs(H.from_dev(outs[l]), ref_l.astype(np.float32), ref_o, ref_l, f"layer {l}")
+    b.same_bits()
+    b.kv.close()
+
+
 @pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 32)])
 @pytest.mark.parametrize("queries", [1, 40])
 @pytest.mark.parametrize("which", ["fork", "write", "streams"])

@@ -77,3 +77,31 @@ def test_only_an_answer_that_has_landed_is_a_work_item(lib):
     for stale in (-1, 0, 7, 99, 100, 2 ** 31 - 1, -2 ** 31):
         assert lib.claimed(0, stale, 100) == -1
     assert [lib.claimed(1, x, 100) for x in (-1, 0, 99, 100, 2 ** 31 - 1)] == [-1, 0, 99, -1, -1]
+
+
+@pytest.mark.parametrize("Hq,Hkv", [(16, 16), (28, 4)])
+def test_rows_that_the_results_overwrite_are_appended_first(lib, Hq, Hkv):
+    """A caller may have a layer's results written over its new K/V rows.  Attention blocks that write the rows of their own items
+    would read rows that other blocks' results have replaced, so such a layer has its append in front."""
+    kv = hp.Handle(lib, Hq=Hq, Hkv=Hkv, layers=2)
+    tasks, T = (0, 1, 2), 3
+    kv.alloc(*tasks)
+    assert kv.append({t: 100 for t in tasks}) == 0
+    assert kv.step_begin([(t, 1, 101) for t in tasks]) == 0
+    k, o, lse = T * Hkv * 128 * 2, T * Hq * 128 * 2, T * Hq * 4
+
+    def kinds(**where):
+        kv.forget()
+        assert kv.step_layer(0, **where) == 0
+        return [(l["kind"], l["writes"], l["run_ahead"]) for l in kv.launches()]
+
+    apart, behind = [(hp.DECODE, 1, 1)], [(hp.APPEND, 1, 0), (hp.DECODE, 0, 1)]
+    K, V, O, X = 1 << 30, 2 << 30, 4 << 30, 5 << 30
+    assert kinds(lse=X) == [(hp.DECODE, 1, 0)]                 # the first layer waits
+    for rows in (K, V):
+        assert kinds(out=rows) == behind and kinds(out=rows + k - 16) == behind and kinds(out=rows - o + 16) == behind
+        assert kinds(lse=rows + k - 4) == behind and kinds(lse=rows - lse + 4) == behind
+        assert kinds(out=rows + k) == apart and kinds(out=rows - o) == apart
+        assert kinds(lse=rows + k) == apart and kinds(lse=rows - lse) == apart
+    assert kinds(q=O) == apart                                 # results over the queries, as ever
+    kv.close()
