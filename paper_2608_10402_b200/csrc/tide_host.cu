@@ -84,6 +84,22 @@ struct PlanHost {
   size_t n_all() const { return seg_dec.size() + seg_tile.size() + seg_umma.size() + seg_merge.size(); }
 };
 
+// Layers of a step of decode-style rows without groups are one launch, which writes the step's rows itself: where every row has one
+// new token, and with several tokens a row up to kStepWritesBytes of new K and V; 64-wide heads up to kStepWritesKv64 of context.
+// It saves the append launch, some 2.5 us (1.5 where another kernel stands between the layers); a block spends about a microsecond on
+// the rows of an item, which many items of short contexts do not hide, above all with two halves of packed rows, and the
+// producer of 64-wide heads, which has half the time per stage, runs half a percent slower.  us a layer, append launch / rows written by
+// the decode launch (in brackets with another kernel between the layers):
+//   one token a row: 28 / 4 heads, D = 128: a row of 4k keys 12.5 / 10.4 (17.2 / 15.0), 60 of 8k 180.9 / 177.2 (185.9 / 183.5), 200 of 1k
+//     88.7 / 85.8 (93.7 / 91.8); 32 / 8 heads, D = 64: 60 of 512 23.1 / 20.1 (27.5 / 25.8), 100 of 1k 47.4 / 44.8 (52.1 / 51.2),
+//     60 of 8k (1.2 GiB) 190.5 / 187.7 (193.7 / 194.9), 60 of 16k (2.4) 373.7 / 373.3 (376.8 / 378.2), 400 of 2k (2.0) 337.7 / 338.5 (342.7 / 344.0)
+//   several: 32 / 8 heads, D = 128, 4 tokens: 64 rows of 1k (1.0 MiB) 62.1 / 57.9 (65.8 / 64.5), 100 of 2k (1.6) 187.3 / 185.8
+//     (191.4 / 191.5), 200 of 1k (3.1) 178.3 / 182.1 (183.0 / 188.8); 16 / 16 heads, D = 64, 16 tokens: 24 of 2k (1.5) 51.5 / 49.3
+//     (55.3 / 55.1), 100 of 1k (6.3) 109.2 / 110.6 (113.4 / 116.7); 28 / 4 heads, 2 tokens: 200 of 1k (0.8) 98.0 / 96.3 (102.7 / 100.4),
+//     400 of 1k (1.6) 178.8 / 180.9 (183.7 / 187.7)
+constexpr int64_t kStepWritesBytes = 5ll << 18;              // 1.25 MiB
+constexpr int64_t kStepWritesKv64 = 3ll << 29;               // 1.5 GiB
+
 // What an extension of tasks did, as host arrays that are reused from call to call.
 struct ExtendOut {
   std::vector<int32_t> idx, val;           // page-table delta: table[idx[i]] = val[i]
@@ -1667,11 +1683,15 @@ int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows, void*
   kv->step_seq = kv->live_keys.seq();
   kv->step_tasks.resize((size_t)n_rows);
   kv->step_from.resize((size_t)n_rows);
+  int64_t context = 0;                                       // tokens
   for (int b = 0; b < n_rows; ++b) {
     kv->step_tasks[(size_t)b] = rows[b].task;
     kv->step_from[(size_t)b] = rows[b].ctx_len - rows[b].q_len;
+    context += rows[b].ctx_len;
   }
-  kv->step_fused = !kv->fixed_grids && P.items_dec > 0 && P.items_tile == 0 && P.items_umma == 0 && P.merge_rows == 0 && P.groups.empty();
+  const int64_t T = indptr[(size_t)n_rows];
+  kv->step_fused = !kv->fixed_grids && P.items_dec > 0 && P.items_tile == 0 && P.items_umma == 0 && P.merge_rows == 0 && P.groups.empty() &&
+                   (T == n_rows || T * g.Hkv * g.D * 4 <= kStepWritesBytes) && (g.D == 128 || context * g.Hkv * g.D * 4 <= kStepWritesKv64);
   kv->step_recs = n_rows;
   kv->step_tokens = indptr[(size_t)n_rows];
   kv->step_valid = true;
@@ -1705,9 +1725,6 @@ int tide_step_layer(tide_kv_t* kv, int32_t layer, const void* new_k, const void*
   ap.early = kv->step_layers > 0 && kv->step_stream == st ? 1 : 0;   // behind another layer, whose kernels waited for the upload
   kv->step_stream = st;
   ++kv->step_layers;
-  // Decode-style rows without groups: one launch a layer.  Us a layer with the append as a launch of its own and without: 28 / 4
-  // heads, D = 128, one row of 4k keys 12.8 and 10.8, 32 rows of 1k 27.5 and 24.1, 60 rows of 8k 203 and 200; 32 / 8 heads, D = 64,
-  // 32 rows of 1k 31.4 and 28.9, 60 rows of 8k 225 and 226; a step of one layer, eight rows of 512, 20.5 and 18.2.
   // The producers run ahead only behind another layer: not right behind the upload of the descriptors and pages that they read,
   // nor behind a writer that came in between, whose keys the step's plan knows nothing of.
   // Results written over the new rows would replace rows that other blocks of such a launch have yet to read: append first.

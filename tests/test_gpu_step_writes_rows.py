@@ -80,7 +80,7 @@ class Both:
                 assert np.array_equal(H.from_dev(gk), ok) and np.array_equal(H.from_dev(gv), ov), (l, t)
 
 
-@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 16), (12, 4, 64, 32), (16, 1, 128, 32), (6, 3, 64, 16)])
+@pytest.mark.parametrize("geom", [(28, 4, 128, 16), (8, 2, 64, 16), (12, 4, 64, 32), (16, 1, 128, 32), (6, 3, 64, 16), (3, 3, 128, 32), (2, 2, 64, 16)])
 def test_rows_are_written_by_the_attention_launch(geom):
     G = geom[0] // geom[1]
     most = 16 // G

@@ -105,3 +105,64 @@ def test_rows_that_the_results_overwrite_are_appended_first(lib, Hq, Hkv):
         assert kinds(lse=rows + k) == apart and kinds(lse=rows - lse) == apart
     assert kinds(q=O) == apart                                 # results over the queries, as ever
     kv.close()
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_which_steps_write_their_rows_in_the_decode_launch(lib, D):
+    """One token a row, or up to 1.25 MiB of new K and V; only decode-style rows, no groups, no fixed launch shapes."""
+    kv = hp.Handle(lib, Hq=16, Hkv=16, D=D, max_rows=400, max_tasks=400, num_pages=16384)
+    kv.alloc(*range(360))
+    assert kv.append({t: 100 for t in range(360)}) == 0
+    length = [100] * 400
+
+    def kinds(new):
+        rows = [(t, c, length[t] + c) for t, c in new.items()]
+        assert kv.step_begin(rows) == 0
+        for t, c in new.items():
+            length[t] += c
+        kv.forget()
+        assert kv.step_layer(0) == 0
+        return [(l["kind"], l["writes"]) for l in kv.launches()]
+
+    one, two = [(hp.DECODE, 1)], [(hp.APPEND, 1), (hp.DECODE, 0)]
+    most = (5 << 18) // (16 * D * 4)                           # tokens: 160, 320
+    assert kinds({t: 1 for t in range(360)}) == one            # beyond it, but one each
+    assert kinds({t: 16 for t in range(most // 16)}) == one
+    assert kinds({t: 16 for t in range(most // 16)} | {350: 1}) == two
+    assert kinds({t: 1 for t in range(most - 2)} | {350: 2}) == one
+    assert kinds({t: 1 for t in range(most - 1)} | {350: 2}) == two
+    assert kinds({0: 1, 1: 17}) == [(hp.APPEND, 1), (hp.UMMA, 0), (hp.DECODE, 0)]       # a resume row
+    assert kv.fix_grids(4096, 0, 0, 0, 4096) == 0
+    assert kinds({0: 1, 1: 1}) == two
+    assert kv.fix_grids(0, 0, 0, 0, 0) == 0
+    assert kinds({0: 1, 1: 1}) == one
+    kv.alloc(390)
+    assert kv.append({390: 600}) == 0 and kv.fork(390, 391) == 0 and kv.fork(390, 392) == 0
+    length[390:393] = [600] * 3
+    assert kinds({390: 1, 391: 1, 392: 1}) == one              # a group would not save enough
+    kv.tune(tide.TUNE_MIN_SAVED_BYTES, 0)
+    assert kinds({390: 1, 391: 1, 392: 1}) == [(hp.APPEND, 1), (hp.DECODE, 0), (hp.MERGE, 0)]
+    kv.close()
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_large_layers_of_64_wide_heads_append_first(lib, D):
+    """Up to 1.5 GiB of K and V: 393216 tokens of 16 heads of 64."""
+    kv = hp.Handle(lib, Hq=16, Hkv=16, D=D, max_rows=8, num_pages=32768, max_pages=4100)
+    kv.alloc(*range(7))
+    for t in range(6):
+        assert kv.append({t: 65534}) == 0
+    assert kv.append({6: 5}) == 0
+
+    def kinds(rows):
+        assert kv.step_begin(rows) == 0
+        kv.forget()
+        assert kv.step_layer(0) == 0
+        return [(l["kind"], l["writes"]) for l in kv.launches()]
+
+    one, two = [(hp.DECODE, 1)], [(hp.APPEND, 1), (hp.DECODE, 0)]
+    assert kinds([(t, 1, 65535) for t in range(6)]) == one
+    assert kinds([(t, 1, 65536) for t in range(6)]) == one     # 6 * 65536 = 393216
+    assert kinds([(t, 1, 65537) for t in range(5)] + [(6, 1, 6)]) == one
+    assert kinds([(t, 1, 65538) for t in range(5)] + [(5, 1, 65537)]) == (two if D == 64 else one)
+    kv.close()
