@@ -154,9 +154,9 @@ int tide_step_host(tide_kv_t* kv, int32_t layer, int32_t n_rows, const tide_row_
  * tasks (tide_kv_extend), plans the attention work and uploads the plan and the write records to a part of the
  * workspace that stays valid until the next tide_step_begin or any call that changes a task.  All-or-nothing.
  * tide_step_layer(layer) then writes that layer's new_k / new_v (device bf16 [sum q_len, Hkv, D], batch order)
- * and attends q against layer `layer` exactly as tide_attend would; it only launches kernels (no copies, no
- * events, no host waits), so the calls of all layers may be captured in one CUDA graph and replayed, as long
- * as the captured pointers stay valid.  scale must be positive and finite.  TIDE_ERR_INVALID_ARG if no step is
+ * and attends q against layer `layer` exactly as tide_attend would (out and lse may overlap the new rows); it
+ * only launches kernels (no copies, no events, no host waits), so the calls of all layers may be captured in one CUDA
+ * graph and replayed, as long as the captured pointers stay valid.  scale must be positive and finite.  TIDE_ERR_INVALID_ARG if no step is
  * open.  Per-phase timing (tide_set_profiling) does not cover tide_step_layer. */
 int tide_step_begin(tide_kv_t* kv, int32_t n_rows, const tide_row_t* rows /*host*/, void* stream);
 /* Fixes the launch shapes of tide_step_layer so that ONE captured CUDA graph of a step's layers can be replayed
@@ -224,8 +224,8 @@ int tide_kv_read(tide_kv_t* kv, int32_t layer, int32_t task, void* out_k /*devic
  * returns by itself.  The word is sticky: from the time-out until this call clears it, thread blocks of that
  * launch and of every later attention launch on the handle leave without computing, so `out` / `lse` of those
  * calls are undefined although the calls themselves returned TIDE_OK.  A caller that needs to know asks
- * tide_status after the step; after a TIDE_ERR_DEVICE_TIMEOUT the cache contents are intact and the attention
- * call can simply be repeated. */
+ * tide_status after the step; after a TIDE_ERR_DEVICE_TIMEOUT the cache contents are intact - a layer of a step has
+ * its new rows in the cache whether its attention ran or not - and the attention call can simply be repeated. */
 int tide_status(tide_kv_t* kv, void* stream);
 
 /* Rows of the most recently planned batch (tide_attend, tide_step_begin) that were planned as groups sharing their
@@ -242,7 +242,8 @@ int tide_last_plan(tide_kv_t* kv, int64_t* decode_items, int64_t* prefill_items,
                    int64_t* kernel_launches);
 
 /* Planner settings and test hooks of one handle.  The defaults are the measured best on B200; nothing reads the
- * environment.  Changing a setting closes an open step (tide_step_begin must be called again).
+ * environment.  Changing a setting closes an open step (tide_step_begin must be called again), except for the test hook
+ * TIDE_TUNE_DROP_FIRST_STAGE, which no plan depends on and which may be armed between two layers.
  * TIDE_ERR_INVALID_ARG for an unknown knob or a value outside its range. */
 typedef enum {
   TIDE_TUNE_ITEMS_PER_SM = 0,     /* work items per SM the KV-split planner aims for, 1..64 (default: for decode    */
