@@ -227,10 +227,7 @@ cudaError_t launch_copy_pages(uint8_t* pool, const int32_t* src, const int32_t* 
 // its first kMoveLinks links, ahead of the block's barrier and stores nothing before it.
 constexpr int kMoveLinks = 4;
 // Bound by latency - two dependent loads, page number and data, for every kMoveLinks links of a thread - until the blocks fill
-// the chip, where it is memory; so a chain is cut no further than that.  us, a thread per chain or, for shifts below 64, runs / this
-// (4 KV heads, D = 128, tail of 1500 / 4000 / 16000 tokens): shift 8 18.4 28.7 90.1 / 8.2 11.2 24.6, shift 64 14.3 24.6 81.9 / 8.2 12.3
-// 22.5, shift 128 10.2 16.4 43.0 / 8.2 12.3 22.6, shift 512 8.2 10.2 20.5 / 8.2 10.2 18.4; eleven tails of 3500 tokens by 107 in a
-// row, with their append and attention, 109 / 59.
+// the chip, where it is memory and the last round of blocks; how far chains are cut is launch_move's choice.
 constexpr int kMovePairsLog2 = 5, kMoveChainThreads = 8 << kMovePairsLog2;   // 32 (segment, chain) pairs of eight lanes, 128 bytes of a row
 template <int SLABS>
 __global__ void __launch_bounds__(kMoveChainThreads, 3) move_chains_kernel(uint8_t* pool0, size_t layer_stride, const int32_t* __restrict__ table_row, int to,
@@ -247,10 +244,13 @@ __global__ void __launch_bounds__(kMoveChainThreads, 3) move_chains_kernel(uint8
   const int c = slab * 8 + (threadIdx.x & 7), pair = threadIdx.x >> 3;
   const int chain = (group << chains_log2) + (pair & ((1 << chains_log2) - 1)), seg = pair >> chains_log2;
   const int links = chain < chains ? (n - chain - 1) / shift + 1 : 0;
-  const int first = min(seg * seg_links, links), end = min(first + seg_links, links), last = end - 1;   // this segment's links
+  const int first = min(seg * seg_links, links), end = min(first + seg_links, links);   // this segment's links ...
+  const bool cut = segs_log2 > 0;
+  const int last = cut ? end - 1 : end;                      // ... in front of the one whose source another thread writes
+  const int s_log2 = g.S == 16 ? 4 : 5;
   auto at = [&](int link) -> uint4* {                        // a link's target: the source of the link before it
-    const int pos = to + chain + link * shift, lp = pos / g.S;
-    return reinterpret_cast<uint4*>(pool + (long long)__ldcg(table_row + lp) * g.page_bytes + head + blk_offset(g, pos - lp * g.S, kv, c));
+    const int pos = to + chain + link * shift, lp = pos >> s_log2;
+    return reinterpret_cast<uint4*>(pool + (long long)__ldcg(table_row + lp) * g.page_bytes + head + blk_offset(g, pos & (g.S - 1), kv, c));
   };
   uint4 *a0[kMoveLinks + 1], *a1[kMoveLinks + 1];
   uint4 v0[kMoveLinks], v1[kMoveLinks];
@@ -260,7 +260,8 @@ __global__ void __launch_bounds__(kMoveChainThreads, 3) move_chains_kernel(uint8
 #pragma unroll
     for (int k = 0; k < kMoveLinks; ++k) a[k + 1] = i + k < last ? at(i + k + 1) : target;
 #pragma unroll
-    for (int k = 0; k < kMoveLinks; ++k) v[k] = __ldcg(a[k + 1]);
+    for (int k = 0; k < kMoveLinks; ++k)
+      if (i + k < last) v[k] = __ldcg(a[k + 1]);
   };
   auto store = [&](int i, uint4* const (&a)[kMoveLinks + 1], const uint4 (&v)[kMoveLinks]) {
 #pragma unroll
@@ -271,11 +272,15 @@ __global__ void __launch_bounds__(kMoveChainThreads, 3) move_chains_kernel(uint8
   uint4 last_value = make_uint4(0, 0, 0, 0);
   int i = first;
   if (first < end) {
-    last_target = at(last);
-    last_value = __ldcg(at(end));
-    if (i < last) load(i, at(i), a0, v0);
+    if (cut) {
+      // the page numbers of all these links side by side, then their data (one link's behind the other's: 1 to 2 us more)
+      uint4* const source = at(end);
+      last_target = at(last);
+      load(i, at(i), a0, v0);
+      last_value = __ldcg(source);
+    } else load(i, at(i), a0, v0);
   }
-  __syncthreads();
+  if (cut) __syncthreads();
   while (i < last) {
     if (i + kMoveLinks < last) load(i + kMoveLinks, a0[kMoveLinks], a1, v1);
     store(i, a0, v0);
@@ -285,7 +290,7 @@ __global__ void __launch_bounds__(kMoveChainThreads, 3) move_chains_kernel(uint8
     store(i, a1, v1);
     i += kMoveLinks;
   }
-  if (first < end) *last_target = last_value;
+  if (last_target != nullptr) *last_target = last_value;
   if (overlapped) grid_dep_wait();
 }
 
@@ -334,30 +339,48 @@ __global__ void __launch_bounds__(kMoveThreads) move_runs_kernel(uint8_t* pool0,
   if (overlapped) grid_dep_wait();
 }
 
-// Runs are left where a chain has more links than its threads share out well: a shift of one (tail of 1500 / 4000 / 16000 tokens 18.4 /
-// 28.7 / 88 us, by chains 20.5 / 43 / 147) and chains of thousands of links, which only tails of 100k tokens and more that move
-// by a few positions have (tests/test_gpu_timeout.py takes such a move for its long launch on few blocks).
-constexpr int kMoveMostLinks = 4096;
+// How many segments (as a power of two) each chain is cut into; groups of chains x `columns` are the blocks, of which three fit an SM.
+// While half of these places would stay empty, down to segments whose links are loaded at once; then up to nine blocks an SM, which
+// even out the last round, down to 16 links.  A last cut that would leave a second round nearly empty is not made.
+// us, cut until the blocks just fill the chip / this (4 KV heads, D = 128): 8 layers, tail of 16000 tokens, shift 64 142 / 101, 100 172 / 102,
+// 128 150 / 99, 512 110 / 101; tail of 65000 566 / 381, 679 / 389, 583 / 373, 444 / 429; one layer, shift 128, tail of 1500 / 4000 / 16000: a
+// thread per chain 10.2 / 16.2 / 43.0, this 8.2 / 9.9 / 17.2; eleven tails of 3500 tokens by 107 in a row, with their append and attention,
+// 109 and 59.
+static int move_segments_log2(int chains, int links, long long columns) {
+  const long long places = 3ll * sm_count();
+  auto blocks = [&](int segs_log2) -> long long {
+    const int per_block_log2 = kMovePairsLog2 - segs_log2;
+    return (((long long)chains + (1 << per_block_log2) - 1) >> per_block_log2) * columns;
+  };
+  int s = 0;
+  for (; s < kMovePairsLog2; ++s) {
+    const int ahead = (links - 1) >> s;                      // of a segment's last link
+    if (!(2 * blocks(s) < places && ahead > kMoveLinks) && !(blocks(s) < 3 * places && ahead >= 32)) break;
+  }
+  if (s > 0 && blocks(s) > places && 2 * blocks(s) < 3 * places && blocks(s - 1) <= places) --s;
+  return s;
+}
+
+// Runs take a shift of one, and long tails that move by two: in so few chains only as many threads move as a chain has segments.
+// us, runs / chains (4 KV heads, D = 128): shift 1, tail of 1500 / 4000 / 16000 tokens 17 29 88 / 21 43 147; shift 2, 16000 88 / 68, 65000 and 300000
+// 391 1811 / 461 2477 (8 layers, 65000 / 120000 584 1024 / 578 1107; these before the loads of a segment were put side by side); shift 3,
+// 16000 / 120000 88 723 / 47 529; shift 17, 120000 723 / 136.
+constexpr int kMoveRunsFrom = 8192;                          // links of a shift of two
 
 cudaError_t launch_move(uint8_t* pool, size_t layer_stride, int layers, const int32_t* table_row, int to, int shift, int n, bool overlapped,
                         const Geom& g, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int links = (n - 1) / shift + 1, slabs = g.D / 64;
-  if (shift == 1 || links > kMoveMostLinks) {
-    const dim3 grid((unsigned)(2 * g.Hkv * slabs), (unsigned)layers);
+  const int links = (n - 1) / shift + 1, columns = 2 * g.Hkv * (g.D / 64);
+  if (shift == 1 || (shift == 2 && links > kMoveRunsFrom)) {
+    const dim3 grid((unsigned)columns, (unsigned)layers);
     return launch_dep(g.D == 128 ? move_runs_kernel<2> : move_runs_kernel<1>, grid, kMoveThreads, 0, s, pool, layer_stride, table_row, to, shift, n,
                       overlapped ? 1 : 0, g);
   }
-  const int chains = std::min(shift, n), fill = 3 * sm_count();        // the resident blocks
-  int segs_log2 = 0;
-  auto blocks = [&] {
-    const int per_block_log2 = kMovePairsLog2 - segs_log2;
-    return (long long)((chains + (1 << per_block_log2) - 1) >> per_block_log2) * 2 * g.Hkv * slabs;
-  };
-  while (segs_log2 < kMovePairsLog2 && (links - 1) >> segs_log2 > kMoveLinks && blocks() * layers < fill) ++segs_log2;
-  const dim3 grid((unsigned)blocks(), (unsigned)layers);
+  const int chains = std::min(shift, n), segs_log2 = move_segments_log2(chains, links, (long long)columns * layers);
+  const int per_block_log2 = kMovePairsLog2 - segs_log2;
+  const dim3 grid((unsigned)((((long long)chains + (1 << per_block_log2) - 1) >> per_block_log2) * columns), (unsigned)layers);
   return launch_dep(g.D == 128 ? move_chains_kernel<2> : move_chains_kernel<1>, grid, kMoveChainThreads, 0, s, pool, layer_stride, table_row, to, shift,
-                    n, segs_log2, (links + (1 << segs_log2) - 1) >> segs_log2, overlapped ? 1 : 0, g);
+                    n, segs_log2, ((links - 1) >> segs_log2) + 1, overlapped ? 1 : 0, g);
 }
 
 // Logical content of one task -> contiguous [len, Hkv, D]; inverse of the scatter above.

@@ -70,14 +70,16 @@ def test_tails_move_in_place(geom, layers):
 
 @pytest.mark.parametrize("geom,layers", [((28, 4, 128, 16), 1), ((8, 2, 64, 32), 2)])
 def test_chains_cut_into_segments(geom, layers):
-    """Chains of as many links as a segment holds, one more and one less, of 32 segments' and of the most that are moved by
-    chains; fewer chains than a block holds, and a last block that is not full; tails that fill the chip with fewer segments."""
+    """Chains of as many links as a segment holds, one more and one less, and of 32 segments'; the longest of a shift of two; fewer
+    chains than a block holds, and a last block that is not full; tails that fill the chip with fewer segments."""
     import torch
     from paper_2608_10402_b200 import tide
     HQ, HKV, D, S = geom
     rng = np.random.default_rng(7 * HQ + D)
     shapes = [(3, 40, 40 * 5), (3, 40, 40 * 5 + 1), (0, 7, 7 * 6 - 1), (1, 2, 2 * 160), (1, 2, 2 * 160 + 1), (15, 33, 33 * 32 + 5), (2, 2, 8192), (2, 2, 8193),
-              (5, 600, 4000), (0, 31, 1), (9, 1000, 6000), (100, 65, 64 * 65)]
+              (5, 600, 4000), (0, 31, 1), (9, 1000, 6000), (100, 65, 64 * 65),
+              # last cuts taken back; a shift of two by runs
+              (3, 64, 64 * 300 + 5), (7, 32, 32 * 520 + 1), (2, 2, 2 * 8192 + 1)]
     length = [sum(x) for x in shapes]
     n, pages = len(shapes), sum((l + S - 1) // S for l in length) + 4
     order = rng.permutation(pages).astype(np.int32)
