@@ -65,6 +65,7 @@ class Both:
                 between(l)
             kv.step_layer(l, dk[l], dv[l], dq[l], 1.0 / math.sqrt(D), out[l], lse[l])
             launches.append(kv.last_plan()["kernel_launches"])
+        self.last = (rows, k, v, q, out, lse)
         if check:
             assert kv.status() == self.tide.OK
             for l in range(LAYERS):
@@ -114,6 +115,13 @@ def test_a_writer_between_two_layers_goes_in_front():
         ok, _ = b.orc.read(l, 2)
         assert np.array_equal(gk[-20:-1], extra["k"][l][:19]) and np.array_equal(gv[-20:-1], extra["v"][l][:19])
         assert np.array_equal(gk[-1], ok[-1] if l else extra["k"][l][19]) and np.array_equal(gk[:-20], ok[:-20])
+    # the layers behind the writer have seen its rows
+    rows, k, v, q, out, lse = b.last
+    b.orc.truncate(2, b.orc.task_len(2) - 20)
+    b.orc.append([2], np.array([0, 20], np.int32), np.concatenate([extra["k"][:, :19], k[:, 2:]], axis=1), np.concatenate([extra["v"][:, :19], v[:, 2:]], axis=1))
+    for l in (1, 2):
+        ref_o, ref_l = cbuild.attend_paged(b.orc.layer(l), rows, q[l], 1.0 / math.sqrt(b.geom[2]))
+        H.check_outputs(H.from_dev(out[l]), lse[l].cpu().numpy(), ref_o, ref_l, f"layer {l}")
     b.kv.close()
 
 
